@@ -177,7 +177,7 @@ struct DeviceWork {       // pointers into the workspace for one run
     int32_t n_units, n_prefill, n_merge, n_dmerge;
     int64_t n_part_slots;              // rows of part_lse / part_o
     const int32_t* prefill_cta_start;  // static prefill partition (n_prefill_ctas + 1 entries), unused when 0
-    int32_t n_prefill_ctas;
+    int32_t n_prefill_ctas;            // entries of that partition: CTAs, or CTA pairs at head dimension 128
 };
 
 struct RunArgs {
@@ -193,6 +193,7 @@ struct RunArgs {
     cudaStream_t stream;
     int num_sms;
     int dec_sms, pf_sms;  // SMs (= CTAs) for the decode and the prefill kernel
+    bool sm_pairs;        // side by side with the pair kernel: the decode kernel's CTAs take whole SM pairs too
     int32_t total_q;      // q tokens of the batch (rows of q and out)
     int32_t n_req;        // requests of the batch (rows of the block table)
     int64_t wait_limit_ns;
@@ -200,6 +201,7 @@ struct RunArgs {
 
 ps_status launch_decode(const RunArgs& a);
 ps_status launch_prefill(const RunArgs& a);
+ps_status launch_prefill_pair(const RunArgs& a);  // head dimension 128
 ps_status launch_merge(const RunArgs& a);
 int decode_warps_per_sm();
 

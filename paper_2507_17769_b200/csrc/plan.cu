@@ -29,14 +29,30 @@ constexpr int kDecodeUnitsPerWarp = 1;  // work units per resident warp (measure
 // partial result for the one warp that combines them (one row of 4096 tokens: 22 us at 32 pieces, 26 at 64).
 constexpr int kDecodeMinPagesLo = 4, kDecodeMinPagesHi = 8, kDecodePiecesPerRow = 16;
 constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
-// Measured on B200 (decode: bandwidth against the number of SMs the kernel runs on; prefill: time of one
-// key-tile step of a q tile pair), used to split the SMs of a mixed batch between the two kernels.
+// Measured on B200 (bandwidth against the number of SMs the decode kernel runs on), used with the prefill kernel's cost
+// model to split the SMs of a mixed batch between the two kernels.
 constexpr double kDecodePeakBytesPerSec = 6.7e12;
 constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a running prefill kernel
 constexpr double kDecodeBytesPerSecPerSm = 115e9;
 constexpr double kDecodeAloneBytesPerSecPerSm = 135e9;  // per SM with the memory system to itself
-constexpr double kPrefillStepSec = 2.5e-6;
 constexpr double kKernelFloorSec = 12e-6;
+
+// Cost model of a prefill kernel in units of one 128-key step of an item (256 rows): an item pays a fixed overhead
+// (pipeline fill, output) plus one unit per key tile.
+struct PrefillModel {
+    double step_sec;      // SM-seconds of a step
+    double fixed;         // steps an item costs beyond its key tiles
+    double masked_extra;  // and the diagonal tile's slower softmax
+    double cut;           // steps that cutting items costs: partial rows, merge kernel
+    int sms_per_worker;   // an item is worked on by one CTA, or by a pair of them
+};
+// head dimension 64 (prefill.cu; fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a
+// masked tile)
+constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 1};
+// head dimension 128 (prefill_pair.cu; 72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of
+// a pair, 2.8 us per item; the merge kernel takes about 8 us)
+constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 2};
+static inline const PrefillModel& prefill_model(const ps_shape& sh) { return sh.head_dim == 128 ? kPairModel : kSingleModel; }
 
 // A chunk of a few tokens runs as that many decode rows (token i of the chunk is a row that sees prior + i + 1 keys
 // of the same sequence) instead of bringing in the prefill kernel for one small item: its launch and pipeline fill
@@ -101,6 +117,7 @@ struct ps_plan {
     // decode kernel (HBM-bound: a fraction of the SMs saturates the memory system) and the prefill kernel
     // (tensor-bound) run side by side on disjoint sets of SMs
     int32_t dec_sms = 0, pf_sms = 0;
+    int32_t pf_workers = 0;  // what prefill items are handed to: CTAs, or CTA pairs (one SM each) at head dimension 128
     bool concurrent = false;
     bool tiny_as_rows = false;  // this batch runs its chunks of a few tokens as decode rows
     std::vector<DecodePiece> pieces;
@@ -243,12 +260,6 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     *n_slots = slots;
 }
 
-// Cost model of the prefill kernel in units of one 128-key tile step: an item pays a fixed
-// overhead (pipeline fill, output) plus one unit per key tile.
-// (fitted to per-CTA run times on B200: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile)
-constexpr double kPrefillFixedCost = 1.5;
-constexpr double kPrefillMaskedExtra = 0.5;  // the diagonal tile of an item takes the slower masked softmax
-constexpr double kPrefillCutCost = 3.0;
 constexpr double kPrefillWholeItemSlack = 1.12;  // uncut items are taken if the busiest CTA stays within this of an even split
 constexpr double kPrefillMinCtaCost = 4.0;  // do not spread the work thinner than this per CTA (two key tiles)
 
@@ -256,6 +267,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                          const ps_plan_opts* opts, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     const int tile_tok = kPrefillRowsPerItem / G;
+    const PrefillModel& cost = prefill_model(pl->shape);
     struct Tile { int r, g, tok0, n_tok, first_pos, key_tiles; };
     std::vector<Tile> tiles;
     size_t n_tiles = 0;
@@ -295,13 +307,13 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 cuts.push_back(Cut{(int)i, kt0});
             }
         }
-    } else if ((int64_t)tiles.size() < 4LL * pl->pf_sms) {
+    } else if ((int64_t)tiles.size() < 4LL * pl->pf_workers) {
         // Few items per SM: give every CTA an equal share of the flattened (item, key tile) cost
         // line, cutting items where a share ends.  Only the cut items need the merge.
         static_partition = true;
         double total = 0;
-        for (const Tile& t : tiles) total += kPrefillFixedCost + t.key_tiles + kPrefillMaskedExtra;
-        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_sms, total / kPrefillMinCtaCost));
+        for (const Tile& t : tiles) total += cost.fixed + t.key_tiles + cost.masked_extra;
+        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_workers, total / kPrefillMinCtaCost));
         // Many short items (fresh prompts): whole items, longest first, each to the CTA with the least work so far.
         // If that comes within kPrefillWholeItemSlack of an even split, nothing is cut: no partial rows, no merge
         // kernel, no item paying its fixed cost twice.
@@ -321,12 +333,12 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 Slot& least = heap.back();
                 owner[i] = least.second;
                 ++count[least.second + 1];
-                least.first += kPrefillFixedCost + tiles[i].key_tiles + kPrefillMaskedExtra;
+                least.first += cost.fixed + tiles[i].key_tiles + cost.masked_extra;
                 makespan = std::max(makespan, least.first);
                 std::push_heap(heap.begin(), heap.end(), std::greater<Slot>());
             }
-            // (cutting is not free either: the merge kernel and the partial rows cost about kPrefillCutCost steps)
-            if (makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + kPrefillCutCost)) {
+            // (cutting is not free either)
+            if (makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.cut)) {
                 for (int c = 0; c < n_cta; ++c) count[c + 1] += count[c];
                 pl->prefill_cta_start.assign(count.begin(), count.end());
                 std::vector<Tile> sorted(tiles.size());
@@ -341,7 +353,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
         // many shares do depends on the quota itself: bisect for the smallest quota that does not leave the
         // last CTA with more than a share.
         int n_items = 0;
-        double q_lo = total / n_cta, q_hi = (total + (n_cta - 1) * kPrefillFixedCost) / n_cta + 0.5;
+        double q_lo = total / n_cta, q_hi = (total + (n_cta - 1) * cost.fixed) / n_cta + 0.5;
         for (int pass = 0; pass < 7; ++pass) {
             const double quota = pass == 6 ? q_hi : 0.5 * (q_lo + q_hi);  // the last pass keeps a quota known to fit
             pl->prefill_cta_start.assign(1, 0);
@@ -358,10 +370,10 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 const int kt = tiles[i].key_tiles;
                 int kt0 = 0;
                 for (;;) {
-                    const double rest = kPrefillFixedCost + (kt - kt0) + kPrefillMaskedExtra;  // the item's remaining tiles as one piece
+                    const double rest = cost.fixed + (kt - kt0) + cost.masked_extra;  // the item's remaining tiles as one piece
                     const double room = (cta + 1) * quota - cum;
                     const bool cta_has_work = pl->prefill_cta_start.back() < n_items;
-                    const double fit = room - kPrefillFixedCost;
+                    const double fit = room - cost.fixed;
                     const int take = fit < 0.5 ? 0 : (int)(fit + 0.5);  // key tiles that fit, to the nearest
                     if (cta == n_cta - 1 || rest <= room + 0.5 || take >= kt - kt0 || (take < 1 && !cta_has_work)) {
                         cum += rest;
@@ -371,7 +383,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                     if (take >= 1) {
                         kt0 += take;
                         cuts.push_back(Cut{(int)i, kt0});
-                        cum += kPrefillFixedCost + take;
+                        cum += cost.fixed + take;
                         ++n_items;
                     }
                     close_cta();  // (with take < 1: no room left for even one key tile; the item starts in the next CTA)
@@ -501,6 +513,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     {
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
         const int G = shape->n_q_heads / shape->n_kv_heads;
+        const PrefillModel& cost = prefill_model(*shape);
         const int tile_tok = kPrefillRowsPerItem / G;
         for (int r = 0; r < n; ++r) {
             if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) {
@@ -509,7 +522,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             } else {
                 for (int t0 = 0; t0 < q_len_host[r]; t0 += tile_tok) {
                     const int n_tok = std::min(tile_tok, q_len_host[r] - t0);
-                    pf_steps += (kPrefillFixedCost + (prior_host[r] + t0 + n_tok + kPrefillKeyTile - 1) / kPrefillKeyTile) * shape->n_kv_heads;
+                    pf_steps += (cost.fixed + (prior_host[r] + t0 + n_tok + kPrefillKeyTile - 1) / kPrefillKeyTile) * shape->n_kv_heads;
                 }
             }
         }
@@ -518,7 +531,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         if (dec_bytes > 0 && pf_steps > 0 && pl->num_sms >= 16) {
             // time models (seconds): decode = bytes / min(side-by-side peak, n * per-SM rate); prefill = steps * step time / m
             auto t_dec = [&](int nd) { return dec_bytes / std::min(kDecodeSharedPeakBytesPerSec, nd * kDecodeBytesPerSecPerSm) + kKernelFloorSec; };
-            auto t_pf = [&](int nd) { return pf_steps * kPrefillStepSec / (pl->num_sms - nd) + kKernelFloorSec; };
+            auto t_pf = [&](int nd) { return pf_steps * cost.step_sec / (pl->num_sms - nd) + kKernelFloorSec; };
             int best_n = 0;
             double best_t = 1e30;
             for (int nd = 8; nd <= pl->num_sms - 8; nd += 4) {
@@ -535,12 +548,12 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             for (int nd = best_n; nd <= pl->num_sms - 8; nd += 4)
                 if (std::max(t_dec(nd), t_pf(nd)) <= 1.015 * best_t && t_pf(nd) <= 0.8 * t_dec(nd)) hi = nd;
             best_n = (best_n + hi) / 2 / 4 * 4;
-            const double t_seq = dec_bytes / kDecodePeakBytesPerSec + pf_steps * kPrefillStepSec / pl->num_sms + 2 * kKernelFloorSec;
+            const double t_seq = dec_bytes / kDecodePeakBytesPerSec + pf_steps * cost.step_sec / pl->num_sms + 2 * kKernelFloorSec;
             // The decode rows pay the shared rate only while the prefill kernel runs; once it has ended they stream
             // at the rate their CTAs reach alone.  A short chunk beside many decode rows is therefore cheaper than
             // the model above says, which matters for the choice against running the two one after the other.
             if (best_n > 0) {
-                const double pf_work = pf_steps * kPrefillStepSec / (pl->num_sms - best_n);
+                const double pf_work = pf_steps * cost.step_sec / (pl->num_sms - best_n);
                 const double shared = std::min(kDecodeSharedPeakBytesPerSec, best_n * kDecodeBytesPerSecPerSm);
                 const double alone = std::min(kDecodePeakBytesPerSec, best_n * kDecodeAloneBytesPerSecPerSm);
                 const double dec_work = dec_bytes <= shared * pf_work ? dec_bytes / shared : pf_work + (dec_bytes - shared * pf_work) / alone;
@@ -553,6 +566,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
         }
     }
+    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(*shape).sms_per_worker);
     int64_t n_slots = 0;
     plan_decode(pl, prior_host, q_len_host, q_start, opts, &n_slots);
     plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);
@@ -638,7 +652,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     pl->info.total_q_tokens = T;
     pl->info.decode_sms = pl->dec_sms;
     pl->info.prefill_sms = pl->pf_sms;
-    pl->info.n_launches = (pl->concurrent && !pl->units.empty() && pl->prefill_cta_start.empty() && (int)pl->prefill.size() > pl->pf_sms ? 1 : 0) + (pl->units.empty() ? 0 : 1) + (pl->prefill.empty() ? 0 : 1) + (pl->merge.empty() ? 0 : 1);
+    pl->info.n_launches = (pl->concurrent && !pl->units.empty() && pl->prefill_cta_start.empty() && (int)pl->prefill.size() > pl->pf_workers ? 1 : 0) + (pl->units.empty() ? 0 : 1) + (pl->prefill.empty() ? 0 : 1) + (pl->merge.empty() ? 0 : 1);
     *plan_inout = pl;
     *workspace_bytes_out = pl->ws_bytes;
     return PS_OK;
@@ -806,13 +820,14 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
         // fails below, it is joined back into the caller's stream before the call returns.
         if (rec) cudaEventRecord(ev[2], side);
         RunArgs ad = a;
+        ad.sm_pairs = pl->pf_workers < pl->pf_sms;
         ad.stream = side;
         st = launch_decode(ad);
         if (rec && st == PS_OK) cudaEventRecord(ev[3], side);
         if (rec && st == PS_OK) cudaEventRecord(ev[0], s);
         if (st == PS_OK) st = launch_prefill(a);
         if (rec && st == PS_OK) cudaEventRecord(ev[1], s);
-        const bool helpers = a.w.n_prefill_ctas == 0 && a.w.n_prefill > a.pf_sms;
+        const bool helpers = a.w.n_prefill_ctas == 0 && a.w.n_prefill > pl->pf_workers;
         if (st == PS_OK && !helpers) {
             // Only this launch writes prefill partials: combine them right behind it, on the SMs it leaves, while
             // the decode kernel is still streaming (decode rows are combined inside the decode kernel).

@@ -1,4 +1,4 @@
-// Prefill-chunk attention on the 5th-generation tensor cores.
+// Prefill-chunk attention on the 5th-generation tensor cores, for head dimension 64 (128: prefill_pair.cu).
 //
 // A chunk's rows attend the prior context plus the chunk's own earlier tokens
 // (paper sections 2.4 and 4.7); this part is a dense contraction and compute
@@ -33,9 +33,7 @@
 //
 // TMEM columns: S_A 0..127, S_B 128..255, O_A 256.., O_B 384.. (512 allocated).
 // Every wait is bounded; on expiry the CTA sets the timeout status and drains.
-#include <cuda.h>
-
-#include "common.cuh"
+#include "tcgen05.cuh"
 
 namespace ps {
 
@@ -51,117 +49,6 @@ constexpr int kProducerWarp = 8, kMmaWarp = 9;
 constexpr int kTileKeys = 128;
 constexpr int kRows = 128;
 constexpr float kRescaleThreshold = 8.f;  // log2 units
-// ---- tcgen05 wrappers -------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// One leader lane of a converged warp (always the same one for the full mask).  Issuing the MMAs under this
-// predicate, rather than under a test of the lane index, keeps the descriptor arithmetic warp-uniform.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}" : "=r"(pred));
-    return pred != 0;
-}
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-// D[tmem] (+)= A[smem desc] * B[smem desc]
-__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
-        "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-          "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
-          "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
-          "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-        : "memory");
-}
-// 3-input max and packed fp32 pairs (two lanes per 64-bit register)
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-// One box of a 3-d tensor map into shared memory; completion is counted in bytes on `bar`.
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// Shared-memory matrix descriptor, 128-byte swizzle, 8-row atoms of 1024 bytes.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version for this architecture
-    d |= (uint64_t)2 << 61;  // SWIZZLE_128B
-    return d;
-}
-// Instruction descriptor: bf16 x bf16 -> fp32, M = 128.
-__host__ __device__ constexpr uint32_t instr_desc(int n, bool b_mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
-           ((uint32_t)(kRows >> 4) << 24);
-}
-
 constexpr int kBarBlockBytes = 512;  // mbarriers, flags and the item record ring
 
 template <int D>
@@ -220,28 +107,6 @@ static_assert(Bars::mma_drained % 8 == 0 && Bars::armed + 24 <= Bars::ring && si
                   Bars::bytes <= kBarBlockBytes,
               "barrier block layout");
 
-// Wait for a phase for at most about the CTA's wait limit (nanoseconds, in the word behind the abort flag; the low
-// half of the nanosecond clock serves, so limits reach 4 s); gives up early when another role of the CTA has already
-// given up.  The role whose wait runs out raises the CTA's abort flag.  One non-blocking probe first; a limit of
-// zero gives up right after it.  The clock is read only every kWaitPollsPerClockRead failed polls.
-__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    if (mbar_test_wait(bar, parity)) return true;
-    const uint32_t limit_ns = (uint32_t)abort_flag[1];  // the wait limit sits behind the abort flag
-    if (limit_ns > 0) {
-        uint32_t t0 = 0;
-        for (uint32_t i = 1;; ++i) {
-            if (mbar_try_wait(bar, parity)) return true;
-            if ((i & (kWaitPollsPerClockRead - 1)) == 0) {
-                if (*abort_flag) return false;
-                const uint32_t now = global_timer_lo() | 1u;
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > limit_ns) break;
-            }
-        }
-    }
-    *abort_flag = 1;
-    return false;
-}
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map) {
     using Cfg = PrefillCfg<D>;
@@ -296,8 +161,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
     // and the mbarriers, so the next item's Q, K and first QK^T overlap the current item's last
     // softmax, PV and output.  Every role counts items and key tiles identically to derive barrier
     // phases; tile B's barriers only move in items that have a second q tile.
-    constexpr uint32_t kIdescQK = instr_desc(kTileKeys, false);
-    constexpr uint32_t kIdescPV = instr_desc(D, true);
+    constexpr uint32_t kIdescQK = instr_desc(kRows, kTileKeys, false);
+    constexpr uint32_t kIdescPV = instr_desc(kRows, D, true);
     static_assert(kPrefillRowsPerItem == 2 * kRows, "the planner pairs two q tiles per item");
     const int tile_tok = kRows / p.G;
     const int g_shift = 31 - __clz(p.G);  // G is a power of two
@@ -815,27 +680,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
 
 }  // namespace
 
-namespace {
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up through the runtime so that the library does not link libcuda.
-EncodeTiledFn tensor_map_encoder() {
-    static EncodeTiledFn fn = [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            f = nullptr;
-        return (EncodeTiledFn)f;
-    }();
-    return fn;
-}
-
-}  // namespace
-
 template <int D>
 static ps_status launch_prefill_d(const RunArgs& a) {
     using Cfg = PrefillCfg<D>;
@@ -866,18 +710,9 @@ static ps_status launch_prefill_d(const RunArgs& a) {
     p.n_part_slots = (int32_t)a.w.n_part_slots;
     p.wait_limit_ns = (uint32_t)a.wait_limit_ns;
 
-    // Q as a [T tokens][Hq heads][D] tensor; a box is one 64-element half of a q tile's 128 rows
-    EncodeTiledFn encode = tensor_map_encoder();
-    if (!encode) return fail(PS_ERR_CUDA, "the driver does not provide cuTensorMapEncodeTiled");
     CUtensorMap q_map;
-    const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)p.Hq, (cuuint64_t)a.total_q};
-    const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)p.Hq * D * 2};
-    const cuuint32_t box[3] = {64, (cuuint32_t)p.G, (cuuint32_t)(kRows / p.G)};
-    const cuuint32_t elem_strides[3] = {1, 1, 1};
-    const CUresult r = encode(&q_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(a.q), dims, strides, box,
-                              elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(PS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
+    const ps_status enc = encode_q_map(a, &q_map);
+    if (enc != PS_OK) return enc;
 
     const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
     prefill_kernel<D><<<grid, kThreads, Cfg::kSmemBytes, a.stream>>>(p, q_map);
@@ -887,7 +722,7 @@ static ps_status launch_prefill_d(const RunArgs& a) {
 
 ps_status launch_prefill(const RunArgs& a) {
     if (a.w.n_prefill == 0) return PS_OK;
-    return a.shape.head_dim == 128 ? launch_prefill_d<128>(a) : launch_prefill_d<64>(a);
+    return a.shape.head_dim == 128 ? launch_prefill_pair(a) : launch_prefill_d<64>(a);
 }
 
 }  // namespace ps

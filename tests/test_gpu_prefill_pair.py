@@ -1,0 +1,73 @@
+"""The CTA-pair prefill kernel (head dimension 128) where its own branches can go wrong: items of one to seven key tiles
+(its score buffers, the groups that begin an item and the stages wrap at three, three and four), ragged ends, several items
+per pair, and rows whose softmax sums leave the range in which weights are taken without their row maximum, which are
+computed again relative to it."""
+import numpy as np
+import pytest
+
+import oracle
+from workloads import gen
+
+from parity_util import compare, kv_bits, q_bits
+
+pytestmark = pytest.mark.gpu
+
+
+def scaled(bits, exps):
+    """bf16 bit patterns [T, H, d] times 2 ** exps[token]: exact, the exponent field moves."""
+    f = (bits.astype(np.uint32) << 16).view(np.float32) * (2.0 ** np.asarray(exps, dtype=np.float32))[:, None, None]
+    return (f.astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
+
+
+def run_and_compare(batch, exps, what):
+    import torch
+    from workloads.device import DeviceBatch
+
+    s = batch.shape
+    db = DeviceBatch(batch)
+    q = np.concatenate([q_bits(batch, r) for r in range(batch.n)])
+    q = scaled(q, exps)
+    db.q = torch.from_numpy(q.view(np.int16)).cuda().view(torch.bfloat16)
+    info = db.plan()
+    assert info.n_prefill_items > 0
+    out, lse = db.run()
+    db.pa.check()
+    ks, vs = zip(*[kv_bits(batch, r) for r in range(batch.n)])
+    kp = oracle.plain_pool(ks, batch.block_table, batch.num_pages, s.page_size)
+    vp = oracle.plain_pool(vs, batch.block_table, batch.num_pages, s.page_size)
+    rr = [r for r in range(batch.n) for _ in range(int(batch.q_len[r]))]
+    rt = [i for r in range(batch.n) for i in range(int(batch.q_len[r]))]
+    want, want_lse = oracle.attn_rows(q, kp, vp, batch.block_table, batch.prior, batch.q_len, s.n_q_heads, s.n_kv_heads, s.head_dim,
+                                      s.page_size, rr, rt)
+    keys = np.array([int(batch.prior[r]) + i + 1 for r, i in zip(rr, rt)])
+    # Large scores make rows see a few keys in effect, however many they have: the outputs are single V values, bf16-rounded
+    # (compare() scales its bound for such rows by the value).  lse: fp32 arithmetic on scores of up to 2^e times the plain
+    # ones, whose products and sums over d = 128 are each good to a few units of 2^-24.
+    peaked = np.asarray(exps) > 1
+    compare(out, None, want, want_lse, what=what, few_key_rows=True, keys=np.where(peaked, 1, keys))
+    err = np.abs(lse.cpu().numpy().astype(np.float64) - want_lse)
+    assert (err <= 2e-3 + 1e-5 * np.abs(want_lse)).all(), "%s: lse off by %.3e" % (what, err.max())
+    again, lse2 = db.run()
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16)) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("shape", [gen.SHAPE_8B, gen.SHAPE_LARGE, gen.Shape(16, 8, 128)])
+@pytest.mark.parametrize("prior", [0, 1, 100, 127, 128, 250, 384, 511, 640, 777])
+def test_items_of_one_to_seven_key_tiles(shape, prior):
+    b = gen.make_batch(shape, 900 + prior, [prior, prior + 60], [40, 21])
+    run_and_compare(b, np.zeros(b.total_q), "prior %d" % prior)
+
+
+def test_many_short_items_per_pair():
+    b = gen.make_batch(gen.SHAPE_8B, 950, [0] * 12, [500, 40, 33, 260, 130, 129, 128, 127, 65, 64, 63, 300])
+    run_and_compare(b, np.zeros(b.total_q), "many short items")
+
+
+@pytest.mark.parametrize("every", [1, 3, 97])
+@pytest.mark.parametrize("exp", [6, 9])
+def test_rows_out_of_range_are_computed_again(every, exp):
+    """Q times 2^6 gives scores of hundreds (weights overflow and underflow without the row maximum), 2^9 of thousands;
+    ``every``: which tokens are scaled (all, a third, a few), so that items mix such rows with ordinary ones."""
+    b = gen.make_batch(gen.SHAPE_8B, 960 + exp, [300, 0, 129], [130, 200, 70])
+    exps = np.where(np.arange(b.total_q) % every == 0, exp, 0)
+    run_and_compare(b, exps, "exp %d every %d" % (exp, every))
