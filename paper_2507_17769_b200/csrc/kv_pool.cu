@@ -37,28 +37,50 @@ ps_status check_shape(const ps_shape* s) {
     return PS_OK;
 }
 
+// Where the new tokens go: request r's are packed tokens q_start[r] .. q_start[r + 1] and follow prior[r] cached ones.  The
+// lengths travel as a kernel parameter: copied to the device first they cost every append a small transfer that its stream
+// has to wait for (about 6 us between two kernels, and 4 us of host time).  Batches of more than kParamRowsMax requests
+// still take that way.
+template <int N>
+struct ParamRows {
+    int32_t q_start_[N + 1], prior_[N];
+    __device__ __forceinline__ int q_start(int r) const { return q_start_[r]; }
+    __device__ __forceinline__ int prior(int r) const { return prior_[r]; }
+};
+struct DeviceRows {
+    const int32_t *q_start_, *prior_;
+    __device__ __forceinline__ int q_start(int r) const { return q_start_[r]; }
+    __device__ __forceinline__ int prior(int r) const { return prior_[r]; }
+};
+constexpr int kParamRowsMax = 4000;  // 32 KB, as much as a kernel's parameters may be
+
+// request of packed token t: last r with q_start(r) <= t
+template <class Rows>
+__device__ __forceinline__ int request_of(const Rows& rows, int n, int t) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (rows.q_start(mid) <= t) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
 // One thread moves one 16-byte unit of K and of V.
 // grid.x covers T * Hkv * (d / 8) units.
+template <class Rows>
 __global__ void kv_write_kernel(char* pool, int64_t num_pages, const uint4* __restrict__ k_new,
                                 const uint4* __restrict__ v_new, const int32_t* __restrict__ block_table,
-                                int max_pages, const int32_t* __restrict__ q_start, const int32_t* __restrict__ prior,
-                                int n, int Hkv, int d, int* flag) {
+                                int max_pages, const __grid_constant__ Rows rows, int n, int Hkv, int d, int* flag) {
     const int units_per_tok = Hkv * (d >> 3);
-    const int64_t total = (int64_t)q_start[n] * units_per_tok;
+    const int64_t total = (int64_t)rows.q_start(n) * units_per_tok;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int t = (int)(idx / units_per_tok);
         const int rem = (int)(idx % units_per_tok);
         const int g = rem / (d >> 3);
         const int u = rem % (d >> 3);
-        // request of packed token t: last r with q_start[r] <= t
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (q_start[mid] <= t) lo = mid; else hi = mid - 1;
-        }
-        const int r = lo;
-        const int pos = prior[r] + (t - q_start[r]);
+        const int r = request_of(rows, n, t);
+        const int pos = rows.prior(r) + (t - rows.q_start(r));
         const int64_t page = block_table[(int64_t)r * max_pages + pos / kPage];
         if (page < 0 || page >= num_pages) { atomicOr(flag, kStatusBounds); continue; }
         const int slot = pos % kPage;
@@ -103,23 +125,18 @@ __device__ __forceinline__ uint32_t quantise4(float x0, float x1, float x2, floa
 }
 
 // One warp quantises K and V of one (new token, kv head): lane l holds elements 4 l .. 4 l + 3 (head_dim = 128).
+template <class Rows>
 __global__ void kv_write_fp8_kernel(char* pool, int64_t num_pages, const uint2* __restrict__ k_new,
                                     const uint2* __restrict__ v_new, const int32_t* __restrict__ block_table, int max_pages,
-                                    const int32_t* __restrict__ q_start, const int32_t* __restrict__ prior, int n, int Hkv,
-                                    int* flag) {
+                                    const __grid_constant__ Rows rows, int n, int Hkv, int* flag) {
     constexpr int d = 128;
     const int lane = threadIdx.x & 31;
-    const int64_t total = (int64_t)q_start[n] * Hkv;
+    const int64_t total = (int64_t)rows.q_start(n) * Hkv;
     for (int64_t vec = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); vec < total;
          vec += (int64_t)gridDim.x * (blockDim.x >> 5)) {
         const int t = (int)(vec / Hkv), g = (int)(vec % Hkv);
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (q_start[mid] <= t) lo = mid; else hi = mid - 1;
-        }
-        const int r = lo;
-        const int pos = prior[r] + (t - q_start[r]);
+        const int r = request_of(rows, n, t);
+        const int pos = rows.prior(r) + (t - rows.q_start(r));
         const int64_t page = block_table[(int64_t)r * max_pages + pos / kPage];
         if (page < 0 || page >= num_pages) {
             if (lane == 0) atomicOr(flag, kStatusBounds);
@@ -176,6 +193,56 @@ using namespace ps;
 struct ps_kv {
     KvPool p;
 };
+
+namespace {
+
+struct KvWrite {
+    const void *k_new, *v_new;
+    const int32_t* block_table;
+    int32_t max_pages;
+    const int32_t *prior, *q_len;
+    int32_t n;
+    int64_t T;
+    cudaStream_t stream;
+};
+
+void fill_rows(const KvWrite& w, int32_t* q_start, int32_t* prior) {
+    int32_t t = 0;
+    for (int r = 0; r < w.n; ++r) {
+        q_start[r] = t;
+        t += w.q_len[r];
+        prior[r] = w.prior[r];
+    }
+    q_start[w.n] = t;
+}
+
+template <class Rows>
+ps_status launch_write(const KvPool& p, const KvWrite& w, const Rows& rows) {
+    const int Hkv = p.shape.n_kv_heads, d = p.shape.head_dim;
+    if (p.shape.dtype == 1) {
+        const int64_t warps = w.T * Hkv;
+        const int blocks = (int)((warps + 7) / 8 < 148 * 16 ? (warps + 7) / 8 : 148 * 16);
+        kv_write_fp8_kernel<<<blocks, 256, 0, w.stream>>>(p.base, p.num_pages, (const uint2*)w.k_new, (const uint2*)w.v_new, w.block_table,
+                                                          w.max_pages, rows, w.n, Hkv, p.flag_dev);
+    } else {
+        const int64_t total = w.T * Hkv * (d / 8);
+        const int threads = 256;
+        const int blocks = (int)((total + threads - 1) / threads < 148 * 32 ? (total + threads - 1) / threads : 148 * 32);
+        kv_write_kernel<<<blocks, threads, 0, w.stream>>>(p.base, p.num_pages, (const uint4*)w.k_new, (const uint4*)w.v_new, w.block_table,
+                                                          w.max_pages, rows, w.n, Hkv, d, p.flag_dev);
+    }
+    PS_CUDA_TRY(cudaGetLastError());
+    return PS_OK;
+}
+
+template <int N>
+ps_status write_with_params(const KvPool& p, const KvWrite& w) {
+    ParamRows<N> rows;  // (entries past n are not read)
+    fill_rows(w, rows.q_start_, rows.prior_);
+    return launch_write(p, w, rows);
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -248,41 +315,25 @@ ps_status ps_kv_write(ps_kv* kv, const void* k_new_dev, const void* v_new_dev, c
         return fail(PS_ERR_INVALID, "null argument");
     if (n < 1 || max_pages < 1) return fail(PS_ERR_INVALID, "n=%d, max_pages=%d must be positive", n, max_pages);
     if (2 * (int64_t)n + 1 > kv->p.meta_cap) return fail(PS_ERR_INVALID, "n=%d exceeds %d requests per call", n, (kv->p.meta_cap - 1) / 2);
-    std::vector<int32_t> meta(2 * (size_t)n + 1);
     int64_t T = 0;
     for (int r = 0; r < n; ++r) {
         if (q_len_host[r] < 1 || prior_host[r] < 0)
             return fail(PS_ERR_INVALID, "request %d: q_len=%d prior=%d", r, q_len_host[r], prior_host[r]);
         if ((int64_t)prior_host[r] + q_len_host[r] > (int64_t)max_pages * kPage)
             return fail(PS_ERR_INVALID, "request %d: kv_len exceeds max_pages * page_size", r);
-        meta[r] = (int32_t)T;
         T += q_len_host[r];
         if (T > 0x7fffffffLL / 64) return fail(PS_ERR_INVALID, "too many new tokens");
-        meta[n + 1 + r] = prior_host[r];
     }
-    meta[n] = (int32_t)T;
-    cudaStream_t s = (cudaStream_t)stream;
+    const KvWrite w{k_new_dev, v_new_dev, block_table_dev, max_pages, prior_host, q_len_host, n, T, (cudaStream_t)stream};
+    if (n <= 64) return write_with_params<64>(kv->p, w);
+    if (n <= 512) return write_with_params<512>(kv->p, w);
+    if (n <= kParamRowsMax) return write_with_params<kParamRowsMax>(kv->p, w);
+    std::vector<int32_t> meta(2 * (size_t)n + 1);
+    fill_rows(w, meta.data(), meta.data() + n + 1);
     // pageable source: the runtime has staged the bytes when the call returns; calls on one
     // pool must be stream-ordered because they share meta_dev
-    PS_CUDA_TRY(cudaMemcpyAsync(kv->p.meta_dev, meta.data(), meta.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    const int Hkv = kv->p.shape.n_kv_heads, d = kv->p.shape.head_dim;
-    if (kv->p.shape.dtype == 1) {
-        const int64_t warps = T * Hkv;
-        const int blocks = (int)((warps + 7) / 8 < 148 * 16 ? (warps + 7) / 8 : 148 * 16);
-        kv_write_fp8_kernel<<<blocks, 256, 0, s>>>(kv->p.base, kv->p.num_pages, (const uint2*)k_new_dev, (const uint2*)v_new_dev,
-                                                   block_table_dev, max_pages, kv->p.meta_dev, kv->p.meta_dev + n + 1, n, Hkv,
-                                                   kv->p.flag_dev);
-        PS_CUDA_TRY(cudaGetLastError());
-        return PS_OK;
-    }
-    const int64_t total = T * Hkv * (d / 8);
-    const int threads = 256;
-    const int blocks = (int)((total + threads - 1) / threads < 148 * 32 ? (total + threads - 1) / threads : 148 * 32);
-    kv_write_kernel<<<blocks, threads, 0, s>>>(kv->p.base, kv->p.num_pages, (const uint4*)k_new_dev,
-                                               (const uint4*)v_new_dev, block_table_dev, max_pages, kv->p.meta_dev,
-                                               kv->p.meta_dev + n + 1, n, Hkv, d, kv->p.flag_dev);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    PS_CUDA_TRY(cudaMemcpyAsync(kv->p.meta_dev, meta.data(), meta.size() * sizeof(int32_t), cudaMemcpyHostToDevice, w.stream));
+    return launch_write(kv->p, w, DeviceRows{kv->p.meta_dev, kv->p.meta_dev + n + 1});
 }
 
 ps_status ps_kv_gather(const ps_kv* kv, const int32_t* block_table_row_dev, int32_t len, void* k_out_dev,
