@@ -87,11 +87,11 @@ def load() -> ctypes.CDLL:
     lib.ps_kv_bytes.argtypes = [sp, _i64, ctypes.POINTER(_sz)]
     lib.ps_kv_alloc.argtypes = [sp, _i64, _vp, _sz, ctypes.POINTER(_vp)]
     lib.ps_kv_free.argtypes = [_vp]
-    lib.ps_kv_write.argtypes = [_vp, _vp, _vp, _vp, _i32, _i32p, _i32p, _i32, _vp]
+    lib.ps_kv_write.argtypes = [_vp, _vp, _vp, _vp, _i32, _vp, _vp, _i32, _vp]
     lib.ps_kv_gather.argtypes = [_vp, _vp, _i32, _vp, _vp, _vp]
     lib.ps_kv_gather_fp8.argtypes = [_vp, _vp, _i32, _vp, _vp, _vp, _vp, _vp]
     lib.ps_kv_status.argtypes = [_vp, _vp]
-    lib.ps_attn_plan.argtypes = [sp, _i32p, _i32p, _i32, _i32, ctypes.POINTER(ps_plan_opts), ctypes.POINTER(_vp),
+    lib.ps_attn_plan.argtypes = [sp, _vp, _vp, _i32, _i32, ctypes.POINTER(ps_plan_opts), ctypes.POINTER(_vp),
                                  ctypes.POINTER(_sz)]
     lib.ps_plan_free.argtypes = [_vp]
     lib.ps_plan_get_info.argtypes = [_vp, ctypes.POINTER(ps_plan_info)]
@@ -121,8 +121,8 @@ def _check(status: int):
 
 
 def _ptr(x):
-    if x is None:
-        return None
+    if x is None or type(x) is int:
+        return x
     if hasattr(x, "data_ptr"):
         return x.data_ptr()
     return int(x)
@@ -131,6 +131,17 @@ def _ptr(x):
 def _host_i32(a):
     arr = np.ascontiguousarray(a, dtype=np.int32)
     return arr, arr.ctypes.data_as(_i32p)
+
+
+_I32 = np.dtype(np.int32)
+
+
+def _host_i32_address(a):
+    """Like _host_i32 with the address as a plain integer, for arguments declared ``void *``: a typed ctypes pointer takes
+    2 us to make, and the calls of every iteration take two arrays each."""
+    if type(a) is not np.ndarray or a.dtype is not _I32 or not a.flags.c_contiguous:
+        a = np.ascontiguousarray(a, dtype=_I32)
+    return a, a.__array_interface__["data"][0]
 
 
 def make_shape(n_q_heads, n_kv_heads, head_dim, page_size=16, dtype=0) -> ps_shape:
@@ -163,8 +174,8 @@ def ps_kv_free(kv):
 
 
 def ps_kv_write(kv, k_new_dev, v_new_dev, block_table_dev, max_pages, prior_host, q_len_host, stream=None):
-    pr, prp = _host_i32(prior_host)
-    ql, qlp = _host_i32(q_len_host)
+    pr, prp = _host_i32_address(prior_host)
+    ql, qlp = _host_i32_address(q_len_host)
     _check(load().ps_kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, prp, qlp,
                               pr.shape[0], _ptr(stream)))
 
@@ -184,8 +195,8 @@ def ps_kv_status(kv, stream=None):
 
 def ps_attn_plan(shape: ps_shape, prior_host, q_len_host, max_pages_per_seq, opts: ps_plan_opts | None = None, plan=None):
     """Returns (plan handle, workspace bytes).  Pass ``plan`` to rebuild an existing handle in place."""
-    pr, prp = _host_i32(prior_host)
-    ql, qlp = _host_i32(q_len_host)
+    pr, prp = _host_i32_address(prior_host)
+    ql, qlp = _host_i32_address(q_len_host)
     handle = _vp(plan or 0)
     ws = _sz(0)
     _check(load().ps_attn_plan(ctypes.byref(shape), prp, qlp, pr.shape[0], max_pages_per_seq,
