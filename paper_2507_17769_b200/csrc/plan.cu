@@ -33,8 +33,10 @@ constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 // model to split the SMs of a mixed batch between the two kernels.
 constexpr double kDecodePeakBytesPerSec = 6.7e12;
 constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a running prefill kernel
-constexpr double kDecodeBytesPerSecPerSm = 115e9;
-constexpr double kDecodeAloneBytesPerSecPerSm = 135e9;  // per SM with the memory system to itself
+// Per SM with the memory system to itself, and 0.85 of it beside a prefill kernel: 16 to 48 SMs stream 130 GB/s each at head
+// dimension 128, 80 GB/s at 64, where a page is half as large and takes a warp as long.
+static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 80e9; }
+static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;
 
 // Cost model of a prefill kernel in units of one 128-key step of an item (256 rows): an item pays a fixed overhead
@@ -511,6 +513,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     }
     // ---- split the SMs between the two kernels of a mixed batch ----
     {
+        double longest = 0;                  // steps of the longest prefill item
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
         const int G = shape->n_q_heads / shape->n_kv_heads;
         const PrefillModel& cost = prefill_model(*shape);
@@ -522,7 +525,9 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             } else {
                 for (int t0 = 0; t0 < q_len_host[r]; t0 += tile_tok) {
                     const int n_tok = std::min(tile_tok, q_len_host[r] - t0);
-                    pf_steps += (cost.fixed + (prior_host[r] + t0 + n_tok + kPrefillKeyTile - 1) / kPrefillKeyTile) * shape->n_kv_heads;
+                    const double steps = cost.fixed + (prior_host[r] + t0 + n_tok + kPrefillKeyTile - 1) / kPrefillKeyTile;
+                    pf_steps += steps * shape->n_kv_heads;
+                    longest = std::max(longest, steps);
                 }
             }
         }
@@ -530,8 +535,14 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         pl->concurrent = false;
         if (dec_bytes > 0 && pf_steps > 0 && pl->num_sms >= 16) {
             // time models (seconds): decode = bytes / min(side-by-side peak, n * per-SM rate); prefill = steps * step time / m
-            auto t_dec = [&](int nd) { return dec_bytes / std::min(kDecodeSharedPeakBytesPerSec, nd * kDecodeBytesPerSecPerSm) + kKernelFloorSec; };
-            auto t_pf = [&](int nd) { return pf_steps * cost.step_sec / (pl->num_sms - nd) + kKernelFloorSec; };
+            auto t_dec = [&](int nd) { return dec_bytes / std::min(kDecodeSharedPeakBytesPerSec, nd * decode_rate_per_sm(*shape)) + kKernelFloorSec; };
+            // Whole items leave some workers idle at the end (about 0.4 of the longest item on average) and take at least the
+            // longest one; cutting them costs cost.cut steps instead.
+            auto pf_time = [&](int sms) {
+                const double even = pf_steps * cost.step_sec / sms, worker_step = cost.step_sec / cost.sms_per_worker;
+                return std::min(std::max(even + 0.4 * longest * worker_step, longest * worker_step), even + cost.cut * worker_step);
+            };
+            auto t_pf = [&](int nd) { return pf_time(pl->num_sms - nd) + kKernelFloorSec; };
             int best_n = 0;
             double best_t = 1e30;
             for (int nd = 8; nd <= pl->num_sms - 8; nd += 4) {
@@ -548,14 +559,14 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             for (int nd = best_n; nd <= pl->num_sms - 8; nd += 4)
                 if (std::max(t_dec(nd), t_pf(nd)) <= 1.015 * best_t && t_pf(nd) <= 0.8 * t_dec(nd)) hi = nd;
             best_n = (best_n + hi) / 2 / 4 * 4;
-            const double t_seq = dec_bytes / kDecodePeakBytesPerSec + pf_steps * cost.step_sec / pl->num_sms + 2 * kKernelFloorSec;
+            const double t_seq = dec_bytes / kDecodePeakBytesPerSec + pf_time(pl->num_sms) + 2 * kKernelFloorSec;
             // The decode rows pay the shared rate only while the prefill kernel runs; once it has ended they stream
             // at the rate their CTAs reach alone.  A short chunk beside many decode rows is therefore cheaper than
             // the model above says, which matters for the choice against running the two one after the other.
             if (best_n > 0) {
-                const double pf_work = pf_steps * cost.step_sec / (pl->num_sms - best_n);
-                const double shared = std::min(kDecodeSharedPeakBytesPerSec, best_n * kDecodeBytesPerSecPerSm);
-                const double alone = std::min(kDecodePeakBytesPerSec, best_n * kDecodeAloneBytesPerSecPerSm);
+                const double pf_work = pf_time(pl->num_sms - best_n);
+                const double shared = std::min(kDecodeSharedPeakBytesPerSec, best_n * decode_rate_per_sm(*shape));
+                const double alone = std::min(kDecodePeakBytesPerSec, best_n * decode_alone_rate_per_sm(*shape));
                 const double dec_work = dec_bytes <= shared * pf_work ? dec_bytes / shared : pf_work + (dec_bytes - shared * pf_work) / alone;
                 best_t = std::min(best_t, std::max(pf_work, dec_work) + kKernelFloorSec);
             }
