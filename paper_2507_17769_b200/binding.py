@@ -1,4 +1,5 @@
-"""ctypes binding of ``libpolyserve_attn.so`` -- argument marshalling only.
+"""Binding of ``libpolyserve_attn.so`` -- argument marshalling only (ctypes; the calls of every iteration through the
+extension module ``_pycalls``).
 
 Every function has the name and argument order of its C declaration in
 ``include/polyserve_attn.h``; all arithmetic runs in the CUDA kernels behind
@@ -70,13 +71,14 @@ EXPORTS = ["ps_kv_bytes", "ps_kv_alloc", "ps_kv_free", "ps_kv_write", "ps_kv_gat
            "ps_last_error", "ps_version"]
 
 _lib = None
+_calls = None  # the extension module of the calls of every iteration
 _vp, _i32, _i64, _sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t
 _i32p = ctypes.POINTER(ctypes.c_int32)
 
 
 def load() -> ctypes.CDLL:
     """Load (building first if the sources are newer) the shared library."""
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     path = LIB
@@ -111,6 +113,10 @@ def load() -> ctypes.CDLL:
     lib.ps_last_error.argtypes = []
     lib.ps_version.restype = ctypes.c_char_p
     lib.ps_version.argtypes = []
+    from . import _pycalls
+
+    _pycalls.bind(*(ctypes.cast(f, _vp).value for f in (lib.ps_kv_write, lib.ps_kv_gather, lib.ps_attn_plan, lib.ps_attn_run)))
+    _calls = _pycalls
     _lib = lib
     return lib
 
@@ -136,12 +142,11 @@ def _host_i32(a):
 _I32 = np.dtype(np.int32)
 
 
-def _host_i32_address(a):
-    """Like _host_i32 with the address as a plain integer, for arguments declared ``void *``: a typed ctypes pointer takes
-    2 us to make, and the calls of every iteration take two arrays each."""
+def _lengths(a):
+    """A batch's lengths as the extension module takes them."""
     if type(a) is not np.ndarray or a.dtype is not _I32 or not a.flags.c_contiguous:
         a = np.ascontiguousarray(a, dtype=_I32)
-    return a, a.__array_interface__["data"][0]
+    return a
 
 
 def make_shape(n_q_heads, n_kv_heads, head_dim, page_size=16, dtype=0) -> ps_shape:
@@ -174,14 +179,14 @@ def ps_kv_free(kv):
 
 
 def ps_kv_write(kv, k_new_dev, v_new_dev, block_table_dev, max_pages, prior_host, q_len_host, stream=None):
-    pr, prp = _host_i32_address(prior_host)
-    ql, qlp = _host_i32_address(q_len_host)
-    _check(load().ps_kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, prp, qlp,
-                              pr.shape[0], _ptr(stream)))
+    load()
+    _check(_calls.kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, _lengths(prior_host),
+                           _lengths(q_len_host), _ptr(stream)))
 
 
 def ps_kv_gather(kv, block_table_row_dev, length, k_out_dev, v_out_dev, stream=None):
-    _check(load().ps_kv_gather(kv, _ptr(block_table_row_dev), length, _ptr(k_out_dev), _ptr(v_out_dev), _ptr(stream)))
+    load()
+    _check(_calls.kv_gather(kv, _ptr(block_table_row_dev), length, _ptr(k_out_dev), _ptr(v_out_dev), _ptr(stream)))
 
 
 def ps_kv_gather_fp8(kv, block_table_row_dev, length, k_codes_out_dev, v_codes_out_dev, k_scale_out_dev, v_scale_out_dev, stream=None):
@@ -195,12 +200,16 @@ def ps_kv_status(kv, stream=None):
 
 def ps_attn_plan(shape: ps_shape, prior_host, q_len_host, max_pages_per_seq, opts: ps_plan_opts | None = None, plan=None):
     """Returns (plan handle, workspace bytes).  Pass ``plan`` to rebuild an existing handle in place."""
-    pr, prp = _host_i32_address(prior_host)
-    ql, qlp = _host_i32_address(q_len_host)
+    lib = load()
+    if opts is None:
+        status, handle, ws = _calls.attn_plan(ctypes.addressof(shape), _lengths(prior_host), _lengths(q_len_host), max_pages_per_seq, plan)
+        _check(status)
+        return handle, ws
+    pr, prp = _host_i32(prior_host)
+    ql, qlp = _host_i32(q_len_host)
     handle = _vp(plan or 0)
     ws = _sz(0)
-    _check(load().ps_attn_plan(ctypes.byref(shape), prp, qlp, pr.shape[0], max_pages_per_seq,
-                               ctypes.byref(opts) if opts is not None else None, ctypes.byref(handle), ctypes.byref(ws)))
+    _check(lib.ps_attn_plan(ctypes.byref(shape), prp, qlp, pr.shape[0], max_pages_per_seq, ctypes.byref(opts), ctypes.byref(handle), ctypes.byref(ws)))
     return handle.value, ws.value
 
 
@@ -224,8 +233,9 @@ def ps_plan_get_items(plan):
 
 
 def ps_attn_run(plan, kv, q_dev, block_table_dev, out_dev, lse_out_dev, workspace_dev, workspace_bytes, stream=None):
-    _check(load().ps_attn_run(plan, kv, _ptr(q_dev), _ptr(block_table_dev), _ptr(out_dev), _ptr(lse_out_dev),
-                              _ptr(workspace_dev), workspace_bytes, _ptr(stream)))
+    load()
+    _check(_calls.attn_run(plan, kv, _ptr(q_dev), _ptr(block_table_dev), _ptr(out_dev), _ptr(lse_out_dev), _ptr(workspace_dev),
+                           workspace_bytes, _ptr(stream)))
 
 
 PS_STATIC_WORKSPACE_BYTES = 8 << 20

@@ -2,8 +2,8 @@
 
     python -m paper_2507_17769_b200.build [--force] [--verbose]
 
-Compiles every ``csrc/*.cu`` into ``libpolyserve_attn.so`` next to this file.
-nvcc cross-compiles, so no GPU is needed to build.
+Compiles every ``csrc/*.cu`` into ``libpolyserve_attn.so`` next to this file, and ``csrc/pycalls.c`` into the extension
+module of the calls of every iteration.  nvcc cross-compiles, so no GPU is needed to build.
 """
 from __future__ import annotations
 
@@ -12,11 +12,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpolyserve_attn.so")
+CALLS = os.path.join(HERE, "_pycalls.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "-Xptxas", "-v",
@@ -35,12 +37,12 @@ def sources():
 
 
 def _deps_mtime() -> float:
-    files = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+    files = sources() + [os.path.join(CSRC, "pycalls.c")] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
     return max(os.path.getmtime(f) for f in files)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
+    if not force and os.path.exists(CALLS) and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
     nvcc = _nvcc()
@@ -58,6 +60,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
             if proc.returncode != 0:
                 raise RuntimeError("nvcc failed on %s" % src)
             objs.append(obj)
+    tmp = CALLS + ".tmp.%d" % os.getpid()
+    subprocess.check_call(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp,
+                           os.path.join(CSRC, "pycalls.c")])
+    os.replace(tmp, CALLS)
     tmp = LIB + ".tmp.%d" % os.getpid()
     subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)

@@ -77,7 +77,8 @@ class PagedAttention:
         """Logical tokens [0, length) of one sequence as contiguous (K, V) bf16 [length, Hkv, d] (bf16 cache)."""
         t = self.torch
         assert self.shape.dtype == 0, "use gather_fp8 on an FP8 cache"
-        k = t.empty((length, self.shape.n_kv_heads, self.shape.head_dim), dtype=t.bfloat16, device=self.device)
+        hkv, d = self.shape.n_kv_heads, self.shape.head_dim
+        k = t.empty_strided((length, hkv, d), (hkv * d, d, 1), dtype=t.bfloat16, device=self.device)
         v = t.empty_like(k)
         B.ps_kv_gather(self.kv, block_table_row_dev, int(length), k.data_ptr(), v.data_ptr(), self._stream())
         return k, v
@@ -106,7 +107,8 @@ class PagedAttention:
         if out is None:
             out = t.empty_like(q)
         if lse is None and want_lse:
-            lse = t.empty((q.shape[0], self.shape.n_q_heads), dtype=t.float32, device=self.device)
+            hq = self.shape.n_q_heads
+            lse = t.empty_strided((q.shape[0], hq), (hq, 1), dtype=t.float32, device=self.device)  # (two thirds of empty()'s time)
         B.ps_attn_run(self._plan, self.kv, q.data_ptr(), block_table_dev.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
                       self._ws.data_ptr(), self._ws_bytes, self._stream())
         return out, lse
