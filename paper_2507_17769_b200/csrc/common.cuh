@@ -51,6 +51,32 @@ ps_status once_per_device(PerDeviceOnce& state, F configure) {
     return st;
 }
 
+// Launches a kernel; clusters of `cluster` CTAs if above 1.  Every kernel of an iteration begins with pdl_wait(), so it may be
+// launched (`early`) while the kernel before it in the stream still runs: its launch and set-up, some 1.5 us, then overlap
+// that kernel's end.  Behind anything but a kernel, a copy or an event for instance, `early` changes nothing.
+template <class... P, class... A>
+ps_status launch_kernel(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t stream, int cluster, bool early, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
+    if (early) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = attr;
+    PS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, args...));
+    return PS_OK;
+}
+
 // ---------------------------------------------------------------------------
 // KV pool layout
 //
@@ -194,6 +220,7 @@ struct RunArgs {
     int num_sms;
     int dec_sms, pf_sms;  // SMs (= CTAs) for the decode and the prefill kernel
     bool sm_pairs;        // side by side with the pair kernel: the decode kernel's CTAs take whole SM pairs too
+    bool early;           // the kernel may be launched while the one before it in the stream still runs
     int32_t total_q;      // q tokens of the batch (rows of q and out)
     int32_t n_req;        // requests of the batch (rows of the block table)
     int64_t wait_limit_ns;
@@ -213,6 +240,12 @@ int decode_warps_per_sm();
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
+
+// Waits until the kernels before this one in the stream have completed and their results can be read; nothing that they may
+// write is read before it, and nothing that they may read is written.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel of the stream may be launched once every CTA has come by here.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

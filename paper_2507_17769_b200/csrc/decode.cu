@@ -123,6 +123,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
         mbar_fence_init();
     }
     __syncwarp();
+    pdl_trigger();
+    pdl_wait();
 
     // K/V pages are read once: marked first to go in L2, they leave the partial rows, Q and the work list resident
     // (measured: 100.9 -> 96.9 us on the 64-sequence decode batch, 465.6 -> 452.7 us on 512 sequences)
@@ -608,28 +610,11 @@ static ps_status launch_decode_d(const RunArgs& a) {
     p.wait_limit_ns = a.wait_limit_ns;
     int grid = (a.w.n_units + kWarps - 1) / kWarps;
     if (grid > a.dec_sms) grid = a.dec_sms;
-    if (a.sm_pairs) {
-        // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
-        // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
-        // before they have left.
-        cudaLaunchConfig_t cfgl = {};
-        cfgl.gridDim = dim3((grid + 1) / 2 * 2);
-        cfgl.blockDim = dim3(kWarps * 32);
-        cfgl.dynamicSmemBytes = Cfg::kSmemBytes;
-        cfgl.stream = a.stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfgl.attrs = attr;
-        cfgl.numAttrs = 1;
-        PS_CUDA_TRY(cudaLaunchKernelEx(&cfgl, decode_kernel<D, FP8>, p));
-        return PS_OK;
-    }
-    decode_kernel<D, FP8><<<grid, kWarps * 32, Cfg::kSmemBytes, a.stream>>>(p);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
+    // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
+    // before they have left.
+    if (a.sm_pairs) grid = (grid + 1) / 2 * 2;
+    return launch_kernel(decode_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
 }
 
 ps_status launch_decode(const RunArgs& a) {

@@ -57,6 +57,8 @@ constexpr int kParamRowsMax = 4000;  // 32 KB, as much as a kernel's parameters 
 // request of packed token t: last r with q_start(r) <= t
 template <class Rows>
 __device__ __forceinline__ int request_of(const Rows& rows, int n, int t) {
+    // (up to the first request of several tokens, which in a serving batch come last, every request has one)
+    if (t < n && rows.q_start(t) == t) return t;
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -65,48 +67,129 @@ __device__ __forceinline__ int request_of(const Rows& rows, int n, int t) {
     return lo;
 }
 
-// One thread moves one 16-byte unit of K and of V.
-// grid.x covers T * Hkv * (d / 8) units.
-template <class Rows>
-__global__ void kv_write_kernel(char* pool, int64_t num_pages, const uint4* __restrict__ k_new,
-                                const uint4* __restrict__ v_new, const int32_t* __restrict__ block_table,
-                                int max_pages, const __grid_constant__ Rows rows, int n, int Hkv, int d, int* flag) {
-    const int units_per_tok = Hkv * (d >> 3);
-    const int64_t total = (int64_t)rows.q_start(n) * units_per_tok;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int t = (int)(idx / units_per_tok);
-        const int rem = (int)(idx % units_per_tok);
-        const int g = rem / (d >> 3);
-        const int u = rem % (d >> 3);
+// Append and gather are copies between a token's row [Hkv][d] and its place in a page, so they are bound by memory, and at
+// these sizes by its latency: a warp moves one token's K and V, 32 bytes a lane, with all loads of a chunk (two pairs of K
+// and of V a lane) under way before its first store.  A 16-byte unit u of token slot t lies at u ^ (t & 7): a pair of units
+// stays a 32-byte pair whose halves change places in odd slots.
+// Measured (6001 tokens of 8 x 128, K and V, 74 MB; cold inputs, append and gather in turn): 22.5 us with one thread per
+// 16-byte unit and a request search in each, 20.6 with two tokens a warp, 19.3 with one, 15.2 (4.9 TB/s) launched early.
+constexpr int kCopyThreads = 256;
+constexpr int kCopyTokens = kCopyThreads / 32;  // of a CTA
+
+struct Pair32 {
+    uint4 a, b;
+};
+__device__ __forceinline__ Pair32 load32(const void* p) {
+    Pair32 x;
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(x.a.x), "=r"(x.a.y), "=r"(x.a.z), "=r"(x.a.w), "=r"(x.b.x), "=r"(x.b.y), "=r"(x.b.z), "=r"(x.b.w)
+                 : "l"(p));
+    return x;
+}
+__device__ __forceinline__ void store32(void* p, const Pair32& x) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(x.a.x), "r"(x.a.y), "r"(x.a.z), "r"(x.a.w),
+                 "r"(x.b.x), "r"(x.b.y), "r"(x.b.z), "r"(x.b.w)
+                 : "memory");
+}
+// a token's row: 32-byte aligned where the caller's tensor is (ALIGNED), else 16
+template <bool ALIGNED>
+__device__ __forceinline__ Pair32 load_row32(const char* p) {
+    if (ALIGNED) return load32(p);
+    return Pair32{reinterpret_cast<const uint4*>(p)[0], reinterpret_cast<const uint4*>(p)[1]};
+}
+template <bool ALIGNED>
+__device__ __forceinline__ void store_row32(char* p, const Pair32& x) {
+    if (ALIGNED) {
+        store32(p, x);
+    } else {
+        reinterpret_cast<uint4*>(p)[0] = x.a;
+        reinterpret_cast<uint4*>(p)[1] = x.b;
+    }
+}
+__device__ __forceinline__ Pair32 swap_if(const Pair32& x, bool odd) { return odd ? Pair32{x.b, x.a} : x; }
+// 32-byte pair c of a token's row -> offset of its (page, kv head)'s pair in the K block, from the page's start
+template <int D>
+__device__ __forceinline__ uint32_t pair_offset(int c, int slot) {
+    constexpr int kPairs = D / 16;
+    return (uint32_t)(c / kPairs) * (uint32_t)page_head_bytes(D) + (unit_offset(slot, (c % kPairs) * 16) & ~16u);
+}
+
+template <int D, bool ALIGNED, class Rows>
+__global__ void __launch_bounds__(kCopyThreads) kv_write_kernel(char* pool, int64_t num_pages, const char* __restrict__ k_new, const char* __restrict__ v_new,
+                                                                const int32_t* __restrict__ block_table, int max_pages, const __grid_constant__ Rows rows, int n,
+                                                                int Hkv, int* flag) {
+    pdl_trigger();
+    const int lane = threadIdx.x & 31;
+    const int t = (int)blockIdx.x * kCopyTokens + (int)(threadIdx.x >> 5);
+    const int pairs = Hkv * (D / 16);
+    pdl_wait();
+    if (t >= rows.q_start(n)) return;
+    for (int c0 = 0; c0 < pairs; c0 += 64) {
+        Pair32 x[2][2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int c = c0 + 32 * j + lane;
+            if (c < pairs) {
+                const int64_t at = ((int64_t)t * pairs + c) * 32;
+                x[j][0] = load_row32<ALIGNED>(k_new + at);
+                x[j][1] = load_row32<ALIGNED>(v_new + at);
+            }
+        }
         const int r = request_of(rows, n, t);
-        const int pos = rows.prior(r) + (t - rows.q_start(r));
+        const int pos = rows.prior(r) + (t - rows.q_start(r)), slot = pos % kPage;
         const int64_t page = block_table[(int64_t)r * max_pages + pos / kPage];
-        if (page < 0 || page >= num_pages) { atomicOr(flag, kStatusBounds); continue; }
-        const int slot = pos % kPage;
-        char* blk = pool + ((page * Hkv + g) * 2) * block_bytes(d);
-        const uint32_t off = unit_offset(slot, u * 8);
-        *reinterpret_cast<uint4*>(blk + off) = k_new[idx];
-        *reinterpret_cast<uint4*>(blk + block_bytes(d) + off) = v_new[idx];
+        if (page < 0 || page >= num_pages) {
+            if (lane == 0) atomicOr(flag, kStatusBounds);
+            return;
+        }
+        char* const dst = pool + page * Hkv * (int64_t)page_head_bytes(D);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int c = c0 + 32 * j + lane;
+            if (c < pairs) {
+                char* const at = dst + pair_offset<D>(c, slot);
+                store32(at, swap_if(x[j][0], slot & 1));
+                store32(at + block_bytes(D), swap_if(x[j][1], slot & 1));
+            }
+        }
     }
 }
 
-__global__ void kv_gather_kernel(const char* pool, int64_t num_pages, const int32_t* __restrict__ bt_row, int len,
-                                 int Hkv, int d, uint4* k_out, uint4* v_out, int* flag) {
-    const int units_per_tok = Hkv * (d >> 3);
-    const int64_t total = (int64_t)len * units_per_tok;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int pos = (int)(idx / units_per_tok);
-        const int rem = (int)(idx % units_per_tok);
-        const int g = rem / (d >> 3);
-        const int u = rem % (d >> 3);
-        const int64_t page = bt_row[pos / kPage];
-        if (page < 0 || page >= num_pages) { atomicOr(flag, kStatusBounds); continue; }
-        const char* blk = pool + ((page * Hkv + g) * 2) * block_bytes(d);
-        const uint32_t off = unit_offset(pos % kPage, u * 8);
-        if (k_out) k_out[idx] = *reinterpret_cast<const uint4*>(blk + off);
-        if (v_out) v_out[idx] = *reinterpret_cast<const uint4*>(blk + block_bytes(d) + off);
+template <int D, bool ALIGNED>
+__global__ void __launch_bounds__(kCopyThreads) kv_gather_kernel(const char* pool, int64_t num_pages, const int32_t* __restrict__ bt_row, int len, int Hkv,
+                                                                 char* k_out, char* v_out, int* flag) {
+    pdl_trigger();
+    const int lane = threadIdx.x & 31;
+    const int t = (int)blockIdx.x * kCopyTokens + (int)(threadIdx.x >> 5), slot = t % kPage;
+    const int pairs = Hkv * (D / 16);
+    pdl_wait();
+    if (t >= len) return;
+    const int64_t page = bt_row[t / kPage];
+    if (page < 0 || page >= num_pages) {
+        if (lane == 0) atomicOr(flag, kStatusBounds);
+        return;
+    }
+    const char* const src = pool + page * Hkv * (int64_t)page_head_bytes(D);
+    for (int c0 = 0; c0 < pairs; c0 += 64) {
+        Pair32 x[2][2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int c = c0 + 32 * j + lane;
+            if (c < pairs) {
+                const char* const at = src + pair_offset<D>(c, slot);
+                x[j][0] = load32(at);
+                x[j][1] = load32(at + block_bytes(D));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int c = c0 + 32 * j + lane;
+            if (c < pairs) {
+                const int64_t at = ((int64_t)t * pairs + c) * 32;
+                if (k_out) store_row32<ALIGNED>(k_out + at, swap_if(x[j][0], slot & 1));
+                if (v_out) store_row32<ALIGNED>(v_out + at, swap_if(x[j][1], slot & 1));
+            }
+        }
     }
 }
 
@@ -130,6 +213,8 @@ __global__ void kv_write_fp8_kernel(char* pool, int64_t num_pages, const uint2* 
                                     const uint2* __restrict__ v_new, const int32_t* __restrict__ block_table, int max_pages,
                                     const __grid_constant__ Rows rows, int n, int Hkv, int* flag) {
     constexpr int d = 128;
+    pdl_trigger();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t total = (int64_t)rows.q_start(n) * Hkv;
     for (int64_t vec = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); vec < total;
@@ -166,6 +251,8 @@ __global__ void kv_write_fp8_kernel(char* pool, int64_t num_pages, const uint2* 
 __global__ void kv_gather_fp8_kernel(const char* pool, int64_t num_pages, const int32_t* __restrict__ bt_row, int len, int Hkv,
                                      uint32_t* k_out, uint32_t* v_out, float* k_scale_out, float* v_scale_out, int* flag) {
     constexpr int d = 128;
+    pdl_trigger();
+    pdl_wait();
     const int64_t total = (int64_t)len * Hkv * (d / 4);
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
         const int pos = (int)(idx / (Hkv * (d / 4)));
@@ -216,23 +303,22 @@ void fill_rows(const KvWrite& w, int32_t* q_start, int32_t* prior) {
     q_start[w.n] = t;
 }
 
+unsigned copy_blocks(int64_t tokens) { return (unsigned)((tokens + kCopyTokens - 1) / kCopyTokens); }
+
 template <class Rows>
 ps_status launch_write(const KvPool& p, const KvWrite& w, const Rows& rows) {
     const int Hkv = p.shape.n_kv_heads, d = p.shape.head_dim;
     if (p.shape.dtype == 1) {
         const int64_t warps = w.T * Hkv;
         const int blocks = (int)((warps + 7) / 8 < 148 * 16 ? (warps + 7) / 8 : 148 * 16);
-        kv_write_fp8_kernel<<<blocks, 256, 0, w.stream>>>(p.base, p.num_pages, (const uint2*)w.k_new, (const uint2*)w.v_new, w.block_table,
-                                                          w.max_pages, rows, w.n, Hkv, p.flag_dev);
-    } else {
-        const int64_t total = w.T * Hkv * (d / 8);
-        const int threads = 256;
-        const int blocks = (int)((total + threads - 1) / threads < 148 * 32 ? (total + threads - 1) / threads : 148 * 32);
-        kv_write_kernel<<<blocks, threads, 0, w.stream>>>(p.base, p.num_pages, (const uint4*)w.k_new, (const uint4*)w.v_new, w.block_table,
-                                                          w.max_pages, rows, w.n, Hkv, d, p.flag_dev);
+        return launch_kernel(kv_write_fp8_kernel<Rows>, blocks, 256, 0, w.stream, 1, true, p.base, p.num_pages, (const uint2*)w.k_new,
+                             (const uint2*)w.v_new, w.block_table, w.max_pages, rows, w.n, Hkv, p.flag_dev);
     }
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    const bool aligned = (((uintptr_t)w.k_new | (uintptr_t)w.v_new) & 31) == 0;
+    auto* const kernel = d == 128 ? (aligned ? kv_write_kernel<128, true, Rows> : kv_write_kernel<128, false, Rows>)
+                                  : (aligned ? kv_write_kernel<64, true, Rows> : kv_write_kernel<64, false, Rows>);
+    return launch_kernel(kernel, copy_blocks(w.T), kCopyThreads, 0, w.stream, 1, true, p.base, p.num_pages, (const char*)w.k_new,
+                         (const char*)w.v_new, w.block_table, w.max_pages, rows, w.n, Hkv, p.flag_dev);
 }
 
 template <int N>
@@ -343,14 +429,11 @@ ps_status ps_kv_gather(const ps_kv* kv, const int32_t* block_table_row_dev, int3
     if (len == 0 || (!k_out_dev && !v_out_dev)) return PS_OK;
     if (kv->p.shape.dtype == 1) return ps_kv_gather_fp8(kv, block_table_row_dev, len, k_out_dev, v_out_dev, nullptr, nullptr, stream);
     const int Hkv = kv->p.shape.n_kv_heads, d = kv->p.shape.head_dim;
-    const int64_t total = (int64_t)len * Hkv * (d / 8);
-    const int threads = 256;
-    const int blocks = (int)((total + threads - 1) / threads < 148 * 32 ? (total + threads - 1) / threads : 148 * 32);
-    kv_gather_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(kv->p.base, kv->p.num_pages, block_table_row_dev,
-                                                                   len, Hkv, d, (uint4*)k_out_dev, (uint4*)v_out_dev,
-                                                                   kv->p.flag_dev);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    const bool aligned = (((uintptr_t)k_out_dev | (uintptr_t)v_out_dev) & 31) == 0;
+    auto* const kernel = d == 128 ? (aligned ? kv_gather_kernel<128, true> : kv_gather_kernel<128, false>)
+                                  : (aligned ? kv_gather_kernel<64, true> : kv_gather_kernel<64, false>);
+    return launch_kernel(kernel, copy_blocks(len), kCopyThreads, 0, (cudaStream_t)stream, 1, true, (const char*)kv->p.base, kv->p.num_pages,
+                         block_table_row_dev, len, Hkv, (char*)k_out_dev, (char*)v_out_dev, kv->p.flag_dev);
 }
 
 ps_status ps_kv_gather_fp8(const ps_kv* kv, const int32_t* block_table_row_dev, int32_t len, void* k_codes_out_dev,
@@ -363,11 +446,9 @@ ps_status ps_kv_gather_fp8(const ps_kv* kv, const int32_t* block_table_row_dev, 
     const int64_t total = (int64_t)len * Hkv * 32;
     const int threads = 256;
     const int blocks = (int)((total + threads - 1) / threads < 148 * 32 ? (total + threads - 1) / threads : 148 * 32);
-    kv_gather_fp8_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(kv->p.base, kv->p.num_pages, block_table_row_dev, len, Hkv,
-                                                                       (uint32_t*)k_codes_out_dev, (uint32_t*)v_codes_out_dev,
-                                                                       k_scale_out_dev, v_scale_out_dev, kv->p.flag_dev);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    return launch_kernel(kv_gather_fp8_kernel, blocks, threads, 0, (cudaStream_t)stream, 1, true, (const char*)kv->p.base, kv->p.num_pages,
+                         block_table_row_dev, len, Hkv, (uint32_t*)k_codes_out_dev, (uint32_t*)v_codes_out_dev, (float*)k_scale_out_dev,
+                         (float*)v_scale_out_dev, kv->p.flag_dev);
 }
 
 ps_status ps_kv_status(ps_kv* kv, void* stream) {

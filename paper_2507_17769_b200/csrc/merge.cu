@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntr
                                                                   int Hq, int G) {
     constexpr int V = D / 32;  // floats per lane
     using Vec = typename std::conditional<V == 4, float4, float2>::type;
+    pdl_wait();
     const MergeEntry e = entries[blockIdx.x];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rows = e.n_tok * G;
@@ -95,12 +96,8 @@ ps_status launch_merge(const RunArgs& a) {
     const int Hq = a.shape.n_q_heads, G = Hq / a.shape.n_kv_heads;
     // blockIdx.x = merge entry (a prefill item cut into segments, up to 256 rows); blockIdx.y = its rows, one per warp
     const dim3 grid(a.w.n_merge, kPrefillRowsPerItem / kMergeWarps);
-    if (a.shape.head_dim == 128)
-        merge_kernel<128><<<grid, kMergeWarps * 32, 0, a.stream>>>(a.w.merge, a.w.part_lse, a.w.part_o, a.out, a.lse, Hq, G);
-    else
-        merge_kernel<64><<<grid, kMergeWarps * 32, 0, a.stream>>>(a.w.merge, a.w.part_lse, a.w.part_o, a.out, a.lse, Hq, G);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    return launch_kernel(a.shape.head_dim == 128 ? merge_kernel<128> : merge_kernel<64>, grid, kMergeWarps * 32, 0, a.stream, 1, a.early, a.w.merge,
+                         (const float*)a.w.part_lse, (const float*)a.w.part_o, a.out, a.lse, Hq, G);
 }
 
 }  // namespace ps

@@ -798,6 +798,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.total_q = (int32_t)pl->info.total_q_tokens;
     a.n_req = pl->n;
     a.wait_limit_ns = pl->wait_limit_ns;
+    a.early = !capturing;
     a.w.hdr = (WsHeader*)ws;
     a.w.pieces = (const DecodePiece*)(ws + pl->off_pieces);
     a.w.units = (const DecodeUnit*)(ws + pl->off_units);
@@ -842,8 +843,12 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
         if (st == PS_OK && !helpers) {
             // Only this launch writes prefill partials: combine them right behind it, on the SMs it leaves, while
             // the decode kernel is still streaming (decode rows are combined inside the decode kernel).
+            // (not launched early: its CTAs, waiting beside the decode kernel's, slowed a batch of 48 decode rows and two chunks
+            // at head dimension 64 from 70 to 81 us)
+            RunArgs am = a;
+            am.early = false;
             if (rec) cudaEventRecord(ev[4], s);
-            st = launch_merge(a);
+            st = launch_merge(am);
             if (rec) cudaEventRecord(ev[5], s);
             merged = true;
         }
@@ -853,6 +858,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
             RunArgs ah = a;
             ah.stream = side;
             ah.pf_sms = a.dec_sms;
+            ah.early = false;  // (waiting for the decode kernel it would hold SMs that the first launch needs)
             st = launch_prefill(ah);
         }
         const cudaError_t ej = cudaEventRecord(pl->ev_join, side);

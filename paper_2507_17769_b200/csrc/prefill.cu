@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         tmem_alloc(bars + Bars::tmem_slot, Cfg::kTmemCols);
         tmem_relinquish();
     }
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -652,6 +653,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         // (the warpgroup's two other warps have no work; they wait at the final barrier)
     }
 
+    pdl_trigger();
     tc_fence_before();
     __syncthreads();  // every role has left its loop
     if (*s_abort) {
@@ -715,9 +717,7 @@ static ps_status launch_prefill_d(const RunArgs& a) {
     if (enc != PS_OK) return enc;
 
     const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
-    prefill_kernel<D><<<grid, kThreads, Cfg::kSmemBytes, a.stream>>>(p, q_map);
-    PS_CUDA_TRY(cudaGetLastError());
-    return PS_OK;
+    return launch_kernel(prefill_kernel<D>, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map);
 }
 
 ps_status launch_prefill(const RunArgs& a) {

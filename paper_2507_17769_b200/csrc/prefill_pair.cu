@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     if (threadIdx.x < Bars::n_armed) s_armed[threadIdx.x] = -1;
     tc_fence_before();
     __syncthreads();
+    pdl_wait();
     cluster_sync();  // the peer's barriers are initialised before anything arrives at them
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(smem + kOffBar + Bars::tmem_slot), 0);
@@ -919,6 +920,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         }
     }
 
+    // (not before: a kernel that waits for this one's end would take the place of the decode kernel's CTAs beside it)
+    pdl_trigger();
     if (warp == kMmaWarp) {
         if (rank == 0) {
             if (elect_one()) pair_commit(bars + Bars::mma_drained);
@@ -1030,20 +1033,7 @@ ps_status launch_prefill_pair(const RunArgs& a) {
         if (r != CUDA_SUCCESS) return fail(PS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
     }
     const int pairs = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms / 2 ? a.w.n_prefill : (a.pf_sms > 1 ? a.pf_sms / 2 : 1));
-    cudaLaunchConfig_t cfgl = {};
-    cfgl.gridDim = dim3(2 * pairs);
-    cfgl.blockDim = dim3(kThreads);
-    cfgl.dynamicSmemBytes = kSmemBytes;
-    cfgl.stream = a.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfgl.attrs = attr;
-    cfgl.numAttrs = 1;
-    PS_CUDA_TRY(cudaLaunchKernelEx(&cfgl, prefill_pair_kernel, p, q_map, pool_map));
-    return PS_OK;
+    return launch_kernel(prefill_pair_kernel, 2 * pairs, kThreads, kSmemBytes, a.stream, 2, a.early, p, q_map, pool_map);
 }
 
 }  // namespace ps
