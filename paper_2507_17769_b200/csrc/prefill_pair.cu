@@ -8,10 +8,10 @@
 // 32 KB per 128-key step from L2 for 128 rows.
 //
 //   warps 0-15 softmax: thread = half a row (64 of a tile's 128 keys); warps 0-7 take the even key tiles, 8-15 the odd ones
-//   warp 16    K producer: in rank 0 also fetches the pair's items; K half tiles (bulk copies of pool blocks) and Q
+//   warp 16    K producer: K half tiles (gathered pool blocks) and Q
 //   warp 17    V producer
-//   warp 18    rank 0: issues the MMAs; rank 1: tells rank 0 that this CTA's K half tiles (and Q) have landed
-//   warp 19    rank 0: waits for V on the MMA warp's behalf; rank 1: as warp 18, for V
+//   warp 18    rank 0: issues the MMAs; rank 1: tells rank 0 that this CTA's K and V half tiles and Q have landed
+//   warp 19    rank 0: waits for V on the MMA warp's behalf; rank 1: fetches the pair's items, well ahead of their use
 //
 // TMEM columns (of each CTA): scores of key tile n at 128 (n % 3), O at 384.  Weights overwrite their own scores (bf16,
 // each half in the first 32 of its 64 columns), so one barrier per tile says both that P is there and that the buffer may
@@ -33,7 +33,8 @@
 //     2048 x 8192  275 -> 215 us (1436 TFLOP/s, 0.87)    2 x 2048 on 19.8 k and 28.9 k, 64 q heads  2890 -> 2330 us (1460)
 // Steps on the way, on 2048 x 8192: pair with two score buffers and eight softmax warps 251 us; three buffers, sixteen
 // warps, no maximum 245; warp-uniform MMA issue and the feeder 241; gathered copies 218; part of the exponentials on the
-// FMA pipe and items begun by the other group 212.
+// FMA pipe and items begun by the other group 212.  Items fetched by a warp of their own: 888 items of one key tile (12 a
+// pair) 70.5 -> 64 us, of five 112 -> 106, four prompts of 1400 to 2000 tokens, whole iteration, 134.1 -> 129.5.
 // Every wait is bounded; on expiry a CTA sets the timeout status and drains.
 #include "tcgen05.cuh"
 
@@ -42,7 +43,7 @@ namespace ps {
 namespace {
 
 constexpr int kThreads = 640;
-constexpr int kKProducerWarp = 16, kVProducerWarp = 17, kMmaWarp = 18;
+constexpr int kKProducerWarp = 16, kVProducerWarp = 17, kMmaWarp = 18, kItemWarp = 19;
 constexpr int kRegsSoftmax = 104, kRegsOther = 64;  // 640 x 96 at launch = 512 x 104 + 128 x 64
 constexpr int D = 128;
 constexpr int kTileKeys = 128;
@@ -65,7 +66,10 @@ constexpr int kOffK = kOffQ + 2 * kQBytes;
 constexpr int kOffV = kOffK + kStagesK * kKBytes;
 constexpr int kOffBar = kOffV + kStagesV * kVBytes;
 constexpr int kItemRing = 8;
-// every warp of both CTAs but rank 0's K producer, which writes the records
+// Key tiles of items fetched ahead.  An item's first K tile is used some 5000 cycles after its record is out, four key tiles;
+// with 6 the tensor core waited for short items' K (four prompts of 1400 to 2000 tokens 131.4 us, with 12 129.5).
+constexpr int kAheadTiles = 12;
+// every warp of both CTAs but rank 1's item warp, which writes the records
 constexpr int kRingConsumers = 2 * 20 - 1;
 constexpr int64_t kPairDrainLimitNs = 100000000ll;
 constexpr uint32_t kColO = 384;
@@ -83,14 +87,14 @@ struct Bars {  // byte offsets from the barrier block
     static constexpr int o_done = p_ready + 8 * 2 * kScoreBufs;  // per item mod 4 (a warp that skips items then never skips a phase it could mistake)
     static constexpr int o_free = o_done + 32;              // rank 0
     static constexpr int mma_drained = o_free + 8;
-    static constexpr int item_full = mma_drained + 8, item_empty = item_full + 8 * kItemRing;  // (item_empty: rank 0)
+    static constexpr int item_full = mma_drained + 8, item_empty = item_full + 8 * kItemRing;  // (item_empty: rank 1)
     static constexpr int n_bars = (item_empty + 8 * kItemRing) / 8;
     static constexpr int tmem_slot = item_empty + 8 * kItemRing, abort_slot = tmem_slot + 4, limit_slot = abort_slot + 4;
     static constexpr int armed = limit_slot + 4;            // parity of the last phase armed with copies: K, V stages, Q buffers
     static constexpr int n_armed = kStagesK + kStagesV + 2;
-    static constexpr int again = armed + 4 * n_armed;       // rank 0, per ring slot a byte per rank and quarter of its rows: sums out of range
+    static constexpr int again = armed + 4 * n_armed;       // rank 1, per ring slot a byte per rank and quarter of its rows: sums out of range
     static constexpr int ring = (again + 8 * kItemRing + 15) / 16 * 16;
-    static constexpr int redo = ring + kItemRing * (int)sizeof(PrefillItem);      // rank 0: records to run again
+    static constexpr int redo = ring + kItemRing * (int)sizeof(PrefillItem);      // rank 1: records to run again
     static constexpr int row_part = redo + kItemRing * (int)sizeof(PrefillItem);  // [item & 3][softmax warpgroup] per row: (sum or maximum, item number and the sum's rounding)
     static constexpr int bytes = row_part + 16 * kRows * 8;
 };
@@ -297,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     uint4* const redo = reinterpret_cast<uint4*>(smem + kOffBar + Bars::redo);
     // next item of this pair's static share, or of the queue all pairs of the run drain
     auto next_item = [&](int cur, int end) { return p.pair_start ? (cur < end ? cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1); };
-    if (rank == 0 && threadIdx.x == kKProducerWarp * 32) {
+    if (rank == 1 && threadIdx.x == kItemWarp * 32) {
         // the first item's record is on its way before the pair meets
         const int pair = blockIdx.x >> 1;
         const int idx = next_item(p.pair_start ? __ldg(p.pair_start + pair) : 0, p.pair_start ? __ldg(p.pair_start + pair + 1) : 0);
@@ -324,7 +328,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     cluster_sync();  // the peer's barriers are initialised before anything arrives at them
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(smem + kOffBar + Bars::tmem_slot), 0);
-    const uint32_t lead = map_to_rank(bars, 0);  // rank 0's barrier block
+    const uint32_t lead = map_to_rank(bars, 0);   // rank 0's barrier block
+    const uint32_t items = map_to_rank(bars, 1);  // rank 1's, where records are given back
     // warp-uniform result, so that the warp-collective instructions that follow stay converged
     auto wait_all = [](uint32_t bar, uint32_t parity, volatile int* abort_flag) {
         return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag));
@@ -336,11 +341,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     auto take_record = [&](uint32_t n, uint4& a, uint4& b, bool give_back) -> bool {
         const uint32_t slot = n % kItemRing;
         if (!wait_all(bars + Bars::item_full + 8 * slot, (n / kItemRing) & 1, s_abort)) return false;
-        acquire_cluster(bars + Bars::item_full + 8 * slot, (n / kItemRing) & 1);  // the record was written by rank 0
+        acquire_cluster(bars + Bars::item_full + 8 * slot, (n / kItemRing) & 1);  // the record was written by rank 1
         a = ring[2 * slot];
         b = ring[2 * slot + 1];
         __syncwarp();
-        if (give_back && lane == 0) arrive_at(lead + Bars::item_empty + 8 * slot);
+        if (give_back && lane == 0) arrive_at(items + Bars::item_empty + 8 * slot);
         return (int32_t)b.y > 0;
     };
     auto tiles_of = [](const uint4& a) { return ((int32_t)a.w - (int32_t)a.z + kTileKeys - 1) / kTileKeys; };
@@ -506,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
             store_tagged(row_part(n_item, 2 * w + h), l, (n_item & 0xffffu) | (pack_bf16(0.f, rounding) & 0xffff0000u));
             auto give_back = [&]() {
                 __syncwarp();
-                arrive_at_if(lead + Bars::item_empty + 8 * (n_item % kItemRing), lane == 0);
+                arrive_at_if(items + Bars::item_empty + 8 * (n_item % kItemRing), lane == 0);
             };
             if (g_last != w) {
                 give_back();
@@ -528,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 const uint32_t quarter = rank * 4 + (warp & 3);
                 bool write = mode == kModeRelative ? ((rb.y >> (16 + quarter)) & 1u) != 0 : mode == kModePlain;
                 if (mode == kModePlain && __any_sync(0xffffffffu, bad)) {
-                    if (lane == 0) store_u8_at(lead + Bars::again + 8 * (n_item % kItemRing) + quarter);
+                    if (lane == 0) store_u8_at(items + Bars::again + 8 * (n_item % kItemRing) + quarter);
                     fence_cluster();
                     write = false;
                 }
@@ -584,131 +589,16 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
         if (warp == kKProducerWarp || warp == kVProducerWarp) {
             // ================================================================
-            // producers: K half tiles (this rank's 64 keys) with the Q tiles and, in rank 0, the item records; V half
-            // tiles (this rank's 64 columns).  K/V tiles of a chunk's sequence are read again by every other item of that
+            // producers: K half tiles (this rank's 64 keys) with the Q tiles; V half tiles (this rank's 64 columns).  K/V tiles of a chunk's sequence are read again by every other item of that
             // sequence: they are marked last to leave L2.
             // ================================================================
             const bool is_k = warp == kKProducerWarp;
             const uint64_t kv_policy = l2_policy_evict_last();
             uint32_t n_item = 0, tc = 0;
             bool ok = true;
-            // Rank 0's K producer publishes the next record while the current item's tiles are being requested: neither the
-            // queue's counter nor the record's load is waited for between items.
-            uint4 na, nb;            // the record published last
-            bool need_record = false, published = false;  // an index has been asked for whose record is not fetched; record n_item + 1 is out
-            uint32_t mode = kModePlain;
-            const bool lead_k = is_k && rank == 0;
-            const int pair = blockIdx.x >> 1;
-            int static_cur = 0, static_end = 0, next_idx = 0;  // (next_idx in lane 0)
-            uint32_t redo_head = 0, redo_tail = 0;             // records put aside
-            uint4 fa = make_uint4(0, 0, 0, 0), fb = fa;        // the record fetched; n_tok = 0: end of work
-            auto check_record = [&]() {
-                if ((int32_t)fb.y == 0) return;
-                // A record that points outside the batch (only a damaged work list has one) ends this pair's work and
-                // flags the run; nothing is read or written through it.
-                const int32_t r_req = (int32_t)fa.x, r_g = (int32_t)fa.y, r_kb = (int32_t)fa.z, r_ke = (int32_t)fa.w;
-                const int32_t r_q = (int32_t)fb.x, r_n = (int32_t)fb.y, r_slot = (int32_t)fb.z, r_pos = (int32_t)fb.w;
-                const bool rec_ok = (uint32_t)r_req < (uint32_t)p.n_req && (uint32_t)r_g < (uint32_t)p.Hkv && r_kb >= 0 &&
-                                    r_kb % kTileKeys == 0 && r_kb < r_ke && r_ke <= p.max_pages * kPage && r_n >= 1 &&
-                                    r_n <= 2 * tile_tok && r_q >= 0 && (int64_t)r_q + r_n <= p.total_q && r_pos >= 0 &&
-                                    (int64_t)r_pos + r_n >= r_ke &&
-                                    (r_slot < 0 || (int64_t)r_slot + (int64_t)r_n * p.G <= p.n_part_slots);
-                if (!rec_ok) {
-                    if (lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
-                    fa = fb = make_uint4(0, 0, 0, 0);
-                }
-            };
-            auto fetch_index = [&]() {
-                if (lane == 0) next_idx = next_item(static_cur, static_end);
-                ++static_cur;
-            };
-            auto fetch_record = [&]() {
-                const int idx = __shfl_sync(0xffffffffu, next_idx, 0);
-                fa = fb = make_uint4(0, 0, 0, 0);
-                if (idx < p.n_items) {
-                    fa = __ldg(reinterpret_cast<const uint4*>(p.items + idx));
-                    fb = __ldg(reinterpret_cast<const uint4*>(p.items + idx) + 1);
-                }
-                check_record();
-            };
-            if (lead_k) {
-                fa = redo[0];
-                fb = redo[1];
-                check_record();
-                if (p.pair_start) {
-                    static_cur = __ldg(p.pair_start + pair) + 1;
-                    static_end = __ldg(p.pair_start + pair + 1);
-                }
-            }
-            // every consumer is done with the record that last used the slot of record n; if its item has to be run again,
-            // the record is put aside
-            auto reclaim = [&](uint32_t n) -> bool {
-                const uint32_t slot = n % kItemRing, par = ((n / kItemRing) & 1) ^ 1;
-                if (!wait_all(bars + Bars::item_empty + 8 * slot, par, s_abort)) return false;
-                acquire_cluster(bars + Bars::item_empty + 8 * slot, par);
-                const uint32_t mask = __ballot_sync(0xffffffffu, lane < 8 && again[8 * slot + (lane & 7)] != 0);
-                if (mask) {
-                    if (lane < 2) {
-                        uint4 x = ring[2 * slot + lane];
-                        if (lane == 1) x.y |= mask << 16;
-                        redo[2 * (redo_tail % kItemRing) + lane] = x;
-                    }
-                    ++redo_tail;
-                    if (lane < 8) again[8 * slot + lane] = 0;
-                    __syncwarp();
-                }
-                return true;
-            };
-            // publishes record n: the second pass of an item run again, the first one of the next such item, or the record
-            // fetched (which stays fetched in the first two cases)
-            auto publish = [&](uint32_t n) -> bool {
-                if (!reclaim(n)) return false;
-                if (mode != kModeMax && redo_head == redo_tail && (int32_t)fb.y == 0) {
-                    // end of work, unless one of the items still under way has to be run again
-                    for (uint32_t k = 1; k < kItemRing; ++k)
-                        if (n >= k && !reclaim(n - k + kItemRing)) return false;
-                }
-                bool from_fetched = false;
-                if (mode == kModeMax) {
-                    mode = kModeRelative;
-                } else if (redo_head != redo_tail) {
-                    na = redo[2 * (redo_head % kItemRing)];
-                    nb = redo[2 * (redo_head % kItemRing) + 1];
-                    ++redo_head;
-                    mode = kModeMax;
-                } else {
-                    na = fa;
-                    nb = fb;
-                    mode = kModePlain;
-                    from_fetched = true;
-                }
-                nb.y = (nb.y & 0xffffffu) | (mode << 24);
-                const uint32_t slot = n % kItemRing;
-                if (lane == 0) {
-                    uint4 plain = na;
-                    ring[2 * slot] = plain;
-                    ring[2 * slot + 1] = nb;
-                    mbar_arrive(bars + Bars::item_full + 8 * slot);
-                    const uint32_t peer = map_to_rank(bars, 1);
-                    store_at(peer + Bars::ring + 32 * slot, plain);
-                    store_at(peer + Bars::ring + 32 * slot + 16, nb);
-                    arrive_at_release_cluster(peer + Bars::item_full + 8 * slot);
-                }
-                __syncwarp();
-                if (from_fetched && (int32_t)nb.y != 0) fetch_index();
-                need_record = from_fetched && (int32_t)nb.y != 0;
-                return true;
-            };
-            if (lead_k) ok = publish(0);
             for (; ok; ++n_item) {
                 uint4 ra, rb;
-                if (lead_k) {
-                    ra = na;
-                    rb = nb;
-                    if ((int32_t)rb.y <= 0) break;
-                } else if (!take_record(n_item, ra, rb, true)) {
-                    break;
-                }
+                if (!take_record(n_item, ra, rb, true)) break;
                 const int kv_head = (int)ra.y;
                 const int key_begin = (int)ra.z;
                 const int n_tiles = tiles_of(ra), n_pages = ((int)ra.w - key_begin + kPage - 1) / kPage;
@@ -761,19 +651,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                         }
                         __syncwarp();
                     }
-                    if (lead_k && j == 1 && need_record) fetch_record();
-                    if (lead_k && j == 2 && !(n_tiles > 3 && (int32_t)fb.y == 0)) {
-                        ok = publish(n_item + 1);
-                        if (!ok) break;
-                        published = true;
-                    }
                 }
-                if (lead_k && ok && !published) {
-                    // (short items, and the last one: the end of work is published when every item has been checked)
-                    if (n_tiles < 2 && need_record) fetch_record();
-                    ok = publish(n_item + 1);
-                }
-                published = false;
             }
             // the arrivals that rank 0's commits still owe this CTA's barriers come before it leaves
             if (ok && !*s_abort) {
@@ -893,29 +771,152 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 }
                 ++n_item;
             }
-        } else {
+        } else if (warp == kMmaWarp) {
             // ================================================================
-            // tell rank 0 that this CTA's half tiles have landed (warp 18: K and Q, warp 19: V)
+            // relay: tells rank 0 that this CTA's half tiles have landed.  V follows K two tiles behind, which is about when
+            // either is asked for, so that neither is told late; when no next record is out, V catches up first (the last
+            // record is not out before every item's V has been used).
             // ================================================================
-            const bool is_k = warp == kMmaWarp;
-            const uint32_t n_st = is_k ? kStagesK : kStagesV, full = is_k ? Bars::k_full : Bars::v_full;
-            uint32_t n_item = 0, n = 0;
+            uint32_t n_item = 0, n = 0, nv = 0;  // key tiles whose K, and V, has been told of
             bool ok = true;
             uint4 ra, rb;
-            while (ok && take_record(n_item, ra, rb, true)) {
+            auto tell_v = [&]() {
+                const uint32_t s = nv % kStagesV;
+                ok = wait_all(bars + Bars::v_full + 8 * s, (nv / kStagesV) & 1, s_abort);
+                if (ok && lane == 0) arrive_at(lead + Bars::v_full + 8 * s);
+                ++nv;
+            };
+            while (ok) {
+                if (!__all_sync(0xffffffffu, mbar_test_wait(bars + Bars::item_full + 8 * (n_item % kItemRing), (n_item / kItemRing) & 1)))
+                    while (ok && nv < n) tell_v();
+                if (!ok || !take_record(n_item, ra, rb, true)) break;
                 const int n_tiles = tiles_of(ra);
-                for (int j = 0; j < n_tiles; ++j, ++n) {
-                    const uint32_t s = n % n_st;
-                    ok = wait_all(bars + full + 8 * s, (n / n_st) & 1, s_abort);
+                for (int j = 0; j < n_tiles && ok; ++j) {
+                    const uint32_t s = n % kStagesK;
+                    ok = wait_all(bars + Bars::k_full + 8 * s, (n / kStagesK) & 1, s_abort);
                     if (!ok) break;
-                    if (lane == 0) arrive_at(lead + full + 8 * s);
-                    if (is_k && j == 0) {
+                    if (lane == 0) arrive_at(lead + Bars::k_full + 8 * s);
+                    if (j == 0) {
                         ok = wait_all(bars + Bars::q_full + 8 * (n_item & 1), (n_item >> 1) & 1, s_abort);
                         if (!ok) break;
                         if (lane == 0) arrive_at(lead + Bars::q_full + 8 * (n_item & 1));
                     }
+                    ++n;
+                    while (ok && nv + 2 < n) tell_v();
                 }
                 ++n_item;
+            }
+        } else {
+            // ================================================================
+            // items: fetches the pair's records, from its static share or the queue, and puts them into both CTAs' rings as
+            // slots come free.  (Done by the K producer between its copies, an item cost 4.0 us beyond its key tiles: some 200
+            // instructions that no hot loop keeps in the instruction cache, and two trips to L2.)
+            // ================================================================
+            const int pair = blockIdx.x >> 1;
+            int static_cur = 0, static_end = 0;
+            if (p.pair_start) {
+                static_cur = __ldg(p.pair_start + pair) + 1;
+                static_end = __ldg(p.pair_start + pair + 1);
+            }
+            uint32_t mode = kModePlain, redo_head = 0, redo_tail = 0;  // records put aside
+            uint4 fa = redo[0], fb = redo[1];                          // the record fetched; n_tok = 0: end of work
+            uint4 na, nb;                                              // the record published last
+            __syncwarp();  // (the ring of records put aside begins with the first one's place)
+            auto check_record = [&]() {
+                if ((int32_t)fb.y == 0) return;
+                // A record that points outside the batch (only a damaged work list has one) ends this pair's work and
+                // flags the run; nothing is read or written through it.
+                const int32_t r_req = (int32_t)fa.x, r_g = (int32_t)fa.y, r_kb = (int32_t)fa.z, r_ke = (int32_t)fa.w;
+                const int32_t r_q = (int32_t)fb.x, r_n = (int32_t)fb.y, r_slot = (int32_t)fb.z, r_pos = (int32_t)fb.w;
+                const bool rec_ok = (uint32_t)r_req < (uint32_t)p.n_req && (uint32_t)r_g < (uint32_t)p.Hkv && r_kb >= 0 &&
+                                    r_kb % kTileKeys == 0 && r_kb < r_ke && r_ke <= p.max_pages * kPage && r_n >= 1 &&
+                                    r_n <= 2 * tile_tok && r_q >= 0 && (int64_t)r_q + r_n <= p.total_q && r_pos >= 0 &&
+                                    (int64_t)r_pos + r_n >= r_ke &&
+                                    (r_slot < 0 || (int64_t)r_slot + (int64_t)r_n * p.G <= p.n_part_slots);
+                if (!rec_ok) {
+                    if (lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
+                    fa = fb = make_uint4(0, 0, 0, 0);
+                }
+            };
+            auto fetch_record = [&]() {
+                int idx = 0;
+                if (lane == 0) idx = next_item(static_cur, static_end);
+                ++static_cur;
+                idx = __shfl_sync(0xffffffffu, idx, 0);
+                fa = fb = make_uint4(0, 0, 0, 0);
+                if (idx < p.n_items) {
+                    fa = __ldg(reinterpret_cast<const uint4*>(p.items + idx));
+                    fb = __ldg(reinterpret_cast<const uint4*>(p.items + idx) + 1);
+                }
+                check_record();
+            };
+            // every consumer is done with the record that last used the slot of record n; if its item has to be run again,
+            // the record is put aside
+            auto reclaim = [&](uint32_t n) -> bool {
+                const uint32_t slot = n % kItemRing, par = ((n / kItemRing) & 1) ^ 1;
+                if (!wait_all(bars + Bars::item_empty + 8 * slot, par, s_abort)) return false;
+                acquire_cluster(bars + Bars::item_empty + 8 * slot, par);
+                const uint32_t mask = __ballot_sync(0xffffffffu, lane < 8 && again[8 * slot + (lane & 7)] != 0);
+                if (mask) {
+                    if (lane < 2) {
+                        uint4 x = ring[2 * slot + lane];
+                        if (lane == 1) x.y |= mask << 16;
+                        redo[2 * (redo_tail % kItemRing) + lane] = x;
+                    }
+                    ++redo_tail;
+                    if (lane < 8) again[8 * slot + lane] = 0;
+                    __syncwarp();
+                }
+                return true;
+            };
+            check_record();
+            uint32_t done = 0;  // records known to be given back
+            int out = 0;        // key tiles of the records published behind them
+            // publishes record n: the second pass of an item run again, the first one of the next such item, or the record
+            // fetched (which stays fetched in the first two cases)
+            bool ok = true;
+            for (uint32_t n = 0; ok; ++n) {
+                if (!reclaim(n)) break;
+                if (mode != kModeMax && redo_head == redo_tail && (int32_t)fb.y == 0) {
+                    // end of work, unless one of the items still under way has to be run again
+                    for (uint32_t k = 1; k < kItemRing && ok; ++k)
+                        if (n >= k) ok = reclaim(n - k + kItemRing);
+                    if (!ok) break;
+                }
+                bool from_fetched = false;
+                if (mode == kModeMax) {
+                    mode = kModeRelative;
+                } else if (redo_head != redo_tail) {
+                    na = redo[2 * (redo_head % kItemRing)];
+                    nb = redo[2 * (redo_head % kItemRing) + 1];
+                    ++redo_head;
+                    mode = kModeMax;
+                } else {
+                    na = fa;
+                    nb = fb;
+                    mode = kModePlain;
+                    from_fetched = true;
+                }
+                nb.y = (nb.y & 0xffffffu) | (mode << 24);
+                const uint32_t slot = n % kItemRing;
+                if (lane == 0) {
+                    ring[2 * slot] = na;
+                    ring[2 * slot + 1] = nb;
+                    mbar_arrive(bars + Bars::item_full + 8 * slot);
+                    store_at(lead + Bars::ring + 32 * slot, na);
+                    store_at(lead + Bars::ring + 32 * slot + 16, nb);
+                    arrive_at_release_cluster(lead + Bars::item_full + 8 * slot);
+                }
+                __syncwarp();
+                if (from_fetched && (int32_t)nb.y == 0) break;
+                // An item taken early from the queue is one that an idle pair cannot take: only one is, beyond kAheadTiles.  (And
+                // `done` stays within a ring of n: a slot's barrier tells its last two phases apart, no more.)
+                out += tiles_of(na);
+                for (; ok && done < n && (out > kAheadTiles || n - done >= kItemRing - 1); ++done) {
+                    ok = reclaim(done + kItemRing);
+                    out -= tiles_of(ring[2 * (done % kItemRing)]);
+                }
+                if (ok && from_fetched) fetch_record();
             }
         }
     }

@@ -63,6 +63,13 @@ def test_many_short_items_per_pair():
     run_and_compare(b, np.zeros(b.total_q), "many short items")
 
 
+@pytest.mark.parametrize("redo", [False, True])
+def test_more_one_tile_items_per_pair_than_records_fit_its_ring(redo):
+    """13 to 15 items of one key tile per pair; with ``redo`` every ninth token's rows are computed again as well."""
+    b = gen.make_batch(gen.SHAPE_8B, 955, [0, 40] * 65, [64, 33] * 65)
+    run_and_compare(b, np.where(np.arange(b.total_q) % 9 == 0, 6, 0) if redo else np.zeros(b.total_q), "one-tile items")
+
+
 @pytest.mark.parametrize("every", [1, 3, 97])
 @pytest.mark.parametrize("exp", [6, 9])
 def test_rows_out_of_range_are_computed_again(every, exp):
