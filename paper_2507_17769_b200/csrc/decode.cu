@@ -100,6 +100,195 @@ __device__ __forceinline__ bool piece_pages_ok(const int4& a, const DecodeParams
     return (uint32_t)a.x < (uint32_t)p.n_req && (uint32_t)a.y < (uint32_t)p.Hkv && a.z >= 0 && a.z < a.w && a.w <= p.max_pages;
 }
 
+// Both halves of a piece; false if something had to be replaced.
+__device__ __forceinline__ bool check_piece(const DecodeParams& p, int4& a, int4& b) {
+    bool ok = true;
+    if (!piece_pages_ok(a, p)) {
+        a = make_int4(0, 0, 0, 1);
+        ok = false;
+    }
+    if ((uint32_t)b.x >= (uint32_t)p.total_q) {
+        b.x = 0;
+        ok = false;
+    }
+    if (b.y >= 0 && ((int64_t)b.y + p.G > p.n_part_slots || (uint32_t)b.w >= (uint32_t)p.n_dmerge)) {
+        b.y = -1;
+        ok = false;
+    }
+    if (b.z <= (a.w - 1) * kPage) {  // the row's keys end inside the piece's last page or behind it
+        b.z = a.w * kPage;
+        ok = false;
+    }
+    return ok;
+}
+
+// What a warp has gathered of one (row, kv head): O^T fragments, and per head column the maximum and this thread's part of the sum.
+template <int D>
+struct Gathered {
+    float o[D / 16][4];
+    float m0, m1, l0, l1;
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int mt = 0; mt < D / 16; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
+        m0 = m1 = -INFINITY;
+        l0 = l1 = 0.f;
+    }
+    // column sums over the 8 row-groups of the fragment
+    __device__ __forceinline__ void sum_rows() {
+#pragma unroll
+        for (int k = 4; k <= 16; k <<= 1) {
+            l0 += __shfl_xor_sync(0xffffffffu, l0, k);
+            l1 += __shfl_xor_sync(0xffffffffu, l1, k);
+        }
+    }
+};
+
+// Q^T of one kv head's group as B fragments: thread holds head (lane / 4), d = 16 ks + 2 (lane % 4) + {0, 1} (+ 8)
+template <int D, bool FP8>
+__device__ __forceinline__ void load_q(const __nv_bfloat16* q, int64_t first_row, int G, int lane, uint32_t (&qb)[D / 16][2]) {
+    const int hh = lane >> 2;
+    const uint32_t* qrow = reinterpret_cast<const uint32_t*>(q + (first_row + hh) * D);
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+        if constexpr (FP8) {  // k-step ks covers d = 16 ks + 4 (lane % 4) + {0, 1 | 2, 3}: the order of the K bytes a thread gets
+            const uint32_t w0 = hh < G ? __ldg(qrow + ks * 8 + 2 * (lane & 3)) : 0u;
+            const uint32_t w1 = hh < G ? __ldg(qrow + ks * 8 + 2 * (lane & 3) + 1) : 0u;
+            qb[ks][0] = pack_f16(bf16_lo(w0), bf16_hi(w0));
+            qb[ks][1] = pack_f16(bf16_lo(w1), bf16_hi(w1));
+        } else {
+            qb[ks][0] = hh < G ? __ldg(qrow + ks * 8 + (lane & 3)) : 0u;
+            qb[ks][1] = hh < G ? __ldg(qrow + ks * 8 + 4 + (lane & 3)) : 0u;
+        }
+    }
+}
+
+// One page (its K, V in a shared-memory stage, nvalid >= 1 of its slots filled) into what the warp has gathered.
+template <int D, bool FP8>
+__device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nvalid, float scale_log2, const uint32_t (&qb)[D / 16][2],
+                                            Gathered<D>& a, int lane) {
+    using Cfg = DecodeCfg<D, FP8>;
+    constexpr int KS = D / 16;  // k-steps of QK^T == m-tiles of PV
+    const uint32_t vbase = kbase + Cfg::kBlockBytes;
+    const int row = lane >> 2;  // token rows row, row + 8 of S^T; d rows of O^T
+    const int mi = lane >> 3, l7 = lane & 7;
+    // ldmatrix row addresses (byte offsets inside a block, before the per-step unit term)
+    const uint32_t k_tok_off = (uint32_t)(((mi & 1) * 8 + l7) * 128);
+    const uint32_t v_tok_off = (uint32_t)(((mi >> 1) * 8 + l7) * 128);
+    if (nvalid < kPage) {
+        // Slots past the sequence end hold whatever the pool holds (possibly NaN):
+        // zero those V rows so that 0 * V stays 0; their scores are masked below.
+        char* vb = stage + Cfg::kBlockBytes;
+        const int units = (kPage - nvalid) * 8;  // 16-byte units per region of 16 rows x 128 bytes
+        for (int h = 0; h < Cfg::kBlockBytes / 2048; ++h)
+            for (int u = lane; u < units; u += 32)
+                *reinterpret_cast<uint4*>(vb + h * 2048 + nvalid * 128 + u * 16) = make_uint4(0, 0, 0, 0);
+        fence_proxy_async_smem();  // order these generic writes before the stage's next bulk copy
+        __syncwarp();
+    }
+
+    // S^T = K Q^T : 16 tokens x 8 head columns
+    float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+    float x0, x1, x2, x3;
+    float sv_lo = 1.f, sv_hi = 1.f;  // FP8: V scales of this thread's two token rows
+    if constexpr (FP8) {
+        // One ldmatrix brings 16 tokens x 32 bytes: the thread gets bytes d = 16 u + 4 (lane % 4) + {0..3} of rows
+        // `row` and `row + 8` for two 16-byte chunks u, each of which is one k-step after conversion.
+#pragma unroll
+        for (int kp = 0; kp < KS / 2; ++kp) {
+            const uint32_t unit = (uint32_t)(((kp * 2 + (mi >> 1)) & 7) ^ l7);
+            uint32_t r0, r1, r2, r3;
+            ldsm_x4(kbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
+            mma_16816_f16(sa, e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16),
+                          qb[2 * kp][0], qb[2 * kp][1]);
+            mma_16816_f16(sb, e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16),
+                          qb[2 * kp + 1][0], qb[2 * kp + 1][1]);
+        }
+        const float* scales = reinterpret_cast<const float*>(stage + 2 * Cfg::kBlockBytes);
+        const float fk_lo = scales[row] * scale_log2, fk_hi = scales[row + 8] * scale_log2;
+        x0 = (sa[0] + sb[0]) * fk_lo, x1 = (sa[1] + sb[1]) * fk_lo;
+        x2 = (sa[2] + sb[2]) * fk_hi, x3 = (sa[3] + sb[3]) * fk_hi;
+        // slots past the sequence end hold arbitrary scales: their weights are zero, keep 0 * scale = 0
+        sv_lo = row < nvalid ? scales[kPage + row] * kWeightScale : 0.f;
+        sv_hi = row + 8 < nvalid ? scales[kPage + row + 8] * kWeightScale : 0.f;
+    } else {
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            const uint32_t unit = (uint32_t)(((ks * 2 + (mi >> 1)) & 7) ^ l7);
+            uint32_t a0, a1, a2, a3;
+            ldsm_x4(kbase + (ks >> 2) * 2048 + k_tok_off + (unit << 4), a0, a1, a2, a3);
+            if (ks & 1) mma_16816(sb, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+            else mma_16816(sa, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+        }
+        x0 = (sa[0] + sb[0]) * scale_log2, x1 = (sa[1] + sb[1]) * scale_log2;
+        x2 = (sa[2] + sb[2]) * scale_log2, x3 = (sa[3] + sb[3]) * scale_log2;
+    }
+    if (row >= nvalid) x0 = x1 = -INFINITY;
+    if (row + 8 >= nvalid) x2 = x3 = -INFINITY;
+
+    float mx0 = fmaxf(x0, x2), mx1 = fmaxf(x1, x3);
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 4));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 4));
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 8));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 8));
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 16));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 16));
+    const float mn0 = fmaxf(a.m0, mx0), mn1 = fmaxf(a.m1, mx1);  // finite: token 0 of the page is valid
+    const float al0 = fast_exp2(a.m0 - mn0), al1 = fast_exp2(a.m1 - mn1);
+    a.m0 = mn0;
+    a.m1 = mn1;
+    const float p0 = fast_exp2(x0 - mn0), p1 = fast_exp2(x1 - mn1);
+    const float p2 = fast_exp2(x2 - mn0), p3 = fast_exp2(x3 - mn1);
+    // the row sum uses the bf16-rounded weights that PV multiplies, so that the
+    // normalised output is an exact convex mix of V rows
+    uint32_t pk0, pk1;
+    if constexpr (FP8) {
+        // each key's V scale rides on its weight into the MMA; the row sum is over the weights themselves
+        pk0 = pack_f16(p0 * sv_lo, p1 * sv_lo), pk1 = pack_f16(p2 * sv_hi, p3 * sv_hi);
+        a.l0 = a.l0 * al0 + p0 + p2;
+        a.l1 = a.l1 * al1 + p1 + p3;
+    } else {
+        pk0 = pack_bf16(p0, p1), pk1 = pack_bf16(p2, p3);
+        a.l0 = a.l0 * al0 + bf16_lo(pk0) + bf16_lo(pk1);
+        a.l1 = a.l1 * al1 + bf16_hi(pk0) + bf16_hi(pk1);
+    }
+    const uint32_t pb0 = movmatrix_t(pk0);
+    const uint32_t pb1 = movmatrix_t(pk1);
+
+    // O^T += V^T P^T : d x 8 head columns
+    if constexpr (FP8) {
+        // A transposed ldmatrix over 16-bit units hands the thread, per 16-byte chunk u, the bytes
+        // V[token 2c][d], V[token 2c][d + 1], V[token 2c + 1][d], V[token 2c + 1][d + 1] with d = 16 u + 2 row
+        // (tokens 2c, 2c + 1 of the first eight in one register, of the second eight in the next); a byte
+        // permute pairs the two tokens of one d, so accumulator row `row` is d and row `row + 8` is d + 1.
+#pragma unroll
+        for (int mp = 0; mp < KS / 2; ++mp) {
+            a.o[2 * mp][0] *= al0, a.o[2 * mp][1] *= al1, a.o[2 * mp][2] *= al0, a.o[2 * mp][3] *= al1;
+            a.o[2 * mp + 1][0] *= al0, a.o[2 * mp + 1][1] *= al1, a.o[2 * mp + 1][2] *= al0, a.o[2 * mp + 1][3] *= al1;
+            const uint32_t unit = (uint32_t)(((mp * 2 + (mi >> 1)) & 7) ^ l7);
+            uint32_t r0, r1, r2, r3;
+            ldsm_x4_t(vbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
+            r0 = __byte_perm(r0, 0, 0x3120), r1 = __byte_perm(r1, 0, 0x3120);
+            r2 = __byte_perm(r2, 0, 0x3120), r3 = __byte_perm(r3, 0, 0x3120);
+            mma_16816_f16(a.o[2 * mp], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r1 >> 16),
+                          pb0, pb1);
+            mma_16816_f16(a.o[2 * mp + 1], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r3 >> 16),
+                          pb0, pb1);
+        }
+    } else {
+#pragma unroll
+        for (int mt = 0; mt < KS; ++mt) {
+            a.o[mt][0] *= al0;
+            a.o[mt][1] *= al1;
+            a.o[mt][2] *= al0;
+            a.o[mt][3] *= al1;
+            const uint32_t unit = (uint32_t)(((mt * 2 + (mi & 1)) & 7) ^ l7);
+            uint32_t a0, a1, a2, a3;
+            ldsm_x4_t(vbase + (mt >> 2) * 2048 + v_tok_off + (unit << 4), a0, a1, a2, a3);
+            mma_16816(a.o[mt], a0, a1, a2, a3, pb0, pb1);
+        }
+    }
+}
+
 template <int D, bool FP8>
 __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodeParams p) {
     using Cfg = DecodeCfg<D, FP8>;
@@ -191,15 +380,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
     uint32_t n_cons = 0, cseq = 0;
 
     uint32_t qb[KS][2];
-    float o[KS][4];
-    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
+    Gathered<D> acc;
+    acc.clear();
 
     const int col = 2 * (lane & 3);  // this thread's head columns: col, col + 1
-    const int row = lane >> 2;       // token rows row, row + 8 of S^T; d rows of O^T
-    const int mi = lane >> 3, l7 = lane & 7;
-    // ldmatrix row addresses (byte offsets inside a block, before the per-step unit term)
-    const uint32_t k_tok_off = (uint32_t)(((mi & 1) * 8 + l7) * 128);
-    const uint32_t v_tok_off = (uint32_t)(((mi >> 1) * 8 + l7) * 128);
+    const int row = lane >> 2;       // d rows of O^T
 
     // Combine the partials of merge record midx (output token qtok, kv head g), in segment order.
     int n_deferred = 0;
@@ -285,17 +470,12 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
     };
 
     auto finalize = [&]() {
-        // column sums over the 8 row-groups of the fragment
-        l0 += __shfl_xor_sync(0xffffffffu, l0, 4);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 4);
-        l0 += __shfl_xor_sync(0xffffffffu, l0, 8);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 8);
-        l0 += __shfl_xor_sync(0xffffffffu, l0, 16);
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 16);
+        acc.sum_rows();
+        const float(&o)[KS][4] = acc.o;
         // (FP8: the accumulators hold the outputs times kWeightScale)
-        const float inv0 = (FP8 ? 1.f / kWeightScale : 1.f) / l0, inv1 = (FP8 ? 1.f / kWeightScale : 1.f) / l1;
-        const float lse0 = (m0 + log2f(l0)) * 0.6931471805599453f;
-        const float lse1 = (m1 + log2f(l1)) * 0.6931471805599453f;
+        const float inv0 = (FP8 ? 1.f / kWeightScale : 1.f) / acc.l0, inv1 = (FP8 ? 1.f / kWeightScale : 1.f) / acc.l1;
+        const float lse0 = (acc.m0 + log2f(acc.l0)) * 0.6931471805599453f;
+        const float lse1 = (acc.m1 + log2f(acc.l1)) * 0.6931471805599453f;
         const int h_base = C_g * p.G;
         // accumulator rows `row` and `row + 8` of m-tile mt hold d = 16 mt + row and + 8 -- in the FP8 variant, whose
         // transposed V fragments pair neighbouring bytes, d = 16 mt + 2 row and the next one
@@ -381,26 +561,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
             }
             int4 a = __ldg(reinterpret_cast<const int4*>(&p.pieces[C_piece]));
             int4 b = __ldg(reinterpret_cast<const int4*>(&p.pieces[C_piece]) + 1);
-            {
-                bool bad = false;
-                if (!piece_pages_ok(a, p)) {
-                    a = make_int4(0, 0, 0, 1);
-                    bad = true;
-                }
-                if ((uint32_t)b.x >= (uint32_t)p.total_q) {
-                    b.x = 0;
-                    bad = true;
-                }
-                if (b.y >= 0 && ((int64_t)b.y + p.G > p.n_part_slots || (uint32_t)b.w >= (uint32_t)p.n_dmerge)) {
-                    b.y = -1;
-                    bad = true;
-                }
-                if (b.z <= (a.w - 1) * kPage) {  // the row's keys end inside the piece's last page or behind it
-                    b.z = a.w * kPage;
-                    bad = true;
-                }
-                if (bad && lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
-            }
+            if (!check_piece(p, a, b) && lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
             C_g = a.y;
             C_page = a.z;
             C_page_end = a.w;
@@ -409,25 +570,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
             C_kvlen = b.z;
             C_midx = b.w;
             have_piece = true;
-            // Q^T as B fragments: thread holds head (lane / 4), d = 16 ks + 2 (lane % 4) + {0, 1} (+ 8)
-            const int hh = lane >> 2;
-            const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + ((int64_t)C_qtok * p.Hq + C_g * p.G + hh) * D);
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                if constexpr (FP8) {  // k-step ks covers d = 16 ks + 4 (lane % 4) + {0, 1 | 2, 3}: the order of the K bytes a thread gets
-                    const uint32_t w0 = hh < p.G ? __ldg(qrow + ks * 8 + 2 * (lane & 3)) : 0u;
-                    const uint32_t w1 = hh < p.G ? __ldg(qrow + ks * 8 + 2 * (lane & 3) + 1) : 0u;
-                    qb[ks][0] = pack_f16(bf16_lo(w0), bf16_hi(w0));
-                    qb[ks][1] = pack_f16(bf16_lo(w1), bf16_hi(w1));
-                } else {
-                    qb[ks][0] = hh < p.G ? __ldg(qrow + ks * 8 + (lane & 3)) : 0u;
-                    qb[ks][1] = hh < p.G ? __ldg(qrow + ks * 8 + 4 + (lane & 3)) : 0u;
-                }
-            }
-#pragma unroll
-            for (int mt = 0; mt < KS; ++mt) o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f;
-            m0 = m1 = -INFINITY;
-            l0 = l1 = 0.f;
+            load_q<D, FP8>(p.q, (int64_t)C_qtok * p.Hq + C_g * p.G, p.G, lane, qb);
+            acc.clear();
         }
 
         const uint32_t stage = n_cons % STAGES;
@@ -436,123 +580,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
             timed_out = true;
             break;
         }
-        const uint32_t kbase = stage0 + stage * Cfg::kStageBytes;
-        const uint32_t vbase = kbase + Cfg::kBlockBytes;
         const int nvalid = C_kvlen - C_page * kPage;  // >= 1
 
-        if (nvalid < kPage) {
-            // Slots past the sequence end hold whatever the pool holds (possibly NaN):
-            // zero those V rows so that 0 * V stays 0; their scores are masked below.
-            char* vb = my_stages + stage * Cfg::kStageBytes + Cfg::kBlockBytes;
-            const int units = (kPage - nvalid) * 8;  // 16-byte units per region of 16 rows x 128 bytes
-            for (int h = 0; h < Cfg::kBlockBytes / 2048; ++h)
-                for (int u = lane; u < units; u += 32)
-                    *reinterpret_cast<uint4*>(vb + h * 2048 + nvalid * 128 + u * 16) = make_uint4(0, 0, 0, 0);
-            fence_proxy_async_smem();  // order these generic writes before the stage's next bulk copy
-            __syncwarp();
-        }
-
-        // S^T = K Q^T : 16 tokens x 8 head columns
-        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
-        float x0, x1, x2, x3;
-        float sv_lo = 1.f, sv_hi = 1.f;  // FP8: V scales of this thread's two token rows
-        if constexpr (FP8) {
-            // One ldmatrix brings 16 tokens x 32 bytes: the thread gets bytes d = 16 u + 4 (lane % 4) + {0..3} of rows
-            // `row` and `row + 8` for two 16-byte chunks u, each of which is one k-step after conversion.
-#pragma unroll
-            for (int kp = 0; kp < KS / 2; ++kp) {
-                const uint32_t unit = (uint32_t)(((kp * 2 + (mi >> 1)) & 7) ^ l7);
-                uint32_t r0, r1, r2, r3;
-                ldsm_x4(kbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
-                mma_16816_f16(sa, e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16),
-                              qb[2 * kp][0], qb[2 * kp][1]);
-                mma_16816_f16(sb, e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16),
-                              qb[2 * kp + 1][0], qb[2 * kp + 1][1]);
-            }
-            const float* scales = reinterpret_cast<const float*>(my_stages + stage * Cfg::kStageBytes + 2 * Cfg::kBlockBytes);
-            const float fk_lo = scales[row] * p.scale_log2, fk_hi = scales[row + 8] * p.scale_log2;
-            x0 = (sa[0] + sb[0]) * fk_lo, x1 = (sa[1] + sb[1]) * fk_lo;
-            x2 = (sa[2] + sb[2]) * fk_hi, x3 = (sa[3] + sb[3]) * fk_hi;
-            // slots past the sequence end hold arbitrary scales: their weights are zero, keep 0 * scale = 0
-            sv_lo = row < nvalid ? scales[kPage + row] * kWeightScale : 0.f;
-            sv_hi = row + 8 < nvalid ? scales[kPage + row + 8] * kWeightScale : 0.f;
-        } else {
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t unit = (uint32_t)(((ks * 2 + (mi >> 1)) & 7) ^ l7);
-                uint32_t a0, a1, a2, a3;
-                ldsm_x4(kbase + (ks >> 2) * 2048 + k_tok_off + (unit << 4), a0, a1, a2, a3);
-                if (ks & 1) mma_16816(sb, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-                else mma_16816(sa, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-            }
-            x0 = (sa[0] + sb[0]) * p.scale_log2, x1 = (sa[1] + sb[1]) * p.scale_log2;
-            x2 = (sa[2] + sb[2]) * p.scale_log2, x3 = (sa[3] + sb[3]) * p.scale_log2;
-        }
-        if (row >= nvalid) x0 = x1 = -INFINITY;
-        if (row + 8 >= nvalid) x2 = x3 = -INFINITY;
-
-        float mx0 = fmaxf(x0, x2), mx1 = fmaxf(x1, x3);
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 4));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 4));
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 8));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 8));
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 16));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 16));
-        const float mn0 = fmaxf(m0, mx0), mn1 = fmaxf(m1, mx1);  // finite: token 0 of the page is valid
-        const float al0 = fast_exp2(m0 - mn0), al1 = fast_exp2(m1 - mn1);
-        m0 = mn0;
-        m1 = mn1;
-        const float p0 = fast_exp2(x0 - mn0), p1 = fast_exp2(x1 - mn1);
-        const float p2 = fast_exp2(x2 - mn0), p3 = fast_exp2(x3 - mn1);
-        // the row sum uses the bf16-rounded weights that PV multiplies, so that the
-        // normalised output is an exact convex mix of V rows
-        uint32_t pk0, pk1;
-        if constexpr (FP8) {
-            // each key's V scale rides on its weight into the MMA; the row sum is over the weights themselves
-            pk0 = pack_f16(p0 * sv_lo, p1 * sv_lo), pk1 = pack_f16(p2 * sv_hi, p3 * sv_hi);
-            l0 = l0 * al0 + p0 + p2;
-            l1 = l1 * al1 + p1 + p3;
-        } else {
-            pk0 = pack_bf16(p0, p1), pk1 = pack_bf16(p2, p3);
-            l0 = l0 * al0 + bf16_lo(pk0) + bf16_lo(pk1);
-            l1 = l1 * al1 + bf16_hi(pk0) + bf16_hi(pk1);
-        }
-        const uint32_t pb0 = movmatrix_t(pk0);
-        const uint32_t pb1 = movmatrix_t(pk1);
-
-        // O^T += V^T P^T : d x 8 head columns
-        if constexpr (FP8) {
-            // A transposed ldmatrix over 16-bit units hands the thread, per 16-byte chunk u, the bytes
-            // V[token 2c][d], V[token 2c][d + 1], V[token 2c + 1][d], V[token 2c + 1][d + 1] with d = 16 u + 2 row
-            // (tokens 2c, 2c + 1 of the first eight in one register, of the second eight in the next); a byte
-            // permute pairs the two tokens of one d, so accumulator row `row` is d and row `row + 8` is d + 1.
-#pragma unroll
-            for (int mp = 0; mp < KS / 2; ++mp) {
-                o[2 * mp][0] *= al0, o[2 * mp][1] *= al1, o[2 * mp][2] *= al0, o[2 * mp][3] *= al1;
-                o[2 * mp + 1][0] *= al0, o[2 * mp + 1][1] *= al1, o[2 * mp + 1][2] *= al0, o[2 * mp + 1][3] *= al1;
-                const uint32_t unit = (uint32_t)(((mp * 2 + (mi >> 1)) & 7) ^ l7);
-                uint32_t r0, r1, r2, r3;
-                ldsm_x4_t(vbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
-                r0 = __byte_perm(r0, 0, 0x3120), r1 = __byte_perm(r1, 0, 0x3120);
-                r2 = __byte_perm(r2, 0, 0x3120), r3 = __byte_perm(r3, 0, 0x3120);
-                mma_16816_f16(o[2 * mp], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r1 >> 16),
-                              pb0, pb1);
-                mma_16816_f16(o[2 * mp + 1], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r3 >> 16),
-                              pb0, pb1);
-            }
-        } else {
-#pragma unroll
-            for (int mt = 0; mt < KS; ++mt) {
-                o[mt][0] *= al0;
-                o[mt][1] *= al1;
-                o[mt][2] *= al0;
-                o[mt][3] *= al1;
-                const uint32_t unit = (uint32_t)(((mt * 2 + (mi & 1)) & 7) ^ l7);
-                uint32_t a0, a1, a2, a3;
-                ldsm_x4_t(vbase + (mt >> 2) * 2048 + v_tok_off + (unit << 4), a0, a1, a2, a3);
-                mma_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
-            }
-        }
+        attend_page<D, FP8>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, nvalid, p.scale_log2, qb, acc, lane);
 
         __syncwarp();  // every lane has read this stage
         ++C_page;
@@ -570,6 +600,172 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
     }
 }
 
+// Batches too small to give every warp of the GPU its share of pages: a CTA per piece of a (row, kv head), its warps taking
+// the piece's pages in turn, and what they have gathered combined in shared memory.  Such a batch is bound by a chain of
+// latencies (record, block table, pages, partial rows, arrival, partial rows again), not by bytes: here a warp has a few
+// pages, and only rows longer than a piece leave partial rows, a twelfth as many as one per warp.
+// Measured (32 q / 8 kv heads, kernel alone, before: a unit per warp): 8 rows of 512 tokens 17.0 -> 10.0 us, 16 of 600 19.1
+// -> 10.9, 8 of 1500 21.1 -> 12.9, one of 256 15.0 -> 8.9, one of 16384 41.8 -> 17.5.
+template <int D>
+struct CtaPart {  // what a warp leaves for the others, in the place of its stages
+    static constexpr int kRow = D + 4;  // floats; the pad spreads the fragment's rows over the banks
+    static constexpr int kBytes = 8 * kRow * 4;
+};
+template <int D, bool FP8>
+__global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const DecodeParams p, int n_pieces) {
+    using Cfg = DecodeCfg<D, FP8>;
+    constexpr int STAGES = Cfg::kStages;
+    constexpr int KS = D / 16;
+    static_assert(CtaPart<D>::kBytes <= STAGES * Cfg::kStageBytes, "a warp's part fits its stages");
+    extern __shared__ char smem_raw[];
+    char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ float s_m[kWarps][8], s_l[kWarps][8];
+    __shared__ int s_arrived;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    char* const my_stages = smem + (size_t)warp * STAGES * Cfg::kStageBytes;
+    const uint32_t stage0 = smem_u32(my_stages);
+    const uint32_t bar0 = smem_u32(smem + (size_t)kWarps * STAGES * Cfg::kStageBytes) + 8 * warp * STAGES;
+    if (lane == 0) {
+        for (int s = 0; s < STAGES; ++s) mbar_init(bar0 + 8 * s, 1);
+        mbar_fence_init();
+    }
+    __syncwarp();
+    pdl_trigger();
+    pdl_wait();
+    if ((int)blockIdx.x >= n_pieces) return;  // (a grid of CTA pairs)
+
+    int4 a = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]));
+    int4 b = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]) + 1);
+    if (!check_piece(p, a, b) && threadIdx.x == 0) atomicOr(&p.hdr->status, kStatusBounds);
+    const int first = a.z + warp, n_mine = a.w > first ? (a.w - first + kWarps - 1) / kWarps : 0;  // my pages: first + 12 i
+    const int32_t* const bt = p.block_table + (int64_t)a.x * p.max_pages + first;
+    const uint64_t kv_policy = l2_policy_evict_first();
+    int pages = lane < n_mine ? __ldg(bt + kWarps * lane) : 0;  // those of 32 turns, one a lane
+    auto produce = [&](int i) {
+        if (i > 0 && i % 32 == 0) pages = i + lane < n_mine ? __ldg(bt + kWarps * (i + lane)) : 0;
+        const int page = __shfl_sync(0xffffffffu, pages, i % 32);
+        if (lane == 0) {
+            const uint32_t bar = bar0 + 8 * (i % STAGES);
+            if ((uint32_t)page < (uint64_t)p.num_pages) {
+                mbar_expect_tx(bar, Cfg::kStageBytes);
+                bulk_g2s_hint(stage0 + (i % STAGES) * Cfg::kStageBytes, p.pool + ((int64_t)page * p.Hkv + a.y) * (int64_t)Cfg::kStageBytes,
+                              Cfg::kStageBytes, bar, kv_policy);
+            } else {
+                atomicOr(&p.hdr->status, kStatusBounds);
+                mbar_arrive(bar);  // complete the phase without data; the run is flagged invalid
+            }
+        }
+    };
+    int n_prod = 0, n_cons = 0;
+    while (n_prod < n_mine && n_prod < STAGES) produce(n_prod++);
+    uint32_t qb[KS][2];
+    const int64_t row0 = (int64_t)b.x * p.Hq + a.y * p.G;  // the group's first row of q and out
+    if (n_mine > 0) load_q<D, FP8>(p.q, row0, p.G, lane, qb);
+    Gathered<D> acc;
+    acc.clear();
+    bool timed_out = false;
+    for (; n_cons < n_mine; ++n_cons) {
+        const int stage = n_cons % STAGES;
+        if (!mbar_wait(bar0 + 8 * stage, (n_cons / STAGES) & 1, p.wait_limit_ns)) {
+            if (lane == 0) atomicOr(&p.hdr->status, kStatusTimeout);
+            timed_out = true;
+            break;
+        }
+        attend_page<D, FP8>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, b.z - (first + kWarps * n_cons) * kPage,
+                            p.scale_log2, qb, acc, lane);
+        __syncwarp();  // every lane has read this stage
+        if (n_prod < n_mine) produce(n_prod++);
+    }
+    if (timed_out)  // let the copies still in flight (the one waited for included) land before their place is used again
+        for (int n = n_cons; n < n_prod; ++n) mbar_wait(bar0 + 8 * (n % STAGES), (n / STAGES) & 1, kDrainLimitNs);
+
+    // ---- the warps' parts: O^T, maximum and sum per head column ----
+    acc.sum_rows();
+    const int col = 2 * (lane & 3), row = lane >> 2;
+    {
+        float* const part = reinterpret_cast<float*>(my_stages);
+        constexpr int kRowStep = FP8 ? 2 : 1, kPairStep = FP8 ? 1 : 8;  // rows of the accumulator: as in decode_kernel
+#pragma unroll
+        for (int mt = 0; mt < KS; ++mt) {
+            float* const o0 = part + col * CtaPart<D>::kRow + mt * 16 + kRowStep * row;
+            o0[0] = acc.o[mt][0];
+            o0[kPairStep] = acc.o[mt][2];
+            o0[CtaPart<D>::kRow] = acc.o[mt][1];
+            o0[CtaPart<D>::kRow + kPairStep] = acc.o[mt][3];
+        }
+        if (row == 0) {
+            s_m[warp][col] = acc.m0, s_m[warp][col + 1] = acc.m1;
+            s_l[warp][col] = acc.l0, s_l[warp][col + 1] = acc.l1;
+        }
+    }
+    __syncthreads();
+    // ---- combined: a thread takes four values of one head (G * D / 4 <= 256 threads have work) ----
+    const int t = threadIdx.x, h = t / (D / 4), d4 = t % (D / 4);
+    if (h < p.G) {
+        float m = s_m[0][h];  // (warp 0 has the piece's first page)
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) m = fmaxf(m, s_m[w][h]);
+        float l = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const float f = fast_exp2(s_m[w][h] - m);  // 0 for a warp without pages
+            l += f * s_l[w][h];
+            const float4 x = reinterpret_cast<const float4*>(smem + (size_t)w * STAGES * Cfg::kStageBytes)[h * (CtaPart<D>::kRow / 4) + d4];
+            o.x += f * x.x, o.y += f * x.y, o.z += f * x.z, o.w += f * x.w;
+        }
+        const float inv = (FP8 ? 1.f / kWeightScale : 1.f) / l;  // (FP8: the accumulators hold the outputs times kWeightScale)
+        const float lse = (m + log2f(l)) * 0.6931471805599453f;
+        o.x *= inv, o.y *= inv, o.z *= inv, o.w *= inv;
+        if (b.y < 0) {
+            reinterpret_cast<uint2*>(p.out + (row0 + h) * D)[d4] = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+            if (p.lse && d4 == 0) p.lse[row0 + h] = lse;
+        } else {
+            reinterpret_cast<float4*>(p.part_o + ((int64_t)b.y + h) * D)[d4] = o;
+            if (d4 == 0) p.part_lse[b.y + h] = lse;
+        }
+    }
+    if (b.y < 0) return;
+    // ---- the CTA that delivers a (row, kv head)'s last piece combines them, in segment order.  (Release and acquire as in
+    // decode_kernel: the barrier orders every thread's partial stores before the increment.) ----
+    const DecodeMerge dm = p.dmerge[b.w];
+    __syncthreads();
+    if (t == 0) asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(s_arrived) : "l"(p.dmerge_cnt + b.w) : "memory");
+    __syncthreads();
+    if (s_arrived != dm.n_seg - 1 || h >= p.G) return;
+    constexpr int kAhead = 8;  // segments whose values are requested before the first is used
+    const float* const lse_in = p.part_lse + dm.base + h;
+    const float4* const o_in = reinterpret_cast<const float4*>(p.part_o + ((int64_t)dm.base + h) * D) + d4;
+    float m = -INFINITY, den = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < dm.n_seg; s0 += kAhead) {
+        float4 x[kAhead];
+        float lw[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const int sk = min(s0 + k, dm.n_seg - 1);
+            lw[k] = s0 + k < dm.n_seg ? __ldcg(lse_in + (int64_t)sk * p.G) : -INFINITY;
+            x[k] = __ldcg(o_in + (int64_t)sk * p.G * (D / 4));
+        }
+        float mn = m;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) mn = fmaxf(mn, lw[k]);
+        const float al = __expf(m - mn);
+        m = mn;
+        den *= al;
+        o.x *= al, o.y *= al, o.z *= al, o.w *= al;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            const float w = __expf(lw[k] - m);
+            den += w;
+            o.x += w * x[k].x, o.y += w * x[k].y, o.z += w * x[k].z, o.w += w * x[k].w;
+        }
+    }
+    const float inv = 1.f / den;
+    reinterpret_cast<uint2*>(p.out + (row0 + h) * D)[d4] = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+    if (p.lse && d4 == 0) p.lse[row0 + h] = m + __logf(den);
+}
+
 }  // namespace
 
 int decode_warps_per_sm() { return kWarps; }
@@ -580,6 +776,7 @@ static ps_status launch_decode_d(const RunArgs& a) {
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
         PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+        PS_CUDA_TRY(cudaFuncSetAttribute(decode_cta_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
         return PS_OK;
     });
     if (cfg != PS_OK) return cfg;
@@ -608,17 +805,19 @@ static ps_status launch_decode_d(const RunArgs& a) {
     p.n_dmerge = a.w.n_dmerge;
     p.n_part_slots = a.w.n_part_slots;
     p.wait_limit_ns = a.wait_limit_ns;
-    int grid = (a.w.n_units + kWarps - 1) / kWarps;
+    int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + kWarps - 1) / kWarps;
     if (grid > a.dec_sms) grid = a.dec_sms;
     // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
     // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
     // before they have left.
     if (a.sm_pairs) grid = (grid + 1) / 2 * 2;
+    if (a.w.n_cta_pieces > 0)
+        return launch_kernel(decode_cta_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p, a.w.n_cta_pieces);
     return launch_kernel(decode_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
 }
 
 ps_status launch_decode(const RunArgs& a) {
-    if (a.w.n_units == 0) return PS_OK;
+    if (a.w.n_units == 0 && a.w.n_cta_pieces == 0) return PS_OK;
     if (a.shape.dtype == 1) return launch_decode_d<128, true>(a);  // the FP8 cache variant exists for head_dim 128
     return a.shape.head_dim == 128 ? launch_decode_d<128, false>(a) : launch_decode_d<64, false>(a);
 }

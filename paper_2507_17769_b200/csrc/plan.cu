@@ -28,6 +28,8 @@ constexpr int kDecodeUnitsPerWarp = 1;  // work units per resident warp (measure
 // 64 tokens: 13 us instead of 20; 8 rows of 512: 16 instead of 23), but every further piece of a row is one more
 // partial result for the one warp that combines them (one row of 4096 tokens: 22 us at 32 pieces, 26 at 64).
 constexpr int kDecodeMinPagesLo = 4, kDecodeMinPagesHi = 8, kDecodePiecesPerRow = 16;
+// A CTA per piece (small batches): pages a warp may get at most, and pages a warp gets before a row is cut.
+constexpr int kCtaPagesPerWarp = 8, kCtaMinPieceTurns = 4;
 constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 // Measured on B200 (bandwidth against the number of SMs the decode kernel runs on), used with the prefill kernel's cost
 // model to split the SMs of a mixed batch between the two kernels.
@@ -124,6 +126,7 @@ struct ps_plan {
     bool tiny_as_rows = false;  // this batch runs its chunks of a few tokens as decode rows
     std::vector<DecodePiece> pieces;
     std::vector<DecodeUnit> units;
+    bool cta_pieces = false;             // a CTA per piece, no units
     std::vector<PrefillItem> prefill;
     std::vector<MergeEntry> merge;       // prefill q tile pairs cut into segments: combined by the merge kernel
     std::vector<DecodeMerge> dmerge;     // combined inside the decode kernel
@@ -171,6 +174,65 @@ static int query_num_sms() {
     return sms;
 }
 
+// Batches too small for a share per warp: a CTA per piece.  Applies where every (row, kv head) gets a CTA of its own and no
+// piece leaves a warp more than kCtaPagesPerWarp pages -- where a warp's share would be the smallest unit, and a piece per
+// warp would be many partial rows.  Rows longer than kCtaMinPiece are cut as far as there are CTAs.
+static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start, int64_t total_pages,
+                             int64_t longest, int64_t* n_slots) {
+    const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv, warps = decode_warps_per_sm();
+    const int64_t max_piece = (int64_t)kCtaPagesPerWarp * warps;
+    if (total_pages > pl->dec_sms * max_piece) return false;
+    std::vector<std::pair<int32_t, int32_t>> rows;  // (request, keys the row sees)
+    for (int r = 0; r < pl->n; ++r) {
+        if (!runs_as_decode(pl->shape, pl->tiny_as_rows, prior[r], q_len[r])) continue;
+        if ((int64_t)(rows.size() + q_len[r]) * Hkv > pl->dec_sms) return false;
+        for (int i = 0; i < q_len[r]; ++i) rows.emplace_back(r, prior[r] + i + 1);
+    }
+    auto pages_of = [](int32_t keys) { return (int64_t)(keys + kPage - 1) / kPage; };
+    auto pieces_at = [&](int64_t piece) {
+        int64_t n = 0;
+        for (const auto& row : rows) n += (pages_of(row.second) + piece - 1) / piece;
+        return n * Hkv;
+    };
+    int64_t lo = kCtaMinPieceTurns * warps, hi = std::max(lo, longest);  // smallest piece that leaves no more pieces than CTAs
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (pieces_at(mid) <= pl->dec_sms) hi = mid; else lo = mid + 1;
+    }
+    if (lo > max_piece) return false;
+    pl->cta_pieces = true;
+    pl->info.decode_segment_tokens = (int32_t)(lo * kPage);
+    pl->pieces.clear();
+    pl->units.clear();
+    pl->dmerge.clear();
+    int32_t tok_req = -1, tok = 0;
+    for (const auto& row : rows) {
+        tok = row.first == tok_req ? tok + 1 : q_start[row.first];
+        tok_req = row.first;
+        const int64_t pages = pages_of(row.second), n_seg = (pages + lo - 1) / lo;
+        for (int g = 0; g < Hkv; ++g) {
+            for (int64_t s = 0; s < n_seg; ++s) {
+                DecodePiece pc{};
+                pc.req = row.first;
+                pc.kv_head = g;
+                pc.page_begin = (int32_t)(pages * s / n_seg);
+                pc.page_end = (int32_t)(pages * (s + 1) / n_seg);
+                pc.q_tok = tok;
+                pc.part_slot = n_seg > 1 ? (int32_t)(*n_slots + s * G) : -1;
+                pc.kv_len = row.second;
+                pc.merge_idx = n_seg > 1 ? (int32_t)pl->dmerge.size() : 0;
+                pl->pieces.push_back(pc);
+            }
+            if (n_seg > 1) {
+                pl->dmerge.push_back(DecodeMerge{(int32_t)*n_slots, (int32_t)n_seg});
+                *n_slots += n_seg * G;
+            }
+        }
+    }
+    pl->decode_merge_rows += (int64_t)pl->dmerge.size() * G;
+    return true;
+}
+
 static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,
                         const ps_plan_opts* opts, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
@@ -188,6 +250,9 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
         pl->dmerge.clear();
         return;
     }
+    pl->cta_pieces = false;
+    pl->info.decode_segment_tokens = 0;
+    if (!(opts && opts->decode_segment_tokens > 0) && plan_decode_ctas(pl, prior, q_len, q_start, total_pages, longest, n_slots)) return;
     const int64_t min_pages = std::min<int64_t>(kDecodeMinPagesHi, std::max<int64_t>(kDecodeMinPagesLo, (longest + kDecodePiecesPerRow - 1) / kDecodePiecesPerRow));
     int64_t per_unit;
     if (opts && opts->decode_segment_tokens > 0) {
@@ -663,7 +728,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     pl->info.total_q_tokens = T;
     pl->info.decode_sms = pl->dec_sms;
     pl->info.prefill_sms = pl->pf_sms;
-    pl->info.n_launches = (pl->concurrent && !pl->units.empty() && pl->prefill_cta_start.empty() && (int)pl->prefill.size() > pl->pf_workers ? 1 : 0) + (pl->units.empty() ? 0 : 1) + (pl->prefill.empty() ? 0 : 1) + (pl->merge.empty() ? 0 : 1);
+    pl->info.n_launches = (pl->concurrent && !pl->pieces.empty() && pl->prefill_cta_start.empty() && (int)pl->prefill.size() > pl->pf_workers ? 1 : 0) + (pl->pieces.empty() ? 0 : 1) + (pl->prefill.empty() ? 0 : 1) + (pl->merge.empty() ? 0 : 1);
     *plan_inout = pl;
     *workspace_bytes_out = pl->ws_bytes;
     return PS_OK;
@@ -807,6 +872,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.w.part_lse = (float*)(ws_base + pl->off_part_lse);
     a.w.part_o = (float*)(ws_base + pl->off_part_o);
     a.w.n_units = (int32_t)pl->units.size();
+    a.w.n_cta_pieces = pl->cta_pieces ? (int32_t)pl->pieces.size() : 0;
     a.w.n_prefill = (int32_t)pl->prefill.size();
     a.w.n_merge = (int32_t)pl->merge.size();
     a.w.n_dmerge = (int32_t)pl->dmerge.size();
