@@ -135,7 +135,7 @@ constexpr int64_t kMaxWaitLimitNs = 4000000000ll;  // the kernels time their wai
 constexpr int64_t kDrainLimitNs = 1000000000ll;
 
 struct WsHeader {         // 64 bytes at the start of the workspace
-    int32_t status;       // sticky OR of kStatus* seen by any kernel of the run
+    int32_t status;       // worst kStatus* seen by any kernel of the run, above it the run's tag (report())
     int32_t decode_next;  // dynamic work counters
     int32_t prefill_next;
     int32_t pad[13];
@@ -190,6 +190,17 @@ struct MergeEntry {
     int32_t pad[2];
 };
 
+// Work lists of small batches travel as kernel parameters: uploaded, a list costs its run an event between two streams (the
+// kernel began 3.6 us after the copy, 8 decode rows) and the host 2.5 us.
+constexpr int kInlinePieces = 148, kInlineItems = 64, kInlineStarts = 76;
+struct InlinePieces {
+    DecodePiece piece[kInlinePieces];
+};
+struct alignas(16) InlineItems {
+    PrefillItem item[kInlineItems];
+    int32_t start[kInlineStarts];  // the static partition
+};
+
 struct DeviceWork {       // pointers into the workspace for one run
     WsHeader* hdr;
     const DecodePiece* pieces;
@@ -221,6 +232,14 @@ struct RunArgs {
     int num_sms;
     int dec_sms, pf_sms;  // SMs (= CTAs) for the decode and the prefill kernel
     bool sm_pairs;        // side by side with the pair kernel: the decode kernel's CTAs take whole SM pairs too
+    // work lists as kernel parameters, on the host; null: they are in the workspace
+    const DecodePiece* inline_pieces;
+    const PrefillItem* inline_items;
+    const int32_t* inline_starts;
+    int32_t tag;          // of the run, a multiple of 4: status words of other runs in the same place are told apart by it
+    // The kernel does not wait for the one before it in the stream until its end: that is the same run's decode kernel, which
+    // lets it be launched only after all that came before has completed.
+    bool beside;
     bool early;           // the kernel may be launched while the one before it in the stream still runs
     int32_t total_q;      // q tokens of the batch (rows of q and out)
     int32_t n_req;        // requests of the batch (rows of the block table)
@@ -245,6 +264,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // Waits until the kernels before this one in the stream have completed and their results can be read; nothing that they may
 // write is read before it, and nothing that they may read is written.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// kStatus* of a run whose tag is `tag`
+__device__ __forceinline__ void report(WsHeader* hdr, int32_t tag, int32_t bits) { atomicMax(&hdr->status, tag | bits); }
 // The next kernel of the stream may be launched once every CTA has come by here.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

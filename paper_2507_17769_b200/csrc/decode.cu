@@ -18,6 +18,7 @@
 //     spanning several (request, kv head) pieces) fetched from one atomic
 //     counter; the producer side of the warp runs STAGES pages ahead of the
 //     consumer side, across piece and unit boundaries.
+#include <cstring>
 #include <type_traits>
 
 #include "common.cuh"
@@ -91,6 +92,7 @@ struct DecodeParams {
     int32_t n_req, total_q, n_dmerge;  // extents the work records are checked against
     int64_t n_part_slots;
     int64_t wait_limit_ns;
+    int32_t tag;
 };
 
 // A work record that points outside the batch (it can only come from a damaged work list) is replaced by one that
@@ -312,8 +314,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
         mbar_fence_init();
     }
     __syncwarp();
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // (in this order: a prefill kernel beside this one relies on all before it being complete)
 
     // K/V pages are read once: marked first to go in L2, they leave the partial rows, Q and the work list resident
     // (measured: 100.9 -> 96.9 us on the 64-sequence decode batch, 465.6 -> 452.7 us on 512 sequences)
@@ -363,7 +365,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
                 bulk_g2s_hint(stage0 + stage * Cfg::kStageBytes,
                               p.pool + ((int64_t)page * p.Hkv + P_g) * (int64_t)Cfg::kStageBytes, Cfg::kStageBytes, bar, kv_policy);
             } else {
-                atomicOr(&p.hdr->status, kStatusBounds);
+                report(p.hdr, p.tag, kStatusBounds);
                 mbar_arrive(bar);  // complete the phase without data; the run is flagged invalid
             }
         }
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
             }
             int4 a = __ldg(reinterpret_cast<const int4*>(&p.pieces[C_piece]));
             int4 b = __ldg(reinterpret_cast<const int4*>(&p.pieces[C_piece]) + 1);
-            if (!check_piece(p, a, b) && lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
+            if (!check_piece(p, a, b) && lane == 0) report(p.hdr, p.tag, kStatusBounds);
             C_g = a.y;
             C_page = a.z;
             C_page_end = a.w;
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
 
         const uint32_t stage = n_cons % STAGES;
         if (!mbar_wait(bar0 + 8 * stage, (n_cons / STAGES) & 1, p.wait_limit_ns)) {
-            if (lane == 0) atomicOr(&p.hdr->status, kStatusTimeout);
+            if (lane == 0) report(p.hdr, p.tag, kStatusTimeout);
             timed_out = true;
             break;
         }
@@ -612,7 +614,7 @@ struct CtaPart {  // what a warp leaves for the others, in the place of its stag
     static constexpr int kBytes = 8 * kRow * 4;
 };
 template <int D, bool FP8>
-__global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const DecodeParams p, int n_pieces) {
+__global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const DecodeParams p, int n_pieces, const __grid_constant__ InlinePieces inl) {
     using Cfg = DecodeCfg<D, FP8>;
     constexpr int STAGES = Cfg::kStages;
     constexpr int KS = D / 16;
@@ -630,13 +632,20 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const Decode
         mbar_fence_init();
     }
     __syncwarp();
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();  // (as in decode_kernel)
     if ((int)blockIdx.x >= n_pieces) return;  // (a grid of CTA pairs)
 
-    int4 a = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]));
-    int4 b = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]) + 1);
-    if (!check_piece(p, a, b) && threadIdx.x == 0) atomicOr(&p.hdr->status, kStatusBounds);
+    int4 a, b;
+    if (p.pieces) {
+        a = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]));
+        b = __ldg(reinterpret_cast<const int4*>(&p.pieces[blockIdx.x]) + 1);
+    } else {
+        const DecodePiece& pc = inl.piece[blockIdx.x];
+        a = make_int4(pc.req, pc.kv_head, pc.page_begin, pc.page_end);
+        b = make_int4(pc.q_tok, pc.part_slot, pc.kv_len, pc.merge_idx);
+    }
+    if (!check_piece(p, a, b) && threadIdx.x == 0) report(p.hdr, p.tag, kStatusBounds);
     const int first = a.z + warp, n_mine = a.w > first ? (a.w - first + kWarps - 1) / kWarps : 0;  // my pages: first + 12 i
     const int32_t* const bt = p.block_table + (int64_t)a.x * p.max_pages + first;
     const uint64_t kv_policy = l2_policy_evict_first();
@@ -651,7 +660,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const Decode
                 bulk_g2s_hint(stage0 + (i % STAGES) * Cfg::kStageBytes, p.pool + ((int64_t)page * p.Hkv + a.y) * (int64_t)Cfg::kStageBytes,
                               Cfg::kStageBytes, bar, kv_policy);
             } else {
-                atomicOr(&p.hdr->status, kStatusBounds);
+                report(p.hdr, p.tag, kStatusBounds);
                 mbar_arrive(bar);  // complete the phase without data; the run is flagged invalid
             }
         }
@@ -667,7 +676,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const Decode
     for (; n_cons < n_mine; ++n_cons) {
         const int stage = n_cons % STAGES;
         if (!mbar_wait(bar0 + 8 * stage, (n_cons / STAGES) & 1, p.wait_limit_ns)) {
-            if (lane == 0) atomicOr(&p.hdr->status, kStatusTimeout);
+            if (lane == 0) report(p.hdr, p.tag, kStatusTimeout);
             timed_out = true;
             break;
         }
@@ -805,14 +814,21 @@ static ps_status launch_decode_d(const RunArgs& a) {
     p.n_dmerge = a.w.n_dmerge;
     p.n_part_slots = a.w.n_part_slots;
     p.wait_limit_ns = a.wait_limit_ns;
+    p.tag = a.tag;
     int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + kWarps - 1) / kWarps;
     if (grid > a.dec_sms) grid = a.dec_sms;
     // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
     // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
     // before they have left.
     if (a.sm_pairs) grid = (grid + 1) / 2 * 2;
-    if (a.w.n_cta_pieces > 0)
-        return launch_kernel(decode_cta_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p, a.w.n_cta_pieces);
+    if (a.w.n_cta_pieces > 0) {
+        InlinePieces inl;  // (entries past the list's end are not read)
+        if (a.inline_pieces) {
+            p.pieces = nullptr;
+            memcpy(inl.piece, a.inline_pieces, a.w.n_cta_pieces * sizeof(DecodePiece));
+        }
+        return launch_kernel(decode_cta_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p, a.w.n_cta_pieces, inl);
+    }
     return launch_kernel(decode_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
 }
 

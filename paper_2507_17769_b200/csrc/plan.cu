@@ -161,6 +161,11 @@ struct ps_plan {
     unsigned run_no = 0;
     void* last_ws = nullptr;
     WsHeader* last_hdr = nullptr;
+    int32_t last_tag = 0;
+    // Small batches: the work list travels as kernel parameters, the run needs no workspace, and its status word is here.
+    bool inline_list = false;
+    WsHeader* own_hdr = nullptr;
+    uint32_t inline_runs = 0;
     // optional per-kernel timing: 6 events per recorded run (begin/end of prefill, decode, merge)
     bool timing = false;
     std::vector<cudaEvent_t> tev;
@@ -194,7 +199,9 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
         for (const auto& row : rows) n += (pages_of(row.second) + piece - 1) / piece;
         return n * Hkv;
     };
-    int64_t lo = kCtaMinPieceTurns * warps, hi = std::max(lo, longest);  // smallest piece that leaves no more pieces than CTAs
+    // Uncut if that leaves no warp too many pages (a list without merges need not be uploaded); else the smallest piece that
+    // leaves no more pieces than CTAs.
+    int64_t lo = std::max<int64_t>(kCtaMinPieceTurns * warps, longest <= max_piece ? longest : 0), hi = std::max(lo, longest);
     while (lo < hi) {
         const int64_t mid = (lo + hi) / 2;
         if (pieces_at(mid) <= pl->dec_sms) hi = mid; else lo = mid + 1;
@@ -646,6 +653,9 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     int64_t n_slots = 0;
     plan_decode(pl, prior_host, q_len_host, q_start, opts, &n_slots);
     plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);
+    pl->inline_list = (pl->pieces.empty() || (pl->cta_pieces && pl->dmerge.empty() && pl->pieces.size() <= kInlinePieces)) &&
+                      (pl->prefill.empty() || (pl->prefill.size() <= kInlineItems && pl->merge.empty() && !pl->prefill_cta_start.empty() &&
+                                               pl->prefill_cta_start.size() <= kInlineStarts));
     if (n_slots > 0x7fffffffLL) {
         if (fresh) delete pl;
         return fail(PS_ERR_UNSUPPORTED, "partial buffer would need %lld slots", (long long)n_slots);
@@ -705,6 +715,12 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             pl->copy_stream = nullptr;  // uploads then go on the caller's stream
             if (pl->side_stream) cudaStreamDestroy(pl->side_stream);
             pl->side_stream = nullptr;  // mixed batches then run their two kernels one after the other
+        } else if (cudaMalloc((void**)&pl->own_hdr, sizeof(WsHeader)) != cudaSuccess ||
+                   cudaMemsetAsync(pl->own_hdr, 0, sizeof(WsHeader), pl->copy_stream) != cudaSuccess ||
+                   cudaStreamSynchronize(pl->copy_stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            if (pl->own_hdr) cudaFree(pl->own_hdr);
+            pl->own_hdr = nullptr;  // every list is uploaded then
         }
     }
     memset(pl->pinned, 0, 256);
@@ -753,6 +769,7 @@ ps_status ps_plan_free(ps_plan* pl) {
     if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
     if (pl->ev_join) cudaEventDestroy(pl->ev_join);
     for (cudaEvent_t e : pl->tev) cudaEventDestroy(e);
+    if (pl->own_hdr) cudaFree(pl->own_hdr);  // (waits for the kernels that may still write it)
     if (pl->pinned) { if (pl->pinned_is_cuda) cudaFreeHost(pl->pinned); else free(pl->pinned); }
     delete pl;
     return PS_OK;
@@ -809,9 +826,11 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     // The upload may run under the kernels of the previous run only if this plan's own record of the two slots is
     // all there is to know about the workspace: same memory as last time, slots where they were, and no other
     // plan's run on it since.
-    const bool mine = claim_workspace(workspace_dev, pl->serial);
-    const bool known = mine && pl->last_ws == workspace_dev && !pl->layout_moved;
-    if (capturing) {
+    const bool as_params = pl->inline_list && pl->own_hdr && !capturing;  // (a graph's replays copy the staging image)
+    const bool known = !as_params && claim_workspace(workspace_dev, pl->serial) && pl->last_ws == workspace_dev && !pl->layout_moved;
+    if (as_params) {
+        // nothing to upload, and nothing of the workspace is used
+    } else if (capturing) {
         // Inside a stream capture the upload is a node of the graph on the caller's stream: every replay copies the
         // staging image as it then stands.  Nothing recorded here may be waited for by a later call outside the
         // capture, so the slot bookkeeping starts afresh.
@@ -841,11 +860,18 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
         PS_CUDA_TRY(cudaStreamSynchronize(s));  // no event to guard the staging image: finish the copy now
     }
     // the upload is in place (or queued): only now does the run count
-    ++pl->run_no;
-    pl->layout_moved = false;
-    pl->last_ws = workspace_dev;
-    pl->last_hdr = (WsHeader*)ws;
-    pl->done_valid[slot] = false;  // until this run's own completion event is recorded below
+    if (as_params) {
+        pl->inline_runs = pl->inline_runs % 0x1fffffffu + 1;
+        pl->last_hdr = pl->own_hdr;
+        pl->last_tag = (int32_t)(pl->inline_runs << 2);
+    } else {
+        ++pl->run_no;
+        pl->layout_moved = false;
+        pl->last_ws = workspace_dev;
+        pl->last_hdr = (WsHeader*)ws;
+        pl->last_tag = 0;
+        pl->done_valid[slot] = false;  // until this run's own completion event is recorded below
+    }
 
     RunArgs a{};
     a.shape = pl->shape;
@@ -864,7 +890,13 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.n_req = pl->n;
     a.wait_limit_ns = pl->wait_limit_ns;
     a.early = !capturing;
-    a.w.hdr = (WsHeader*)ws;
+    if (as_params) {
+        a.inline_pieces = pl->pieces.data();
+        a.inline_items = pl->prefill.empty() ? nullptr : pl->prefill.data();
+        a.inline_starts = pl->prefill_cta_start.data();
+    }
+    a.tag = pl->last_tag;
+    a.w.hdr = pl->last_hdr;
     a.w.pieces = (const DecodePiece*)(ws + pl->off_pieces);
     a.w.units = (const DecodeUnit*)(ws + pl->off_units);
     a.w.prefill = (const PrefillItem*)(ws + pl->off_prefill);
@@ -887,7 +919,22 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     cudaEvent_t* ev = rec ? &pl->tev[(size_t)pl->timed_runs * 6] : nullptr;
     ps_status st = PS_OK;
     bool merged = false;  // the merge kernel has been launched already
-    if (pl->concurrent && pl->side_stream) {
+    if (as_params && pl->concurrent) {
+        // Small mixed batch: both kernels on the caller's stream, the prefill kernel launched as soon as the decode kernel has
+        // begun and waiting for its end only at its own.  (A second stream costs two events, which take some 3 us each between
+        // kernels, as much as such a kernel takes.)
+        RunArgs ad = a;
+        ad.sm_pairs = pl->pf_workers < pl->pf_sms;
+        if (rec) cudaEventRecord(ev[2], s);
+        st = launch_decode(ad);
+        if (rec && st == PS_OK) cudaEventRecord(ev[3], s);
+        if (rec && st == PS_OK) cudaEventRecord(ev[0], s);
+        RunArgs ap = a;
+        ap.beside = true;
+        if (st == PS_OK) st = launch_prefill(ap);
+        if (rec && st == PS_OK) cudaEventRecord(ev[1], s);
+        if (st != PS_OK) return st;
+    } else if (pl->concurrent && pl->side_stream) {
         // Mixed batch: the decode kernel runs on its share of the SMs on a second stream while the
         // prefill kernel runs on the rest.  Both need about 200 KB of shared memory per CTA, so each SM
         // holds one CTA of either kernel.
@@ -947,7 +994,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
         if (rec) cudaEventRecord(ev[5], s);
     }
     if (rec) ++pl->timed_runs;
-    if (pl->copy_stream && st == PS_OK && !capturing) {
+    if (pl->copy_stream && st == PS_OK && !capturing && !as_params) {
         PS_CUDA_TRY(cudaEventRecord(pl->ev_done[slot], s));
         pl->done_valid[slot] = true;
     }
@@ -1000,6 +1047,7 @@ ps_status ps_plan_status(ps_plan* pl, void* stream) {
     if (!pl->last_hdr) return PS_OK;
     int32_t status = 0;
     PS_CUDA_TRY(cudaMemcpy(&status, &pl->last_hdr->status, sizeof status, cudaMemcpyDeviceToHost));
+    status = (status & ~3) == pl->last_tag ? status & 3 : 0;  // (else an earlier run's)
     if (status & kStatusTimeout) return fail(PS_ERR_TIMEOUT, "a bounded device-side wait expired; output is invalid");
     if (status & kStatusBounds) return fail(PS_ERR_BOUNDS, "a block-table entry pointed outside the pool");
     return PS_OK;

@@ -87,6 +87,8 @@ struct PrefillParams {
     int32_t n_items;
     int32_t Hq, Hkv, G;
     int32_t n_req, total_q, n_part_slots;  // extents the item records are checked against
+    int32_t tag;
+    int16_t inline_list, beside;
 };
 static_assert(sizeof(PrefillParams) <= 128, "parameter block");
 
@@ -108,7 +110,7 @@ static_assert(Bars::mma_drained % 8 == 0 && Bars::armed + 24 <= Bars::ring && si
               "barrier block layout");
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map) {
+__global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map, const __grid_constant__ InlineItems inl) {
     using Cfg = PrefillCfg<D>;
     extern __shared__ char smem_raw[];
     char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         tmem_alloc(bars + Bars::tmem_slot, Cfg::kTmemCols);
         tmem_relinquish();
     }
-    pdl_wait();
+    if (!p.beside) pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -447,21 +449,29 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
             const int pg = lane >> 2, which = lane & 3;  // page in tile; 0/1 = K half 0/1, 2/3 = V half 0/1
             constexpr uint32_t kPieceBytes = kPage * 128;  // 16 tokens x 64 elements
             uint32_t n_item = 0, tile_ctr = 0, items_x[2] = {0, 0};
-            int static_cur = p.cta_start ? p.cta_start[blockIdx.x] : 0;
-            const int static_end = p.cta_start ? p.cta_start[blockIdx.x + 1] : 0;
+            const bool static_share = p.inline_list || p.cta_start;
+            auto start_of = [&](int cta) { return p.inline_list ? inl.start[cta] : p.cta_start ? p.cta_start[cta] : 0; };
+            int static_cur = start_of(blockIdx.x);
+            const int static_end = start_of(blockIdx.x + 1);
             bool ok = true;
             while (ok) {
                 // next item of this CTA's static share, or of the queue all CTAs of the run drain
                 int idx = 0;
                 if (lane == 0)
-                    idx = p.cta_start ? (static_cur < static_end ? static_cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1);
+                    idx = static_share ? (static_cur < static_end ? static_cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1);
                 ++static_cur;
                 idx = __shfl_sync(0xffffffffu, idx, 0);
                 uint4 rec0 = make_uint4(0, 0, 0, 0), rec1 = make_uint4(0, 0, 0, 0);  // n_tok = 0: end of work
                 if (idx < p.n_items) {
-                    const uint4* src = reinterpret_cast<const uint4*>(p.items + idx);
-                    rec0 = __ldg(src);
-                    rec1 = __ldg(src + 1);
+                    if (p.inline_list) {
+                        const PrefillItem& it = inl.item[idx];
+                        rec0 = make_uint4(it.req, it.kv_head, it.key_begin, it.key_end);
+                        rec1 = make_uint4(it.q_tok, it.n_tok, it.part_slot, it.first_pos);
+                    } else {
+                        const uint4* src = reinterpret_cast<const uint4*>(p.items + idx);
+                        rec0 = __ldg(src);
+                        rec1 = __ldg(src + 1);
+                    }
                     // A record that points outside the batch (only a damaged work list has one) ends this CTA's
                     // work and flags the run; nothing is read or written through it.
                     const int32_t r_req = (int32_t)rec0.x, r_g = (int32_t)rec0.y, r_kb = (int32_t)rec0.z, r_ke = (int32_t)rec0.w;
@@ -472,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                                         (int64_t)r_pos + r_n >= r_ke &&
                                         (r_slot < 0 || (int64_t)r_slot + (int64_t)r_n * p.G <= p.n_part_slots);
                     if (!rec_ok) {
-                        if (lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
+                        if (lane == 0) report(p.hdr, p.tag, kStatusBounds);
                         rec0 = rec1 = make_uint4(0, 0, 0, 0);
                     }
                 }
@@ -500,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                     const int page = (lane < n_pages) ? __ldg(bt + j * 8 + lane) : 0;
                     const bool in_range = (uint32_t)page < (uint64_t)p.num_pages;
                     const uint32_t good = __ballot_sync(0xffffffffu, lane < n_pages && in_range);
-                    if (__popc(good) != n_pages && lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
+                    if (__popc(good) != n_pages && lane == 0) report(p.hdr, p.tag, kStatusBounds);
                     const int my_page = __shfl_sync(0xffffffffu, page, pg);
                     const bool mine = (good >> pg) & 1u;
                     const uint32_t tile_bytes = (uint32_t)__popc(good) * Cfg::kHalves * kPieceBytes;
@@ -660,7 +670,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         // A bounded wait ran out somewhere in this CTA: the output is invalid and the run is flagged.  Before the CTA
         // gives back its shared and tensor memory, the copies the producer has requested get a bounded time to land
         // and the MMAs issued so far (they read shared memory and write tensor memory) to retire.
-        if (threadIdx.x == 0) atomicOr(&p.hdr->status, kStatusTimeout);
+        if (threadIdx.x == 0) report(p.hdr, p.tag, kStatusTimeout);
         if (warp == kProducerWarp) {
             for (int k = 0; k < 2; ++k) {
                 const int ak = s_armed[k], av = s_armed[2 + k], aq = s_armed[4 + k];
@@ -677,6 +687,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         tc_fence_before();
         __syncthreads();
     }
+    if (p.beside) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
     if (warp == 0) tmem_dealloc(tmem, Cfg::kTmemCols);
 }
 
@@ -712,12 +723,18 @@ static ps_status launch_prefill_d(const RunArgs& a) {
     p.n_part_slots = (int32_t)a.w.n_part_slots;
     p.wait_limit_ns = (uint32_t)a.wait_limit_ns;
 
+    p.tag = a.tag;
+    p.inline_list = a.inline_items != nullptr;
+    p.beside = a.beside;
+    InlineItems inl;
+    fill_inline_items(a, inl);
+
     CUtensorMap q_map;
     const ps_status enc = encode_q_map(a, &q_map);
     if (enc != PS_OK) return enc;
 
     const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
-    return launch_kernel(prefill_kernel<D>, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map);
+    return launch_kernel(prefill_kernel<D>, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
 }
 
 ps_status launch_prefill(const RunArgs& a) {

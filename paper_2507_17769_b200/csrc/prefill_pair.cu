@@ -121,8 +121,10 @@ struct PairParams {
     int32_t n_items;
     int32_t Hq, Hkv, G;
     int32_t n_req, total_q, n_part_slots;  // extents the item records are checked against
-    int32_t out_aligned32;
+    int32_t tag;
+    int32_t flags;
 };
+constexpr int32_t kOutAligned32 = 1, kInlineList = 2, kBeside = 4;
 static_assert(sizeof(PairParams) <= 128, "parameter block");
 
 // ---- cluster-wide variants of the wrappers ----------------------------------
@@ -272,7 +274,7 @@ __device__ __forceinline__ void store32(char* dst, const uint32_t* v, bool align
     }
 }
 __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairParams p, const __grid_constant__ CUtensorMap q_map,
-                                                                    const __grid_constant__ CUtensorMap pool_map) {
+                                                                    const __grid_constant__ CUtensorMap pool_map, const __grid_constant__ InlineItems inl) {
     extern __shared__ char smem_raw[];
     char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -300,13 +302,27 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     uint4* const ring = reinterpret_cast<uint4*>(smem + kOffBar + Bars::ring);  // two uint4 per record
     uint4* const redo = reinterpret_cast<uint4*>(smem + kOffBar + Bars::redo);
     // next item of this pair's static share, or of the queue all pairs of the run drain
-    auto next_item = [&](int cur, int end) { return p.pair_start ? (cur < end ? cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1); };
+    const bool inline_list = (p.flags & kInlineList) != 0, static_share = inline_list || p.pair_start != nullptr;
+    auto next_item = [&](int cur, int end) { return static_share ? (cur < end ? cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1); };
+    auto start_of = [&](int pair) { return inline_list ? inl.start[pair] : __ldg(p.pair_start + pair); };
+    auto record = [&](int idx, uint4& a, uint4& b) {
+        if (inline_list) {
+            const PrefillItem& it = inl.item[idx];
+            a = make_uint4(it.req, it.kv_head, it.key_begin, it.key_end);
+            b = make_uint4(it.q_tok, it.n_tok, it.part_slot, it.first_pos);
+        } else {
+            a = __ldg(reinterpret_cast<const uint4*>(p.items + idx));
+            b = __ldg(reinterpret_cast<const uint4*>(p.items + idx) + 1);
+        }
+    };
     if (rank == 1 && threadIdx.x == kItemWarp * 32) {
         // the first item's record is on its way before the pair meets
         const int pair = blockIdx.x >> 1;
-        const int idx = next_item(p.pair_start ? __ldg(p.pair_start + pair) : 0, p.pair_start ? __ldg(p.pair_start + pair + 1) : 0);
-        redo[0] = idx < p.n_items ? __ldg(reinterpret_cast<const uint4*>(p.items + idx)) : make_uint4(0, 0, 0, 0);
-        redo[1] = idx < p.n_items ? __ldg(reinterpret_cast<const uint4*>(p.items + idx) + 1) : make_uint4(0, 0, 0, 0);
+        const int idx = next_item(static_share ? start_of(pair) : 0, static_share ? start_of(pair + 1) : 0);
+        uint4 a = make_uint4(0, 0, 0, 0), b = a;
+        if (idx < p.n_items) record(idx, a, b);
+        redo[0] = a;
+        redo[1] = b;
     }
     for (int k = threadIdx.x; k < Bars::n_bars; k += kThreads) {
         const int off = 8 * k;
@@ -324,7 +340,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     if (threadIdx.x < Bars::n_armed) s_armed[threadIdx.x] = -1;
     tc_fence_before();
     __syncthreads();
-    pdl_wait();
+    if (!(p.flags & kBeside)) pdl_wait();
     cluster_sync();  // the peer's barriers are initialised before anything arrives at them
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(smem + kOffBar + Bars::tmem_slot), 0);
@@ -563,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
 #pragma unroll
                             for (int c = 0; c < 8; ++c)
                                 x[c] = pack_bf16(__uint_as_float(v[u >> 1][(u & 1) * 16 + 2 * c]) * inv, __uint_as_float(v[u >> 1][(u & 1) * 16 + 2 * c + 1]) * inv);
-                            store32(dst + 32 * u, x, p.out_aligned32);
+                            store32(dst + 32 * u, x, p.flags & kOutAligned32);
                         }
                     } else {
                         char* dst = reinterpret_cast<char*>(p.part_o + prow * D + h * 64);
@@ -607,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 // lane, requested four tiles ahead; -8 for a page that is not there.
                 auto pool_row = [&](int page, int idx) {
                     const bool has = idx < n_pages, good = has && (uint32_t)page < (uint64_t)p.num_pages;
-                    if (has && !good) atomicOr(&p.hdr->status, kStatusBounds);
+                    if (has && !good) report(p.hdr, p.tag, kStatusBounds);
                     return good ? (page * p.Hkv + kv_head) * 4 : -8;
                 };
                 int row = -8, bt_next = lane < n_pages ? __ldg(bt + lane) : 0;
@@ -814,9 +830,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
             // ================================================================
             const int pair = blockIdx.x >> 1;
             int static_cur = 0, static_end = 0;
-            if (p.pair_start) {
-                static_cur = __ldg(p.pair_start + pair) + 1;
-                static_end = __ldg(p.pair_start + pair + 1);
+            if (static_share) {
+                static_cur = start_of(pair) + 1;
+                static_end = start_of(pair + 1);
             }
             uint32_t mode = kModePlain, redo_head = 0, redo_tail = 0;  // records put aside
             uint4 fa = redo[0], fb = redo[1];                          // the record fetched; n_tok = 0: end of work
@@ -834,7 +850,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                                     (int64_t)r_pos + r_n >= r_ke &&
                                     (r_slot < 0 || (int64_t)r_slot + (int64_t)r_n * p.G <= p.n_part_slots);
                 if (!rec_ok) {
-                    if (lane == 0) atomicOr(&p.hdr->status, kStatusBounds);
+                    if (lane == 0) report(p.hdr, p.tag, kStatusBounds);
                     fa = fb = make_uint4(0, 0, 0, 0);
                 }
             };
@@ -844,10 +860,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 ++static_cur;
                 idx = __shfl_sync(0xffffffffu, idx, 0);
                 fa = fb = make_uint4(0, 0, 0, 0);
-                if (idx < p.n_items) {
-                    fa = __ldg(reinterpret_cast<const uint4*>(p.items + idx));
-                    fb = __ldg(reinterpret_cast<const uint4*>(p.items + idx) + 1);
-                }
+                if (idx < p.n_items) record(idx, fa, fb);
                 check_record();
             };
             // every consumer is done with the record that last used the slot of record n; if its item has to be run again,
@@ -936,7 +949,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
     if (*s_abort) {
         // A bounded wait ran out somewhere in this CTA: the output is invalid and the run is flagged.  Before the pair
         // gives back its shared and tensor memory, the copies requested get a bounded time to land (the MMAs have retired).
-        if (threadIdx.x == 0) atomicOr(&p.hdr->status, kStatusTimeout);
+        if (threadIdx.x == 0) report(p.hdr, p.tag, kStatusTimeout);
         if (warp == kKProducerWarp) {
             // (rank 0's barriers also count the peer's relay, which may never come: the copies land in microseconds, so one
             // limit serves them all)
@@ -952,6 +965,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         }
         __syncthreads();
     }
+    if (p.flags & kBeside) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
     cluster_sync();
     if (warp == 0) pair_tmem_dealloc(tmem, 512);
 }
@@ -1017,7 +1031,10 @@ ps_status launch_prefill_pair(const RunArgs& a) {
     p.total_q = a.total_q;
     p.n_part_slots = (int32_t)a.w.n_part_slots;
     p.wait_limit_ns = (uint32_t)a.wait_limit_ns;
-    p.out_aligned32 = (uintptr_t)a.out % 32 == 0;
+    p.tag = a.tag;
+    p.flags = ((uintptr_t)a.out % 32 == 0 ? kOutAligned32 : 0) | (a.inline_items ? kInlineList : 0) | (a.beside ? kBeside : 0);
+    InlineItems inl;
+    fill_inline_items(a, inl);
     CUtensorMap q_map;
     const ps_status enc = encode_q_map(a, &q_map);
     if (enc != PS_OK) return enc;
@@ -1034,7 +1051,7 @@ ps_status launch_prefill_pair(const RunArgs& a) {
         if (r != CUDA_SUCCESS) return fail(PS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
     }
     const int pairs = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms / 2 ? a.w.n_prefill : (a.pf_sms > 1 ? a.pf_sms / 2 : 1));
-    return launch_kernel(prefill_pair_kernel, 2 * pairs, kThreads, kSmemBytes, a.stream, 2, a.early, p, q_map, pool_map);
+    return launch_kernel(prefill_pair_kernel, 2 * pairs, kThreads, kSmemBytes, a.stream, 2, a.early, p, q_map, pool_map, inl);
 }
 
 }  // namespace ps

@@ -4,11 +4,20 @@
 
 #include <cuda.h>
 
+#include <cstring>
+
 #include "common.cuh"
 
 namespace ps {
 
 // Q as a [T tokens][Hq heads][D] tensor; a box is one 64-element half of a q tile's 128 (token, head) rows.
+// (entries past the list's end are not read)
+inline void fill_inline_items(const RunArgs& a, InlineItems& inl) {
+    if (!a.inline_items) return;
+    memcpy(inl.item, a.inline_items, a.w.n_prefill * sizeof(PrefillItem));
+    memcpy(inl.start, a.inline_starts, (a.w.n_prefill_ctas + 1) * sizeof(int32_t));
+}
+
 ps_status encode_q_map(const RunArgs& a, CUtensorMap* map);
 
 #ifdef __CUDACC__
