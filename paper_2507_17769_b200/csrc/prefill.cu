@@ -687,8 +687,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         tc_fence_before();
         __syncthreads();
     }
-    if (p.beside) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
     if (warp == 0) tmem_dealloc(tmem, Cfg::kTmemCols);
+    if (p.beside && blockIdx.x == 0) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
 }
 
 }  // namespace

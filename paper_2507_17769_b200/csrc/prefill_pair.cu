@@ -965,9 +965,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         }
         __syncthreads();
     }
-    if (p.flags & kBeside) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
     cluster_sync();
     if (warp == 0) pair_tmem_dealloc(tmem, 512);
+    // This kernel's end also means that of the decode kernel beside it.  (One CTA's last instruction: what follows a wait is
+    // time between this run and the next kernel.)
+    if ((p.flags & kBeside) && blockIdx.x == 0) pdl_wait();
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
