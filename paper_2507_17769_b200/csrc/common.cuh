@@ -250,7 +250,7 @@ ps_status launch_decode(const RunArgs& a);
 ps_status launch_prefill(const RunArgs& a);
 ps_status launch_prefill_pair(const RunArgs& a);  // head dimension 128
 ps_status launch_merge(const RunArgs& a);
-int decode_warps_per_sm();
+int decode_warps_per_sm(int head_dim);
 
 // ---------------------------------------------------------------------------
 // PTX wrappers

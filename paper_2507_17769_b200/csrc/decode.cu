@@ -27,9 +27,10 @@ namespace ps {
 
 namespace {
 
-// streaming warps per CTA (one CTA per SM) and ring depth per warp: 12 x 2 x 8 KB = 192 KB in flight per SM;
-// measured on B200: 12 x 2 and 10 x 2 beat 8 x 3, 6 x 4 and 4 x 6 by 2-6 %
-constexpr int kWarps = 12;
+// Streaming warps per CTA (one CTA per SM) and ring depth per warp: 12 x 2 x 8 KB = 192 KB in flight per SM at head dimension
+// 128; measured on B200: 12 x 2 and 10 x 2 beat 8 x 3, 6 x 4 and 4 x 6 by 2-6 %.  At 64 a page is half as large and takes a
+// warp nearly as long: 24 x 2 x 4 KB (an SM streams 87 GB/s, 12 x 4 x 4 KB 80).
+__host__ __device__ constexpr int warps_at(int d) { return d == 128 ? 12 : 24; }
 constexpr int kStagesPerWarp = 2;
 constexpr int kRing = 8;  // unit ids in flight between the producer and consumer cursors of a warp
 constexpr int kDeferred = 8;  // merges a warp can postpone until its KV stream has drained
@@ -41,7 +42,8 @@ struct DecodeCfg {
     static constexpr int kBlockBytes = FP8 ? kPage * D : kPage * D * 2;                  // K (or V) of one page, one kv head
     static constexpr int kStageBytes = FP8 ? (int)fp8_page_head_bytes(D) : 2 * kBlockBytes;  // K then V (then the scales)
     // 8 KB (4 KB at D = 64) stages per warp; the FP8 blocks are half as large, so twice as many are kept in flight
-    static constexpr int kStages = (FP8 ? 2 : 1) * ((D == 128) ? kStagesPerWarp : 2 * kStagesPerWarp);
+    static constexpr int kWarps = warps_at(D);
+    static constexpr int kStages = (FP8 ? 2 : 1) * kStagesPerWarp;
     static constexpr int kSmemBytes =
         kWarps * kStages * kStageBytes + kWarps * kStages * 8 + kWarps * kRing * 4 + kWarps * kDeferred * 12 + 1024;
 };
@@ -292,8 +294,9 @@ __device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nva
 }
 
 template <int D, bool FP8>
-__global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodeParams p) {
+__global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_kernel(const DecodeParams p) {
     using Cfg = DecodeCfg<D, FP8>;
+    constexpr int kWarps = Cfg::kWarps;
     constexpr int STAGES = Cfg::kStages;
     constexpr int KS = D / 16;  // k-steps of QK^T == m-tiles of PV
 
@@ -418,7 +421,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
             for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
             // fixed segment order; kAhead segments' rows are requested before the first is used, so that a long
             // list of segments costs about one trip to L2 per kAhead of them
-            constexpr int kAhead = NV <= 2 ? 8 : NV <= 4 ? 4 : 2;  // at most 16 float4 in flight per lane
+            constexpr int kAhead = (NV <= 2 ? 8 : NV <= 4 ? 4 : 2) * D / 128;  // at most 16 float4 in flight per lane (8 with 24 warps)
             for (int s0 = 0; s0 < dm.n_seg; s0 += kAhead) {
                 float4 x[kAhead][NV];
                 float lw[kAhead];
@@ -449,7 +452,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_kernel(const DecodePara
         };
         // NV = D * G / 128: one float4 at (D, G) = (64, 2) or (128, 1) up to eight at (128, 8)
         switch (D * p.G / 128) {
-            case 8: run(std::integral_constant<int, 8>{}); break;
+            case 8:
+                if constexpr (D == 128) run(std::integral_constant<int, 8>{});  // (at D = 64 a group of 8 has 4)
+                break;
             case 4: run(std::integral_constant<int, 4>{}); break;
             case 2: run(std::integral_constant<int, 2>{}); break;
             case 1: run(std::integral_constant<int, 1>{}); break;
@@ -614,8 +619,9 @@ struct CtaPart {  // what a warp leaves for the others, in the place of its stag
     static constexpr int kBytes = 8 * kRow * 4;
 };
 template <int D, bool FP8>
-__global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const DecodeParams p, int n_pieces, const __grid_constant__ InlinePieces inl) {
+__global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_cta_kernel(const DecodeParams p, int n_pieces, const __grid_constant__ InlinePieces inl) {
     using Cfg = DecodeCfg<D, FP8>;
+    constexpr int kWarps = Cfg::kWarps;
     constexpr int STAGES = Cfg::kStages;
     constexpr int KS = D / 16;
     static_assert(CtaPart<D>::kBytes <= STAGES * Cfg::kStageBytes, "a warp's part fits its stages");
@@ -646,7 +652,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const Decode
         b = make_int4(pc.q_tok, pc.part_slot, pc.kv_len, pc.merge_idx);
     }
     if (!check_piece(p, a, b) && threadIdx.x == 0) report(p.hdr, p.tag, kStatusBounds);
-    const int first = a.z + warp, n_mine = a.w > first ? (a.w - first + kWarps - 1) / kWarps : 0;  // my pages: first + 12 i
+    const int first = a.z + warp, n_mine = a.w > first ? (a.w - first + kWarps - 1) / kWarps : 0;  // my pages: first + kWarps i
     const int32_t* const bt = p.block_table + (int64_t)a.x * p.max_pages + first;
     const uint64_t kv_policy = l2_policy_evict_first();
     int pages = lane < n_mine ? __ldg(bt + kWarps * lane) : 0;  // those of 32 turns, one a lane
@@ -777,11 +783,12 @@ __global__ void __launch_bounds__(kWarps * 32, 1) decode_cta_kernel(const Decode
 
 }  // namespace
 
-int decode_warps_per_sm() { return kWarps; }
+int decode_warps_per_sm(int head_dim) { return warps_at(head_dim); }
 
 template <int D, bool FP8>
 static ps_status launch_decode_d(const RunArgs& a) {
     using Cfg = DecodeCfg<D, FP8>;
+    constexpr int kWarps = Cfg::kWarps;
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
         PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));

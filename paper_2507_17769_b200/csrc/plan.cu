@@ -28,8 +28,8 @@ constexpr int kDecodeUnitsPerWarp = 1;  // work units per resident warp (measure
 // 64 tokens: 13 us instead of 20; 8 rows of 512: 16 instead of 23), but every further piece of a row is one more
 // partial result for the one warp that combines them (one row of 4096 tokens: 22 us at 32 pieces, 26 at 64).
 constexpr int kDecodeMinPagesLo = 4, kDecodeMinPagesHi = 8, kDecodePiecesPerRow = 16;
-// A CTA per piece (small batches): pages a warp may get at most, and pages a warp gets before a row is cut.
-constexpr int kCtaPagesPerWarp = 8, kCtaMinPieceTurns = 4;
+// A CTA per piece (small batches): pages of a piece at most, and before a row is cut (8 and 4 for each of 12 warps).
+constexpr int kCtaMaxPiece = 96, kCtaMinPiece = 48;
 constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 // Measured on B200 (bandwidth against the number of SMs the decode kernel runs on), used with the prefill kernel's cost
 // model to split the SMs of a mixed batch between the two kernels.
@@ -180,12 +180,12 @@ static int query_num_sms() {
 }
 
 // Batches too small for a share per warp: a CTA per piece.  Applies where every (row, kv head) gets a CTA of its own and no
-// piece leaves a warp more than kCtaPagesPerWarp pages -- where a warp's share would be the smallest unit, and a piece per
+// piece is longer than kCtaMaxPiece -- where a warp's share would be the smallest unit, and a piece per
 // warp would be many partial rows.  Rows longer than kCtaMinPiece are cut as far as there are CTAs.
 static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start, int64_t total_pages,
                              int64_t longest, int64_t* n_slots) {
-    const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv, warps = decode_warps_per_sm();
-    const int64_t max_piece = (int64_t)kCtaPagesPerWarp * warps;
+    const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
+    const int64_t max_piece = kCtaMaxPiece;
     if (total_pages > pl->dec_sms * max_piece) return false;
     std::vector<std::pair<int32_t, int32_t>> rows;  // (request, keys the row sees)
     for (int r = 0; r < pl->n; ++r) {
@@ -201,7 +201,7 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
     };
     // Uncut if that leaves no warp too many pages (a list without merges need not be uploaded); else the smallest piece that
     // leaves no more pieces than CTAs.
-    int64_t lo = std::max<int64_t>(kCtaMinPieceTurns * warps, longest <= max_piece ? longest : 0), hi = std::max(lo, longest);
+    int64_t lo = std::max<int64_t>(kCtaMinPiece, longest <= max_piece ? longest : 0), hi = std::max(lo, longest);
     while (lo < hi) {
         const int64_t mid = (lo + hi) / 2;
         if (pieces_at(mid) <= pl->dec_sms) hi = mid; else lo = mid + 1;
@@ -265,7 +265,7 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     if (opts && opts->decode_segment_tokens > 0) {
         per_unit = std::max(1, opts->decode_segment_tokens / kPage);
     } else {
-        const int64_t target = (int64_t)pl->dec_sms * decode_warps_per_sm() * kDecodeUnitsPerWarp;
+        const int64_t target = (int64_t)pl->dec_sms * decode_warps_per_sm(pl->shape.head_dim) * kDecodeUnitsPerWarp;
         per_unit = std::max<int64_t>(min_pages, (total_pages + target - 1) / target);
     }
     pl->info.decode_segment_tokens = (int32_t)(per_unit * kPage);
