@@ -121,6 +121,12 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+def calls():
+    """The extension module of the calls of every iteration (addresses as integers, lengths as given by lengths())."""
+    load()
+    return _calls
+
+
 def _check(status: int):
     if status != PS_OK:
         raise PsError(status, load().ps_last_error().decode())
@@ -142,7 +148,7 @@ def _host_i32(a):
 _I32 = np.dtype(np.int32)
 
 
-def _lengths(a):
+def lengths(a):
     """A batch's lengths as the extension module takes them."""
     if type(a) is not np.ndarray or a.dtype is not _I32 or not a.flags.c_contiguous:
         a = np.ascontiguousarray(a, dtype=_I32)
@@ -180,8 +186,8 @@ def ps_kv_free(kv):
 
 def ps_kv_write(kv, k_new_dev, v_new_dev, block_table_dev, max_pages, prior_host, q_len_host, stream=None):
     load()
-    _check(_calls.kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, _lengths(prior_host),
-                           _lengths(q_len_host), _ptr(stream)))
+    _check(_calls.kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, lengths(prior_host),
+                           lengths(q_len_host), _ptr(stream)))
 
 
 def ps_kv_gather(kv, block_table_row_dev, length, k_out_dev, v_out_dev, stream=None):
@@ -202,7 +208,7 @@ def ps_attn_plan(shape: ps_shape, prior_host, q_len_host, max_pages_per_seq, opt
     """Returns (plan handle, workspace bytes).  Pass ``plan`` to rebuild an existing handle in place."""
     lib = load()
     if opts is None:
-        status, handle, ws = _calls.attn_plan(ctypes.addressof(shape), _lengths(prior_host), _lengths(q_len_host), max_pages_per_seq, plan)
+        status, handle, ws = _calls.attn_plan(ctypes.addressof(shape), lengths(prior_host), lengths(q_len_host), max_pages_per_seq, plan)
         _check(status)
         return handle, ws
     pr, prp = _host_i32(prior_host)

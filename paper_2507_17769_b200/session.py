@@ -22,6 +22,7 @@ class PagedAttention:
         import torch
 
         self.torch = torch
+        self._calls = B.calls()
         self.device = torch.device(device)
         self.shape = B.make_shape(n_q_heads, n_kv_heads, head_dim, page_size, kv_dtype)
         self.num_pages = int(num_pages)
@@ -36,7 +37,9 @@ class PagedAttention:
         self._plan = None
         self._ws = None
         self._ws_bytes = 0
+        self._ws_ptr = 0
         self._total_q = 0
+        self._n_q_heads = int(n_q_heads)
         index = self.pool.device.index
         raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # (a tenth of the time that current_stream() takes)
         self._stream = (lambda: raw(index)) if raw else (lambda: torch.cuda.current_stream(index).cuda_stream)
@@ -58,9 +61,10 @@ class PagedAttention:
     def write(self, k_new, v_new, block_table_dev, prior, q_len, max_pages=None):
         """Scatter new tokens' K, V (bf16 [T, Hkv, d]) into their pages."""
         if max_pages is None:
-            max_pages = block_table_dev.shape[-1]
+            max_pages = block_table_dev.size(-1)
         assert k_new.is_contiguous() and v_new.is_contiguous() and block_table_dev.is_contiguous()
-        B.ps_kv_write(self.kv, k_new.data_ptr(), v_new.data_ptr(), block_table_dev.data_ptr(), int(max_pages), prior, q_len, self._stream())
+        B._check(self._calls.kv_write(self.kv, k_new.data_ptr(), v_new.data_ptr(), block_table_dev.data_ptr(), int(max_pages), B.lengths(prior),
+                                     B.lengths(q_len), self._stream()))
 
     def gather_fp8(self, block_table_row_dev, length):
         """FP8 cache: logical tokens [0, length) of one sequence as (K codes, V codes) uint8 [length, Hkv, d] and
@@ -92,6 +96,7 @@ class PagedAttention:
         if need > self._ws_bytes:
             self._ws = self.torch.empty(int(need * 1.25) + 256, dtype=self.torch.uint8, device=self.device)
             self._ws_bytes = self._ws.numel()
+            self._ws_ptr = self._ws.data_ptr()
         info = B.ps_plan_get_info(self._plan)
         self._total_q = info.total_q_tokens
         return info
@@ -103,14 +108,14 @@ class PagedAttention:
         """Attention for the planned batch.  q: bf16 [T, Hq, d].  Returns (out, lse)."""
         t = self.torch
         assert self._plan is not None, "call plan() first"
-        assert q.is_contiguous() and q.shape[0] == self._total_q and block_table_dev.is_contiguous()
+        total_q, hq = self._total_q, self._n_q_heads
+        assert q.is_contiguous() and q.size(0) == total_q and block_table_dev.is_contiguous()
         if out is None:
             out = t.empty_like(q)
         if lse is None and want_lse:
-            hq = self.shape.n_q_heads
-            lse = t.empty_strided((q.shape[0], hq), (hq, 1), dtype=t.float32, device=self.device)  # (two thirds of empty()'s time)
-        B.ps_attn_run(self._plan, self.kv, q.data_ptr(), block_table_dev.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
-                      self._ws.data_ptr(), self._ws_bytes, self._stream())
+            lse = t.empty_strided((total_q, hq), (hq, 1), dtype=t.float32, device=self.device)  # (two thirds of empty()'s time)
+        B._check(self._calls.attn_run(self._plan, self.kv, q.data_ptr(), block_table_dev.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(),
+                                     self._ws_ptr, self._ws_bytes, self._stream()))
         return out, lse
 
     def check(self):
