@@ -224,6 +224,11 @@ ps_status ps_plan_get_items(const ps_plan *plan, int32_t *decode_items_out, int6
  * merge kernel then follows the prefill kernel at once, under the decode
  * kernel), and is joined back into `stream` before the call's work is
  * complete in stream order.
+ * Small batches (at most 148 decode pieces and 64 prefill items, none of them
+ * cut) differ: their work list travels with the kernels' parameters, nothing
+ * is uploaded and the workspace is not touched.  Kernels may be launched while
+ * the kernel before them in `stream` still runs; each waits for its end before
+ * it reads or writes device memory, so stream order holds as usual.
  * Ordering rule for the workspace: all runs that use one workspace -- of one
  * plan, re-planned or not, and of different plans that take turns on it --
  * must be issued to the same stream, or be ordered by the caller.  Under that
