@@ -790,8 +790,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         } else if (warp == kMmaWarp) {
             // ================================================================
             // relay: tells rank 0 that this CTA's half tiles have landed.  V follows K two tiles behind, which is about when
-            // either is asked for, so that neither is told late; when no next record is out, V catches up first (the last
-            // record is not out before every item's V has been used).
+            // either is asked for, so that neither is told late; when no next record is out, V catches up first.  It also does
+            // once the last record is out, which may be before the last two tiles' V has landed: the softmax warps give an
+            // item back when its sums are checked, and only the one of a ragged last tile has waited for V.
             // ================================================================
             uint32_t n_item = 0, n = 0, nv = 0;  // key tiles whose K, and V, has been told of
             bool ok = true;
@@ -822,6 +823,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 }
                 ++n_item;
             }
+            while (ok && nv < n) tell_v();
         } else {
             // ================================================================
             // items: fetches the pair's records, from its static share or the queue, and puts them into both CTAs' rings as

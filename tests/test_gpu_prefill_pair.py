@@ -78,3 +78,33 @@ def test_rows_out_of_range_are_computed_again(every, exp):
     b = gen.make_batch(gen.SHAPE_8B, 960 + exp, [300, 0, 129], [130, 200, 70])
     exps = np.where(np.arange(b.total_q) % every == 0, exp, 0)
     run_and_compare(b, exps, "exp %d every %d" % (exp, every))
+
+
+@pytest.mark.parametrize("segment", [0, 128, 256, 384, 512])
+def test_pairs_whose_last_item_ends_on_a_full_key_tile(segment):
+    """A pair's last record may be out before V of its last tiles has landed: their softmax does not wait for V unless the
+    last tile is ragged.  Chunks whose keys end on a tile boundary, cold in L2, beside decode rows that keep the memory system
+    busy; ``segment``: the planner's own cuts, or items of one to four full tiles."""
+    import torch
+    import paper_2507_17769_b200 as ps
+    from workloads.device import DeviceBatch
+
+    rng = np.random.default_rng(970)
+    rows, chunks = 64, 16
+    b = gen.make_batch(gen.SHAPE_8B, 970, rng.integers(3000, 5000, rows).tolist() + [64 + 256 * (8 + k) for k in range(chunks)],
+                       [1] * rows + [64] * chunks)
+    db = DeviceBatch(b)
+    first = {}
+    for k in list(range(chunks)) * 3:
+        idx = list(range(rows)) + [rows + k]
+        q = torch.cat([db.q[:rows], db.q[rows + 64 * k : rows + 64 * (k + 1)]])
+        bt = db.block_table[idx].contiguous()
+        info = db.pa.plan(b.prior[idx], b.q_len[idx], b.max_pages, ps.ps_plan_opts(0, segment, 0) if segment else None)
+        assert info.n_prefill_items > 0
+        ps.ps_plan_set_wait_limit(db.pa._plan, 200_000_000)
+        out, lse = db.pa.run(q, bt)
+        db.pa.check()  # (a wait that runs out is an error here)
+        if k in first:
+            assert torch.equal(out.view(torch.int16), first[k][0].view(torch.int16)) and torch.equal(lse, first[k][1])
+        first[k] = (out, lse)
+    db.pa.close()
