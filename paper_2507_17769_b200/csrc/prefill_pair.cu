@@ -221,12 +221,18 @@ __device__ __forceinline__ void pair_commit(uint32_t bar) {
         : "memory");
 }
 
-// exp2 of a pair on the FMA pipe: 2^n by exponent arithmetic, 2^f by a polynomial that is as close (2e-7) as ex2.approx.
-// x below -126 gives 2^-126.
+// NaN stays NaN
+__device__ __forceinline__ float clamp_nan(float x, float lo, float hi) {
+    asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lo), "f"(hi));
+    return x;
+}
+// exp2 of a pair on the FMA pipe: 2^n from exponent arithmetic times 2^f by a polynomial that is as close (2e-7) as ex2.approx.
+// Scores come here without their row maximum taken off: above 127 the result stays 2^127, which takes the row's sum out of
+// range as infinity would, and below -126.5 it is zero.
 __device__ __forceinline__ void exp2_poly2(uint64_t x, float& e0, float& e1) {
     float x0, x1;
     unpack2(x, x0, x1);
-    x = pack2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    x = pack2(clamp_nan(x0, -127.f, 127.f), clamp_nan(x1, -127.f, 127.f));
     constexpr float kRound = 12582912.f;  // 1.5 * 2^23: adding it leaves round(x) in the low bits
     const uint64_t t = add2(x, pack2(kRound, kRound));
     const uint64_t f = fma2(add2(t, pack2(-kRound, -kRound)), pack2(-1.f, -1.f), x);
@@ -235,11 +241,10 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x, float& e0, float& e1) {
     uint64_t y = pack2(c[5], c[5]);
 #pragma unroll
     for (int k = 4; k >= 0; --k) y = fma2(y, f, pack2(c[k], c[k]));
-    float y0, y1, t0, t1;
-    unpack2(y, y0, y1);
+    float t0, t1;
     unpack2(t, t0, t1);
-    e0 = __int_as_float(__float_as_int(y0) + (__float_as_int(t0) << 23));
-    e1 = __int_as_float(__float_as_int(y1) + (__float_as_int(t1) << 23));
+    const uint64_t two_n = pack2(__int_as_float((__float_as_int(t0) << 23) + 0x3f800000), __int_as_float((__float_as_int(t1) << 23) + 0x3f800000));
+    unpack2(fma2(y, two_n, 0ull), e0, e1);
 }
 
 // 32 weights exp2(scale * s - ref) of one row as bf16 pairs, added to the packed row sums: two scores per instruction

@@ -19,7 +19,23 @@ def scaled(bits, exps):
     return (f.astype(np.float32).view(np.uint32) >> 16).astype(np.uint16)
 
 
-def run_and_compare(batch, exps, what):
+def bf16_bits(x):
+    u = np.ascontiguousarray(x, dtype=np.float32).view(np.uint32)
+    return ((u + 0x7FFF + ((u >> 16) & 1)) >> 16).astype(np.uint16)
+
+
+def f32(bits):
+    return (bits.astype(np.uint32) << 16).view(np.float32)
+
+
+def on_device(bits):
+    import torch
+
+    return torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
+
+
+def run_and_compare(batch, exps, what, plant=None, opts=None):
+    """``plant``: changes request 0's K bit patterns [kv_len, Hkv, d], given them and q's; returns the positions changed."""
     import torch
     from workloads.device import DeviceBatch
 
@@ -27,12 +43,15 @@ def run_and_compare(batch, exps, what):
     db = DeviceBatch(batch)
     q = np.concatenate([q_bits(batch, r) for r in range(batch.n)])
     q = scaled(q, exps)
-    db.q = torch.from_numpy(q.view(np.int16)).cuda().view(torch.bfloat16)
-    info = db.plan()
+    db.q = on_device(q)
+    ks, vs = zip(*[kv_bits(batch, r) for r in range(batch.n)])
+    if plant:
+        for at in plant(ks[0], q):
+            db.pa.write(on_device(ks[0][at : at + 1]), on_device(vs[0][at : at + 1]), db.block_table[0], [at], [1], max_pages=batch.max_pages)
+    info = db.plan(opts)
     assert info.n_prefill_items > 0
     out, lse = db.run()
     db.pa.check()
-    ks, vs = zip(*[kv_bits(batch, r) for r in range(batch.n)])
     kp = oracle.plain_pool(ks, batch.block_table, batch.num_pages, s.page_size)
     vp = oracle.plain_pool(vs, batch.block_table, batch.num_pages, s.page_size)
     rr = [r for r in range(batch.n) for _ in range(int(batch.q_len[r]))]
@@ -43,7 +62,7 @@ def run_and_compare(batch, exps, what):
     # Large scores make rows see a few keys in effect, however many they have: the outputs are single V values, bf16-rounded
     # (compare() scales its bound for such rows by the value).  lse: fp32 arithmetic on scores of up to 2^e times the plain
     # ones, whose products and sums over d = 128 are each good to a few units of 2^-24.
-    peaked = np.asarray(exps) > 1
+    peaked = (np.asarray(exps) > 1) | (plant is not None)
     compare(out, None, want, want_lse, what=what, few_key_rows=True, keys=np.where(peaked, 1, keys))
     err = np.abs(lse.cpu().numpy().astype(np.float64) - want_lse)
     assert (err <= 2e-3 + 1e-5 * np.abs(want_lse)).all(), "%s: lse off by %.3e" % (what, err.max())
@@ -108,3 +127,53 @@ def test_pairs_whose_last_item_ends_on_a_full_key_tile(segment):
             assert torch.equal(out.view(torch.int16), first[k][0].view(torch.int16)) and torch.equal(lse, first[k][1])
         first[k] = (out, lse)
     db.pa.close()
+
+
+@pytest.mark.parametrize("segment", [0, 4096])
+@pytest.mark.parametrize("score", [50.0, 85.0, 104.0, 139.0, 173.0, 177.4, 355.0, 5000.0])
+def test_one_key_with_a_large_score(score, segment):
+    """Ordinary rows of some 2000 keys in which one key has nearly all the weight, orthogonal to the other rows of its item,
+    so that nothing else takes the item's sums out of range.  A kv head each for the positions (modulo 32) whose
+    exponentials go to the exp2 unit and to the FMA pipe; 50 to 177.4 are 72 to 256 in powers of two, where exponent
+    arithmetic without a bound first overflows, then wraps."""
+    import paper_2507_17769_b200 as ps
+
+    b = gen.make_batch(gen.SHAPE_8B, 980, [2100], [16])
+    places = [640 + c for c in (1, 2, 3, 5, 64 + 2, 64 + 3, 34, 35)]
+
+    def plant(k, q):
+        for g, at in enumerate(places):
+            rows = f32(q[:, 4 * g : 4 * g + 4]).reshape(64, 128).astype(np.float64)
+            want = np.zeros(64)
+            want[(7 * g) % 64] = score * np.sqrt(128)
+            k[at, g] = bf16_bits(np.linalg.lstsq(rows, want, rcond=None)[0])
+        return places
+
+    run_and_compare(b, np.zeros(b.total_q), "score %g" % score, plant, ps.ps_plan_opts(0, segment, 0) if segment else None)
+
+
+@pytest.mark.parametrize("past", [0, 384])
+def test_a_nan_key_reaches_the_rows_that_see_it(past):
+    """A NaN in one key makes the output of every row that sees it NaN, whichever unit exponentiates its column; other rows
+    are not touched.  ``past``: first position of the keys' tile (the second one some rows see and others do not)."""
+    import torch
+    from workloads.device import DeviceBatch
+
+    b = gen.make_batch(gen.SHAPE_8B, 981, [300], [200])
+    db = DeviceBatch(b)
+    ks, vs = kv_bits(b, 0)
+    places = [past + c for c in (1, 2, 3, 5, 66, 67, 34, 35)]
+    db.plan()
+    clean = db.run()[0]
+    for g, at in enumerate(places):
+        ks[at, g] = 0x7FC0
+        db.pa.write(on_device(ks[at : at + 1]), on_device(vs[at : at + 1]), db.block_table[0], [at], [1], max_pages=b.max_pages)
+    out, _ = db.run()
+    db.pa.check()
+    for g, at in enumerate(places):
+        sees = torch.arange(300, 500, device="cuda") >= at
+        heads = slice(4 * g, 4 * g + 4)
+        assert bool(torch.isnan(out[sees][:, heads].float()).all()), "key %d" % at
+        assert bool(torch.isfinite(out[~sees][:, heads].float()).all()), "key %d" % at
+        if bool((~sees).any()):
+            assert (out[~sees][:, heads].float() - clean[~sees][:, heads].float()).abs().max().item() <= 1e-2
