@@ -17,10 +17,12 @@
 // each half in the first 32 of its 64 columns), so one barrier per tile says both that P is there and that the buffer may
 // be written behind the PV that reads it: QK^T of tile n + 3 is issued right behind PV of tile n, three tiles ahead of use.
 //
-// The softmax needs no row maximum.  Weights are exp2 of the scaled scores themselves: fp32 sums and accumulators and
-// bf16 weights keep their relative precision from 2^-60 to 2^60, far beyond the scores of trained heads.  An item whose
-// row sums leave that range is run again, first for its rows' maxima and then relative to them.  Only rows that see fewer
-// than 64 keys are always taken relative to their maximum.
+// The softmax needs no row maximum.  Weights are exp2 of the scaled scores less a reference, the maximum of 32 of the row's
+// scores in the item's first tile: fp32 sums and accumulators and bf16 weights keep their relative precision wherever the
+// exponents are, and the reference's own weight keeps a sum from being small.  An item with a row whose sum exceeds 2^100
+// (scores of some 69 above the sample's, in natural units) is run again, first for its rows' maxima and then relative to them:
+// 640 us instead of 240 on 2048 x 8192 if every item has such a row.  Rows that see fewer than 64 keys are always taken
+// relative to their maximum.
 //
 // What bounds it: a 128-key step of the pair takes 1310 cycles, of which the tensor core needs 1024; the exp2 unit would need
 // as many.  What is left is issue time: the MMA warp needs about 1150 cycles a step (16 MMAs and their commits 700, three
@@ -49,7 +51,9 @@ constexpr int D = 128;
 constexpr int kTileKeys = 128;
 constexpr int kRows = 128;                // rows of one CTA
 constexpr float kScaleLog2 = 0.12751743f;  // log2(e) / sqrt(128)
-constexpr float kSumMin = 8.7e-19f, kSumMax = 1.15e18f;  // 2^-60, 2^60: row sums outside are recomputed
+// 2^-60, 2^100: row sums outside are recomputed.  (Below 2^100 the accumulators are finite for |V| up to 2^27; only a row whose
+// sample was not finite can have a sum below 1.)
+constexpr float kSumMin = 8.7e-19f, kSumMax = 1.26e30f;
 // Pairs of every 16 whose exponentials go to the FMA pipe instead of the exp2 unit, which at full tensor rate would be just
 // as busy as the tensor core (measured: 0 / 1 / 2 pairs 96.8 / 92.5 / 91.1 us on 1536 tokens after 3885, four prompts of 500
 // to 1900 tokens 75.7 / 75.7 / 77.9).
@@ -96,7 +100,8 @@ struct Bars {  // byte offsets from the barrier block
     static constexpr int ring = (again + 8 * kItemRing + 15) / 16 * 16;
     static constexpr int redo = ring + kItemRing * (int)sizeof(PrefillItem);      // rank 1: records to run again
     static constexpr int row_part = redo + kItemRing * (int)sizeof(PrefillItem);  // [item & 3][softmax warpgroup] per row: (sum or maximum, item number and the sum's rounding)
-    static constexpr int bytes = row_part + 16 * kRows * 8;
+    static constexpr int row_ref = row_part + 16 * kRows * 8;  // [item & 3] per row: (reference, item number)
+    static constexpr int bytes = row_ref + 4 * kRows * 8;
 };
 constexpr int kSmemBytes = kOffBar + Bars::bytes + 1024;  // + alignment slack
 static_assert(kSmemBytes <= 232448 && Bars::armed % 4 == 0 && sizeof(PrefillItem) == 32, "shared memory");
@@ -340,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         mbar_init(bars + off, count);
         mbar_fence_init();
     }
-    for (int k = threadIdx.x; k < 16 * kRows; k += kThreads) store_tagged(bars + Bars::row_part + 8 * k, 0.f, 0xffffffffu);
+    for (int k = threadIdx.x; k < 20 * kRows; k += kThreads) store_tagged(bars + Bars::row_part + 8 * k, 0.f, 0xffffffffu);
     if (threadIdx.x < 8 * kItemRing) again[threadIdx.x] = 0;
     if (threadIdx.x < Bars::n_armed) s_armed[threadIdx.x] = -1;
     tc_fence_before();
@@ -383,6 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
         const uint32_t lane_tm = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         // this row's entry in slot [item & 3][warpgroup]
         auto row_part = [&](uint32_t item, uint32_t wg) { return bars + Bars::row_part + 8 * (((item & 3) * 4 + wg) * kRows + t); };
+        auto row_ref = [&](uint32_t item) { return bars + Bars::row_ref + 8 * ((item & 3) * kRows + t); };
         // another warpgroup's entry for this row, once it carries `tag`
         auto read_tagged = [&](uint32_t addr, uint32_t item, float& v, float& rounding) -> bool {
             uint32_t t0 = 0;
@@ -426,10 +432,32 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 if (ref == -INFINITY) ref = 0.f;
             }
             if (mode == kModeMax) l = -INFINITY;
+            if (mode == kModePlain && w == g0) {
+                // The row's reference, the same in both halves.  (Columns 32 to 63 hold scores until the tile's PV: a half's
+                // weights go over its first 32.)
+                const uint32_t buf6 = tc0 % (2 * kScoreBufs), buf = buf6 >= 3 ? buf6 - 3 : buf6;
+                ok = wait_all(bars + Bars::s_full + 8 * buf6, (tc0 / (2 * kScoreBufs)) & 1, s_abort);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t sv[32];
+                tmem_ld32(lane_tm + buf * 128 + 32, sv);
+                tmem_wait_ld();
+                float mx = -INFINITY;
+#pragma unroll
+                for (int c = 0; c < 32; c += 2) mx = max3(mx, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
+                // (rows that see fewer than 64 keys: below; they are in items of at most three tiles)
+                if (limit - key_begin >= 64 && fabsf(mx) < INFINITY) ref = mx * kScaleLog2;
+                if (h == 0 && n_tiles > 3) store_tagged(row_ref(n_item), ref, n_item & 0xffffu);
+            } else if (mode == kModePlain && n_tiles > 3) {
+                float unused;
+                ok = read_tagged(row_ref(n_item), n_item, ref, unused);
+                if (!ok) break;
+            }
             for (int j = w == g0 ? 0 : 3; j < n_tiles; j += j < 2 ? 1 : 2) {
                 const uint32_t tc = tc0 + j;
                 const uint32_t buf6 = tc % (2 * kScoreBufs), buf = buf6 >= 3 ? buf6 - 3 : buf6;
-                ok = wait_all(bars + Bars::s_full + 8 * buf6, (tc / (2 * kScoreBufs)) & 1, s_abort);
+                // (the first tile's scores have been waited for, for the reference)
+                if (j > 0 || mode != kModePlain) ok = wait_all(bars + Bars::s_full + 8 * buf6, (tc / (2 * kScoreBufs)) & 1, s_abort);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t s_addr = lane_tm + buf * 128 + h * 64;

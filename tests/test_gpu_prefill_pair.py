@@ -46,7 +46,9 @@ def run_and_compare(batch, exps, what, plant=None, opts=None):
     db.q = on_device(q)
     ks, vs = zip(*[kv_bits(batch, r) for r in range(batch.n)])
     if plant:
-        for at in plant(ks[0], q):
+        changed = plant(ks[0], q)
+        db.q = on_device(q)
+        for at in changed:
             db.pa.write(on_device(ks[0][at : at + 1]), on_device(vs[0][at : at + 1]), db.block_table[0], [at], [1], max_pages=batch.max_pages)
     info = db.plan(opts)
     assert info.n_prefill_items > 0
@@ -150,6 +152,28 @@ def test_one_key_with_a_large_score(score, segment):
         return places
 
     run_and_compare(b, np.zeros(b.total_q), "score %g" % score, plant, ps.ps_plan_opts(0, segment, 0) if segment else None)
+
+
+@pytest.mark.parametrize("prior", [0, 90, 700])
+@pytest.mark.parametrize("where,offset", [("all", 60.0), ("all", -60.0), ("all", 300.0), ("all", -300.0), ("sample", -40.0), ("sample", -66.0),
+                                          ("sample", -72.0), ("sample", -300.0), ("sample", 300.0), ("first", 60.0), ("first", 100.0)])
+def test_scores_away_from_the_rows_reference(where, offset, prior):
+    """Scores moved by an offset on all keys, on the 32 of every tile of which the first tile's are a row's reference, or on
+    the first key: weights are relative to the reference, and -72 below the others the sums leave their range."""
+    b = gen.make_batch(gen.SHAPE_8B, 990, [prior], [150])
+    unit = np.full(128, 128 ** -0.5)
+
+    def along(x, to):  # x's component along `unit` set to `to`
+        return bf16_bits(x + (to - x @ unit)[..., None] * unit)
+
+    def plant(k, q):
+        q[:] = along(f32(q).astype(np.float64), 16.0)
+        kv = np.arange(k.shape[0])
+        hit = np.ones_like(kv, dtype=bool) if where == "all" else (kv % 64 >= 32) & (kv % 128 < 64) if where == "sample" else kv == 0
+        k[:] = along(f32(k).astype(np.float64), np.where(hit, offset * 128 ** 0.5 / 16, 0.0)[:, None])
+        return kv
+
+    run_and_compare(b, np.zeros(b.total_q), "%s %g" % (where, offset), plant)
 
 
 @pytest.mark.parametrize("past", [0, 384])
