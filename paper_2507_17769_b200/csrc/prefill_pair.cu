@@ -24,8 +24,8 @@
 // 640 us instead of 240 on 2048 x 8192 if every item has such a row.  Rows that see fewer than 64 keys are always taken
 // relative to their maximum.
 //
-// What bounds it: a 128-key step of the pair takes 1310 cycles, of which the tensor core needs 1024; the exp2 unit would need
-// as many.  What is left is issue time: the MMA warp needs about 1150 cycles a step (16 MMAs and their commits 700, three
+// What bounds it: a 128-key step of the pair takes 1310 cycles, of which the tensor core needs 1024 and the exp2 unit as many.
+// What is left is issue time: the MMA warp needs about 1150 cycles a step (16 MMAs and their commits 700, three
 // waits), and every instruction that is not in a hot loop costs its warp some 6 cycles, because four softmax warps per
 // scheduler evict it.  Hence one barrier per tile for that warp (a feeder warp waits for V on its behalf), gathered tensor
 // copies, short code at the item's end, and items begun by the group that is not writing output.
@@ -34,9 +34,11 @@
 //     1536 x 3885  119 -> 92.5 us (1266 TFLOP/s, 0.77 of the measured cuBLAS rate)    512 x 8192  76.1 -> 60.0
 //     2048 x 8192  275 -> 215 us (1436 TFLOP/s, 0.87)    2 x 2048 on 19.8 k and 28.9 k, 64 q heads  2890 -> 2330 us (1460)
 // Steps on the way, on 2048 x 8192: pair with two score buffers and eight softmax warps 251 us; three buffers, sixteen
-// warps, no maximum 245; warp-uniform MMA issue and the feeder 241; gathered copies 218; part of the exponentials on the
-// FMA pipe and items begun by the other group 212.  Items fetched by a warp of their own: 888 items of one key tile (12 a
-// pair) 70.5 -> 64 us, of five 112 -> 106, four prompts of 1400 to 2000 tokens, whole iteration, 134.1 -> 129.5.
+// warps, no maximum 245; warp-uniform MMA issue and the feeder 241; gathered copies 218; items begun by the other group and
+// part of the exponentials as a polynomial on the FMA pipe 212.  (The polynomial was taken out again: beside the maximum that
+// the sums' rounding needs it cost more than it saved, 278 us a run back to back with it and 263 without.)  Items fetched by a
+// warp of their own: 888 items of one key tile (12 a pair) 70.5 -> 64 us, of five 112 -> 106, four prompts of 1400 to 2000
+// tokens, whole iteration, 134.1 -> 129.5.
 // Every wait is bounded; on expiry a CTA sets the timeout status and drains.
 #include "tcgen05.cuh"
 
@@ -54,10 +56,6 @@ constexpr float kScaleLog2 = 0.12751743f;  // log2(e) / sqrt(128)
 // 2^-60, 2^100: row sums outside are recomputed.  (Below 2^100 the accumulators are finite for |V| up to 2^27; only a row whose
 // sample was not finite can have a sum below 1.)
 constexpr float kSumMin = 8.7e-19f, kSumMax = 1.26e30f;
-// Pairs of every 16 whose exponentials go to the FMA pipe instead of the exp2 unit, which at full tensor rate would be just
-// as busy as the tensor core (measured: 0 / 1 / 2 pairs 96.8 / 92.5 / 91.1 us on 1536 tokens after 3885, four prompts of 500
-// to 1900 tokens 75.7 / 75.7 / 77.9).
-constexpr int kPolyPairs = 1;
 constexpr int kStagesK = 4, kStagesV = 4;
 static_assert(kStagesV <= 5, "the feeder counts on a key tile's weights being six tiles away from the next on its barrier");
 constexpr int kScoreBufs = 3;
@@ -99,7 +97,7 @@ struct Bars {  // byte offsets from the barrier block
     static constexpr int again = armed + 4 * n_armed;       // rank 1, per ring slot a byte per rank and quarter of its rows: sums out of range
     static constexpr int ring = (again + 8 * kItemRing + 15) / 16 * 16;
     static constexpr int redo = ring + kItemRing * (int)sizeof(PrefillItem);      // rank 1: records to run again
-    static constexpr int row_part = redo + kItemRing * (int)sizeof(PrefillItem);  // [item & 3][softmax warpgroup] per row: (sum or maximum, item number and the sum's rounding)
+    static constexpr int row_part = redo + kItemRing * (int)sizeof(PrefillItem);  // [item & 3][softmax warpgroup] per row: (sum or maximum, item number in the low byte of the sum's rounding)
     static constexpr int row_ref = row_part + 16 * kRows * 8;  // [item & 3] per row: (reference, item number)
     static constexpr int bytes = row_ref + 4 * kRows * 8;
 };
@@ -226,47 +224,16 @@ __device__ __forceinline__ void pair_commit(uint32_t bar) {
         : "memory");
 }
 
-// NaN stays NaN
-__device__ __forceinline__ float clamp_nan(float x, float lo, float hi) {
-    asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(x) : "f"(lo), "f"(hi));
-    return x;
-}
-// exp2 of a pair on the FMA pipe: 2^n from exponent arithmetic times 2^f by a polynomial that is as close (2e-7) as ex2.approx.
-// Scores come here without their row maximum taken off: above 127 the result stays 2^127, which takes the row's sum out of
-// range as infinity would, and below -126.5 it is zero.
-__device__ __forceinline__ void exp2_poly2(uint64_t x, float& e0, float& e1) {
-    float x0, x1;
-    unpack2(x, x0, x1);
-    x = pack2(clamp_nan(x0, -127.f, 127.f), clamp_nan(x1, -127.f, 127.f));
-    constexpr float kRound = 12582912.f;  // 1.5 * 2^23: adding it leaves round(x) in the low bits
-    const uint64_t t = add2(x, pack2(kRound, kRound));
-    const uint64_t f = fma2(add2(t, pack2(-kRound, -kRound)), pack2(-1.f, -1.f), x);
-    // least relative error on [-1/2, 1/2], fitted by reweighted least squares
-    constexpr float c[6] = {1.0000001f, 0.69314694f, 0.2402212f, 0.05550713f, 0.009675541f, 0.0013276472f};
-    uint64_t y = pack2(c[5], c[5]);
-#pragma unroll
-    for (int k = 4; k >= 0; --k) y = fma2(y, f, pack2(c[k], c[k]));
-    float t0, t1;
-    unpack2(t, t0, t1);
-    const uint64_t two_n = pack2(__int_as_float((__float_as_int(t0) << 23) + 0x3f800000), __int_as_float((__float_as_int(t1) << 23) + 0x3f800000));
-    unpack2(fma2(y, two_n, 0ull), e0, e1);
-}
-
 // 32 weights exp2(scale * s - ref) of one row as bf16 pairs, added to the packed row sums: two scores per instruction
-// (packed fp32 FMA and add), POLY of the 16 pairs exponentiated on the FMA pipe.
-template <int POLY>
-__device__ __forceinline__ void weights32(const uint32_t (&s)[32], float ref, uint64_t& ls0, uint64_t& ls1, uint32_t* packed) {
+// (packed fp32 FMA and add).  `top`: largest score so far.
+__device__ __forceinline__ void weights32(const uint32_t (&s)[32], float ref, uint64_t& ls0, uint64_t& ls1, float& top, uint32_t* packed) {
     const uint64_t sc2 = pack2(kScaleLog2, kScaleLog2), nm2 = pack2(-ref, -ref);
 #pragma unroll
     for (int c = 0; c < 32; c += 2) {
-        const uint64_t x = fma2(pack2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, nm2);
+        top = max3(top, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
         float e0, e1;
-        if (((c >> 1) * POLY + 15) % 16 < POLY) {
-            exp2_poly2(x, e0, e1);
-        } else {
-            unpack2(x, e0, e1);
-            e0 = fast_exp2(e0), e1 = fast_exp2(e1);
-        }
+        unpack2(fma2(pack2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, nm2), e0, e1);
+        e0 = fast_exp2(e0), e1 = fast_exp2(e1);
         if (c & 2) ls1 = add2(ls1, pack2(e0, e1));
         else ls0 = add2(ls0, pack2(e0, e1));
         packed[c >> 1] = pack_bf16(e0, e1);
@@ -394,8 +361,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
             uint32_t t0 = 0;
             for (uint32_t i = 1;; ++i) {
                 const uint32_t tag = load_tagged(addr, v);
-                rounding = bf16_hi(tag);
-                if (__all_sync(0xffffffffu, (tag & 0xffffu) == (item & 0xffffu))) return true;
+                rounding = __uint_as_float(tag & ~0xffu);
+                if (__all_sync(0xffffffffu, (tag & 0xffu) == (item & 0xffu))) return true;
                 if ((i & (kWaitPollsPerClockRead - 1)) == 0 || s_abort[1] == 0) {
                     const uint32_t now = global_timer_lo() | 1u;
                     if (t0 == 0) t0 = now;
@@ -419,8 +386,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
             const int i = (int)rank * tile_tok + (t >> g_shift);  // token of this row within the item
             const int limit = min(first_pos + i + 1, key_end);     // first key this row does not see
             const int plain_keys = min(first_pos + (int)rank * tile_tok + 1, key_end);  // keys that every row of this CTA sees
-            float rounding = 0.f;      // what rounding the weights of masked halves has added to l
+            float rounding = 0.f;      // what rounding the weights has added to l
             float ref = 0.f, l = 0.f;  // l: sum of this thread's weights (or their maximum)
+            float top = -INFINITY;     // largest score of its halves that needed no mask
             if (mode == kModeRelative) {
                 ref = -INFINITY;
                 for (uint32_t wg = 0; wg < 4 && ok; ++wg) {
@@ -447,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                 for (int c = 0; c < 32; c += 2) mx = max3(mx, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]));
                 // (rows that see fewer than 64 keys: below; they are in items of at most three tiles)
                 if (limit - key_begin >= 64 && fabsf(mx) < INFINITY) ref = mx * kScaleLog2;
-                if (h == 0 && n_tiles > 3) store_tagged(row_ref(n_item), ref, n_item & 0xffffu);
+                if (h == 0 && n_tiles > 3) store_tagged(row_ref(n_item), ref, n_item & 0xffu);
             } else if (mode == kModePlain && n_tiles > 3) {
                 float unused;
                 ok = read_tagged(row_ref(n_item), n_item, ref, unused);
@@ -471,8 +439,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                     tmem_ld32(s_addr + 32, s1);
                     tmem_wait_ld();
                     uint64_t ls0 = 0ull, ls1 = 0ull;
-                    weights32<kPolyPairs>(s0, ref, ls0, ls1, packed);
-                    weights32<kPolyPairs>(s1, ref, ls0, ls1, packed + 16);
+                    weights32(s0, ref, ls0, ls1, top, packed);
+                    weights32(s1, ref, ls0, ls1, top, packed + 16);
                     tmem_st32(s_addr, packed);
                     float a0, a1, a2, a3;
                     unpack2(ls0, a0, a1);
@@ -557,7 +525,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
             // ---- end of the item.  Every warpgroup leaves its sums; the two of the last tile wait for its PV and write the
             // output (64 columns each), the others go on with the next item, so that the tensor core does not run dry. ----
             const uint32_t g_last = n_tiles <= 3 ? g0 : g0 ^ (uint32_t)((n_tiles & 1) ^ 1);
-            store_tagged(row_part(n_item, 2 * w + h), l, (n_item & 0xffffu) | (pack_bf16(0.f, rounding) & 0xffff0000u));
+            if (mode != kModeMax) {
+                // PV multiplies rounded weights, and their sum is what normalises the output.  Where rounding matters a few keys
+                // have most of the weight; counting it for the largest weight of each of a row's four threads leaves as small an
+                // error as summing all the rounded weights (which would take two additions a pair of scores more).
+                const float e = fast_exp2(fmaf(top, kScaleLog2, -ref)), d = bf16_lo(pack_bf16(e, 0.f)) - e;
+                l += d;
+                rounding += d;
+            }
+            store_tagged(row_part(n_item, 2 * w + h), l, (n_item & 0xffu) | (__float_as_uint(rounding) & ~0xffu));
             auto give_back = [&]() {
                 __syncwarp();
                 arrive_at_if(items + Bars::item_empty + 8 * (n_item % kItemRing), lane == 0);
