@@ -162,8 +162,9 @@ ps_status ps_kv_status(ps_kv *kv, void *stream);
  * *plan_inout == NULL creates a plan; otherwise the existing plan is rebuilt
  * in place, reusing its pinned staging memory (the call first waits until the
  * plan's last ps_attn_run has finished reading that memory).  Running the
- * device is not needed: the only CUDA calls are pinned-memory management and,
- * if opts->num_sms == 0, a device-attribute query.
+ * device is not needed, and no device memory is allocated: the only CUDA calls
+ * are pinned-memory management, the creation of the plan's own streams and
+ * events and, if opts->num_sms == 0, a device-attribute query.
  * *workspace_bytes_out: device bytes ps_attn_run needs for this plan.
  * Errors: PS_ERR_INVALID (n < 1, q_len < 1, prior < 0, kv_len too long),
  * PS_ERR_UNSUPPORTED (shape), PS_ERR_OOM.
@@ -227,8 +228,11 @@ ps_status ps_plan_get_items(const ps_plan *plan, int32_t *decode_items_out, int6
  * Small batches (at most 148 decode pieces and 64 prefill items, none of them
  * cut) differ: their work list travels with the kernels' parameters, nothing
  * is uploaded and the workspace is not touched.  Kernels may be launched while
- * the kernel before them in `stream` still runs; each waits for its end before
- * it reads or writes device memory, so stream order holds as usual.
+ * the kernel before them in `stream` still runs; until all kernels of earlier
+ * calls have completed they read no more than their own run's work list and
+ * count in its header, so stream order holds as usual.  (A prefill kernel
+ * beside the decode kernel of its own run starts when that one has seen them
+ * complete, and ends after it.)
  * Ordering rule for the workspace: all runs that use one workspace -- of one
  * plan, re-planned or not, and of different plans that take turns on it --
  * must be issued to the same stream, or be ordered by the caller.  Under that
@@ -257,7 +261,9 @@ ps_status ps_attn_run(ps_plan *plan, const ps_kv *kv, const void *q_dev, const i
  * or a work record pointing outside the batch, which was not followed; the
  * output is invalid) or PS_ERR_TIMEOUT (a bounded wait expired; output is
  * invalid).  The status word lives in the workspace: read it before another
- * plan runs on the same workspace. */
+ * plan runs on the same workspace.  (A small batch's, whose run does not touch
+ * the workspace, is one of 256 in the library's device image, a plan's own
+ * until it is freed; further plans alive upload small batches' lists too.) */
 ps_status ps_plan_status(ps_plan *plan, void *stream);
 
 /*

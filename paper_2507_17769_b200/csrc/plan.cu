@@ -106,6 +106,48 @@ bool claim_workspace(const void* ws, uint64_t serial) {
     return false;
 }
 
+// Status words of runs whose work list travels as kernel parameters: such a run touches no workspace, and a plan allocates no
+// device memory, so they are part of the library's device image, one for each of up to kOwnHeaders plans alive (others upload
+// their lists).  Tags (report()) go on rising from one owner of a word to the next, which tells a late report of the last
+// owner apart.
+constexpr int kOwnHeaders = 256, kMaxDevices = 64;
+__device__ WsHeader g_own_hdr[kOwnHeaders];
+std::mutex g_own_mu;
+int32_t g_own_given_back[kOwnHeaders], g_own_n_given_back = 0, g_own_never_used = 0;
+uint32_t g_own_runs[kOwnHeaders];
+
+int32_t acquire_own_header(uint32_t* runs) {
+    std::lock_guard<std::mutex> lock(g_own_mu);
+    int32_t k = -1;
+    if (g_own_n_given_back > 0) k = g_own_given_back[--g_own_n_given_back];
+    else if (g_own_never_used < kOwnHeaders) k = g_own_never_used++;
+    if (k >= 0) *runs = g_own_runs[k];
+    return k;
+}
+
+void release_own_header(int32_t k, uint32_t runs) {
+    if (k < 0) return;
+    std::lock_guard<std::mutex> lock(g_own_mu);
+    g_own_runs[k] = runs;
+    g_own_given_back[g_own_n_given_back++] = k;
+}
+
+// its address on the current device, or null
+WsHeader* own_header(int32_t k) {
+    static std::atomic<WsHeader*> base[kMaxDevices];
+    int dev = -1;
+    if (k < 0 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    WsHeader* p = base[dev].load(std::memory_order_relaxed);
+    if (!p) {
+        if (cudaGetSymbolAddress((void**)&p, g_own_hdr) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        base[dev].store(p, std::memory_order_relaxed);
+    }
+    return p + k;
+}
+
 void forget_plan(uint64_t serial) {
     std::lock_guard<std::mutex> lock(g_ws_mu);
     for (auto it = g_ws_owner.begin(); it != g_ws_owner.end();)
@@ -162,9 +204,9 @@ struct ps_plan {
     void* last_ws = nullptr;
     WsHeader* last_hdr = nullptr;
     int32_t last_tag = 0;
-    // Small batches: the work list travels as kernel parameters, the run needs no workspace, and its status word is here.
+    // Small batches: the work list travels as kernel parameters, and the run's status word is one of the library's.
     bool inline_list = false;
-    WsHeader* own_hdr = nullptr;
+    int32_t own_hdr = -1;
     uint32_t inline_runs = 0;
     // optional per-kernel timing: 6 events per recorded run (begin/end of prefill, decode, merge)
     bool timing = false;
@@ -553,6 +595,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         pl = new (std::nothrow) ps_plan();
         if (!pl) return fail(PS_ERR_OOM, "host allocation failed");
         pl->serial = next_plan_serial();
+        pl->own_hdr = acquire_own_header(&pl->inline_runs);
     } else if (pl->copy_pending && pl->ev_copied[pl->last_slot]) {
         cudaError_t e = cudaEventSynchronize(pl->ev_copied[pl->last_slot]);
         if (e != cudaSuccess) return fail(PS_ERR_CUDA, "cudaEventSynchronize failed: %s", cudaGetErrorString(e));
@@ -568,7 +611,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         pl->num_sms = pl->device_sms;
     }
     if (pl->num_sms <= 0) {
-        if (fresh) delete pl;
+        if (fresh) ps_plan_free(pl);
         return fail(PS_ERR_CUDA, "no CUDA device to plan for (pass opts->num_sms to plan without one)");
     }
     pl->prefill.clear();
@@ -657,7 +700,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
                       (pl->prefill.empty() || (pl->prefill.size() <= kInlineItems && pl->merge.empty() && !pl->prefill_cta_start.empty() &&
                                                pl->prefill_cta_start.size() <= kInlineStarts));
     if (n_slots > 0x7fffffffLL) {
-        if (fresh) delete pl;
+        if (fresh) ps_plan_free(pl);
         return fail(PS_ERR_UNSUPPORTED, "partial buffer would need %lld slots", (long long)n_slots);
     }
 
@@ -695,7 +738,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         }
         if (!pl->pinned) {
             pl->pinned_cap = 0;
-            if (fresh) delete pl;
+            if (fresh) ps_plan_free(pl);
             return fail(PS_ERR_OOM, "cannot allocate %zu bytes of staging memory", cap);
         }
         pl->pinned_cap = cap;
@@ -715,12 +758,6 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             pl->copy_stream = nullptr;  // uploads then go on the caller's stream
             if (pl->side_stream) cudaStreamDestroy(pl->side_stream);
             pl->side_stream = nullptr;  // mixed batches then run their two kernels one after the other
-        } else if (cudaMalloc((void**)&pl->own_hdr, sizeof(WsHeader)) != cudaSuccess ||
-                   cudaMemsetAsync(pl->own_hdr, 0, sizeof(WsHeader), pl->copy_stream) != cudaSuccess ||
-                   cudaStreamSynchronize(pl->copy_stream) != cudaSuccess) {
-            (void)cudaGetLastError();
-            if (pl->own_hdr) cudaFree(pl->own_hdr);
-            pl->own_hdr = nullptr;  // every list is uploaded then
         }
     }
     memset(pl->pinned, 0, 256);
@@ -769,7 +806,7 @@ ps_status ps_plan_free(ps_plan* pl) {
     if (pl->ev_fork) cudaEventDestroy(pl->ev_fork);
     if (pl->ev_join) cudaEventDestroy(pl->ev_join);
     for (cudaEvent_t e : pl->tev) cudaEventDestroy(e);
-    if (pl->own_hdr) cudaFree(pl->own_hdr);  // (waits for the kernels that may still write it)
+    release_own_header(pl->own_hdr, pl->inline_runs);
     if (pl->pinned) { if (pl->pinned_is_cuda) cudaFreeHost(pl->pinned); else free(pl->pinned); }
     delete pl;
     return PS_OK;
@@ -826,7 +863,8 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     // The upload may run under the kernels of the previous run only if this plan's own record of the two slots is
     // all there is to know about the workspace: same memory as last time, slots where they were, and no other
     // plan's run on it since.
-    const bool as_params = pl->inline_list && pl->own_hdr && !capturing;  // (a graph's replays copy the staging image)
+    WsHeader* const own_hdr = pl->inline_list && !capturing ? own_header(pl->own_hdr) : nullptr;  // (a graph's replays copy the staging image)
+    const bool as_params = own_hdr != nullptr;
     const bool known = !as_params && claim_workspace(workspace_dev, pl->serial) && pl->last_ws == workspace_dev && !pl->layout_moved;
     if (as_params) {
         // nothing to upload, and nothing of the workspace is used
@@ -861,8 +899,12 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     }
     // the upload is in place (or queued): only now does the run count
     if (as_params) {
-        pl->inline_runs = pl->inline_runs % 0x1fffffffu + 1;
-        pl->last_hdr = pl->own_hdr;
+        if (pl->inline_runs == 0x1fffffffu) {  // tags begin again
+            PS_CUDA_TRY(cudaMemsetAsync(own_hdr, 0, sizeof(WsHeader), s));
+            pl->inline_runs = 0;
+        }
+        ++pl->inline_runs;
+        pl->last_hdr = own_hdr;
         pl->last_tag = (int32_t)(pl->inline_runs << 2);
     } else {
         ++pl->run_no;
