@@ -324,7 +324,10 @@ ps_status ps_attn_run_static(ps_plan *plan, const ps_kv *kv, const void *q_dev, 
  * ps_attn_run record CUDA events around the prefill, decode and merge launches
  * (on the stream each is launched on; max_runs = 0 switches recording off;
  * when the two kernels of a mixed batch run side by side their intervals
- * overlap and each is longer than the kernel would take alone); calling it again
+ * overlap and each is longer than the kernel would take alone; such a run puts
+ * the decode kernel on the plan's second stream even where it would otherwise
+ * launch both on `stream`, so as a whole it takes some microseconds longer than
+ * one that is not recorded); calling it again
  * restarts the count.  ps_plan_get_timing synchronises `stream` and returns
  * the mean duration in milliseconds of each kernel over the runs recorded so
  * far, and how many there were.  A kernel the plan does not launch reports the

@@ -963,15 +963,16 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     bool merged = false;  // the merge kernel has been launched already
     // dynamic item queue with more items than workers: the decode kernel's SMs help once it has ended
     const bool helpers = a.w.n_prefill_ctas == 0 && a.w.n_prefill > pl->pf_workers;
-    if (pl->concurrent && (as_params || (!capturing && !helpers && a.w.n_merge == 0))) {
+    if (pl->concurrent && !(rec && pl->side_stream) && (as_params || (!capturing && !helpers && a.w.n_merge == 0))) {
         // Mixed batch without more to launch than its two kernels: both on the caller's stream, the prefill kernel launched as
         // soon as the decode kernel has begun and waiting for its end only at its own.  (A second stream costs two events,
         // which take some 3 us each between kernels: tiny mixed batch 22.5 -> 16.8 us, with the list as parameters; 32 rows of
         // 2048 tokens beside a 512-token chunk 58.1 -> 57.2.  A merge kernel would have to wait for the decode kernel too, and
-        // helpers have to start as soon as that ends, so such batches keep the second stream.)
+        // helpers have to start as soon as that ends, so such batches keep the second stream.  So do runs that record events:
+        // one between the two launches would hold the prefill kernel back until the decode kernel's end.)
         RunArgs ad = a;
         ad.sm_pairs = pl->pf_workers < pl->pf_sms;
-        if (rec) cudaEventRecord(ev[2], s);
+        if (rec) cudaEventRecord(ev[2], s);  // (without a second stream the kernels follow one another)
         st = launch_decode(ad);
         if (rec && st == PS_OK) cudaEventRecord(ev[3], s);
         if (rec && st == PS_OK) cudaEventRecord(ev[0], s);

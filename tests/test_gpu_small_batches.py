@@ -1,5 +1,6 @@
 """Small batches, whose work lists travel as kernel parameters: the status words of their runs, which the library keeps for a
-limited number of plans and hands from a freed plan to the next."""
+limited number of plans and hands from a freed plan to the next.  And batches whose two kernels are launched on one stream: what
+per-kernel timing reports of them."""
 import numpy as np
 import pytest
 
@@ -70,3 +71,30 @@ def test_more_plans_alive_than_status_words():
     finally:
         for plan in plans:
             ps.ps_plan_free(plan)
+
+
+@pytest.mark.parametrize("rows,ctx,chunk", [(32, 2000, 256), (16, 4000, 96)])
+def test_recording_times_leaves_the_kernels_side_by_side(rows, ctx, chunk):
+    """The two kernels' recorded intervals overlap as the kernels of a run that is not recorded do: recorded one after the
+    other, a run takes more than their sum.  Outputs are the same."""
+    import torch
+    from workloads.device import DeviceBatch
+
+    rng = np.random.default_rng(1020)
+    db = DeviceBatch(gen.make_batch(gen.SHAPE_8B, 1020, rng.integers(ctx * 3 // 4, ctx * 5 // 4, rows).tolist() + [2000], [1] * rows + [chunk]))
+    info = db.plan()
+    assert info.decode_sms + info.prefill_sms == torch.cuda.get_device_properties(0).multi_processor_count and info.n_launches == 2
+    want = db.run()
+    runs, total = 20, []
+    ps.ps_plan_set_timing(db.pa._plan, runs)
+    for _ in range(runs):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        out, lse = db.run()
+        e1.record()
+        torch.cuda.synchronize()
+        total.append(e0.elapsed_time(e1))
+    prefill, decode, _, n = ps.ps_plan_get_timing(db.pa._plan, torch.cuda.current_stream().cuda_stream)
+    db.pa.check()
+    assert n == runs and torch.equal(out.view(torch.int16), want[0].view(torch.int16)) and torch.equal(lse, want[1])
+    assert np.median(total) < prefill + decode, (np.median(total), prefill, decode)
