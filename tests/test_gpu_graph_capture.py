@@ -48,3 +48,48 @@ def test_captured_run_replays_the_plan(which):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, eager)
+
+
+@pytest.mark.parametrize("joined", [False, True])
+def test_captured_append_and_gather_follow_the_kernels_that_make_their_inputs(joined):
+    """Appends and gathers are launched early behind a kernel; in a graph they still wait for what they read, one producer or
+    (``joined``) two on different branches, and what follows them waits for them."""
+    import torch
+
+    n, hkv, d = 700, 8, 128
+    pa = ps.PagedAttention(32, hkv, d, 64, poison=True)
+    bt = torch.randperm(64, device="cuda").to(torch.int32)[None].contiguous()
+    src = torch.zeros((n, hkv, d), dtype=torch.bfloat16, device="cuda")
+    k, v = torch.empty_like(src), torch.empty_like(src)
+    other, side = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def step():
+        if joined:
+            other.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(other):
+                for _ in range(20):
+                    v.copy_(src).mul_(2)
+        for _ in range(20):
+            torch.add(src, 1, out=k)
+        if joined:
+            torch.cuda.current_stream().wait_stream(other)
+        else:
+            torch.mul(src, 2, out=v)
+        pa.write(k, v, bt, [100], [n])
+        gk, gv = pa.gather(bt[0], 100 + n)
+        return gk[100:] + 0, gv[100:] + 0
+
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        gk, gv = step()
+    for i in range(1, 6):
+        src.copy_(torch.randn_like(src))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(gk, src + 1) and torch.equal(gv, src * 2), "replay %d" % i
+    pa.check_pool()
+    pa.close()
