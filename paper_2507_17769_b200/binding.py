@@ -140,6 +140,11 @@ def _ptr(x):
     return int(x)
 
 
+def _plain(x):
+    """A handle or a number, which may be a ctypes object, as the extension module takes it."""
+    return x.value if isinstance(x, ctypes._SimpleCData) else x
+
+
 def _host_i32(a):
     arr = np.ascontiguousarray(a, dtype=np.int32)
     return arr, arr.ctypes.data_as(_i32p)
@@ -186,13 +191,13 @@ def ps_kv_free(kv):
 
 def ps_kv_write(kv, k_new_dev, v_new_dev, block_table_dev, max_pages, prior_host, q_len_host, stream=None):
     load()
-    _check(_calls.kv_write(kv, _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), max_pages, lengths(prior_host),
+    _check(_calls.kv_write(_plain(kv), _ptr(k_new_dev), _ptr(v_new_dev), _ptr(block_table_dev), _plain(max_pages), lengths(prior_host),
                            lengths(q_len_host), _ptr(stream)))
 
 
 def ps_kv_gather(kv, block_table_row_dev, length, k_out_dev, v_out_dev, stream=None):
     load()
-    _check(_calls.kv_gather(kv, _ptr(block_table_row_dev), length, _ptr(k_out_dev), _ptr(v_out_dev), _ptr(stream)))
+    _check(_calls.kv_gather(_plain(kv), _ptr(block_table_row_dev), _plain(length), _ptr(k_out_dev), _ptr(v_out_dev), _ptr(stream)))
 
 
 def ps_kv_gather_fp8(kv, block_table_row_dev, length, k_codes_out_dev, v_codes_out_dev, k_scale_out_dev, v_scale_out_dev, stream=None):
@@ -208,7 +213,7 @@ def ps_attn_plan(shape: ps_shape, prior_host, q_len_host, max_pages_per_seq, opt
     """Returns (plan handle, workspace bytes).  Pass ``plan`` to rebuild an existing handle in place."""
     lib = load()
     if opts is None:
-        status, handle, ws = _calls.attn_plan(ctypes.addressof(shape), lengths(prior_host), lengths(q_len_host), max_pages_per_seq, plan)
+        status, handle, ws = _calls.attn_plan(ctypes.addressof(shape), lengths(prior_host), lengths(q_len_host), _plain(max_pages_per_seq), plan)
         _check(status)
         return handle, ws
     pr, prp = _host_i32(prior_host)
@@ -240,8 +245,8 @@ def ps_plan_get_items(plan):
 
 def ps_attn_run(plan, kv, q_dev, block_table_dev, out_dev, lse_out_dev, workspace_dev, workspace_bytes, stream=None):
     load()
-    _check(_calls.attn_run(plan, kv, _ptr(q_dev), _ptr(block_table_dev), _ptr(out_dev), _ptr(lse_out_dev), _ptr(workspace_dev),
-                           workspace_bytes, _ptr(stream)))
+    _check(_calls.attn_run(_plain(plan), _plain(kv), _ptr(q_dev), _ptr(block_table_dev), _ptr(out_dev), _ptr(lse_out_dev), _ptr(workspace_dev),
+                           _plain(workspace_bytes), _ptr(stream)))
 
 
 PS_STATIC_WORKSPACE_BYTES = 8 << 20

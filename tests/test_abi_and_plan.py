@@ -28,6 +28,23 @@ def test_library_exports_every_declared_symbol():
     assert "sm_100a" in ps.ps_version()
 
 
+def test_per_iteration_calls_take_ctypes_handles_and_numbers():
+    """The calls that go through the extension module accept what ctypes would: handles as c_void_p, numbers as c_int32 and so
+    on.  (Null handles: the library refuses them before it looks at anything else.)"""
+    import ctypes
+
+    one = np.ones(1, np.int32)
+    null = ctypes.c_void_p(None)
+    for call in (lambda: B.ps_kv_write(null, 16, 16, 16, ctypes.c_int32(4), one, one), lambda: B.ps_kv_gather(null, 16, ctypes.c_int32(4), 16, 16),
+                 lambda: B.ps_attn_run(null, null, 16, 16, 16, None, 16, ctypes.c_size_t(256))):
+        with pytest.raises(ps.PsError) as e:
+            call()
+        assert e.value.status == B.PS_ERR_INVALID
+    with pytest.raises(ps.PsError) as e:
+        ps.ps_attn_plan(ps.make_shape(32, 8, 128), one, one, ctypes.c_int32(0))
+    assert e.value.status == B.PS_ERR_INVALID
+
+
 def test_kv_bytes_and_shape_validation():
     s = ps.make_shape(32, 8, 128)
     assert ps.ps_kv_bytes(s, 10) == 10 * 8 * 2 * 16 * 128 * 2
