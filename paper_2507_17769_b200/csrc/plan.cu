@@ -423,8 +423,9 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 cuts.push_back(Cut{(int)i, kt0});
             }
         }
-    } else if ((int64_t)tiles.size() < 4LL * pl->pf_workers) {
-        // Few items per SM: give every CTA an equal share of the flattened (item, key tile) cost
+    } else if ((int64_t)tiles.size() < 4LL * pl->pf_sms) {
+        // Few items per SM (of a pair's two as well: with a queue from 4 items a pair, mixed batches that split evenly enough
+        // brought in helpers which found it empty, 6 us behind the decode kernel's end): give every CTA an equal share of the flattened (item, key tile) cost
         // line, cutting items where a share ends.  Only the cut items need the merge.
         static_partition = true;
         double total = 0;

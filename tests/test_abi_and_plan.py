@@ -302,3 +302,20 @@ def test_fp8_cache_shapes_plan_decode_rows_only():
     with pytest.raises(ps.PsError) as e:
         ps.ps_kv_bytes(ps.make_shape(8, 8, 64, 16, 1), 3)
     assert e.value.status == B.PS_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("hq,rows,ctx,chunks", [(32, 100, 2000, [600, 420]), (64, 146, 1200, [290, 160, 200, 260]), (32, 64, 1000, [600] * 4)])
+def test_mixed_batches_that_split_evenly_launch_two_kernels(hq, rows, ctx, chunks):
+    """Four items per SM and fewer are divided among the prefill kernel's workers beforehand, pairs of SMs or single ones:
+    from a queue the decode kernel's SMs would have to be sent helpers as well."""
+    prior = np.array([ctx - 1] * rows + [1000] * len(chunks), np.int32)
+    q_len = np.array([1] * rows + chunks, np.int32)
+    plan, _ = ps.ps_attn_plan(ps.make_shape(hq, 8, 128), prior, q_len, 2048, opts())
+    try:
+        info = ps.ps_plan_get_info(plan)
+        assert info.decode_sms + info.prefill_sms == 148  # side by side
+        cut = (ps.ps_plan_get_items(plan)[1][:, 6] >= 0).any()  # (cut items: a merge kernel as well)
+        assert info.n_prefill_items > 4 * (info.prefill_sms // 2) or cut
+        assert info.n_launches == (3 if cut else 2)
+    finally:
+        ps.ps_plan_free(plan)
