@@ -217,7 +217,7 @@ struct DeviceWork {       // pointers into the workspace for one run
     int32_t n_units, n_prefill, n_merge, n_dmerge;
     int64_t n_part_slots;              // rows of part_lse / part_o
     const int32_t* prefill_cta_start;  // static prefill partition (n_prefill_ctas + 1 entries), unused when 0
-    int32_t n_prefill_ctas;            // entries of that partition: CTAs, or CTA pairs at head dimension 128
+    int32_t n_prefill_ctas;            // entries of that partition: CTAs, or CTA pairs
 };
 
 struct RunArgs {
@@ -233,6 +233,7 @@ struct RunArgs {
     cudaStream_t stream;
     int num_sms;
     int dec_sms, pf_sms;  // SMs (= CTAs) for the decode and the prefill kernel
+    bool pairs;           // the prefill items go to CTA pairs
     bool sm_pairs;        // side by side with the pair kernel: the decode kernel's CTAs take whole SM pairs too
     // work lists as kernel parameters, on the host; null: they are in the workspace
     const DecodePiece* inline_pieces;

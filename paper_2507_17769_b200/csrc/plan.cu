@@ -50,13 +50,22 @@ struct PrefillModel {
     double cut;           // steps that cutting items costs: partial rows, merge kernel
     int sms_per_worker;   // an item is worked on by one CTA, or by a pair of them
 };
-// head dimension 64 (prefill.cu; fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a
-// masked tile)
+// prefill.cu (fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile)
 constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 1};
-// head dimension 128 (prefill_pair.cu; 72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of
-// a pair, 2.8 us per item; the merge kernel takes about 8 us)
+// prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
+// item; the merge kernel takes about 8 us)
 constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 2};
-static inline const PrefillModel& prefill_model(const ps_shape& sh) { return sh.head_dim == 128 ? kPairModel : kSingleModel; }
+static inline const PrefillModel& prefill_model(bool pairs) { return pairs ? kPairModel : kSingleModel; }
+// Which kernel runs the prefill items.  Head dimension 64: a CTA per item.  128: a pair of CTAs, unless the items are short and
+// there are enough for all SMs.  An item costs a CTA 3.5 us and 2.2 more a key tile, a pair 3.2 us and 0.73, so up to some
+// four key tiles two items on two CTAs are done sooner; of few items a pair does each in less time.
+// Measured (a run, us, single / pair): fresh prompts of 64 tokens 24 of them 19.4 / 23.5, 188 74 / 98; of 256 6 20.9 / 25.2,
+// 24 48.5 / 61; of 512 6 35 / 42, 48 200 / 229; of 1024 12 151 / 148; 64 tokens on 192 40 times 45 / 34, 94 times 53 / 65; on
+// 320 188 times 116 / 123; on 576 164 / 159.
+static inline bool prefill_on_pairs(const ps_shape& sh, int num_sms, int64_t items, int64_t key_tiles) {
+    const bool many = items >= 2.5 * num_sms && key_tiles <= 4.0 * items, some = items >= 1.25 * num_sms && key_tiles <= 1.75 * items;
+    return sh.head_dim == 128 && !many && !some;
+}
 
 // A chunk of a few tokens runs as that many decode rows (token i of the chunk is a row that sees prior + i + 1 keys
 // of the same sequence) instead of bringing in the prefill kernel for one small item: its launch and pipeline fill
@@ -163,7 +172,8 @@ struct ps_plan {
     // decode kernel (HBM-bound: a fraction of the SMs saturates the memory system) and the prefill kernel
     // (tensor-bound) run side by side on disjoint sets of SMs
     int32_t dec_sms = 0, pf_sms = 0;
-    int32_t pf_workers = 0;  // what prefill items are handed to: CTAs, or CTA pairs (one SM each) at head dimension 128
+    bool pairs = false;      // prefill items go to CTA pairs
+    int32_t pf_workers = 0;  // what they are handed to: CTAs, or CTA pairs (one SM each)
     bool concurrent = false;
     bool tiny_as_rows = false;  // this batch runs its chunks of a few tokens as decode rows
     std::vector<DecodePiece> pieces;
@@ -383,7 +393,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                          const ps_plan_opts* opts, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     const int tile_tok = kPrefillRowsPerItem / G;
-    const PrefillModel& cost = prefill_model(pl->shape);
+    const PrefillModel& cost = prefill_model(pl->pairs);
     struct Tile { int r, g, tok0, n_tok, first_pos, key_tiles; };
     std::vector<Tile> tiles;
     size_t n_tiles = 0;
@@ -404,6 +414,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
     }
     pl->prefill_cta_start.clear();
     if (tiles.empty()) return;
+    const bool many_short = pl->shape.head_dim == 128 && !pl->pairs;  // (cutting them never pays)
 
     // (tile, key-tile index) of every cut, ascending in both: tile i is cut into pieces at these key tiles
     // (exclusive of 0 and key_tiles)
@@ -423,7 +434,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 cuts.push_back(Cut{(int)i, kt0});
             }
         }
-    } else if ((int64_t)tiles.size() < 4LL * pl->pf_sms) {
+    } else if ((int64_t)tiles.size() < 4LL * pl->pf_sms && !many_short) {
         // Few items per SM (of a pair's two as well: with a queue from 4 items a pair, mixed batches that split evenly enough
         // brought in helpers which found it empty, 6 us behind the decode kernel's end): give every CTA an equal share of the flattened (item, key tile) cost
         // line, cutting items where a share ends.  Only the cut items need the merge.
@@ -627,12 +638,25 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         // (forced prefill segments: the caller wants every chunk on the prefill kernel)
         pl->tiny_as_rows = !(opts && opts->prefill_segment_tokens > 0) && true_dec_bytes <= kTinyChunkMaxDecodeBytes;
     }
+    {
+        const int tile_tok = kPrefillRowsPerItem / (shape->n_q_heads / shape->n_kv_heads);
+        int64_t items = 0, key_tiles = 0;
+        for (int r = 0; r < n; ++r) {
+            if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) continue;
+            for (int t0 = 0; t0 < q_len_host[r]; t0 += tile_tok) {
+                items += shape->n_kv_heads;
+                key_tiles += (int64_t)shape->n_kv_heads * ((prior_host[r] + std::min(t0 + tile_tok, q_len_host[r]) + kPrefillKeyTile - 1) / kPrefillKeyTile);
+            }
+        }
+        // (forced segments: the kernel of the larger batches)
+        pl->pairs = (opts && opts->prefill_segment_tokens > 0) ? shape->head_dim == 128 : prefill_on_pairs(*shape, pl->num_sms, items, key_tiles);
+    }
     // ---- split the SMs between the two kernels of a mixed batch ----
     {
         double longest = 0;                  // steps of the longest prefill item
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
         const int G = shape->n_q_heads / shape->n_kv_heads;
-        const PrefillModel& cost = prefill_model(*shape);
+        const PrefillModel& cost = prefill_model(pl->pairs);
         const int tile_tok = kPrefillRowsPerItem / G;
         for (int r = 0; r < n; ++r) {
             if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) {
@@ -693,7 +717,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
         }
     }
-    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(*shape).sms_per_worker);
+    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->pairs).sms_per_worker);
     int64_t n_slots = 0;
     plan_decode(pl, prior_host, q_len_host, q_start, opts, &n_slots);
     plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);
@@ -929,6 +953,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.num_sms = pl->num_sms;
     a.dec_sms = pl->dec_sms;
     a.pf_sms = pl->pf_sms;
+    a.pairs = pl->pairs;
     a.total_q = (int32_t)pl->info.total_q_tokens;
     a.n_req = pl->n;
     a.wait_limit_ns = pl->wait_limit_ns;

@@ -1,4 +1,5 @@
-// Prefill-chunk attention on the 5th-generation tensor cores, for head dimension 64 (128: prefill_pair.cu).
+// Prefill-chunk attention on the 5th-generation tensor cores, a CTA per item: for head dimension 64, and at 128 for batches of
+// many short items (others: prefill_pair.cu; the rule is prefill_on_pairs() in plan.cu).
 //
 // A chunk's rows attend the prior context plus the chunk's own earlier tokens
 // (paper sections 2.4 and 4.7); this part is a dense contraction and compute
@@ -20,18 +21,18 @@
 //   warps 4-7  the same for tile B
 //   warp 8     producer: fetches the CTA's next item and publishes its record in
 //              a shared-memory ring; Q tiles by tensor-map loads (128-byte
-//              swizzle); one 2 KB bulk async copy per (page, K|V) into
+//              swizzle); one 2 KB bulk async copy per (page, K|V, d half) into
 //              2-stage K and V rings -- the pool's page layout already is the
 //              128-byte-swizzled operand layout, so blocks are consumed in place
 //   warp 9     MMA issue: S_X = Q_X K^T (SS form, M128 N128 K16) and
 //              O_X += P_X V (A operand from TMEM, V as MN-major B operand,
-//              M128 N64 K16); completion signalled with tcgen05.commit
+//              M128 N=d K16); completion signalled with tcgen05.commit
 //
 // The roles synchronise through mbarriers only, so consecutive items overlap:
 // the next item's Q, first K/V tiles and first QK^T are under way while the
 // current item's last softmax, PV and output are still running.
 //
-// TMEM columns: S_A 0..127, S_B 128..255, O_A 256..319, O_B 384..447 (512 allocated).
+// TMEM columns: S_A 0..127, S_B 128..255, O_A 256.., O_B 384.. (512 allocated).
 // Every wait is bounded; on expiry the CTA sets the timeout status and drains.
 #include "tcgen05.cuh"
 
@@ -46,16 +47,18 @@ constexpr int kSoftmaxThreads = 256;
 constexpr int kThreads = kSoftmaxThreads + 128;
 constexpr int kRegsSoftmax = 192, kRegsOther = 120;
 constexpr int kProducerWarp = 8, kMmaWarp = 9;
-constexpr int D = 64;
 constexpr int kTileKeys = 128;
 constexpr int kRows = 128;
-constexpr float kScaleLog2 = 0.18033688f;  // log2(e) / sqrt(64)
 constexpr float kRescaleThreshold = 8.f;  // log2 units
 constexpr int kBarBlockBytes = 512;  // mbarriers, flags and the item record ring
 
-struct Cfg {
-    static constexpr int kTileBytes = kTileKeys * D * 2;         // a Q tile, a K stage or a V stage: [128 rows][128 B]
-    static constexpr int kQBytes = kTileBytes, kKBytes = kTileBytes, kVBytes = kTileBytes;
+template <int D>
+struct PrefillCfg {
+    static constexpr int kHalves = D / 64;
+    static constexpr int kHalfBytes = kTileKeys * 128;          // [128 rows][128 B]
+    static constexpr int kQBytes = kHalves * kHalfBytes;         // one Q tile
+    static constexpr int kKBytes = kHalves * kHalfBytes;         // one K stage
+    static constexpr int kVBytes = kHalves * kHalfBytes;         // one V stage
     static constexpr int kStages = 2;
     static constexpr int kOffQ = 0;                              // Q_A, Q_B
     static constexpr int kOffK = kOffQ + 2 * kQBytes;
@@ -107,7 +110,9 @@ static_assert(Bars::mma_drained % 8 == 0 && Bars::armed + 24 <= Bars::ring && si
                   Bars::bytes <= kBarBlockBytes,
               "barrier block layout");
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map, const __grid_constant__ InlineItems inl) {
+    using Cfg = PrefillCfg<D>;
     extern __shared__ char smem_raw[];
     char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -165,6 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
     static_assert(kPrefillRowsPerItem == 2 * kRows, "the planner pairs two q tiles per item");
     const int tile_tok = kRows / p.G;
     const int g_shift = 31 - __clz(p.G);  // G is a power of two
+    constexpr float kScaleLog2 = D == 128 ? 0.12751743f : 0.18033688f;  // log2(e) / sqrt(D)
 
     // consumer side of the record ring: record number n into `it`; false at the end-of-work record or on abort
     auto take_item = [&](uint32_t n, PrefillItem& it) -> bool {
@@ -214,6 +220,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                 const int limit = it.first_pos + i;            // last visible key of this row
                 const int tile_first_pos = it.first_pos + x * tile_tok;
                 float m = -INFINITY, l = 0.f;
+                float lu = 0.f;  // D = 128: the sum without the masked tiles' rounding, for the log-sum-exp
                 for (int j = 0; j < n_tiles && ok; ++j) {
                     const uint32_t tc = tile_ctr + j;  // K/V stage phase
                     ok = wait_all(bars + Bars::s_full + 8 * x, (tiles_x + j) & 1, s_abort);
@@ -273,6 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         tmem_wait_st();
                     }
                     l *= alpha;
+                    if (D == 128) lu *= alpha;
                     m = m_new;
                     const float m_sub = (m == -INFINITY) ? 0.f : m;
 
@@ -282,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         // Diagonal and ragged tiles (the only tiles of rows with few visible keys): mask by
                         // select, and sum the bf16-rounded weights that PV multiplies, so that the output
                         // of a row with a handful of keys stays an exact convex mix of V rows.
+                        uint64_t ls = 0ull;
 #pragma unroll
                         for (int hhalf = 0; hhalf < 2; ++hhalf) {
                             uint32_t packed[32];
@@ -297,10 +306,16 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                                     const uint32_t pk = pack_bf16(p0, p1);
                                     l0 += bf16_lo(pk);
                                     l1 += bf16_hi(pk);
+                                    if (D == 128) ls = add2(ls, pack2(p0, p1));
                                     packed[qq * 16 + (c >> 1)] = pk;
                                 }
                             }
                             tmem_st32(s_addr + hhalf * 32, packed);
+                        }
+                        if (D == 128) {
+                            float a0, a1;
+                            unpack2(ls, a0, a1);
+                            lu += a0 + a1;
                         }
                     } else {
                         // Interior tiles: two scores per instruction (packed fp32 FMA and add); four sum chains.
@@ -334,6 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         unpack2(ls1, a2, a3);
                         l0 = a0 + a2;
                         l1 = a1 + a3;
+                        if (D == 128) lu += l0 + l1;
                     }
                     l += l0 + l1;
                     tmem_wait_st();
@@ -347,7 +363,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         if (t >= n_keys) {
                             char* vrow = smem + Cfg::kOffV + s * Cfg::kVBytes + t * 128;
 #pragma unroll
-                            for (int u = 0; u < 8; ++u) *reinterpret_cast<uint4*>(vrow + u * 16) = make_uint4(0, 0, 0, 0);
+                            for (int h = 0; h < Cfg::kHalves; ++h)
+#pragma unroll
+                                for (int u = 0; u < 8; ++u)
+                                    *reinterpret_cast<uint4*>(vrow + h * Cfg::kHalfBytes + u * 16) = make_uint4(0, 0, 0, 0);
                         }
                         fence_proxy_async_smem();
                     }
@@ -360,38 +379,41 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                 if (ok) {
                     tc_fence_after();
                     const float inv = l > 0.f ? 1.f / l : 0.f;
-                    const float lse_v = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+                    const float lse_v = l > 0.f ? (m + log2f(D == 128 ? lu : l)) * 0.6931471805599453f : -INFINITY;
                     const int row0 = (warp & 3) * 32;          // first tile row of this warp
                     const int sub = lane >> 3, unit = lane & 7;  // write-out: 4 rows per instruction, 8 lanes x 16 bytes per row
                     char* const my_row = stg + lane * 128;
                     if (it.part_slot < 0) {
-                        // final output: bf16, 128 bytes a row
-                        uint32_t v[2][32];
-                        tmem_ld32(o_addr, v[0]);
-                        tmem_ld32(o_addr + 32, v[1]);
-                        tmem_wait_ld();
+                        // final output: bf16, 64 columns (128 bytes of each row) per pass
+#pragma unroll 1
+                        for (int c0 = 0; c0 < D; c0 += 64) {
+                            uint32_t v[2][32];
+                            tmem_ld32(o_addr + c0, v[0]);
+                            tmem_ld32(o_addr + c0 + 32, v[1]);
+                            tmem_wait_ld();
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const uint32_t* s = &v[u >> 2][(u & 3) * 8];
-                            uint4 w;
-                            w.x = pack_bf16(__uint_as_float(s[0]) * inv, __uint_as_float(s[1]) * inv);
-                            w.y = pack_bf16(__uint_as_float(s[2]) * inv, __uint_as_float(s[3]) * inv);
-                            w.z = pack_bf16(__uint_as_float(s[4]) * inv, __uint_as_float(s[5]) * inv);
-                            w.w = pack_bf16(__uint_as_float(s[6]) * inv, __uint_as_float(s[7]) * inv);
-                            *reinterpret_cast<uint4*>(my_row + ((u ^ (lane & 7)) << 4)) = w;
-                        }
-                        __syncwarp();
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int r = k * 4 + sub, tt = row0 + r;
-                            const int i_r = x * tile_tok + (tt >> g_shift);
-                            if (i_r < it.n_tok) {
-                                const uint4 w = *reinterpret_cast<const uint4*>(stg + r * 128 + ((unit ^ (r & 7)) << 4));
-                                const int64_t orow_r = (int64_t)(it.q_tok + i_r) * p.Hq + it.kv_head * p.G + (tt & (p.G - 1));
-                                *reinterpret_cast<uint4*>(p.out + orow_r * D + unit * 8) = w;
+                            for (int u = 0; u < 8; ++u) {
+                                const uint32_t* s = &v[u >> 2][(u & 3) * 8];
+                                uint4 w;
+                                w.x = pack_bf16(__uint_as_float(s[0]) * inv, __uint_as_float(s[1]) * inv);
+                                w.y = pack_bf16(__uint_as_float(s[2]) * inv, __uint_as_float(s[3]) * inv);
+                                w.z = pack_bf16(__uint_as_float(s[4]) * inv, __uint_as_float(s[5]) * inv);
+                                w.w = pack_bf16(__uint_as_float(s[6]) * inv, __uint_as_float(s[7]) * inv);
+                                *reinterpret_cast<uint4*>(my_row + ((u ^ (lane & 7)) << 4)) = w;
                             }
+                            __syncwarp();
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                const int r = k * 4 + sub, tt = row0 + r;
+                                const int i_r = x * tile_tok + (tt >> g_shift);
+                                if (i_r < it.n_tok) {
+                                    const uint4 w = *reinterpret_cast<const uint4*>(stg + r * 128 + ((unit ^ (r & 7)) << 4));
+                                    const int64_t orow_r = (int64_t)(it.q_tok + i_r) * p.Hq + it.kv_head * p.G + (tt & (p.G - 1));
+                                    *reinterpret_cast<uint4*>(p.out + orow_r * D + c0 + unit * 8) = w;
+                                }
+                            }
+                            __syncwarp();
                         }
-                        __syncwarp();
                         if (valid && p.lse) p.lse[(int64_t)(it.q_tok + i) * p.Hq + it.kv_head * p.G + hh] = lse_v;
                     } else {
                         // partial result of a cut item: fp32 rows at consecutive slots, 32 columns per pass
@@ -428,12 +450,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
         if (warp == kProducerWarp) {
             // K/V tiles of a chunk's sequence are read again by every q tile of that sequence (and of its other chunks' items
-            // on other CTAs): they are marked last to leave L2, the decode kernel's streamed pages first.
+            // on other CTAs): they are marked last to leave L2, the decode kernel's streamed pages first.  Measured beside decode
+            // rows: a 2048-token chunk on 8 K with 32 decode rows 275 -> 266 us, 512 on 2 K with 128 rows 171 -> 169 us; alone
+            // within 1 %.
             const uint64_t kv_policy = l2_policy_evict_last();
             // ================================================================
             // producer: item records, Q tiles (tensor-map loads), K and V tiles (bulk copies of pool blocks)
             // ================================================================
-            const int pg = lane >> 2;  // page in tile, copied by the first of its four lanes
+            const int pg = lane >> 2, which = lane & 3;  // page in tile; 0/1 = K half 0/1, 2/3 = V half 0/1
             constexpr uint32_t kPieceBytes = kPage * 128;  // 16 tokens x 64 elements
             uint32_t n_item = 0, tile_ctr = 0, items_x[2] = {0, 0};
             const bool static_share = p.inline_list || p.cta_start;
@@ -499,9 +523,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                     const uint32_t good = __ballot_sync(0xffffffffu, lane < n_pages && in_range);
                     if (__popc(good) != n_pages && lane == 0) report(p.hdr, p.tag, kStatusBounds);
                     const int my_page = __shfl_sync(0xffffffffu, page, pg);
-                    const bool mine = (lane & 3) == 0 && ((good >> pg) & 1u);
-                    const uint32_t tile_bytes = (uint32_t)__popc(good) * kPieceBytes;
-                    const char* src = p.pool + ((int64_t)my_page * p.Hkv + it.kv_head) * (int64_t)(2 * kPieceBytes);
+                    const bool mine = (good >> pg) & 1u;
+                    const uint32_t tile_bytes = (uint32_t)__popc(good) * Cfg::kHalves * kPieceBytes;
+                    const char* src = p.pool + ((int64_t)my_page * p.Hkv + it.kv_head) * (int64_t)(2 * Cfg::kHalves * kPieceBytes);
 
                     ok = wait_all(bars + Bars::k_empty + 8 * s, par ^ 1, s_abort);
                     if (!ok) break;
@@ -510,13 +534,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         s_armed[s] = (int)par;
                     }
                     __syncwarp();
-                    if (mine)
-                        bulk_g2s_hint(sbase + Cfg::kOffK + s * Cfg::kKBytes + pg * kPieceBytes, src, kPieceBytes,
-                                      bars + Bars::k_full + 8 * s, kv_policy);
+                    if (mine && which < Cfg::kHalves)
+                        bulk_g2s_hint(sbase + Cfg::kOffK + s * Cfg::kKBytes + which * Cfg::kHalfBytes + pg * kPieceBytes,
+                                      src + which * kPieceBytes, kPieceBytes, bars + Bars::k_full + 8 * s, kv_policy);
 
                     if (j == 0) {
                         // Q tile x: rows (token, head of the group) in token-major order, one box of
-                        // [128 / G tokens][G heads][64 elements], written with the
+                        // [128 / G tokens][G heads][64 elements] per 64-element half, written with the
                         // 128-byte swizzle the MMA descriptors expect.  The buffer is free once the
                         // previous item's last QK^T of that tile has run.
                         for (int x = 0; x < n_x && ok; ++x) {
@@ -525,8 +549,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                             if (lane == 0) {
                                 mbar_expect_tx(bars + Bars::q_full + 8 * x, Cfg::kQBytes);
                                 s_armed[4 + x] = (int)(items_x[x] & 1);
-                                tma_load_3d(sbase + Cfg::kOffQ + x * Cfg::kQBytes, &q_map, 0, it.kv_head * p.G, it.q_tok + x * tile_tok,
-                                            bars + Bars::q_full + 8 * x);
+#pragma unroll
+                                for (int h = 0; h < Cfg::kHalves; ++h)
+                                    tma_load_3d(sbase + Cfg::kOffQ + x * Cfg::kQBytes + h * Cfg::kHalfBytes, &q_map, h * 64,
+                                                it.kv_head * p.G, it.q_tok + x * tile_tok, bars + Bars::q_full + 8 * x);
                             }
                             __syncwarp();
                         }
@@ -540,9 +566,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         s_armed[2 + s] = (int)par;
                     }
                     __syncwarp();
-                    if (mine)
-                        bulk_g2s_hint(sbase + Cfg::kOffV + s * Cfg::kVBytes + pg * kPieceBytes, src + kPieceBytes, kPieceBytes,
-                                      bars + Bars::v_full + 8 * s, kv_policy);
+                    if (mine && which >= 2 && which - 2 < Cfg::kHalves)
+                        bulk_g2s_hint(sbase + Cfg::kOffV + s * Cfg::kVBytes + (which - 2) * Cfg::kHalfBytes + pg * kPieceBytes,
+                                      src + (Cfg::kHalves + which - 2) * kPieceBytes, kPieceBytes, bars + Bars::v_full + 8 * s, kv_policy);
                 }
                 tile_ctr += n_tiles;
                 ++items_x[0];
@@ -554,7 +580,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
             // ================================================================
             // descriptors without their start address; a k-step adds its byte offset / 16 to the low word
             const uint64_t desc_kmajor = smem_desc(0, 16, 1024);
-            const uint64_t desc_v = smem_desc(0, Cfg::kVBytes, 1024);
+            const uint64_t desc_v = smem_desc(0, Cfg::kHalfBytes, 1024);
             uint32_t n_item = 0, tile_ctr = 0, tiles_x[2] = {0, 0}, items_x[2] = {0, 0};
             bool ok = true;
             // S_x = Q_x K^T for key tile number tc (counted over all items) of an item with n_x q tiles.
@@ -576,7 +602,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                     const uint64_t qd = desc_kmajor + ((sbase + Cfg::kOffQ + x * Cfg::kQBytes) >> 4);
                     const uint64_t kd = desc_kmajor + ((sbase + Cfg::kOffK + s * Cfg::kKBytes) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) tc_mma_ss(d_addr, qd + (kk * 32 >> 4), kd + (kk * 32 >> 4), kIdescQK, kk > 0);
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        const uint32_t off = ((kk >> 2) * Cfg::kHalfBytes + (kk & 3) * 32) >> 4;
+                        tc_mma_ss(d_addr, qd + off, kd + off, kIdescQK, kk > 0);
+                    }
                     tc_commit(bars + Bars::s_full + 8 * x);
                     if (x == n_x - 1) tc_commit(bars + Bars::k_empty + 8 * s);
                     if (last) tc_commit(bars + Bars::q_empty + 8 * x);
@@ -675,10 +704,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
 
 }  // namespace
 
-static ps_status launch_prefill_single(const RunArgs& a) {
+template <int D>
+static ps_status launch_prefill_d(const RunArgs& a) {
+    using Cfg = PrefillCfg<D>;
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
-        PS_CUDA_TRY(cudaFuncSetAttribute(prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+        PS_CUDA_TRY(cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
         return PS_OK;
     });
     if (cfg != PS_OK) return cfg;
@@ -714,12 +745,13 @@ static ps_status launch_prefill_single(const RunArgs& a) {
     if (enc != PS_OK) return enc;
 
     const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
-    return launch_kernel(prefill_kernel, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
+    return launch_kernel(prefill_kernel<D>, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
 }
 
 ps_status launch_prefill(const RunArgs& a) {
     if (a.w.n_prefill == 0) return PS_OK;
-    return a.shape.head_dim == 128 ? launch_prefill_pair(a) : launch_prefill_single(a);
+    if (a.pairs) return launch_prefill_pair(a);
+    return a.shape.head_dim == 128 ? launch_prefill_d<128>(a) : launch_prefill_d<64>(a);
 }
 
 }  // namespace ps

@@ -97,9 +97,12 @@ def test_many_short_items_per_pair():
 
 @pytest.mark.parametrize("redo", [False, True])
 def test_more_one_tile_items_per_pair_than_records_fit_its_ring(redo):
-    """13 to 15 items of one key tile per pair; with ``redo`` every ninth token's rows are computed again as well."""
+    """13 to 15 items of one key tile per pair; with ``redo`` every ninth token's rows are computed again as well.  (With a
+    segment longer than any item: the planner would otherwise give so many short items to the single-CTA kernel.)"""
+    import paper_2507_17769_b200 as ps
+
     b = gen.make_batch(gen.SHAPE_8B, 955, [0, 40] * 65, [64, 33] * 65)
-    run_and_compare(b, np.where(np.arange(b.total_q) % 9 == 0, 6, 0) if redo else np.zeros(b.total_q), "one-tile items")
+    run_and_compare(b, np.where(np.arange(b.total_q) % 9 == 0, 9, 0) if redo else np.zeros(b.total_q), "one-tile items", opts=ps.ps_plan_opts(0, 4096, 0))
 
 
 @pytest.mark.parametrize("every", [1, 3, 97])
