@@ -434,10 +434,11 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 cuts.push_back(Cut{(int)i, kt0});
             }
         }
-    } else if ((int64_t)tiles.size() < 4LL * pl->pf_sms && !many_short) {
-        // Few items per SM (of a pair's two as well: with a queue from 4 items a pair, mixed batches that split evenly enough
-        // brought in helpers which found it empty, 6 us behind the decode kernel's end): give every CTA an equal share of the flattened (item, key tile) cost
-        // line, cutting items where a share ends.  Only the cut items need the merge.
+    } else if ((int64_t)tiles.size() < 4LL * pl->num_sms && !many_short) {
+        // Few items per SM of all the device has, whatever the prefill kernel's share: the shares are planned to end together,
+        // and then the helpers that a queue brings find it empty 6 us behind the decode kernel's end (128 rows of about 2500
+        // tokens and 256 items on 60 SMs 224 us, 236 from a queue).  Give every CTA an equal share of the flattened (item, key
+        // tile) cost line, cutting items where a share ends.  Only the cut items need the merge.
         static_partition = true;
         double total = 0;
         for (const Tile& t : tiles) total += cost.fixed + t.key_tiles + cost.masked_extra;

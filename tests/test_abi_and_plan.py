@@ -304,11 +304,12 @@ def test_fp8_cache_shapes_plan_decode_rows_only():
     assert e.value.status == B.PS_ERR_UNSUPPORTED
 
 
-@pytest.mark.parametrize("hq,rows,ctx,chunks", [(32, 100, 2000, [600, 420]), (64, 146, 1200, [290, 160, 200, 260]), (32, 64, 1000, [600] * 4)])
-def test_mixed_batches_that_split_evenly_launch_two_kernels(hq, rows, ctx, chunks):
-    """Four items per SM and fewer are divided among the prefill kernel's workers beforehand, pairs of SMs or single ones:
-    from a queue the decode kernel's SMs would have to be sent helpers as well."""
-    prior = np.array([ctx - 1] * rows + [1000] * len(chunks), np.int32)
+@pytest.mark.parametrize("hq,rows,ctx,chunks,before", [(32, 100, 2000, [600, 420], 1000), (64, 146, 1200, [290, 160, 200, 260], 1000),
+                                                       (32, 64, 1000, [600] * 4, 1000), (32, 128, 2500, [2048], 0)])
+def test_mixed_batches_that_split_evenly_launch_two_kernels(hq, rows, ctx, chunks, before):
+    """Four items per SM of the device and fewer are divided among the prefill kernel's workers beforehand, pairs of SMs or
+    single ones: from a queue the decode kernel's SMs would have to be sent helpers as well."""
+    prior = np.array([ctx - 1] * rows + [before] * len(chunks), np.int32)
     q_len = np.array([1] * rows + chunks, np.int32)
     plan, _ = ps.ps_attn_plan(ps.make_shape(hq, 8, 128), prior, q_len, 2048, opts())
     try:
