@@ -695,9 +695,11 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
             // Once the decode rows saturate HBM the modelled time is flat in n; measured step times keep
             // improving a little as the decode kernel gets more SMs, as long as the prefill kernel still ends
-            // well before it.  Take the middle of that flat stretch.
+            // well before it.  Take the middle of that flat stretch.  (Not at head dimension 64, where it begins at 92 SMs and
+            // more of them gain nothing: 400 rows of about 1000 tokens and a 1024-token chunk 138.6 us at 88, 140 at 96, 146 at
+            // 112, the middle.)
             int hi = best_n;
-            for (int nd = best_n; nd <= pl->num_sms - 8; nd += 4)
+            for (int nd = best_n; shape->head_dim == 128 && nd <= pl->num_sms - 8; nd += 4)
                 if (std::max(t_dec(nd), t_pf(nd)) <= 1.015 * best_t && t_pf(nd) <= 0.8 * t_dec(nd)) hi = nd;
             best_n = (best_n + hi) / 2 / 4 * 4;
             const double t_seq = dec_bytes / kDecodePeakBytesPerSec + pf_time(pl->num_sms) + 2 * kKernelFloorSec;

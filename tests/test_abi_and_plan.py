@@ -320,3 +320,14 @@ def test_mixed_batches_that_split_evenly_launch_two_kernels(hq, rows, ctx, chunk
         assert info.n_launches == (3 if cut else 2)
     finally:
         ps.ps_plan_free(plan)
+
+
+@pytest.mark.parametrize("rows,ctx,chunks,before", [(400, 1000, [1024], 3000), (200, 4000, [400, 300], 3000), (237, 4600, [10, 10, 9, 11], 6500)])
+def test_decode_share_at_head_dimension_64(rows, ctx, chunks, before):
+    """Beside a prefill kernel that ends first the decode kernel gets the SMs with which it streams at full rate, and no more."""
+    plan, _ = ps.ps_attn_plan(ps.make_shape(8, 8, 64), np.array([ctx - 1] * rows + [before] * len(chunks), np.int32),
+                              np.array([1] * rows + chunks, np.int32), 2048, opts())
+    try:
+        assert 84 <= ps.ps_plan_get_info(plan).decode_sms <= 96
+    finally:
+        ps.ps_plan_free(plan)
