@@ -343,10 +343,15 @@ def components_alone(pa, batch, db, out, steps, peaks):
             res.append(kernel_record("decode_kernel", "decode rows alone on all SMs", dec_ms, float(batch.decode_bytes()), peaks,
                                      step_ms=step_ms))
         else:
-            res.append(kernel_record("prefill_kernel", "prefill rows alone on all SMs", pre_ms, float(batch.prefill_flops()), peaks,
+            res.append(kernel_record(prefill_kernel_name(batch), "prefill rows alone on all SMs", pre_ms, float(batch.prefill_flops()), peaks,
                                      step_ms=step_ms))
     pa.plan(batch.prior, batch.q_len, batch.max_pages)  # back to the full batch
     return res
+
+
+def prefill_kernel_name(batch):
+    """The kernel of the timed workloads' chunks (batches of many short ones would take prefill_kernel<128>)."""
+    return "prefill_pair_kernel" if batch.shape.head_dim == 128 else "prefill_kernel<64>"
 
 
 def kernel_record(kernel, where, launch_ms, units, peaks, step_ms=None):
@@ -572,7 +577,7 @@ def run_ours(args):
         if dec_bytes > 0:
             kernels.append(kernel_record("decode_kernel", where + " (%d SMs)" % info.decode_sms, dec_ms, dec_bytes, peaks))
         if pf_flops > 0:
-            kernels.append(kernel_record("prefill_kernel", where + " (%d SMs)" % info.prefill_sms, pre_ms, pf_flops, peaks))
+            kernels.append(kernel_record(prefill_kernel_name(batch), where + " (%d SMs)" % info.prefill_sms, pre_ms, pf_flops, peaks))
         if mixed:
             kernels.extend(components_alone(pa, batch, db, out, args.steps, peaks))
         if t_hbm >= t_tensor:
@@ -582,8 +587,8 @@ def run_ours(args):
         else:
             ach = pf_flops / (ms * 1e-3) / 1e12
             roof = {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
-                    "frac": ach / peaks["bf16_tflops"], "traffic": ncu_traffic("prefill_kernel", pf_flops),
-                    "dominant_kernel": "prefill_kernel"}
+                    "frac": ach / peaks["bf16_tflops"], "traffic": ncu_traffic(prefill_kernel_name(batch), pf_flops),
+                    "dominant_kernel": prefill_kernel_name(batch)}
         roof.update({"peak_source": peaks["source"], "of": "the whole step (ms_per_step)",
                      "bound_times_ms": {"hbm": t_hbm * 1e3, "tensor": t_tensor * 1e3},
                      "traffic_source": NCU_TRAFFIC_SOURCE, "launches_timed": n_timed, "merge_kernel_ms": mrg_ms,

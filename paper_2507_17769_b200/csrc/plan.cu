@@ -28,7 +28,8 @@ constexpr int kDecodeUnitsPerWarp = 1;  // work units per resident warp (measure
 // 64 tokens: 13 us instead of 20; 8 rows of 512: 16 instead of 23), but every further piece of a row is one more
 // partial result for the one warp that combines them (one row of 4096 tokens: 22 us at 32 pieces, 26 at 64).
 constexpr int kDecodeMinPagesLo = 4, kDecodeMinPagesHi = 8, kDecodePiecesPerRow = 16;
-// A CTA per piece (small batches): pages of a piece at most, and before a row is cut (8 and 4 for each of 12 warps).
+// A CTA per piece (small batches): pages of a piece at most, and before a row is cut (8 and 4 for each of the 12 warps that a
+// CTA has at head dimension 128, 4 and 2 for each of 24 at 64).
 constexpr int kCtaMaxPiece = 96, kCtaMinPiece = 48;
 constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 // Measured on B200 (bandwidth against the number of SMs the decode kernel runs on), used with the prefill kernel's cost
@@ -36,7 +37,8 @@ constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 constexpr double kDecodePeakBytesPerSec = 6.7e12;
 constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a running prefill kernel
 // Per SM with the memory system to itself, and 0.85 of it beside a prefill kernel: 16 to 48 SMs stream 130 GB/s each at head
-// dimension 128, 80 GB/s at 64, where a page is half as large and takes a warp as long.
+// dimension 128 and 81 to 89 GB/s at 64, where a page is half as large and takes a warp as long.  (At 64 the lower end is
+// taken: with 87 the planner gave the prefill kernel of 48 rows and two chunks too many SMs, 68.2 us instead of 66.8.)
 static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 80e9; }
 static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;

@@ -29,11 +29,14 @@
 // waits), and every instruction that is not in a hot loop costs its warp some 6 cycles, because four softmax warps per
 // scheduler evict it.  Hence one barrier per tile for that warp (a feeder warp waits for V on its behalf), gathered tensor
 // copies, short code at the item's end, and items begun by the group that is not writing output.
-// Measured (B200, 32 q / 8 kv heads, chunk x prior; kernel alone, CUDA events), before: one CTA per item with two q tiles
-// in turn, P in tensor memory, running row maximum.
-//     1536 x 3885  119 -> 92.5 us (1266 TFLOP/s, 0.77 of the measured cuBLAS rate)    512 x 8192  76.1 -> 60.0
-//     2048 x 8192  275 -> 215 us (1436 TFLOP/s, 0.87)    2 x 2048 on 19.8 k and 28.9 k, 64 q heads  2890 -> 2330 us (1460)
-// Steps on the way, on 2048 x 8192: pair with two score buffers and eight softmax warps 251 us; three buffers, sixteen
+// Measured (B200, 32 q / 8 kv heads, N(0,1) data, chunk x prior; kernel alone on all SMs, mean of 50 back to back between CUDA
+// events, SM clock 1965 MHz), against one CTA per item with two q tiles in turn, P in tensor memory, running row maximum
+// (prefill.cu), on the same GPU:
+//     1536 x 3885  123.7 -> 100.0 us (1171 TFLOP/s, 0.70 of the measured cuBLAS burst rate)    512 x 8192  79.2 -> 67.8
+//     2048 x 2048  116.5 -> 97.7    2048 x 8192  280.6 -> 222 us (1392 TFLOP/s, 0.83)
+//     2 x 2048 on 19.8 k and 28.9 k, 64 q heads  3080 -> 2470 us (1380); in a long run power holds it to 2770 (1230, 0.87 of
+//     cuBLAS's sustained rate).  Without the references and the rounding of the sums it takes 2 % less.
+// Steps on the way, on 2048 x 8192 (shorter runs): pair with two score buffers and eight softmax warps 251 us; three buffers, sixteen
 // warps, no maximum 245; warp-uniform MMA issue and the feeder 241; gathered copies 218; items begun by the other group and
 // part of the exponentials as a polynomial on the FMA pipe 212.  (The polynomial was taken out again: beside the maximum that
 // the sums' rounding needs it cost more than it saved, 278 us a run back to back with it and 263 without.)  Items fetched by a
