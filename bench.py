@@ -61,7 +61,7 @@ def measured_peaks():
 # proportion to the KV a launch reads, so a full launch is the ratio times its algorithmic bytes).  The decode
 # kernel's algorithmic bytes are the KV it streams; for the prefill kernel the ratio is per KV byte of its chunks'
 # sequences (its K/V tiles are re-read from L2, not from DRAM).  Re-captured whenever a kernel changes.
-NCU_TRAFFIC_RATIO = {"decode_kernel": 1.009}
+NCU_TRAFFIC_RATIO = {"decode_kernel": 1.010}
 NCU_TRAFFIC_SOURCE = "profiles/mixed_step_config2.md"
 
 
