@@ -468,8 +468,9 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 makespan = std::max(makespan, least.first);
                 std::push_heap(heap.begin(), heap.end(), std::greater<Slot>());
             }
-            // (cutting is not free either)
-            if (makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.cut)) {
+            // (cutting is not free either, and from four items a worker on it has less to gain than the partial rows cost in
+            // space, 19 MB in a batch that needs none)
+            if ((int64_t)tiles.size() >= 4LL * pl->pf_workers || makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.cut)) {
                 for (int c = 0; c < n_cta; ++c) count[c + 1] += count[c];
                 pl->prefill_cta_start.assign(count.begin(), count.end());
                 std::vector<Tile> sorted(tiles.size());

@@ -331,3 +331,15 @@ def test_decode_share_at_head_dimension_64(rows, ctx, chunks, before):
         assert 84 <= ps.ps_plan_get_info(plan).decode_sms <= 96
     finally:
         ps.ps_plan_free(plan)
+
+
+@pytest.mark.parametrize("d,n", [(128, 38), (128, 50), (128, 60), (64, 75)])
+def test_items_enough_for_a_queue_are_never_cut(d, n):
+    """From four items a worker on, items that cannot be divided evenly stay whole: cut, they would leave partial rows, and the
+    plan would outgrow the built-in scratch."""
+    plan, ws = ps.ps_attn_plan(ps.make_shape(32 if d == 128 else 8, 8, d), np.full(n, 4160, np.int32), np.full(n, 64, np.int32), 2048, opts())
+    try:
+        info = ps.ps_plan_get_info(plan)
+        assert info.n_prefill_items == 8 * n and info.n_partial_slots == 0 and ws <= ps.PS_STATIC_WORKSPACE_BYTES
+    finally:
+        ps.ps_plan_free(plan)
