@@ -252,6 +252,7 @@ struct RunArgs {
 ps_status launch_decode(const RunArgs& a);
 ps_status launch_prefill(const RunArgs& a);
 ps_status launch_prefill_pair(const RunArgs& a);  // head dimension 128
+ps_status launch_prefill_d64(const RunArgs& a);
 ps_status launch_merge(const RunArgs& a);
 int decode_warps_per_sm(int head_dim);
 
@@ -283,6 +284,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// from one lane of a converged warp, without a branch
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool yes) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)yes) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -333,6 +338,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int64_t
             else if (now - t0 > (uint64_t)limit_ns) return false;
         }
     }
+}
+
+// Wait for a phase for at most about the CTA's wait limit (nanoseconds, in the word behind the abort flag; the low
+// half of the nanosecond clock serves, so limits reach 4 s); gives up early when another role of the CTA has already
+// given up.  The role whose wait runs out raises the CTA's abort flag.  One non-blocking probe first; a limit of
+// zero gives up right after it.  The clock is read only every kWaitPollsPerClockRead failed polls.
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (mbar_test_wait(bar, parity)) return true;
+    const uint32_t limit_ns = (uint32_t)abort_flag[1];  // the wait limit sits behind the abort flag
+    if (limit_ns > 0) {
+        uint32_t t0 = 0;
+        for (uint32_t i = 1;; ++i) {
+            if (mbar_try_wait(bar, parity)) return true;
+            if ((i & (kWaitPollsPerClockRead - 1)) == 0) {
+                if (*abort_flag) return false;
+                const uint32_t now = global_timer_lo() | 1u;
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > limit_ns) break;
+            }
+        }
+    }
+    *abort_flag = 1;
+    return false;
 }
 
 // global -> shared bulk copy with an L2 eviction priority; bytes multiple of 16, both addresses 16-byte aligned

@@ -57,7 +57,10 @@ constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 1};
 // prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
 // item; the merge kernel takes about 8 us)
 constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 2};
-static inline const PrefillModel& prefill_model(bool pairs) { return pairs ? kPairModel : kSingleModel; }
+// prefill_d64.cu (148 CTAs of 1 to 3 items of 6 to 29 key tiles, beside a decode kernel: 9.4 us a CTA, 3.1 an item, 1.28 a step; the
+// merge kernel and the gap before it 7.5 us)
+constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 1};
+static inline const PrefillModel& prefill_model(const ps_shape& sh, bool pairs) { return sh.head_dim == 64 ? kD64Model : pairs ? kPairModel : kSingleModel; }
 // Which kernel runs the prefill items.  Head dimension 64: a CTA per item.  128: a pair of CTAs, unless the items are short and
 // there are enough for all SMs.  An item costs a CTA 3.5 us and 2.2 more a key tile, a pair 3.2 us and 0.73, so up to some
 // four key tiles two items on two CTAs are done sooner; of few items a pair does each in less time.
@@ -395,7 +398,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                          const ps_plan_opts* opts, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     const int tile_tok = kPrefillRowsPerItem / G;
-    const PrefillModel& cost = prefill_model(pl->pairs);
+    const PrefillModel& cost = prefill_model(pl->shape, pl->pairs);
     struct Tile { int r, g, tok0, n_tok, first_pos, key_tiles; };
     std::vector<Tile> tiles;
     size_t n_tiles = 0;
@@ -660,7 +663,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         double longest = 0;                  // steps of the longest prefill item
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
         const int G = shape->n_q_heads / shape->n_kv_heads;
-        const PrefillModel& cost = prefill_model(pl->pairs);
+        const PrefillModel& cost = prefill_model(pl->shape, pl->pairs);
         const int tile_tok = kPrefillRowsPerItem / G;
         for (int r = 0; r < n; ++r) {
             if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) {
@@ -723,7 +726,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
         }
     }
-    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->pairs).sms_per_worker);
+    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
     int64_t n_slots = 0;
     plan_decode(pl, prior_host, q_len_host, q_start, opts, &n_slots);
     plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);

@@ -1,5 +1,5 @@
-// Prefill-chunk attention on the 5th-generation tensor cores, a CTA per item: for head dimension 64, and at 128 for batches of
-// many short items (others: prefill_pair.cu; the rule is prefill_on_pairs() in plan.cu).
+// Prefill-chunk attention on the 5th-generation tensor cores, a CTA per item, for batches of many short items at head dimension
+// 128 (others: prefill_pair.cu; the rule is prefill_on_pairs() in plan.cu.  64: prefill_d64.cu).
 //
 // A chunk's rows attend the prior context plus the chunk's own earlier tokens
 // (paper sections 2.4 and 4.7); this part is a dense contraction and compute
@@ -26,7 +26,7 @@
 //              128-byte-swizzled operand layout, so blocks are consumed in place
 //   warp 9     MMA issue: S_X = Q_X K^T (SS form, M128 N128 K16) and
 //              O_X += P_X V (A operand from TMEM, V as MN-major B operand,
-//              M128 N=d K16); completion signalled with tcgen05.commit
+//              M128 N128 K16); completion signalled with tcgen05.commit
 //
 // The roles synchronise through mbarriers only, so consecutive items overlap:
 // the next item's Q, first K/V tiles and first QK^T are under way while the
@@ -52,8 +52,8 @@ constexpr int kRows = 128;
 constexpr float kRescaleThreshold = 8.f;  // log2 units
 constexpr int kBarBlockBytes = 512;  // mbarriers, flags and the item record ring
 
-template <int D>
-struct PrefillCfg {
+constexpr int D = 128;
+struct Cfg {
     static constexpr int kHalves = D / 64;
     static constexpr int kHalfBytes = kTileKeys * 128;          // [128 rows][128 B]
     static constexpr int kQBytes = kHalves * kHalfBytes;         // one Q tile
@@ -110,9 +110,7 @@ static_assert(Bars::mma_drained % 8 == 0 && Bars::armed + 24 <= Bars::ring && si
                   Bars::bytes <= kBarBlockBytes,
               "barrier block layout");
 
-template <int D>
 __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map, const __grid_constant__ InlineItems inl) {
-    using Cfg = PrefillCfg<D>;
     extern __shared__ char smem_raw[];
     char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -170,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
     static_assert(kPrefillRowsPerItem == 2 * kRows, "the planner pairs two q tiles per item");
     const int tile_tok = kRows / p.G;
     const int g_shift = 31 - __clz(p.G);  // G is a power of two
-    constexpr float kScaleLog2 = D == 128 ? 0.12751743f : 0.18033688f;  // log2(e) / sqrt(D)
+    constexpr float kScaleLog2 = scale_log2(D);
 
     // consumer side of the record ring: record number n into `it`; false at the end-of-work record or on abort
     auto take_item = [&](uint32_t n, PrefillItem& it) -> bool {
@@ -220,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                 const int limit = it.first_pos + i;            // last visible key of this row
                 const int tile_first_pos = it.first_pos + x * tile_tok;
                 float m = -INFINITY, l = 0.f;
-                float lu = 0.f;  // D = 128: the sum without the masked tiles' rounding, for the log-sum-exp
+                float lu = 0.f;  // the sum without the masked tiles' rounding, for the log-sum-exp
                 for (int j = 0; j < n_tiles && ok; ++j) {
                     const uint32_t tc = tile_ctr + j;  // K/V stage phase
                     ok = wait_all(bars + Bars::s_full + 8 * x, (tiles_x + j) & 1, s_abort);
@@ -280,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         tmem_wait_st();
                     }
                     l *= alpha;
-                    if (D == 128) lu *= alpha;
+                    lu *= alpha;
                     m = m_new;
                     const float m_sub = (m == -INFINITY) ? 0.f : m;
 
@@ -306,17 +304,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                                     const uint32_t pk = pack_bf16(p0, p1);
                                     l0 += bf16_lo(pk);
                                     l1 += bf16_hi(pk);
-                                    if (D == 128) ls = add2(ls, pack2(p0, p1));
+                                    ls = add2(ls, pack2(p0, p1));
                                     packed[qq * 16 + (c >> 1)] = pk;
                                 }
                             }
                             tmem_st32(s_addr + hhalf * 32, packed);
                         }
-                        if (D == 128) {
-                            float a0, a1;
-                            unpack2(ls, a0, a1);
-                            lu += a0 + a1;
-                        }
+                        float a0, a1;
+                        unpack2(ls, a0, a1);
+                        lu += a0 + a1;
                     } else {
                         // Interior tiles: two scores per instruction (packed fp32 FMA and add); four sum chains.
                         const uint64_t sc2 = pack2(kScaleLog2, kScaleLog2), nm2 = pack2(-m_sub, -m_sub);
@@ -349,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                         unpack2(ls1, a2, a3);
                         l0 = a0 + a2;
                         l1 = a1 + a3;
-                        if (D == 128) lu += l0 + l1;
+                        lu += l0 + l1;
                     }
                     l += l0 + l1;
                     tmem_wait_st();
@@ -379,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                 if (ok) {
                     tc_fence_after();
                     const float inv = l > 0.f ? 1.f / l : 0.f;
-                    const float lse_v = l > 0.f ? (m + log2f(D == 128 ? lu : l)) * 0.6931471805599453f : -INFINITY;
+                    const float lse_v = l > 0.f ? (m + log2f(lu)) * 0.6931471805599453f : -INFINITY;
                     const int row0 = (warp & 3) * 32;          // first tile row of this warp
                     const int sub = lane >> 3, unit = lane & 7;  // write-out: 4 rows per instruction, 8 lanes x 16 bytes per row
                     char* const my_row = stg + lane * 128;
@@ -704,12 +700,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
 
 }  // namespace
 
-template <int D>
-static ps_status launch_prefill_d(const RunArgs& a) {
-    using Cfg = PrefillCfg<D>;
+static ps_status launch_prefill_single(const RunArgs& a) {
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
-        PS_CUDA_TRY(cudaFuncSetAttribute(prefill_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+        PS_CUDA_TRY(cudaFuncSetAttribute(prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
         return PS_OK;
     });
     if (cfg != PS_OK) return cfg;
@@ -745,13 +739,13 @@ static ps_status launch_prefill_d(const RunArgs& a) {
     if (enc != PS_OK) return enc;
 
     const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
-    return launch_kernel(prefill_kernel<D>, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
+    return launch_kernel(prefill_kernel, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
 }
 
 ps_status launch_prefill(const RunArgs& a) {
     if (a.w.n_prefill == 0) return PS_OK;
     if (a.pairs) return launch_prefill_pair(a);
-    return a.shape.head_dim == 128 ? launch_prefill_d<128>(a) : launch_prefill_d<64>(a);
+    return a.shape.head_dim == 128 ? launch_prefill_single(a) : launch_prefill_d64(a);
 }
 
 }  // namespace ps

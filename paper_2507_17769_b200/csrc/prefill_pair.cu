@@ -55,7 +55,7 @@ constexpr int kRegsSoftmax = 104, kRegsOther = 64;  // 640 x 96 at launch = 512 
 constexpr int D = 128;
 constexpr int kTileKeys = 128;
 constexpr int kRows = 128;                // rows of one CTA
-constexpr float kScaleLog2 = 0.12751743f;  // log2(e) / sqrt(128)
+constexpr float kScaleLog2 = scale_log2(D);
 // 2^-60, 2^100: row sums outside are recomputed.  (Below 2^100 the accumulators are finite for |V| up to 2^27; only a row whose
 // sample was not finite can have a sum below 1.)
 constexpr float kSumMin = 8.7e-19f, kSumMax = 1.26e30f;
@@ -65,7 +65,6 @@ constexpr int kScoreBufs = 3;
 constexpr int kQBytes = 2 * kRows * 128;   // one CTA's Q tile: two 64-element halves
 constexpr int kKBytes = 2 * 64 * 128;      // this CTA's 64 keys: two halves
 constexpr int kVBytes = kTileKeys * 128;   // this CTA's 64 of the 128 output columns
-constexpr int kBlock = kPage * 128;        // 16 tokens x 64 elements: one bulk copy
 constexpr int kOffQ = 0;
 constexpr int kOffK = kOffQ + 2 * kQBytes;
 constexpr int kOffV = kOffK + kStagesK * kKBytes;
@@ -169,27 +168,8 @@ __device__ __forceinline__ void acquire_cluster(uint32_t bar, uint32_t parity) {
                  : "memory");
 }
 __device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
-// Four 2 KB blocks of the pool, one after the other into shared memory (box: one row of the pool seen as rows of 2 KB; rows
-// outside the pool read as zero).  A bulk copy per block costs the issuing warp some 100 cycles each, because its operands
-// are uniform registers and the lanes take turns; with 8 of them the producers could not keep up (1500 cycles a key tile).
-__device__ __forceinline__ void gather4(uint32_t dst, const CUtensorMap* map, int r0, int r1, int r2, int r3, uint32_t bar, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes.L2::cache_hint "
-        "[%0], [%1, {%2, %3, %4, %5, %6}], [%7], %8;" ::"r"(dst), "l"(map), "r"(0), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(bar),
-        "l"(policy)
-        : "memory");
-}
 __device__ __forceinline__ void store_u8_at(uint32_t cluster_addr) {
     asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(cluster_addr), "h"((unsigned short)1) : "memory");
-}
-__device__ __forceinline__ void store_tagged(uint32_t addr, float v, uint32_t tag) {
-    asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_uint(v)), "r"(tag) : "memory");
-}
-__device__ __forceinline__ uint32_t load_tagged(uint32_t addr, float& v) {
-    uint32_t bits, tag;
-    asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(bits), "=r"(tag) : "r"(addr) : "memory");
-    v = __uint_as_float(bits);
-    return tag;
 }
 __device__ __forceinline__ void pair_tmem_alloc(uint32_t smem_dst, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(cols) : "memory");
@@ -214,11 +194,6 @@ __device__ __forceinline__ void pair_mma_ts(uint32_t d_tmem, uint32_t a_tmem, ui
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
 // arrives on the barrier at this offset in both CTAs once this thread's earlier MMAs have retired
 __device__ __forceinline__ void pair_commit(uint32_t bar) {
     asm volatile(
@@ -227,32 +202,6 @@ __device__ __forceinline__ void pair_commit(uint32_t bar) {
         : "memory");
 }
 
-// 32 weights exp2(scale * s - ref) of one row as bf16 pairs, added to the packed row sums: two scores per instruction
-// (packed fp32 FMA and add).  `top`: largest score so far.
-__device__ __forceinline__ void weights32(const uint32_t (&s)[32], float ref, uint64_t& ls0, uint64_t& ls1, float& top, uint32_t* packed) {
-    const uint64_t sc2 = pack2(kScaleLog2, kScaleLog2), nm2 = pack2(-ref, -ref);
-#pragma unroll
-    for (int c = 0; c < 32; c += 2) {
-        top = max3(top, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
-        float e0, e1;
-        unpack2(fma2(pack2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, nm2), e0, e1);
-        e0 = fast_exp2(e0), e1 = fast_exp2(e1);
-        if (c & 2) ls1 = add2(ls1, pack2(e0, e1));
-        else ls0 = add2(ls0, pack2(e0, e1));
-        packed[c >> 1] = pack_bf16(e0, e1);
-    }
-}
-// 32 bytes to a 16-byte aligned address, in one store where it is 32-byte aligned
-__device__ __forceinline__ void store32(char* dst, const uint32_t* v, bool aligned32) {
-    if (aligned32) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
-                     "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                     : "memory");
-    } else {
-        reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
-        reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
-    }
-}
 __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairParams p, const __grid_constant__ CUtensorMap q_map,
                                                                     const __grid_constant__ CUtensorMap pool_map, const __grid_constant__ InlineItems inl) {
     extern __shared__ char smem_raw[];
@@ -442,8 +391,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                     tmem_ld32(s_addr + 32, s1);
                     tmem_wait_ld();
                     uint64_t ls0 = 0ull, ls1 = 0ull;
-                    weights32(s0, ref, ls0, ls1, top, packed);
-                    weights32(s1, ref, ls0, ls1, top, packed + 16);
+                    weights32<D>(s0, ref, ls0, ls1, top, packed);
+                    weights32<D>(s1, ref, ls0, ls1, top, packed + 16);
                     tmem_st32(s_addr, packed);
                     float a0, a1, a2, a3;
                     unpack2(ls0, a0, a1);
@@ -655,12 +604,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_pair_kernel(const PairPar
                     ok = wait_all(bars + (is_k ? Bars::k_empty : Bars::v_empty) + 8 * s, par ^ 1, s_abort);
                     if (!ok) break;
                     if (elect_one()) {
-                        mbar_expect_tx(land, 8 * kBlock);
+                        mbar_expect_tx(land, 8 * kPoolBlock);
                         s_armed[is_k ? s : kStagesK + s] = (int)par;
                         const uint32_t dst = sbase + (is_k ? kOffK + s * kKBytes : kOffV + s * kVBytes);
                         gather4(dst, &pool_map, r[0], r[1], r[2], r[3], land, kv_policy);
-                        if (is_k) gather4(dst + 4 * kBlock, &pool_map, r[0] + 1, r[1] + 1, r[2] + 1, r[3] + 1, land, kv_policy);
-                        else gather4(dst + 4 * kBlock, &pool_map, r[4], r[5], r[6], r[7], land, kv_policy);
+                        if (is_k) gather4(dst + 4 * kPoolBlock, &pool_map, r[0] + 1, r[1] + 1, r[2] + 1, r[3] + 1, land, kv_policy);
+                        else gather4(dst + 4 * kPoolBlock, &pool_map, r[4], r[5], r[6], r[7], land, kv_policy);
                     }
                     __syncwarp();
                     if (is_k && j == 0) {
@@ -1020,6 +969,20 @@ ps_status encode_q_map(const RunArgs& a, CUtensorMap* map) {
     return PS_OK;
 }
 
+ps_status encode_pool_map(const RunArgs& a, CUtensorMap* map) {
+    EncodeTiledFn encode = tensor_map_encoder();
+    if (!encode) return fail(PS_ERR_CUDA, "the driver does not provide cuTensorMapEncodeTiled");
+    const cuuint64_t dims[2] = {kPoolBlock / 8, (cuuint64_t)a.num_pages * a.shape.n_kv_heads * (a.shape.head_dim / 32)};
+    const cuuint64_t strides[1] = {kPoolBlock};
+    const cuuint32_t box[2] = {kPoolBlock / 8, 1};
+    const cuuint32_t elem_strides[2] = {1, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<char*>(a.pool), dims, strides, box, elem_strides,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(PS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
+    return PS_OK;
+}
+
 ps_status launch_prefill_pair(const RunArgs& a) {
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
@@ -1054,18 +1017,9 @@ ps_status launch_prefill_pair(const RunArgs& a) {
     CUtensorMap q_map;
     const ps_status enc = encode_q_map(a, &q_map);
     if (enc != PS_OK) return enc;
-    // the pool as rows of 2 KB blocks; a box is one row, gathered four at a time
     CUtensorMap pool_map;
-    {
-        const cuuint64_t dims[2] = {kBlock / 8, (cuuint64_t)a.num_pages * p.Hkv * 4};
-        const cuuint64_t strides[1] = {kBlock};
-        const cuuint32_t box[2] = {kBlock / 8, 1};
-        const cuuint32_t elem_strides[2] = {1, 1};
-        const CUresult r = tensor_map_encoder()(&pool_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<char*>(a.pool), dims, strides,
-                                                box, elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(PS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code %d", (int)r);
-    }
+    const ps_status enc_pool = encode_pool_map(a, &pool_map);
+    if (enc_pool != PS_OK) return enc_pool;
     const int pairs = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms / 2 ? a.w.n_prefill : (a.pf_sms > 1 ? a.pf_sms / 2 : 1));
     return launch_kernel(prefill_pair_kernel, 2 * pairs, kThreads, kSmemBytes, a.stream, 2, a.early, p, q_map, pool_map, inl);
 }

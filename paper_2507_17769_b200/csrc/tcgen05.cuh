@@ -1,5 +1,5 @@
-// What the two prefill kernels share: wrappers over the tcgen05 and tensor-map PTX they use, the matrix descriptors,
-// the bounded wait of a CTA whose warps have different roles, and the tensor map of Q.
+// What the two prefill kernels share: wrappers over the tcgen05 and tensor-map PTX they use, the matrix descriptors
+// and the tensor maps of Q and the pool.
 #pragma once
 
 #include <cuda.h>
@@ -19,6 +19,11 @@ inline void fill_inline_items(const RunArgs& a, InlineItems& inl) {
 }
 
 ps_status encode_q_map(const RunArgs& a, CUtensorMap* map);
+// The pool as rows of 2 KB blocks (16 tokens x 64 elements); a box is one row, gathered four at a time.
+constexpr int kPoolBlock = kPage * 128;
+ps_status encode_pool_map(const RunArgs& a, CUtensorMap* map);
+
+__host__ __device__ constexpr float scale_log2(int d) { return d == 128 ? 0.12751743f : 0.18033688f; }  // log2(e) / sqrt(d)
 
 #ifdef __CUDACC__
 
@@ -130,6 +135,57 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// Four 2 KB blocks of the pool, one after the other into shared memory (box: one row of the pool seen as rows of 2 KB; rows
+// outside the pool read as zero).  A bulk copy per block costs the issuing warp some 100 cycles each, because its operands
+// are uniform registers and the lanes take turns; with 8 of them the producers could not keep up (1500 cycles a key tile).
+__device__ __forceinline__ void gather4(uint32_t dst, const CUtensorMap* map, int r0, int r1, int r2, int r3, uint32_t bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%2, %3, %4, %5, %6}], [%7], %8;" ::"r"(dst), "l"(map), "r"(0), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(bar),
+        "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void store_tagged(uint32_t addr, float v, uint32_t tag) {
+    asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_uint(v)), "r"(tag) : "memory");
+}
+__device__ __forceinline__ uint32_t load_tagged(uint32_t addr, float& v) {
+    uint32_t bits, tag;
+    asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(bits), "=r"(tag) : "r"(addr) : "memory");
+    v = __uint_as_float(bits);
+    return tag;
+}
+__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+// 32 weights exp2(scale * s - ref) of one row as bf16 pairs, added to the packed row sums: two scores per instruction
+// (packed fp32 FMA and add).  `top`: largest score so far.
+template <int D>
+__device__ __forceinline__ void weights32(const uint32_t (&s)[32], float ref, uint64_t& ls0, uint64_t& ls1, float& top, uint32_t* packed) {
+    const uint64_t sc2 = pack2(scale_log2(D), scale_log2(D)), nm2 = pack2(-ref, -ref);
+#pragma unroll
+    for (int c = 0; c < 32; c += 2) {
+        top = max3(top, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
+        float e0, e1;
+        unpack2(fma2(pack2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, nm2), e0, e1);
+        e0 = fast_exp2(e0), e1 = fast_exp2(e1);
+        if (c & 2) ls1 = add2(ls1, pack2(e0, e1));
+        else ls0 = add2(ls0, pack2(e0, e1));
+        packed[c >> 1] = pack_bf16(e0, e1);
+    }
+}
+// 32 bytes to a 16-byte aligned address, in one store where it is 32-byte aligned
+__device__ __forceinline__ void store32(char* dst, const uint32_t* v, bool aligned32) {
+    if (aligned32) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                     "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
+    } else {
+        reinterpret_cast<uint4*>(dst)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4*>(dst)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+}
 // Shared-memory matrix descriptor, 128-byte swizzle, 8-row atoms of 1024 bytes.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
     uint64_t d = 0;
@@ -144,29 +200,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 __host__ __device__ constexpr uint32_t instr_desc(int m, int n, bool b_mn_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
            ((uint32_t)(m >> 4) << 24);
-}
-
-// Wait for a phase for at most about the CTA's wait limit (nanoseconds, in the word behind the abort flag; the low
-// half of the nanosecond clock serves, so limits reach 4 s); gives up early when another role of the CTA has already
-// given up.  The role whose wait runs out raises the CTA's abort flag.  One non-blocking probe first; a limit of
-// zero gives up right after it.  The clock is read only every kWaitPollsPerClockRead failed polls.
-__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    if (mbar_test_wait(bar, parity)) return true;
-    const uint32_t limit_ns = (uint32_t)abort_flag[1];  // the wait limit sits behind the abort flag
-    if (limit_ns > 0) {
-        uint32_t t0 = 0;
-        for (uint32_t i = 1;; ++i) {
-            if (mbar_try_wait(bar, parity)) return true;
-            if ((i & (kWaitPollsPerClockRead - 1)) == 0) {
-                if (*abort_flag) return false;
-                const uint32_t now = global_timer_lo() | 1u;
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > limit_ns) break;
-            }
-        }
-    }
-    *abort_flag = 1;
-    return false;
 }
 
 #endif  // __CUDACC__
