@@ -28,8 +28,8 @@ namespace ps {
 namespace {
 
 // Streaming warps per CTA (one CTA per SM) and ring depth per warp: 12 x 2 x 8 KB = 192 KB in flight per SM at head dimension
-// 128; measured on B200: 12 x 2 and 10 x 2 beat 8 x 3, 6 x 4 and 4 x 6 by 2-6 %.  At 64 a page is half as large and takes a
-// warp nearly as long: 24 x 2 x 4 KB (an SM streams 87 GB/s, 12 x 4 x 4 KB 80).
+// 128; measured on B200: 12 x 2 and 10 x 2 beat 8 x 3, 6 x 4 and 4 x 6 by 2-6 %.  At 64, where a page is half as large, 24 x 2 x
+// 4 KB in the kernel with a CTA per piece; for the one with a unit per warp see StreamCfg.
 __host__ __device__ constexpr int warps_at(int d) { return d == 128 ? 12 : 24; }
 constexpr int kStagesPerWarp = 2;
 constexpr int kRing = 8;  // unit ids in flight between the producer and consumer cursors of a warp
@@ -44,6 +44,19 @@ struct DecodeCfg {
     // 8 KB (4 KB at D = 64) stages per warp; the FP8 blocks are half as large, so twice as many are kept in flight
     static constexpr int kWarps = warps_at(D);
     static constexpr int kStages = (FP8 ? 2 : 1) * kStagesPerWarp;
+    static constexpr int kSmemBytes =
+        kWarps * kStages * kStageBytes + kWarps * kStages * 8 + kWarps * kRing * 4 + kWarps * kDeferred * 12 + 1024;
+};
+
+// The kernel with a unit per warp.  At head dimension 64 a page is half as large and takes a warp nearly as long: two pages a
+// stage, whose softmax costs little more than one's, on as many warps as at 128.  An SM streams 100 GB/s instead of 87 with a page
+// a stage on 24 warps (32 SMs, 256 rows of 3000 tokens, 8 heads: 559 -> 492 us; all SMs 253 -> 245).
+template <int D, bool FP8>
+struct StreamCfg {
+    static constexpr int kPages = D == 128 ? 1 : 2;
+    static constexpr int kPageBytes = DecodeCfg<D, FP8>::kStageBytes, kStageBytes = kPages * kPageBytes;
+    static constexpr int kWarps = 12;
+    static constexpr int kStages = DecodeCfg<D, FP8>::kStages;
     static constexpr int kSmemBytes =
         kWarps * kStages * kStageBytes + kWarps * kStages * 8 + kWarps * kRing * 4 + kWarps * kDeferred * 12 + 1024;
 };
@@ -166,70 +179,82 @@ __device__ __forceinline__ void load_q(const __nv_bfloat16* q, int64_t first_row
     }
 }
 
-// One page (its K, V in a shared-memory stage, nvalid >= 1 of its slots filled) into what the warp has gathered.
-template <int D, bool FP8>
-__device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nvalid, float scale_log2, const uint32_t (&qb)[D / 16][2],
-                                            Gathered<D>& a, int lane) {
+// PP pages (K, V of one after the other in a shared-memory stage, nvalid >= 1 of their slots filled) into what the warp has
+// gathered.
+template <int D, bool FP8, int PP = 1>
+__device__ __forceinline__ void attend_pages(char* stage, uint32_t kbase, int nvalid, float scale_log2, const uint32_t (&qb)[D / 16][2],
+                                             Gathered<D>& a, int lane) {
     using Cfg = DecodeCfg<D, FP8>;
     constexpr int KS = D / 16;  // k-steps of QK^T == m-tiles of PV
-    const uint32_t vbase = kbase + Cfg::kBlockBytes;
     const int row = lane >> 2;  // token rows row, row + 8 of S^T; d rows of O^T
     const int mi = lane >> 3, l7 = lane & 7;
     // ldmatrix row addresses (byte offsets inside a block, before the per-step unit term)
     const uint32_t k_tok_off = (uint32_t)(((mi & 1) * 8 + l7) * 128);
     const uint32_t v_tok_off = (uint32_t)(((mi >> 1) * 8 + l7) * 128);
-    if (nvalid < kPage) {
-        // Slots past the sequence end hold whatever the pool holds (possibly NaN):
+    if (nvalid < PP * kPage) {
+        // Slots past the sequence end hold whatever the pool (or, where there is no page, the stage) holds, possibly NaN:
         // zero those V rows so that 0 * V stays 0; their scores are masked below.
-        char* vb = stage + Cfg::kBlockBytes;
-        const int units = (kPage - nvalid) * 8;  // 16-byte units per region of 16 rows x 128 bytes
-        for (int h = 0; h < Cfg::kBlockBytes / 2048; ++h)
-            for (int u = lane; u < units; u += 32)
-                *reinterpret_cast<uint4*>(vb + h * 2048 + nvalid * 128 + u * 16) = make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int pp = 0; pp < PP; ++pp) {
+            char* vb = stage + pp * Cfg::kStageBytes + Cfg::kBlockBytes;
+            const int filled = min(max(nvalid - pp * kPage, 0), kPage);
+            const int units = (kPage - filled) * 8;  // 16-byte units per region of 16 rows x 128 bytes
+            for (int h = 0; h < Cfg::kBlockBytes / 2048; ++h)
+                for (int u = lane; u < units; u += 32)
+                    *reinterpret_cast<uint4*>(vb + h * 2048 + filled * 128 + u * 16) = make_uint4(0, 0, 0, 0);
+        }
         fence_proxy_async_smem();  // order these generic writes before the stage's next bulk copy
         __syncwarp();
     }
 
-    // S^T = K Q^T : 16 tokens x 8 head columns
-    float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
-    float x0, x1, x2, x3;
-    float sv_lo = 1.f, sv_hi = 1.f;  // FP8: V scales of this thread's two token rows
-    if constexpr (FP8) {
-        // One ldmatrix brings 16 tokens x 32 bytes: the thread gets bytes d = 16 u + 4 (lane % 4) + {0..3} of rows
-        // `row` and `row + 8` for two 16-byte chunks u, each of which is one k-step after conversion.
+    // S^T = K Q^T : 16 tokens a page x 8 head columns
+    float x[PP][4];
+    float sv_lo[PP], sv_hi[PP];  // FP8: V scales of this thread's two token rows
 #pragma unroll
-        for (int kp = 0; kp < KS / 2; ++kp) {
-            const uint32_t unit = (uint32_t)(((kp * 2 + (mi >> 1)) & 7) ^ l7);
-            uint32_t r0, r1, r2, r3;
-            ldsm_x4(kbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
-            mma_16816_f16(sa, e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16),
-                          qb[2 * kp][0], qb[2 * kp][1]);
-            mma_16816_f16(sb, e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16),
-                          qb[2 * kp + 1][0], qb[2 * kp + 1][1]);
-        }
-        const float* scales = reinterpret_cast<const float*>(stage + 2 * Cfg::kBlockBytes);
-        const float fk_lo = scales[row] * scale_log2, fk_hi = scales[row + 8] * scale_log2;
-        x0 = (sa[0] + sb[0]) * fk_lo, x1 = (sa[1] + sb[1]) * fk_lo;
-        x2 = (sa[2] + sb[2]) * fk_hi, x3 = (sa[3] + sb[3]) * fk_hi;
-        // slots past the sequence end hold arbitrary scales: their weights are zero, keep 0 * scale = 0
-        sv_lo = row < nvalid ? scales[kPage + row] * kWeightScale : 0.f;
-        sv_hi = row + 8 < nvalid ? scales[kPage + row + 8] * kWeightScale : 0.f;
-    } else {
+    for (int pp = 0; pp < PP; ++pp) {
+        const uint32_t kb = kbase + pp * Cfg::kStageBytes;
+        const int filled = nvalid - pp * kPage;
+        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+        sv_lo[pp] = sv_hi[pp] = 1.f;
+        if constexpr (FP8) {
+            // One ldmatrix brings 16 tokens x 32 bytes: the thread gets bytes d = 16 u + 4 (lane % 4) + {0..3} of rows
+            // `row` and `row + 8` for two 16-byte chunks u, each of which is one k-step after conversion.
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-            const uint32_t unit = (uint32_t)(((ks * 2 + (mi >> 1)) & 7) ^ l7);
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4(kbase + (ks >> 2) * 2048 + k_tok_off + (unit << 4), a0, a1, a2, a3);
-            if (ks & 1) mma_16816(sb, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-            else mma_16816(sa, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+            for (int kp = 0; kp < KS / 2; ++kp) {
+                const uint32_t unit = (uint32_t)(((kp * 2 + (mi >> 1)) & 7) ^ l7);
+                uint32_t r0, r1, r2, r3;
+                ldsm_x4(kb + k_tok_off + (unit << 4), r0, r1, r2, r3);
+                mma_16816_f16(sa, e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1 >> 16),
+                              qb[2 * kp][0], qb[2 * kp][1]);
+                mma_16816_f16(sb, e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3 >> 16),
+                              qb[2 * kp + 1][0], qb[2 * kp + 1][1]);
+            }
+            const float* scales = reinterpret_cast<const float*>(stage + pp * Cfg::kStageBytes + 2 * Cfg::kBlockBytes);
+            const float fk_lo = scales[row] * scale_log2, fk_hi = scales[row + 8] * scale_log2;
+            x[pp][0] = (sa[0] + sb[0]) * fk_lo, x[pp][1] = (sa[1] + sb[1]) * fk_lo;
+            x[pp][2] = (sa[2] + sb[2]) * fk_hi, x[pp][3] = (sa[3] + sb[3]) * fk_hi;
+            // slots past the sequence end hold arbitrary scales: their weights are zero, keep 0 * scale = 0
+            sv_lo[pp] = row < filled ? scales[kPage + row] * kWeightScale : 0.f;
+            sv_hi[pp] = row + 8 < filled ? scales[kPage + row + 8] * kWeightScale : 0.f;
+        } else {
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint32_t unit = (uint32_t)(((ks * 2 + (mi >> 1)) & 7) ^ l7);
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4(kb + (ks >> 2) * 2048 + k_tok_off + (unit << 4), a0, a1, a2, a3);
+                if (ks & 1) mma_16816(sb, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+                else mma_16816(sa, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+            }
+            x[pp][0] = (sa[0] + sb[0]) * scale_log2, x[pp][1] = (sa[1] + sb[1]) * scale_log2;
+            x[pp][2] = (sa[2] + sb[2]) * scale_log2, x[pp][3] = (sa[3] + sb[3]) * scale_log2;
         }
-        x0 = (sa[0] + sb[0]) * scale_log2, x1 = (sa[1] + sb[1]) * scale_log2;
-        x2 = (sa[2] + sb[2]) * scale_log2, x3 = (sa[3] + sb[3]) * scale_log2;
+        if (row >= filled) x[pp][0] = x[pp][1] = -INFINITY;
+        if (row + 8 >= filled) x[pp][2] = x[pp][3] = -INFINITY;
     }
-    if (row >= nvalid) x0 = x1 = -INFINITY;
-    if (row + 8 >= nvalid) x2 = x3 = -INFINITY;
 
-    float mx0 = fmaxf(x0, x2), mx1 = fmaxf(x1, x3);
+    float mx0 = fmaxf(x[0][0], x[0][2]), mx1 = fmaxf(x[0][1], x[0][3]);
+#pragma unroll
+    for (int pp = 1; pp < PP; ++pp) mx0 = fmaxf(mx0, fmaxf(x[pp][0], x[pp][2])), mx1 = fmaxf(mx1, fmaxf(x[pp][1], x[pp][3]));
     mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 4));
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 4));
     mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 8));
@@ -240,23 +265,29 @@ __device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nva
     const float al0 = fast_exp2(a.m0 - mn0), al1 = fast_exp2(a.m1 - mn1);
     a.m0 = mn0;
     a.m1 = mn1;
-    const float p0 = fast_exp2(x0 - mn0), p1 = fast_exp2(x1 - mn1);
-    const float p2 = fast_exp2(x2 - mn0), p3 = fast_exp2(x3 - mn1);
+    a.l0 *= al0;
+    a.l1 *= al1;
     // the row sum uses the bf16-rounded weights that PV multiplies, so that the
     // normalised output is an exact convex mix of V rows
-    uint32_t pk0, pk1;
-    if constexpr (FP8) {
-        // each key's V scale rides on its weight into the MMA; the row sum is over the weights themselves
-        pk0 = pack_f16(p0 * sv_lo, p1 * sv_lo), pk1 = pack_f16(p2 * sv_hi, p3 * sv_hi);
-        a.l0 = a.l0 * al0 + p0 + p2;
-        a.l1 = a.l1 * al1 + p1 + p3;
-    } else {
-        pk0 = pack_bf16(p0, p1), pk1 = pack_bf16(p2, p3);
-        a.l0 = a.l0 * al0 + bf16_lo(pk0) + bf16_lo(pk1);
-        a.l1 = a.l1 * al1 + bf16_hi(pk0) + bf16_hi(pk1);
+    uint32_t pb0[PP], pb1[PP];
+#pragma unroll
+    for (int pp = 0; pp < PP; ++pp) {
+        const float p0 = fast_exp2(x[pp][0] - mn0), p1 = fast_exp2(x[pp][1] - mn1);
+        const float p2 = fast_exp2(x[pp][2] - mn0), p3 = fast_exp2(x[pp][3] - mn1);
+        uint32_t pk0, pk1;
+        if constexpr (FP8) {
+            // each key's V scale rides on its weight into the MMA; the row sum is over the weights themselves
+            pk0 = pack_f16(p0 * sv_lo[pp], p1 * sv_lo[pp]), pk1 = pack_f16(p2 * sv_hi[pp], p3 * sv_hi[pp]);
+            a.l0 = a.l0 + p0 + p2;
+            a.l1 = a.l1 + p1 + p3;
+        } else {
+            pk0 = pack_bf16(p0, p1), pk1 = pack_bf16(p2, p3);
+            a.l0 = a.l0 + bf16_lo(pk0) + bf16_lo(pk1);
+            a.l1 = a.l1 + bf16_hi(pk0) + bf16_hi(pk1);
+        }
+        pb0[pp] = movmatrix_t(pk0);
+        pb1[pp] = movmatrix_t(pk1);
     }
-    const uint32_t pb0 = movmatrix_t(pk0);
-    const uint32_t pb1 = movmatrix_t(pk1);
 
     // O^T += V^T P^T : d x 8 head columns
     if constexpr (FP8) {
@@ -269,14 +300,17 @@ __device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nva
             a.o[2 * mp][0] *= al0, a.o[2 * mp][1] *= al1, a.o[2 * mp][2] *= al0, a.o[2 * mp][3] *= al1;
             a.o[2 * mp + 1][0] *= al0, a.o[2 * mp + 1][1] *= al1, a.o[2 * mp + 1][2] *= al0, a.o[2 * mp + 1][3] *= al1;
             const uint32_t unit = (uint32_t)(((mp * 2 + (mi >> 1)) & 7) ^ l7);
-            uint32_t r0, r1, r2, r3;
-            ldsm_x4_t(vbase + k_tok_off + (unit << 4), r0, r1, r2, r3);
-            r0 = __byte_perm(r0, 0, 0x3120), r1 = __byte_perm(r1, 0, 0x3120);
-            r2 = __byte_perm(r2, 0, 0x3120), r3 = __byte_perm(r3, 0, 0x3120);
-            mma_16816_f16(a.o[2 * mp], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r1 >> 16),
-                          pb0, pb1);
-            mma_16816_f16(a.o[2 * mp + 1], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r3 >> 16),
-                          pb0, pb1);
+#pragma unroll
+            for (int pp = 0; pp < PP; ++pp) {
+                uint32_t r0, r1, r2, r3;
+                ldsm_x4_t(kbase + pp * Cfg::kStageBytes + Cfg::kBlockBytes + k_tok_off + (unit << 4), r0, r1, r2, r3);
+                r0 = __byte_perm(r0, 0, 0x3120), r1 = __byte_perm(r1, 0, 0x3120);
+                r2 = __byte_perm(r2, 0, 0x3120), r3 = __byte_perm(r3, 0, 0x3120);
+                mma_16816_f16(a.o[2 * mp], e4m3x2_to_f16x2(r0), e4m3x2_to_f16x2(r0 >> 16), e4m3x2_to_f16x2(r1), e4m3x2_to_f16x2(r1 >> 16),
+                              pb0[pp], pb1[pp]);
+                mma_16816_f16(a.o[2 * mp + 1], e4m3x2_to_f16x2(r2), e4m3x2_to_f16x2(r2 >> 16), e4m3x2_to_f16x2(r3), e4m3x2_to_f16x2(r3 >> 16),
+                              pb0[pp], pb1[pp]);
+            }
         }
     } else {
 #pragma unroll
@@ -286,16 +320,20 @@ __device__ __forceinline__ void attend_page(char* stage, uint32_t kbase, int nva
             a.o[mt][2] *= al0;
             a.o[mt][3] *= al1;
             const uint32_t unit = (uint32_t)(((mt * 2 + (mi & 1)) & 7) ^ l7);
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4_t(vbase + (mt >> 2) * 2048 + v_tok_off + (unit << 4), a0, a1, a2, a3);
-            mma_16816(a.o[mt], a0, a1, a2, a3, pb0, pb1);
+#pragma unroll
+            for (int pp = 0; pp < PP; ++pp) {
+                uint32_t a0, a1, a2, a3;
+                ldsm_x4_t(kbase + pp * Cfg::kStageBytes + Cfg::kBlockBytes + (mt >> 2) * 2048 + v_tok_off + (unit << 4), a0, a1, a2, a3);
+                mma_16816(a.o[mt], a0, a1, a2, a3, pb0[pp], pb1[pp]);
+            }
         }
     }
 }
 
 template <int D, bool FP8>
-__global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_kernel(const DecodeParams p) {
-    using Cfg = DecodeCfg<D, FP8>;
+__global__ void __launch_bounds__(StreamCfg<D, FP8>::kWarps * 32, 1) decode_kernel(const DecodeParams p) {
+    using Cfg = StreamCfg<D, FP8>;
+    constexpr int PP = Cfg::kPages;  // of a stage
     constexpr int kWarps = Cfg::kWarps;
     constexpr int STAGES = Cfg::kStages;
     constexpr int KS = D / 16;  // k-steps of QK^T == m-tiles of PV
@@ -359,20 +397,32 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_kern
             P_bt0 += 32;
             P_bt = (P_bt0 + lane < P_page_end) ? __ldg(P_row + P_bt0 + lane) : 0;
         }
-        const int page = __shfl_sync(0xffffffffu, P_bt, P_page - P_bt0);
         const uint32_t stage = n_prod % STAGES;
-        if (lane == 0) {
-            const uint32_t bar = bar0 + 8 * stage;
-            if ((uint32_t)page < (uint64_t)p.num_pages) {
-                mbar_expect_tx(bar, Cfg::kStageBytes);
-                bulk_g2s_hint(stage0 + stage * Cfg::kStageBytes,
-                              p.pool + ((int64_t)page * p.Hkv + P_g) * (int64_t)Cfg::kStageBytes, Cfg::kStageBytes, bar, kv_policy);
+        const uint32_t bar = bar0 + 8 * stage;
+        int page[PP];
+        uint32_t n_good = 0;
+#pragma unroll
+        for (int pp = 0; pp < PP; ++pp) {
+            page[pp] = __shfl_sync(0xffffffffu, P_bt, P_page + pp - P_bt0);
+            if (pp > 0 && P_page + pp >= P_page_end) {
+                page[pp] = -1;  // the piece ends in an odd page
+            } else if ((uint32_t)page[pp] < (uint64_t)p.num_pages) {
+                ++n_good;
             } else {
-                report(p.hdr, p.tag, kStatusBounds);
-                mbar_arrive(bar);  // complete the phase without data; the run is flagged invalid
+                if (lane == 0) report(p.hdr, p.tag, kStatusBounds);  // the phase completes without its data; the run is flagged invalid
+                page[pp] = -1;
             }
         }
-        ++P_page;
+        if (lane == 0) {
+            if (n_good > 0) mbar_expect_tx(bar, n_good * Cfg::kPageBytes);
+            else mbar_arrive(bar);
+#pragma unroll
+            for (int pp = 0; pp < PP; ++pp)
+                if (page[pp] >= 0)
+                    bulk_g2s_hint(stage0 + stage * Cfg::kStageBytes + pp * Cfg::kPageBytes,
+                                  p.pool + ((int64_t)page[pp] * p.Hkv + P_g) * (int64_t)Cfg::kPageBytes, Cfg::kPageBytes, bar, kv_policy);
+        }
+        P_page += PP;
         ++n_prod;
     };
 
@@ -421,7 +471,7 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_kern
             for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
             // fixed segment order; kAhead segments' rows are requested before the first is used, so that a long
             // list of segments costs about one trip to L2 per kAhead of them
-            constexpr int kAhead = (NV <= 2 ? 8 : NV <= 4 ? 4 : 2) * D / 128;  // at most 16 float4 in flight per lane (8 with 24 warps)
+            constexpr int kAhead = NV <= 2 ? 8 : NV <= 4 ? 4 : 2;  // at most 16 float4 in flight per lane
             for (int s0 = 0; s0 < dm.n_seg; s0 += kAhead) {
                 float4 x[kAhead][NV];
                 float lw[kAhead];
@@ -587,12 +637,12 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_kern
             timed_out = true;
             break;
         }
-        const int nvalid = C_kvlen - C_page * kPage;  // >= 1
+        const int nvalid = min(C_kvlen, C_page_end * kPage) - C_page * kPage;  // >= 1
 
-        attend_page<D, FP8>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, nvalid, p.scale_log2, qb, acc, lane);
+        attend_pages<D, FP8, PP>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, nvalid, p.scale_log2, qb, acc, lane);
 
         __syncwarp();  // every lane has read this stage
-        ++C_page;
+        C_page += PP;
         ++n_cons;
         produce();     // refill the stage just released
     }
@@ -686,7 +736,7 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_cta_
             timed_out = true;
             break;
         }
-        attend_page<D, FP8>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, b.z - (first + kWarps * n_cons) * kPage,
+        attend_pages<D, FP8>(my_stages + stage * Cfg::kStageBytes, stage0 + stage * Cfg::kStageBytes, b.z - (first + kWarps * n_cons) * kPage,
                             p.scale_log2, qb, acc, lane);
         __syncwarp();  // every lane has read this stage
         if (n_prod < n_mine) produce(n_prod++);
@@ -783,7 +833,7 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_cta_
 
 }  // namespace
 
-int decode_warps_per_sm(int head_dim) { return warps_at(head_dim); }
+int decode_warps_per_sm(int head_dim) { return head_dim == 128 ? StreamCfg<128, false>::kWarps : StreamCfg<64, false>::kWarps; }
 
 template <int D, bool FP8>
 static ps_status launch_decode_d(const RunArgs& a) {
@@ -791,7 +841,7 @@ static ps_status launch_decode_d(const RunArgs& a) {
     constexpr int kWarps = Cfg::kWarps;
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
-        PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+        PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<D, FP8>::kSmemBytes));
         PS_CUDA_TRY(cudaFuncSetAttribute(decode_cta_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
         return PS_OK;
     });
@@ -822,7 +872,8 @@ static ps_status launch_decode_d(const RunArgs& a) {
     p.n_part_slots = a.w.n_part_slots;
     p.wait_limit_ns = a.wait_limit_ns;
     p.tag = a.tag;
-    int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + kWarps - 1) / kWarps;
+    constexpr int kUnitWarps = StreamCfg<D, FP8>::kWarps;
+    int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + kUnitWarps - 1) / kUnitWarps;
     if (grid > a.dec_sms) grid = a.dec_sms;
     // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
     // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
@@ -836,7 +887,7 @@ static ps_status launch_decode_d(const RunArgs& a) {
         }
         return launch_kernel(decode_cta_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p, a.w.n_cta_pieces, inl);
     }
-    return launch_kernel(decode_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
+    return launch_kernel(decode_kernel<D, FP8>, grid, kUnitWarps * 32, StreamCfg<D, FP8>::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
 }
 
 ps_status launch_decode(const RunArgs& a) {

@@ -37,9 +37,9 @@ constexpr int kPrefillKeyTile = 128;    // keys per tensor-core tile
 constexpr double kDecodePeakBytesPerSec = 6.7e12;
 constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a running prefill kernel
 // Per SM with the memory system to itself, and 0.85 of it beside a prefill kernel: 16 to 48 SMs stream 130 GB/s each at head
-// dimension 128 and 81 to 89 GB/s at 64, where a page is half as large and takes a warp as long.  (At 64 the lower end is
-// taken: with 87 the planner gave the prefill kernel of 48 rows and two chunks too many SMs, 68.2 us instead of 66.8.)
-static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 80e9; }
+// dimension 128 and 99 to 104 GB/s at 64.  (Less is taken at 64, where shares up to 92 SMs gain: 400 rows of 1000 tokens and a
+// 1024-token chunk 148 us on 72 SMs, as 100 would have it, 144.5 on 84.)
+static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 88e9; }
 static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;
 
@@ -324,6 +324,7 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     } else {
         const int64_t target = (int64_t)pl->dec_sms * decode_warps_per_sm(pl->shape.head_dim) * kDecodeUnitsPerWarp;
         per_unit = std::max<int64_t>(min_pages, (total_pages + target - 1) / target);
+        if (pl->shape.head_dim == 64) per_unit += per_unit & 1;  // (two pages a stage)
     }
     pl->info.decode_segment_tokens = (int32_t)(per_unit * kPage);
 
