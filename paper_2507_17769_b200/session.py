@@ -7,6 +7,24 @@ from __future__ import annotations
 
 from . import binding as B
 
+_torch_calls = None
+
+
+def torch_calls():
+    """The extension module of the calls of every iteration that takes torch tensors."""
+    global _torch_calls
+    if _torch_calls is None:
+        import ctypes
+
+        import torch  # noqa: F401  (the extension needs its libraries)
+
+        lib = B.load()
+        from . import _torch_calls as module
+
+        module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.ps_kv_write, lib.ps_kv_gather, lib.ps_attn_run)))
+        _torch_calls = module
+    return _torch_calls
+
 
 class PagedAttention:
     """A paged K/V pool with the per-iteration plan / run cycle.
@@ -23,6 +41,7 @@ class PagedAttention:
 
         self.torch = torch
         self._calls = B.calls()
+        self._tensor_calls, self._tensor = torch_calls(), torch.Tensor
         self.device = torch.device(device)
         self.shape = B.make_shape(n_q_heads, n_kv_heads, head_dim, page_size, kv_dtype)
         self.num_pages = int(num_pages)
@@ -60,6 +79,11 @@ class PagedAttention:
 
     def write(self, k_new, v_new, block_table_dev, prior, q_len, max_pages=None):
         """Scatter new tokens' K, V (bf16 [T, Hkv, d]) into their pages."""
+        t = self._tensor
+        if type(k_new) is t and type(v_new) is t and type(block_table_dev) is t:
+            B._check(self._tensor_calls.write(self.kv, k_new, v_new, block_table_dev, None if max_pages is None else int(max_pages), B.lengths(prior),
+                                              B.lengths(q_len), self._stream()))
+            return
         if max_pages is None:
             max_pages = block_table_dev.size(-1)
         assert k_new.is_contiguous() and v_new.is_contiguous() and block_table_dev.is_contiguous()
@@ -82,6 +106,10 @@ class PagedAttention:
         t = self.torch
         assert self.shape.dtype == 0, "use gather_fp8 on an FP8 cache"
         hkv, d = self.shape.n_kv_heads, self.shape.head_dim
+        if type(block_table_row_dev) is self._tensor:
+            status, k, v = self._tensor_calls.gather(self.kv, block_table_row_dev, int(length), hkv, d, self.pool, self._stream())
+            B._check(status)
+            return k, v
         k = t.empty_strided((length, hkv, d), (hkv * d, d, 1), dtype=t.bfloat16, device=self.device)
         v = t.empty_like(k)
         B.ps_kv_gather(self.kv, block_table_row_dev, int(length), k.data_ptr(), v.data_ptr(), self._stream())
@@ -109,6 +137,12 @@ class PagedAttention:
         t = self.torch
         assert self._plan is not None, "call plan() first"
         total_q, hq = self._total_q, self._n_q_heads
+        exact = self._tensor
+        if type(q) is exact and type(block_table_dev) is exact and (out is None or type(out) is exact) and (lse is None or type(lse) is exact):
+            status, out, lse = self._tensor_calls.run(self._plan, self.kv, q, block_table_dev, out, lse, bool(want_lse), total_q, hq, self.pool, self._ws_ptr,
+                                                      self._ws_bytes, self._stream())
+            B._check(status)
+            return out, lse
         assert q.is_contiguous() and q.size(0) == total_q and block_table_dev.is_contiguous()
         if out is None:
             out = t.empty_like(q)
