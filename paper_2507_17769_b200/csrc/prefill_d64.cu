@@ -289,60 +289,19 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_d64_kernel(const Params p
                     unpack2(ls1, a2, a3);
                     l += (a0 + a2) + (a1 + a3);
                 } else {
-                    // Diagonal and ragged halves: mask by select, and sum the bf16-rounded weights that PV multiplies, so that the
-                    // output of a row with a handful of keys stays an exact convex mix of V rows; the log-sum-exp is taken without
-                    // that rounding.
-                    float l0 = 0.f, l1 = 0.f;
+                    // Diagonal and ragged halves, the only ones of rows with few visible keys.
+                    const int vis_any = __shfl_sync(0xffffffffu, vis, 31);  // columns that some row of the warp sees
                     ok = wait_all(bars + Bars::p_free + 8 * x, par ^ 1, s_abort);
                     if (!ok) break;
                     tc_fence_after();
-                    const int vis_any = __shfl_sync(0xffffffffu, vis, 31);  // columns that some row of the warp sees
                     if (mode == kModePlain && j == 0 && h == 0 && __any_sync(0xffffffffu, vis < 64)) {
                         // Rows that see fewer than 64 keys of the item, all of them here: relative to their maximum, so that the
                         // weight that counts most is 1 and rounds to itself.  (This thread also writes their log-sum-exp.)
-                        float mx = -INFINITY;
-#pragma unroll 1
-                        for (int q = 0; q < 4 && 16 * q < vis_any; ++q) {
-                            uint32_t sv[16];
-                            tmem_ld16(s_addr + 16 * q, sv);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) mx = 16 * q + c < vis ? fmaxf(mx, __uint_as_float(sv[c])) : mx;
-                        }
+                        const float mx = masked_max64(s_addr, vis, vis_any);
                         if (vis < 64 && mx > -INFINITY) ref = mx * kScaleLog2;
                     }
-#pragma unroll 1
-                    for (int q = 0; q < 4; ++q) {
-                        const int v = vis - 16 * q;
-                        if (vis_any <= 16 * q) {
-                            const uint32_t zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                            if (mode != kModeMax) tmem_st8(p_addr + 8 * q, zero);
-                            continue;
-                        }
-                        uint32_t sv[16];
-                        tmem_ld16(s_addr + 16 * q, sv);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) sv[c] = c < v ? sv[c] : 0xff800000u;
-                        if (mode == kModeMax) {
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) l = fmaxf(l, __uint_as_float(sv[c]) * kScaleLog2);
-                        } else {
-                            uint32_t packed[8];
-#pragma unroll
-                            for (int c = 0; c < 16; c += 2) {
-                                const float e0 = fast_exp2(fmaf(__uint_as_float(sv[c]), kScaleLog2, -ref));
-                                const float e1 = fast_exp2(fmaf(__uint_as_float(sv[c + 1]), kScaleLog2, -ref));
-                                const uint32_t pk = pack_bf16(e0, e1);
-                                l0 += bf16_lo(pk);
-                                l1 += bf16_hi(pk);
-                                rounding += (bf16_lo(pk) - e0) + (bf16_hi(pk) - e1);
-                                packed[c >> 1] = pk;
-                            }
-                            tmem_st8(p_addr + 8 * q, packed);
-                        }
-                    }
-                    l += l0 + l1;
+                    if (mode == kModeMax) l = fmaxf(l, masked_max64(s_addr, vis, vis_any) * kScaleLog2);
+                    else masked_weights64<D>(s_addr, p_addr, vis, vis_any, ref, l, rounding);
                     tc_fence_before();
                     __syncwarp();
                     mbar_arrive_if(bars + Bars::s_free + 8 * x, lane == 0);

@@ -76,15 +76,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
@@ -120,10 +111,12 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
-                 "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+        "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
+        "r"(r[15])
+        : "memory");
 }
 // One box of a 3-d tensor map into shared memory; completion is counted in bytes on `bar`.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
@@ -174,6 +167,61 @@ __device__ __forceinline__ void weights32(const uint32_t (&s)[32], float ref, ui
         else ls0 = add2(ls0, pack2(e0, e1));
         packed[c >> 1] = pack_bf16(e0, e1);
     }
+}
+// The same for the 64 scores of a half tile of which this row sees the first `vis`, and some row of the warp the first `vis_any`:
+// masked by select.  l is the sum of the bf16-rounded weights that PV multiplies, so that the output of a row with a handful of keys
+// stays an exact convex mix of V rows; `rounding` is what that adds to their exact sum, of which the log-sum-exp is taken.
+// (Rolled: this code runs once or twice an item, so its instructions come from far; written out for all 64 scores it took 4700
+// cycles a tile.  In steps of 16 scores, with the rounding added up weight by weight, four fresh prompts of 1400 to 2000 tokens took
+// 120 us; so 111.)
+template <int D>
+__device__ __forceinline__ void masked_weights64(uint32_t s_addr, uint32_t p_addr, int vis, int vis_any, float ref, float& l, float& rounding) {
+    const uint64_t sc2 = pack2(scale_log2(D), scale_log2(D)), nm2 = pack2(-ref, -ref);
+    float l0 = 0.f, l1 = 0.f;
+    uint64_t exact = 0ull;
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+        uint32_t packed[16];
+        if (vis_any <= 32 * q) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) packed[c] = 0u;
+        } else {
+            uint32_t s[32];
+            tmem_ld32(s_addr + 32 * q, s);
+            tmem_wait_ld();
+            const int v = vis - 32 * q;
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) {
+                s[c] = c < v ? s[c] : 0xff800000u;
+                s[c + 1] = c + 1 < v ? s[c + 1] : 0xff800000u;
+                float e0, e1;
+                unpack2(fma2(pack2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, nm2), e0, e1);
+                e0 = fast_exp2(e0), e1 = fast_exp2(e1);
+                exact = add2(exact, pack2(e0, e1));
+                packed[c >> 1] = pack_bf16(e0, e1);
+                l0 += bf16_lo(packed[c >> 1]);
+                l1 += bf16_hi(packed[c >> 1]);
+            }
+        }
+        tmem_st16(p_addr + 16 * q, packed);
+    }
+    float x0, x1;
+    unpack2(exact, x0, x1);
+    l += l0 + l1;
+    rounding += (l0 - x0) + (l1 - x1);
+}
+// the largest of the first `vis` of them
+__device__ __forceinline__ float masked_max64(uint32_t s_addr, int vis, int vis_any) {
+    float mx = -INFINITY;
+#pragma unroll 1
+    for (int q = 0; q < 2 && 32 * q < vis_any; ++q) {
+        uint32_t s[32];
+        tmem_ld32(s_addr + 32 * q, s);
+        tmem_wait_ld();
+#pragma unroll
+        for (int c = 0; c < 32; ++c) mx = 32 * q + c < vis ? fmaxf(mx, __uint_as_float(s[c])) : mx;
+    }
+    return mx;
 }
 // 32 bytes to a 16-byte aligned address, in one store where it is 32-byte aligned
 __device__ __forceinline__ void store32(char* dst, const uint32_t* v, bool aligned32) {
