@@ -42,6 +42,8 @@ constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a
 static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 88e9; }
 static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;
+constexpr double kDecodeManyBytes = 0.75e9;
+constexpr int kDecodeAloneSms = 128;
 
 // Cost model of a prefill kernel in units of one 128-key step of an item (256 rows): an item pays a fixed overhead
 // (pipeline fill, output) plus one unit per key tile.
@@ -681,6 +683,12 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         }
         pl->dec_sms = pl->pf_sms = pl->num_sms;
         pl->concurrent = false;
+        // Decode rows alone stream a little faster from 128 SMs: all 148 ask for more than HBM gives, and their requests get in each
+        // other's way.  (bf16 cache; a launch on 148 / 128 SMs, us, on four boxes: 512 rows lognormal 482 / 468, 256 rows of 8000
+        // tokens at 64 heads 1290 / 1230, or 2021 / 2024 for 299 of 11200; 140 of 1700 165 / 161; 256 of 3000 at head dimension 64 250 /
+        // 238; below the line 64 rows, 0.57 GB, 95.0 / 93.6, 32 of 1000 32.6 / 32.3.  Pages of the FP8 cache cost the SMs too much
+        // arithmetic for that.)
+        if (pf_steps == 0 && shape->dtype == 0 && dec_bytes >= kDecodeManyBytes) pl->dec_sms = std::min(pl->num_sms, kDecodeAloneSms);
         if (dec_bytes > 0 && pf_steps > 0 && pl->num_sms >= 16) {
             // time models (seconds): decode = bytes / min(side-by-side peak, n * per-SM rate); prefill = steps * step time / m
             auto t_dec = [&](int nd) { return dec_bytes / std::min(kDecodeSharedPeakBytesPerSec, nd * decode_rate_per_sm(*shape)) + kKernelFloorSec; };
