@@ -52,16 +52,19 @@ struct PrefillModel {
     double fixed;         // steps an item costs beyond its key tiles
     double masked_extra;  // and the diagonal tile's slower softmax
     double cut;           // steps that cutting items costs: partial rows, merge kernel
+    double whole;         // steps by which whole items may end later than an even split: what cutting costs a small batch, a kernel
+                          // more and a list that has to be uploaded
     int sms_per_worker;   // an item is worked on by one CTA, or by a pair of them
 };
 // prefill.cu (fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile)
-constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 1};
+constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 3.0, 1};
 // prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
-// item; the merge kernel takes about 8 us)
-constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 2};
+// item; the merge kernel takes about 8 us).  Whole items, us, instead of cut ones: 8 items of 10 key tiles 25.9 -> 19.0, of 17
+// 26.9 -> 24.4, 40 of up to 26 35.8 -> 31.7, 16 of 33 35.3 -> 40.7 beside 6 decode rows, 8 of 63 31.2 -> 55.
+constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 20.0, 2};
 // prefill_d64.cu (148 CTAs of 1 to 3 items of 6 to 29 key tiles, beside a decode kernel: 9.4 us a CTA, 3.1 an item, 1.28 a step; the
-// merge kernel and the gap before it 7.5 us)
-constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 1};
+// merge kernel and the gap before it 7.5 us).  Whole items instead of cut ones: 8 of 10 key tiles 22.4 -> 18.4, of 17 22.1 -> 26.1.
+constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 10.0, 1};
 static inline const PrefillModel& prefill_model(const ps_shape& sh, bool pairs) { return sh.head_dim == 64 ? kD64Model : pairs ? kPairModel : kSingleModel; }
 // Which kernel runs the prefill items.  Head dimension 64: a CTA per item.  128: a pair of CTAs, unless the items are short and
 // there are enough for all SMs.  An item costs a CTA 3.5 us and 2.2 more a key tile, a pair 3.2 us and 0.73, so up to some
@@ -476,7 +479,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
             }
             // (cutting is not free either, and from four items a worker on it has less to gain than the partial rows cost in
             // space, 19 MB in a batch that needs none)
-            if ((int64_t)tiles.size() >= 4LL * pl->pf_workers || makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.cut)) {
+            if ((int64_t)tiles.size() >= 4LL * pl->pf_workers || makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.whole)) {
                 for (int c = 0; c < n_cta; ++c) count[c + 1] += count[c];
                 pl->prefill_cta_start.assign(count.begin(), count.end());
                 std::vector<Tile> sorted(tiles.size());
@@ -1007,13 +1010,15 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     bool merged = false;  // the merge kernel has been launched already
     // dynamic item queue with more items than workers: the decode kernel's SMs help once it has ended
     const bool helpers = a.w.n_prefill_ctas == 0 && a.w.n_prefill > pl->pf_workers;
-    if (pl->concurrent && !(rec && pl->side_stream) && (as_params || (!capturing && !helpers && a.w.n_merge == 0))) {
-        // Mixed batch without more to launch than its two kernels: both on the caller's stream, the prefill kernel launched as
-        // soon as the decode kernel has begun and waiting for its end only at its own.  (A second stream costs two events,
-        // which take some 3 us each between kernels: tiny mixed batch 22.5 -> 16.8 us, with the list as parameters; 32 rows of
-        // 2048 tokens beside a 512-token chunk 58.1 -> 57.2.  A merge kernel would have to wait for the decode kernel too, and
-        // helpers have to start as soon as that ends, so such batches keep the second stream.  So do runs that record events:
-        // one between the two launches would hold the prefill kernel back until the decode kernel's end.)
+    if (pl->concurrent && !(rec && pl->side_stream) && (as_params || (!capturing && !helpers))) {
+        // Mixed batch: both kernels on the caller's stream, the prefill kernel launched as soon as the decode kernel has begun and
+        // waiting for its end only at its own, and the merge kernel behind both.  (A second stream costs two events, which take
+        // some 3 us each between kernels: tiny mixed batch 22.5 -> 16.8 us, with the list as parameters; 32 rows of 2048 tokens
+        // beside a 512-token chunk 58.1 -> 57.2.  On a second stream the merge kernel could run while the decode kernel still
+        // does, which is worth no more than that even where it does for long: 200 rows of 2500 tokens and 40 on 8000 338 -> 330;
+        // where it ends first, 6 rows of 1500 and 500 on 1500 at head dimension 64 36.1 -> 29.0, 48 rows and two chunks 62.9 ->
+        // 57.5.  Helpers have to start as soon as the decode kernel ends, so batches with a queue keep the second stream.  So do
+        // runs that record events: one between the two launches would hold the prefill kernel back until the decode kernel's end.)
         RunArgs ad = a;
         ad.sm_pairs = pl->pf_workers < pl->pf_sms;
         if (rec) cudaEventRecord(ev[2], s);  // (without a second stream the kernels follow one another)
