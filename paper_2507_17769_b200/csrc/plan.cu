@@ -687,7 +687,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         pl->dec_sms = pl->pf_sms = pl->num_sms;
         pl->concurrent = false;
         // Decode rows alone stream a little faster from 128 SMs: all 148 ask for more than HBM gives, and their requests get in each
-        // other's way.  (bf16 cache; a launch on 148 / 128 SMs, us, on four boxes: 512 rows lognormal 482 / 468, 256 rows of 8000
+        // other's way.  (bf16 cache; a launch on 148 / 128 SMs, us, on four GPUs: 512 rows lognormal 482 / 468, 256 rows of 8000
         // tokens at 64 heads 1290 / 1230, or 2021 / 2024 for 299 of 11200; 140 of 1700 165 / 161; 256 of 3000 at head dimension 64 250 /
         // 238; below the line 64 rows, 0.57 GB, 95.0 / 93.6, 32 of 1000 32.6 / 32.3.  Pages of the FP8 cache cost the SMs too much
         // arithmetic for that.)
