@@ -215,6 +215,7 @@ struct DeviceWork {       // pointers into the workspace for one run
     float* part_o;
     int32_t n_cta_pieces;              // above 0: a CTA per decode piece (small batches), and no units
     int32_t n_units, n_prefill, n_merge, n_dmerge;
+    int32_t merge_segs;                // most segments of a merge entry
     int64_t n_part_slots;              // rows of part_lse / part_o
     const int32_t* prefill_cta_start;  // static prefill partition (n_prefill_ctas + 1 entries), unused when 0
     int32_t n_prefill_ctas;            // entries of that partition: CTAs, or CTA pairs

@@ -996,6 +996,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.w.n_cta_pieces = pl->cta_pieces ? (int32_t)pl->pieces.size() : 0;
     a.w.n_prefill = (int32_t)pl->prefill.size();
     a.w.n_merge = (int32_t)pl->merge.size();
+    for (const MergeEntry& me : pl->merge) a.w.merge_segs = std::max(a.w.merge_segs, me.n_seg);
     a.w.n_dmerge = (int32_t)pl->dmerge.size();
     a.w.n_part_slots = pl->info.n_partial_slots;
     a.w.dmerge = (const DecodeMerge*)(ws + pl->off_dmerge);
