@@ -30,7 +30,11 @@ bool as_ptr(PyObject* o, void** p) {
     *p = PyLong_AsVoidPtr(o);
     return !(*p == nullptr && PyErr_Occurred());
 }
-bool as_i64(PyObject* o, int64_t* v) {
+bool as_i64(PyObject* o, int64_t* v) {  // (what has __index__; a truth value is no size to torch either)
+    if (PyBool_Check(o)) {
+        PyErr_SetString(PyExc_TypeError, "an integer expected, got bool");
+        return false;
+    }
     *v = PyLong_AsLongLong(o);
     return !(*v == -1 && PyErr_Occurred());
 }

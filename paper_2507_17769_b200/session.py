@@ -107,7 +107,7 @@ class PagedAttention:
         assert self.shape.dtype == 0, "use gather_fp8 on an FP8 cache"
         hkv, d = self.shape.n_kv_heads, self.shape.head_dim
         if type(block_table_row_dev) is self._tensor:
-            status, k, v = self._tensor_calls.gather(self.kv, block_table_row_dev, int(length), hkv, d, self.pool, self._stream())
+            status, k, v = self._tensor_calls.gather(self.kv, block_table_row_dev, length, hkv, d, self.pool, self._stream())
             B._check(status)
             return k, v
         k = t.empty_strided((length, hkv, d), (hkv * d, d, 1), dtype=t.bfloat16, device=self.device)
