@@ -26,7 +26,12 @@ bool count_is(Py_ssize_t n, Py_ssize_t want) {
     PyErr_Format(PyExc_TypeError, "%zd arguments expected, got %zd", want, n);
     return false;
 }
+// an address, or None, which the library refuses: a closed session's handles are None
 bool as_ptr(PyObject* o, void** p) {
+    if (o == Py_None) {
+        *p = nullptr;
+        return true;
+    }
     *p = PyLong_AsVoidPtr(o);
     return !(*p == nullptr && PyErr_Occurred());
 }

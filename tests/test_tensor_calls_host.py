@@ -37,3 +37,14 @@ def test_lengths_of_integer_types_are_taken():
             with pytest.raises(ps.PsError) as e:  # (as far as the null pool)
                 host_session().gather(table, length)
             assert e.value.status == ps.binding.PS_ERR_INVALID
+
+
+def test_a_closed_pool_is_reported_as_the_library_does():
+    pa = host_session()
+    pa.kv = None
+    k, row = torch.zeros((1, 2, 64), dtype=torch.bfloat16), torch.zeros((1, 4), dtype=torch.int32)
+    for cast in (lambda x: x, lambda x: x.as_subclass(Sub)):
+        for call in (lambda: pa.write(cast(k), cast(k), cast(row), [0], [1]), lambda: pa.gather(cast(row), 1)):
+            with pytest.raises(ps.PsError) as e:
+                call()
+            assert e.value.status == ps.binding.PS_ERR_INVALID
