@@ -72,7 +72,9 @@ struct Lengths {
     }
 };
 
-struct Unlocked {  // the interpreter lock is given back while the library runs
+// The interpreter lock is given back while the library runs and while results are allocated: an allocation may wait for the device, and
+// what that waits for may need the interpreter.
+struct Unlocked {
     PyThreadState* s = PyEval_SaveThread();
     ~Unlocked() { PyEval_RestoreThread(s); }
 };
@@ -146,11 +148,12 @@ PyObject* py_gather(PyObject*, PyObject* const* a, Py_ssize_t n) {
         PyErr_SetString(PyExc_OverflowError, "argument does not fit 32 bits");
         return nullptr;
     }
-    const auto opts = pool->options().dtype(at::kBFloat16);
-    at::Tensor k = at::empty({len, hkv, d}, opts), v = at::empty({len, hkv, d}, opts);
+    at::Tensor k, v;
     int st;
     {
         Unlocked u;
+        const auto opts = pool->options().dtype(at::kBFloat16);
+        k = at::empty({len, hkv, d}, opts), v = at::empty({len, hkv, d}, opts);
         st = f_gather(kv, (const int32_t*)bt->data_ptr(), (int32_t)len, k.data_ptr(), v.data_ptr(), stream);
     }
     return three(st, THPVariable_Wrap(std::move(k)), THPVariable_Wrap(std::move(v)));
@@ -162,33 +165,24 @@ PyObject* py_gather(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_run(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     void *plan, *kv, *ws, *stream;
-    const at::Tensor *q, *bt, *pool, *given;
+    const at::Tensor *q, *bt, *pool;
     int64_t total_q, hq, bytes;
     if (!count_is(n, 13) || !as_ptr(a[0], &plan) || !as_ptr(a[1], &kv) || !as_tensor(a[2], &q) || !as_tensor(a[3], &bt) || !as_i64(a[7], &total_q) ||
         !as_i64(a[8], &hq) || !as_tensor(a[9], &pool) || !as_ptr(a[10], &ws) || !as_i64(a[11], &bytes) || !as_ptr(a[12], &stream))
         return nullptr;
     if (!holds(q->is_contiguous() && q->size(0) == total_q && bt->is_contiguous(), "q must be contiguous with a row per planned token, and the block table contiguous"))
         return nullptr;
-    void *out_ptr = nullptr, *lse_ptr = nullptr;
+    const at::Tensor *given_out = nullptr, *given_lse = nullptr;
+    if ((a[4] != Py_None && !as_tensor(a[4], &given_out)) || (a[5] != Py_None && !as_tensor(a[5], &given_lse))) return nullptr;
     at::Tensor out, lse;
-    if (a[4] == Py_None) {
-        out = at::empty(q->sizes(), q->options());
-        out_ptr = out.data_ptr();
-    } else {
-        if (!as_tensor(a[4], &given)) return nullptr;
-        out_ptr = given->data_ptr();
-    }
-    if (a[5] != Py_None) {
-        if (!as_tensor(a[5], &given)) return nullptr;
-        lse_ptr = given->data_ptr();
-    } else if (a[6] == Py_True) {
-        lse = at::empty({total_q, hq}, pool->options().dtype(at::kFloat));
-        lse_ptr = lse.data_ptr();
-    }
     int st;
     {
         Unlocked u;
-        st = f_run(plan, kv, q->data_ptr(), (const int32_t*)bt->data_ptr(), out_ptr, (float*)lse_ptr, ws, (size_t)bytes, stream);
+        if (!given_out) out = at::empty(q->sizes(), q->options());
+        if (!given_lse && a[6] == Py_True) lse = at::empty({total_q, hq}, pool->options().dtype(at::kFloat));
+        void* const lse_ptr = given_lse ? given_lse->data_ptr() : lse.defined() ? lse.data_ptr() : nullptr;
+        st = f_run(plan, kv, q->data_ptr(), (const int32_t*)bt->data_ptr(), given_out ? given_out->data_ptr() : out.data_ptr(), (float*)lse_ptr, ws, (size_t)bytes,
+                   stream);
     }
     return three(st, out.defined() ? THPVariable_Wrap(std::move(out)) : again(a[4]), lse.defined() ? THPVariable_Wrap(std::move(lse)) : again(a[5]));
     END_HANDLE_TH_ERRORS

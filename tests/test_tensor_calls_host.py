@@ -1,4 +1,9 @@
 """What PagedAttention's calls with tensors refuse before they reach the device, against the calls through addresses."""
+import os
+import subprocess
+import sys
+import sysconfig
+
 import numpy as np
 import pytest
 import torch
@@ -48,3 +53,59 @@ def test_a_closed_pool_is_reported_as_the_library_does():
             with pytest.raises(ps.PsError) as e:
                 call()
             assert e.value.status == ps.binding.PS_ERR_INVALID
+
+
+ALLOCATOR = r"""
+#include <Python.h>
+#include <c10/core/Allocator.h>
+// forwards to the allocator it replaces and counts the allocations of at least `floor` bytes, and those made with the interpreter lock held
+static c10::Allocator* before;
+static size_t floor_bytes;
+static int counted, held;
+struct Counting : c10::Allocator {
+    c10::DataPtr allocate(size_t n) override {
+        if (n >= floor_bytes) ++counted, held += PyGILState_Check();
+        return before->allocate(n);
+    }
+    c10::DeleterFnPtr raw_deleter() const override { return before->raw_deleter(); }
+    void copy_data(void* d, const void* s, size_t n) const override { before->copy_data(d, s, n); }
+};
+extern "C" void install(long n) {
+    static Counting mine;
+    floor_bytes = (size_t)n;
+    before = c10::GetAllocator(c10::DeviceType::CPU);
+    c10::SetAllocator(c10::DeviceType::CPU, &mine, 100);
+}
+extern "C" int counts(int which) { return which ? held : counted; }
+"""
+
+ALLOCATE = """
+import ctypes, sys
+import torch
+sys.path[:0] = %r
+import test_tensor_calls_host as t
+lib = ctypes.CDLL(%r)
+pa = t.host_session()
+pa._plan, pa._total_q, pa._n_q_heads, pa._ws_ptr, pa._ws_bytes = 0, 4096, 8, 0, 0
+q, row = torch.zeros((4096, 8, 64), dtype=torch.bfloat16), torch.zeros((1, 256), dtype=torch.int32)
+lib.install(4096 * 8 * 4)
+for call in (lambda: pa.gather(row, 4096), lambda: pa.run(q, row)):
+    try:
+        call()
+    except t.ps.PsError:
+        pass
+print(lib.counts(0), lib.counts(1))
+"""
+
+
+def test_results_are_allocated_without_the_interpreter_lock(tmp_path):
+    """An allocation may wait for the device, and what it waits for may need the interpreter (a host function of a stream)."""
+    src, so = tmp_path / "counting.cpp", str(tmp_path / "counting.so")
+    src.write_text(ALLOCATOR)
+    root = os.path.dirname(torch.__file__)
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I",
+                           os.path.join(root, "include"), "-I", sysconfig.get_paths()["include"], str(src), "-o", so, "-L", os.path.join(root, "lib"), "-lc10"])
+    here = os.path.dirname(os.path.abspath(__file__))
+    run = subprocess.run([sys.executable, "-c", ALLOCATE % ([here, os.path.dirname(here)], so)], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr
+    assert run.stdout.split() == ["4", "0"]  # K and V, out and lse
