@@ -5,25 +5,45 @@ call through the C ABI.
 """
 from __future__ import annotations
 
-from . import binding as B
+import subprocess
+import threading
 
-_torch_calls = None
+from . import binding as B
+from . import build
+
+_torch_calls = None  # False: this torch has none
+_torch_calls_lock = threading.Lock()
 
 
 def torch_calls():
-    """The extension module of the calls of every iteration that takes torch tensors."""
+    """The extension module of the calls of every iteration that takes torch tensors, or None where it can be neither loaded nor
+    built: the calls through addresses do the same, some microseconds slower."""
     global _torch_calls
-    if _torch_calls is None:
-        import ctypes
+    with _torch_calls_lock:
+        if _torch_calls is None:
+            import ctypes
+            import importlib.util
+            import os
+            import warnings
 
-        import torch  # noqa: F401  (the extension needs its libraries)
+            lib = B.load()
+            try:
+                path = build.build_torch_calls(build=os.environ.get("PS_ATTN_NO_BUILD") != "1")
+                spec = importlib.util.spec_from_file_location(__package__ + "._torch_calls", path)
+                module = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(module)
+                module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.ps_kv_write, lib.ps_kv_gather, lib.ps_attn_run)))
+                _torch_calls = module
+            except (ImportError, OSError, subprocess.SubprocessError) as e:
+                warnings.warn("the calls with tensors go through addresses: %s" % e, RuntimeWarning)
+                _torch_calls = False
+    return _torch_calls or None
 
-        lib = B.load()
-        from . import _torch_calls as module
 
-        module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.ps_kv_write, lib.ps_kv_gather, lib.ps_attn_run)))
-        _torch_calls = module
-    return _torch_calls
+def take_tensors(pa):
+    """The class whose instances `pa` hands to the extension: torch.Tensor itself, or none."""
+    pa._tensor_calls = torch_calls()
+    pa._tensor = pa.torch.Tensor if pa._tensor_calls else object()  # (the class of nothing)
 
 
 class PagedAttention:
@@ -41,7 +61,7 @@ class PagedAttention:
 
         self.torch = torch
         self._calls = B.calls()
-        self._tensor_calls, self._tensor = torch_calls(), torch.Tensor
+        take_tensors(self)
         self.device = torch.device(device)
         self.shape = B.make_shape(n_q_heads, n_kv_heads, head_dim, page_size, kv_dtype)
         self.num_pages = int(num_pages)

@@ -109,3 +109,47 @@ def test_results_are_allocated_without_the_interpreter_lock(tmp_path):
     run = subprocess.run([sys.executable, "-c", ALLOCATE % ([here, os.path.dirname(here)], so)], capture_output=True, text=True, timeout=300)
     assert run.returncode == 0, run.stderr
     assert run.stdout.split() == ["4", "0"]  # K and V, out and lse
+
+
+def test_the_library_is_built_without_torch(tmp_path):
+    """The C ABI and the planner need no torch, neither to be built nor to be loaded."""
+    (tmp_path / "torch").mkdir()
+    (tmp_path / "torch" / "__init__.py").write_text("raise ImportError('no torch here')\n")
+    here = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import sys; sys.path[:0] = [%r, %r]\nfrom paper_2507_17769_b200 import binding as B, build\nbuild.build_library()\n"
+            "B.load(); assert 'torch' not in sys.modules\nassert not any('torch' in f for f in build.library_files())" % (str(tmp_path), here))
+    run = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr
+
+
+def test_the_extension_belongs_to_one_torch(monkeypatch):
+    """Its file carries the version of torch that it was built against: another torch builds its own."""
+    from paper_2507_17769_b200 import build
+
+    here = build.torch_calls_path()
+    monkeypatch.setattr(torch, "__version__", "1.2.3")
+    assert build.torch_calls_path() != here and "1.2.3" in os.path.basename(build.torch_calls_path())
+
+
+def test_without_the_extension_tensors_take_the_calls_through_addresses(monkeypatch):
+    from paper_2507_17769_b200 import build
+
+    monkeypatch.setattr(session, "_torch_calls", None)
+    monkeypatch.setattr(build, "build_torch_calls", lambda *a, **k: (_ for _ in ()).throw(OSError("no compiler here")))
+    with pytest.warns(RuntimeWarning, match="no compiler here"):
+        assert session.torch_calls() is None
+    assert session.torch_calls() is None  # (tried and told once)
+    monkeypatch.setattr(session.PagedAttention, "__del__", lambda self: None)
+    pa = host_session()
+    session.take_tensors(pa)
+    seen = []
+
+    class Calls:
+        def kv_write(self, *a):
+            seen.append(a)
+            return 0
+
+    pa._calls = Calls()
+    k, row = torch.zeros((1, 2, 64), dtype=torch.bfloat16), torch.zeros((1, 4), dtype=torch.int32)
+    pa.write(k, k, row, [0], [1])
+    assert seen[0][1:5] == (k.data_ptr(), k.data_ptr(), row.data_ptr(), 4)
