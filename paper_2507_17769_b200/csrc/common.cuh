@@ -53,9 +53,10 @@ ps_status once_per_device(PerDeviceOnce& state, F configure) {
 
 // Launches a kernel; clusters of `cluster` CTAs if above 1.  Every kernel of an iteration calls pdl_wait() before it touches
 // what kernels of other calls write or read (a prefill kernel reads its own run's work list, and takes from its own run's
-// queue, before it; one that runs beside its run's decode kernel relies on that one's wait instead, RunArgs::beside), so it may
-// be launched (`early`) while the kernel before it in the stream still runs: its launch and set-up, some 1.5 us, then
-// overlap that kernel's end.  Behind anything but a kernel, a copy or an event for instance, `early` changes nothing.
+// queue, before it, and the merge kernel its entry of that list; a prefill kernel that runs beside its run's decode kernel relies
+// on that one's wait instead, RunArgs::beside), so it may be launched (`early`) while the kernel before it in the stream still
+// runs: its launch and set-up, some 1.5 us, then overlap that kernel's end.  Behind anything but a kernel, a copy or an event for
+// instance, `early` changes nothing.
 template <class... P, class... A>
 ps_status launch_kernel(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t stream, int cluster, bool early, const A&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -9,7 +9,8 @@
 // A warp combines R output rows.  Their partial rows are requested before the log-sum-exps have arrived (their addresses
 // do not depend on them), the log-sum-exps of all (row, segment) pairs are fetched one per lane, and the weights travel by
 // shuffle, so the rows cost about one round trip to L2 together, after the entry record, which belongs to the run's own list and
-// is read while the kernels before are still running.  Bound by latency: rows of few segments go four to a warp, so that all
+// is read while the kernels before are still running.  (The partial rows are not read-only memory for this kernel: it may be there
+// while the prefill kernel still writes them.  They are read from L2, behind the wait.)  Bound by latency: rows of few segments go four to a warp, so that all
 // are under way at once (48 rows and two chunks at head dimension 64, whole iteration, 56.7 -> 55.8 us); rows of more than
 // four segments, of which a batch has few, one to a warp with four segments in flight (100 tokens on 4000, ten segments, four rows
 // a warp with two in flight: 18.5 -> 20.8).
@@ -27,8 +28,7 @@ constexpr int kFewSegs = 4;
 // AHEAD: segments whose partial rows are in flight
 template <int D, int R, int AHEAD>
 __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntry* __restrict__ entries,
-                                                                  const float* __restrict__ part_lse,
-                                                                  const float* __restrict__ part_o,
+                                                                  float* part_lse, float* part_o,
                                                                   __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                                                   int Hq, int G) {
     constexpr int V = D / 32;  // floats per lane
@@ -49,18 +49,19 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntr
     for (int k = 0; k < R; ++k)
 #pragma unroll
         for (int a = 0; a < AHEAD; ++a)
-            if (a < n_seg) x[k][a] = *row_ptr(k, a);
+            if (a < n_seg) x[k][a] = __ldcg(row_ptr(k, a));
     // Lanes kLaneSegs k .. have row k's segments.  A segment that saw no visible key for a row carries lse = -inf and weight 0.
     const float* const my_lse = part_lse + e.base + row_of(lane / kLaneSegs);
+    auto lse_of = [&](int s) { return __ldcg(my_lse + (int64_t)s * e.seg_stride); };
     const int my_seg = lane % kLaneSegs;
-    const float lse_mine = my_seg < n_seg ? my_lse[(int64_t)my_seg * e.seg_stride] : -INFINITY;
+    const float lse_mine = my_seg < n_seg ? lse_of(my_seg) : -INFINITY;
     float M = lse_mine;
-    for (int s = my_seg + kLaneSegs; s < n_seg; s += kLaneSegs) M = fmaxf(M, my_lse[(int64_t)s * e.seg_stride]);
+    for (int s = my_seg + kLaneSegs; s < n_seg; s += kLaneSegs) M = fmaxf(M, lse_of(s));
 #pragma unroll
     for (int o = kLaneSegs / 2; o >= 1; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     const float w_mine = __expf(lse_mine - M);  // exp(-inf) = 0
     float denom = w_mine;
-    for (int s = my_seg + kLaneSegs; s < n_seg; s += kLaneSegs) denom += __expf(my_lse[(int64_t)s * e.seg_stride] - M);
+    for (int s = my_seg + kLaneSegs; s < n_seg; s += kLaneSegs) denom += __expf(lse_of(s) - M);
 #pragma unroll
     for (int o = kLaneSegs / 2; o >= 1; o >>= 1) denom += __shfl_xor_sync(0xffffffffu, denom, o);
 
@@ -76,13 +77,13 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntr
             for (int k = 0; k < R; ++k)
 #pragma unroll
                 for (int a = 0; a < AHEAD; ++a)
-                    if (s0 + a < n_seg) x[k][a] = *row_ptr(k, s0 + a);
+                    if (s0 + a < n_seg) x[k][a] = __ldcg(row_ptr(k, s0 + a));
         }
 #pragma unroll
         for (int a = 0; a < AHEAD; ++a) {
             const int s = s0 + a;
             if (s < n_seg) {  // warp-uniform
-                const float w_far = s < kLaneSegs ? 0.f : __expf(my_lse[(int64_t)s * e.seg_stride] - M);  // of this lane's row
+                const float w_far = s < kLaneSegs ? 0.f : __expf(lse_of(s) - M);  // of this lane's row
 #pragma unroll
                 for (int k = 0; k < R; ++k) {
                     const float w = __shfl_sync(0xffffffffu, s < kLaneSegs ? w_mine : w_far, k * kLaneSegs + s % kLaneSegs);
@@ -119,7 +120,7 @@ ps_status launch_merge(const RunArgs& a) {
     // blockIdx.x = merge entry (a prefill item cut into segments, up to 256 rows); blockIdx.y = its rows
     auto launch = [&](auto* kernel, int rows_of_warp) {
         return launch_kernel(kernel, dim3(a.w.n_merge, kPrefillRowsPerItem / (kMergeWarps * rows_of_warp)), kMergeWarps * 32, 0, a.stream, 1, a.early, a.w.merge,
-                             (const float*)a.w.part_lse, (const float*)a.w.part_o, a.out, a.lse, Hq, G);
+                             a.w.part_lse, a.w.part_o, a.out, a.lse, Hq, G);
     };
     if (a.w.merge_segs <= kFewSegs) return a.shape.head_dim == 128 ? launch(merge_kernel<128, 4, 2>, 4) : launch(merge_kernel<64, 4, 2>, 4);
     return a.shape.head_dim == 128 ? launch(merge_kernel<128, 1, 4>, 1) : launch(merge_kernel<64, 1, 4>, 1);
