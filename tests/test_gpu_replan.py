@@ -145,3 +145,34 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(kind):
     out2, lse2 = db.run()
     db.pa.check()
     assert torch.equal(out.view(torch.int16), out2.view(torch.int16)) and torch.equal(lse, lse2)
+
+
+@pytest.mark.parametrize("kind", ["decode", "prefill", "mixed"])
+def test_waits_that_run_out_at_head_dimension_64(kind):
+    """The same for the kernels of head dimension 64: decode with a unit per warp (two copies a phase in flight), prefill with
+    items of one q tile and of two (two MMA warps, stages that one of them passes over), and both side by side."""
+    import torch
+    from workloads.device import DeviceBatch
+
+    decode = ([1999, 2500, 1200, 900, 3000, 1700, 2100, 800] * 3, [1] * 24)
+    chunks = ([700, 0, 300], [200, 100, 385])
+    rows = decode if kind == "decode" else chunks if kind == "prefill" else (decode[0] + chunks[0], decode[1] + chunks[1])
+    b = gen.make_batch(gen.Shape(8, 8, 64), 8203, *rows)
+    db = DeviceBatch(b)
+    info = db.plan()
+    assert (info.n_prefill_items == 0) == (kind == "decode") and (info.n_decode_items == 0) == (kind == "prefill")
+    assert kind == "prefill" or info.n_decode_items > 148  # (a unit per warp)
+    for _ in range(2):
+        ps.ps_plan_set_wait_limit(db.pa._plan, 0)
+        db.run()
+        with pytest.raises(ps.PsError) as e:
+            db.pa.check()
+        assert e.value.status == B.PS_ERR_TIMEOUT
+        ps.ps_plan_set_wait_limit(db.pa._plan, 2_000_000_000)
+        out, lse = db.run()
+        db.pa.check()
+        want, want_lse, _ = oracle_subset(b, range(b.n))
+        compare(out, lse, want, want_lse, what="after a timed-out run (%s)" % kind)
+    out2, lse2 = db.run()
+    db.pa.check()
+    assert torch.equal(out.view(torch.int16), out2.view(torch.int16)) and torch.equal(lse, lse2)
