@@ -235,6 +235,7 @@ struct RunArgs {
     cudaStream_t stream;
     int num_sms;
     int dec_sms, pf_sms;  // SMs (= CTAs) for the decode and the prefill kernel
+    int dec_pages = 1;    // pages a stage of the decode kernel with a unit per warp
     bool pairs;           // the prefill items go to CTA pairs
     bool sm_pairs;        // side by side with the pair kernel: the decode kernel's CTAs take whole SM pairs too
     // work lists as kernel parameters, on the host; null: they are in the workspace
@@ -256,7 +257,8 @@ ps_status launch_prefill(const RunArgs& a);
 ps_status launch_prefill_pair(const RunArgs& a);  // head dimension 128
 ps_status launch_prefill_d64(const RunArgs& a);
 ps_status launch_merge(const RunArgs& a);
-int decode_warps_per_sm(int head_dim);
+// streaming warps of a CTA of the decode kernel with a unit per warp, by pages a stage
+__host__ __device__ constexpr int decode_unit_warps(int head_dim, int pages) { return head_dim == 64 && pages == 1 ? 24 : 12; }
 
 // ---------------------------------------------------------------------------
 // PTX wrappers

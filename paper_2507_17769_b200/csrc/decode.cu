@@ -48,14 +48,15 @@ struct DecodeCfg {
         kWarps * kStages * kStageBytes + kWarps * kStages * 8 + kWarps * kRing * 4 + kWarps * kDeferred * 12 + 1024;
 };
 
-// The kernel with a unit per warp.  At head dimension 64 a page is half as large and takes a warp nearly as long: two pages a
-// stage, whose softmax costs little more than one's, on as many warps as at 128.  An SM streams 100 GB/s instead of 87 with a page
-// a stage on 24 warps (32 SMs, 256 rows of 3000 tokens, 8 heads: 559 -> 492 us; all SMs 253 -> 245).
-template <int D, bool FP8>
+// The kernel with a unit per warp, PAGES pages a stage.  At head dimension 64 a page is half as large and takes a warp nearly as long:
+// two pages a stage, whose softmax costs little more than one's, on as many warps as at 128.  An SM streams 100 GB/s instead of 87
+// with a page a stage on 24 warps (32 SMs, 256 rows of 3000 tokens, 8 heads: 559 -> 492 us; all SMs 253 -> 245).  But batches of many
+// short rows are bound by what a row costs a warp beside its pages, and there 24 warps are faster: one_page_a_stage() in plan.cu.
+template <int D, bool FP8, int PAGES>
 struct StreamCfg {
-    static constexpr int kPages = D == 128 ? 1 : 2;
+    static constexpr int kPages = PAGES;
     static constexpr int kPageBytes = DecodeCfg<D, FP8>::kStageBytes, kStageBytes = kPages * kPageBytes;
-    static constexpr int kWarps = 12;
+    static constexpr int kWarps = decode_unit_warps(D, PAGES);
     static constexpr int kStages = DecodeCfg<D, FP8>::kStages;
     static constexpr int kSmemBytes =
         kWarps * kStages * kStageBytes + kWarps * kStages * 8 + kWarps * kRing * 4 + kWarps * kDeferred * 12 + 1024;
@@ -330,9 +331,9 @@ __device__ __forceinline__ void attend_pages(char* stage, uint32_t kbase, int nv
     }
 }
 
-template <int D, bool FP8>
-__global__ void __launch_bounds__(StreamCfg<D, FP8>::kWarps * 32, 1) decode_kernel(const DecodeParams p) {
-    using Cfg = StreamCfg<D, FP8>;
+template <int D, bool FP8, int PAGES>
+__global__ void __launch_bounds__(StreamCfg<D, FP8, PAGES>::kWarps * 32, 1) decode_kernel(const DecodeParams p) {
+    using Cfg = StreamCfg<D, FP8, PAGES>;
     constexpr int PP = Cfg::kPages;  // of a stage
     constexpr int kWarps = Cfg::kWarps;
     constexpr int STAGES = Cfg::kStages;
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(StreamCfg<D, FP8>::kWarps * 32, 1) decode_kern
             for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
             // fixed segment order; kAhead segments' rows are requested before the first is used, so that a long
             // list of segments costs about one trip to L2 per kAhead of them
-            constexpr int kAhead = NV <= 2 ? 8 : NV <= 4 ? 4 : 2;  // at most 16 float4 in flight per lane
+            constexpr int kAhead = (NV <= 2 ? 8 : NV <= 4 ? 4 : 2) * 12 / kWarps;  // at most 16 float4 in flight per lane (8 with 24 warps)
             for (int s0 = 0; s0 < dm.n_seg; s0 += kAhead) {
                 float4 x[kAhead][NV];
                 float lw[kAhead];
@@ -850,15 +851,14 @@ __global__ void __launch_bounds__(DecodeCfg<D, FP8>::kWarps * 32, 1) decode_cta_
 
 }  // namespace
 
-int decode_warps_per_sm(int head_dim) { return head_dim == 128 ? StreamCfg<128, false>::kWarps : StreamCfg<64, false>::kWarps; }
-
-template <int D, bool FP8>
+template <int D, bool FP8, int PAGES>
 static ps_status launch_decode_d(const RunArgs& a) {
     using Cfg = DecodeCfg<D, FP8>;
+    using Stream = StreamCfg<D, FP8, PAGES>;
     constexpr int kWarps = Cfg::kWarps;
     static PerDeviceOnce configured;
     const ps_status cfg = once_per_device(configured, []() -> ps_status {
-        PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<D, FP8>::kSmemBytes));
+        PS_CUDA_TRY(cudaFuncSetAttribute(decode_kernel<D, FP8, PAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, Stream::kSmemBytes));
         PS_CUDA_TRY(cudaFuncSetAttribute(decode_cta_kernel<D, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
         return PS_OK;
     });
@@ -889,8 +889,7 @@ static ps_status launch_decode_d(const RunArgs& a) {
     p.n_part_slots = a.w.n_part_slots;
     p.wait_limit_ns = a.wait_limit_ns;
     p.tag = a.tag;
-    constexpr int kUnitWarps = StreamCfg<D, FP8>::kWarps;
-    int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + kUnitWarps - 1) / kUnitWarps;
+    int grid = a.w.n_cta_pieces > 0 ? a.w.n_cta_pieces : (a.w.n_units + Stream::kWarps - 1) / Stream::kWarps;
     if (grid > a.dec_sms) grid = a.dec_sms;
     // Beside the prefill kernel whose CTAs come in pairs: launched in clusters of two, this kernel's CTAs leave whole SM
     // pairs free.  Launched singly they are spread over the pairs, one SM of each, and no prefill pair finds a place
@@ -904,13 +903,14 @@ static ps_status launch_decode_d(const RunArgs& a) {
         }
         return launch_kernel(decode_cta_kernel<D, FP8>, grid, kWarps * 32, Cfg::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p, a.w.n_cta_pieces, inl);
     }
-    return launch_kernel(decode_kernel<D, FP8>, grid, kUnitWarps * 32, StreamCfg<D, FP8>::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
+    return launch_kernel(decode_kernel<D, FP8, PAGES>, grid, Stream::kWarps * 32, Stream::kSmemBytes, a.stream, a.sm_pairs ? 2 : 1, a.early, p);
 }
 
 ps_status launch_decode(const RunArgs& a) {
     if (a.w.n_units == 0 && a.w.n_cta_pieces == 0) return PS_OK;
-    if (a.shape.dtype == 1) return launch_decode_d<128, true>(a);  // the FP8 cache variant exists for head_dim 128
-    return a.shape.head_dim == 128 ? launch_decode_d<128, false>(a) : launch_decode_d<64, false>(a);
+    if (a.shape.dtype == 1) return launch_decode_d<128, true, 1>(a);  // the FP8 cache variant exists for head_dim 128
+    if (a.shape.head_dim == 128) return launch_decode_d<128, false, 1>(a);
+    return a.dec_pages == 2 ? launch_decode_d<64, false, 2>(a) : launch_decode_d<64, false, 1>(a);
 }
 
 }  // namespace ps

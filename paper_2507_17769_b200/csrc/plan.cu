@@ -189,6 +189,7 @@ struct ps_plan {
     std::vector<DecodePiece> pieces;
     std::vector<DecodeUnit> units;
     bool cta_pieces = false;             // a CTA per piece, no units
+    int dec_pages = 1;                   // pages a stage of the decode kernel with a unit per warp
     std::vector<PrefillItem> prefill;
     std::vector<MergeEntry> merge;       // prefill q tile pairs cut into segments: combined by the merge kernel
     std::vector<DecodeMerge> dmerge;     // combined inside the decode kernel
@@ -302,13 +303,25 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
     return true;
 }
 
+// Which form of the decode kernel with a unit per warp takes a batch at head dimension 64: two pages a stage on 12 warps an SM, or one
+// on 24.  A row costs a warp some 2 us beside its pages, so short rows of which a warp has several are done sooner by twice the warps:
+// where there are 1.2 times as many (row, kv head)s as warps and more than the smallest units' pages, up to 9 pages a row.
+// Measured (12 warps / 24, us, 8 kv heads, contexts within half of the mean): 512 rows of 28 tokens 20.3 / 18.3, of 40 22.3 / 18.7, of 64
+// 25.9 / 23.9, of 128 35.1 / 34.4, of 256 55.6 / 54.7; 350 of 40 18.7 / 18.2, of 64 20.9 / 19.8, of 96 24.5 / 22.5, of 256 41.3 / 41.3; 280 of
+// 64 19.8 / 18.6, of 96 21.0 / 22.4, of 128 24.4 / 24.0, of 192 29.7 / 31.0; 230 of 64 18.2 / 18.3, of 128 20.8 / 22.3; few pages: 512 of 20
+// 15.7 / 16.1, 350 of 28 15.4 / 18.1; 2 kv heads: 512 of 128 18.7 / 19.5.
+static bool one_page_a_stage(const ps_plan& pl, int64_t n_rows, int64_t total_pages) {
+    const int64_t warps = (int64_t)pl.dec_sms * decode_unit_warps(64, 2);
+    return n_rows * 5 >= warps * 6 && total_pages > kDecodeMinPagesLo * warps && total_pages <= 9 * n_rows;
+}
+
 static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,
                         const ps_plan_opts* opts, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
-    int64_t total_pages = 0, longest = 0;
+    int64_t total_pages = 0, longest = 0, n_rows = 0;  // (n_rows, total_pages: of all kv heads)
     for (int r = 0; r < pl->n; ++r)
         if (runs_as_decode(pl->shape, pl->tiny_as_rows, prior[r], q_len[r]))
-            for (int i = 0; i < q_len[r]; ++i) {
+            for (int i = 0; i < q_len[r]; ++i, n_rows += Hkv) {
                 const int64_t pages = (prior[r] + i + 1 + kPage - 1) / kPage;
                 total_pages += pages * Hkv;
                 longest = std::max(longest, pages);
@@ -322,21 +335,20 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     pl->cta_pieces = false;
     pl->info.decode_segment_tokens = 0;
     if (!(opts && opts->decode_segment_tokens > 0) && plan_decode_ctas(pl, prior, q_len, q_start, total_pages, longest, n_slots)) return;
+    pl->dec_pages = pl->shape.head_dim == 64 && !one_page_a_stage(*pl, n_rows, total_pages) ? 2 : 1;
     const int64_t min_pages = std::min<int64_t>(kDecodeMinPagesHi, std::max<int64_t>(kDecodeMinPagesLo, (longest + kDecodePiecesPerRow - 1) / kDecodePiecesPerRow));
     int64_t per_unit;
     if (opts && opts->decode_segment_tokens > 0) {
         per_unit = std::max(1, opts->decode_segment_tokens / kPage);
     } else {
-        const int64_t target = (int64_t)pl->dec_sms * decode_warps_per_sm(pl->shape.head_dim) * kDecodeUnitsPerWarp;
+        const int64_t target = (int64_t)pl->dec_sms * decode_unit_warps(pl->shape.head_dim, pl->dec_pages) * kDecodeUnitsPerWarp;
         per_unit = std::max<int64_t>(min_pages, (total_pages + target - 1) / target);
-        if (pl->shape.head_dim == 64) per_unit += per_unit & 1;  // (two pages a stage)
+        if (pl->dec_pages == 2) per_unit += per_unit & 1;
     }
     pl->info.decode_segment_tokens = (int32_t)(per_unit * kPage);
 
     // Upper bounds on the counts (a piece ends where its row or its unit ends), so that the lists are filled
     // in place and trimmed once.
-    int64_t n_rows = 0;
-    for (int r = 0; r < pl->n; ++r) n_rows += runs_as_decode(pl->shape, pl->tiny_as_rows, prior[r], q_len[r]) ? (int64_t)q_len[r] * Hkv : 0;
     const size_t max_units = (size_t)((total_pages + per_unit - 1) / per_unit);
     pl->pieces.resize((size_t)n_rows + max_units);
     pl->units.resize(max_units);
@@ -975,6 +987,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     a.dec_sms = pl->dec_sms;
     a.pf_sms = pl->pf_sms;
     a.pairs = pl->pairs;
+    a.dec_pages = pl->dec_pages;
     a.total_q = (int32_t)pl->info.total_q_tokens;
     a.n_req = pl->n;
     a.wait_limit_ns = pl->wait_limit_ns;

@@ -1,0 +1,26 @@
+"""Which form of the decode kernel a batch of head dimension 64 takes, on both sides of the lines: seen in the size of its units, which
+follows from the number of warps that share the pages."""
+import numpy as np
+import pytest
+
+import paper_2507_17769_b200 as ps
+
+
+def unit_pages(rows, ctx, kv_heads=8, group=1, sms=148):
+    shape = ps.make_shape(kv_heads * group, kv_heads, 64)
+    plan, _ = ps.ps_attn_plan(shape, np.full(rows, ctx - 1), np.ones(rows, dtype=np.int32), (ctx + 15) // 16, ps.ps_plan_opts(0, 0, sms))
+    info = ps.ps_plan_get_info(plan)
+    items = ps.ps_plan_get_items(plan)[0]
+    ps.ps_plan_free(plan)
+    assert sum(-(-int(e) // 16) - int(b) // 16 for b, e in items[:, 2:4]) == rows * kv_heads * ((ctx + 15) // 16)
+    return info.decode_segment_tokens // 16
+
+
+@pytest.mark.parametrize("rows,ctx,warps", [
+    (512, 40, 24), (512, 144, 24), (512, 145, 12),  # nine pages a row, ten
+    (267, 64, 24), (266, 64, 12),                   # 1.2 rows a warp
+])
+def test_many_short_rows_take_24_warps(rows, ctx, warps):
+    pages = rows * 8 * ((ctx + 15) // 16)
+    share = -(-pages // (148 * warps))
+    assert unit_pages(rows, ctx) in ((max(4, share),) if warps == 24 else (max(4, share), max(4, share) + 1))
