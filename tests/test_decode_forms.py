@@ -24,3 +24,8 @@ def test_many_short_rows_take_24_warps(rows, ctx, warps):
     pages = rows * 8 * ((ctx + 15) // 16)
     share = -(-pages // (148 * warps))
     assert unit_pages(rows, ctx) in ((max(4, share),) if warps == 24 else (max(4, share), max(4, share) + 1))
+
+
+@pytest.mark.parametrize("rows,ctx,pages", [(30, 500, 5), (30, 1000, 9), (80, 500, 12)])
+def test_small_units_are_not_rounded_to_whole_stages(rows, ctx, pages):
+    assert unit_pages(rows, ctx) == pages
