@@ -10,7 +10,7 @@
 // do not depend on them), the log-sum-exps of all (row, segment) pairs are fetched one per lane, and the weights travel by
 // shuffle, so the rows cost about one round trip to L2 together, after the entry record, which belongs to the run's own list and
 // is read while the kernels before are still running.  (The partial rows are not read-only memory for this kernel: it may be there
-// while the prefill kernel still writes them.  They are read from L2, behind the wait.)  Bound by latency: rows of few segments go four to a warp, so that all
+// while the prefill kernel still writes them.  They are ordinary loads, behind the wait.)  Bound by latency: rows of few segments go four to a warp, so that all
 // are under way at once (48 rows and two chunks at head dimension 64, whole iteration, 56.7 -> 55.8 us); rows of more than
 // four segments, of which a batch has few, one to a warp with four segments in flight (100 tokens on 4000, ten segments, four rows
 // a warp with two in flight: 18.5 -> 20.8).
@@ -49,10 +49,10 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntr
     for (int k = 0; k < R; ++k)
 #pragma unroll
         for (int a = 0; a < AHEAD; ++a)
-            if (a < n_seg) x[k][a] = __ldcg(row_ptr(k, a));
+            if (a < n_seg) x[k][a] = *row_ptr(k, a);
     // Lanes kLaneSegs k .. have row k's segments.  A segment that saw no visible key for a row carries lse = -inf and weight 0.
     const float* const my_lse = part_lse + e.base + row_of(lane / kLaneSegs);
-    auto lse_of = [&](int s) { return __ldcg(my_lse + (int64_t)s * e.seg_stride); };
+    auto lse_of = [&](int s) { return my_lse[(int64_t)s * e.seg_stride]; };
     const int my_seg = lane % kLaneSegs;
     const float lse_mine = my_seg < n_seg ? lse_of(my_seg) : -INFINITY;
     float M = lse_mine;
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const MergeEntr
             for (int k = 0; k < R; ++k)
 #pragma unroll
                 for (int a = 0; a < AHEAD; ++a)
-                    if (s0 + a < n_seg) x[k][a] = __ldcg(row_ptr(k, s0 + a));
+                    if (s0 + a < n_seg) x[k][a] = *row_ptr(k, s0 + a);
         }
 #pragma unroll
         for (int a = 0; a < AHEAD; ++a) {
