@@ -305,14 +305,15 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
 
 // Which form of the decode kernel with a unit per warp takes a batch at head dimension 64: two pages a stage on 12 warps an SM, or one
 // on 24.  A row costs a warp some 2 us beside its pages, so short rows of which a warp has several are done sooner by twice the warps:
-// where there are 1.2 times as many (row, kv head)s as warps and more than the smallest units' pages, up to 9 pages a row.
-// Measured (12 warps / 24, us, 8 kv heads, contexts within half of the mean): 512 rows of 28 tokens 20.3 / 18.3, of 40 22.3 / 18.7, of 64
-// 25.9 / 23.9, of 128 35.1 / 34.4, of 256 55.6 / 54.7; 350 of 40 18.7 / 18.2, of 64 20.9 / 19.8, of 96 24.5 / 22.5, of 256 41.3 / 41.3; 280 of
-// 64 19.8 / 18.6, of 96 21.0 / 22.4, of 128 24.4 / 24.0, of 192 29.7 / 31.0; 230 of 64 18.2 / 18.3, of 128 20.8 / 22.3; few pages: 512 of 20
-// 15.7 / 16.1, 350 of 28 15.4 / 18.1; 2 kv heads: 512 of 128 18.7 / 19.5.
+// from 1.2 (row, kv head)s a warp up to 5 pages a row, from 1.5 up to 9, where the smallest units do not leave warps idle anyway.
+// Measured (12 warps / 24, us, 8 kv heads, 1 and 4 q heads each, contexts within half of the mean): 512 rows of 28 tokens 20.5 / 18.6,
+// of 40 22.6 / 19.3, of 64 26.1 / 24.3, of 96 30.0 / 30.7, of 128 35.9 / 34.7, of 256 55.5 / 55.3; 350 of 40 19.5 / 18.3, of 64 21.8 / 20.1, of
+// 96 25.2 / 23.6, of 128 28.7 / 28.0, of 192 35.3 / 35.2; 280 of 64 20.3 / 18.6, of 96 21.3 / 22.4, of 192 30.7 / 31.8; 230 of 64 18.5 / 18.4,
+// of 128 21.4 / 22.1; few pages: 512 of 20 16.0 / 16.4, 350 of 28 15.8 / 18.2; 2 kv heads: 512 of 128 18.7 / 19.5.
 static bool one_page_a_stage(const ps_plan& pl, int64_t n_rows, int64_t total_pages) {
     const int64_t warps = (int64_t)pl.dec_sms * decode_unit_warps(64, 2);
-    return n_rows * 5 >= warps * 6 && total_pages > kDecodeMinPagesLo * warps && total_pages <= 9 * n_rows;
+    if (total_pages <= kDecodeMinPagesLo * warps) return false;
+    return (n_rows * 5 >= warps * 6 && total_pages <= 5 * n_rows) || (n_rows * 2 >= warps * 3 && total_pages <= 9 * n_rows);
 }
 
 static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,

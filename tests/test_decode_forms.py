@@ -18,7 +18,8 @@ def unit_pages(rows, ctx, kv_heads=8, group=1, sms=148):
 
 @pytest.mark.parametrize("rows,ctx,warps", [
     (512, 40, 24), (512, 144, 24), (512, 145, 12),  # nine pages a row, ten
-    (267, 64, 24), (266, 64, 12),                   # 1.2 rows a warp
+    (267, 80, 24), (266, 80, 12), (267, 81, 12),     # 1.2 rows a warp, five pages a row, six
+    (333, 96, 24), (332, 96, 12),                   # 1.5 rows a warp
 ])
 def test_many_short_rows_take_24_warps(rows, ctx, warps):
     pages = rows * 8 * ((ctx + 15) // 16)
@@ -26,6 +27,6 @@ def test_many_short_rows_take_24_warps(rows, ctx, warps):
     assert unit_pages(rows, ctx) in ((max(4, share),) if warps == 24 else (max(4, share), max(4, share) + 1))
 
 
-@pytest.mark.parametrize("rows,ctx,pages", [(30, 500, 5), (30, 1000, 9), (80, 500, 12)])
+@pytest.mark.parametrize("rows,ctx,pages", [(30, 500, 5), (30, 1000, 9), (80, 480, 12)])
 def test_small_units_are_not_rounded_to_whole_stages(rows, ctx, pages):
     assert unit_pages(rows, ctx) == pages
