@@ -468,7 +468,9 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
         static_partition = true;
         double total = 0;
         for (const Tile& t : tiles) total += cost.fixed + t.key_tiles + cost.masked_extra;
-        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_workers, total / kPrefillMinCtaCost));
+        // (No two items on one CTA while another has none: two fresh items of one key tile, 16 q / 2 kv heads of 64, 14.1 us on one
+        // CTA, 9.7 on two; 56 items of 1 and 2 key tiles 15.2 on 50 CTAs, 12.0 on 56.)
+        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_workers, std::max<double>((double)tiles.size(), total / kPrefillMinCtaCost)));
         // Many short items (fresh prompts): whole items, longest first, each to the CTA with the least work so far.
         // If that comes within kPrefillWholeItemSlack of an even split, nothing is cut: no partial rows, no merge
         // kernel, no item paying its fixed cost twice.
