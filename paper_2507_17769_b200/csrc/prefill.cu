@@ -79,17 +79,13 @@ struct PrefillParams {
     float* lse;
     WsHeader* hdr;
     const PrefillItem* items;
-    const int32_t* cta_start;  // static partition: this CTA runs items [cta_start[b], cta_start[b + 1]); null = dynamic queue
-    float* part_lse;
-    float* part_o;
     int64_t num_pages;
     uint32_t wait_limit_ns;
     int32_t max_pages;
     int32_t n_items;
     int32_t Hq, Hkv, G;
-    int32_t n_req, total_q, n_part_slots;  // extents the item records are checked against
+    int32_t n_req, total_q;  // extents the item records are checked against
     int32_t tag;
-    int16_t inline_list, beside;
 };
 static_assert(sizeof(PrefillParams) <= 128, "parameter block");
 
@@ -110,7 +106,7 @@ static_assert(Bars::mma_drained % 8 == 0 && Bars::armed + 24 <= Bars::ring && si
                   Bars::bytes <= kBarBlockBytes,
               "barrier block layout");
 
-__global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map, const __grid_constant__ InlineItems inl) {
+__global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap q_map) {
     extern __shared__ char smem_raw[];
     char* smem = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -149,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         tmem_alloc(bars + Bars::tmem_slot, Cfg::kTmemCols);
         tmem_relinquish();
     }
-    if (!p.beside) pdl_wait();
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -379,6 +375,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                     const int row0 = (warp & 3) * 32;          // first tile row of this warp
                     const int sub = lane >> 3, unit = lane & 7;  // write-out: 4 rows per instruction, 8 lanes x 16 bytes per row
                     char* const my_row = stg + lane * 128;
+                    // (Always so: these batches' items are not cut.  Without the branch ptxas spills 64 bytes of the softmax loop's registers
+                    // instead of 28: 188 chunks of 64 tokens on 320, 64 q heads, 262 us instead of 250.)
                     if (it.part_slot < 0) {
                         // final output: bf16, 64 columns (128 bytes of each row) per pass
 #pragma unroll 1
@@ -411,30 +409,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                             __syncwarp();
                         }
                         if (valid && p.lse) p.lse[(int64_t)(it.q_tok + i) * p.Hq + it.kv_head * p.G + hh] = lse_v;
-                    } else {
-                        // partial result of a cut item: fp32 rows at consecutive slots, 32 columns per pass
-                        const int64_t prow0 = (int64_t)it.part_slot + x * kRows + row0;
-#pragma unroll 1
-                        for (int c0 = 0; c0 < D; c0 += 32) {
-                            uint32_t v[32];
-                            tmem_ld32(o_addr + c0, v);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int u = 0; u < 8; ++u)
-                                *reinterpret_cast<float4*>(my_row + ((u ^ (lane & 7)) << 4)) =
-                                    make_float4(__uint_as_float(v[4 * u]) * inv, __uint_as_float(v[4 * u + 1]) * inv,
-                                                __uint_as_float(v[4 * u + 2]) * inv, __uint_as_float(v[4 * u + 3]) * inv);
-                            __syncwarp();
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const int r = k * 4 + sub, tt = row0 + r;
-                                if (x * tile_tok + (tt >> g_shift) < it.n_tok)
-                                    *reinterpret_cast<float4*>(p.part_o + (prow0 + r) * D + c0 + unit * 4) =
-                                        *reinterpret_cast<const float4*>(stg + r * 128 + ((unit ^ (r & 7)) << 4));
-                            }
-                            __syncwarp();
-                        }
-                        if (valid) p.part_lse[prow0 + lane] = lse_v;
                     }
                 }
                 tiles_x += n_tiles;
@@ -456,29 +430,17 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
             const int pg = lane >> 2, which = lane & 3;  // page in tile; 0/1 = K half 0/1, 2/3 = V half 0/1
             constexpr uint32_t kPieceBytes = kPage * 128;  // 16 tokens x 64 elements
             uint32_t n_item = 0, tile_ctr = 0, items_x[2] = {0, 0};
-            const bool static_share = p.inline_list || p.cta_start;
-            auto start_of = [&](int cta) { return p.inline_list ? inl.start[cta] : p.cta_start ? p.cta_start[cta] : 0; };
-            int static_cur = start_of(blockIdx.x);
-            const int static_end = start_of(blockIdx.x + 1);
             bool ok = true;
             while (ok) {
-                // next item of this CTA's static share, or of the queue all CTAs of the run drain
+                // next item of the queue all CTAs of the run drain
                 int idx = 0;
-                if (lane == 0)
-                    idx = static_share ? (static_cur < static_end ? static_cur : p.n_items) : atomicAdd(&p.hdr->prefill_next, 1);
-                ++static_cur;
+                if (lane == 0) idx = atomicAdd(&p.hdr->prefill_next, 1);
                 idx = __shfl_sync(0xffffffffu, idx, 0);
                 uint4 rec0 = make_uint4(0, 0, 0, 0), rec1 = make_uint4(0, 0, 0, 0);  // n_tok = 0: end of work
                 if (idx < p.n_items) {
-                    if (p.inline_list) {
-                        const PrefillItem& it = inl.item[idx];
-                        rec0 = make_uint4(it.req, it.kv_head, it.key_begin, it.key_end);
-                        rec1 = make_uint4(it.q_tok, it.n_tok, it.part_slot, it.first_pos);
-                    } else {
-                        const uint4* src = reinterpret_cast<const uint4*>(p.items + idx);
-                        rec0 = __ldg(src);
-                        rec1 = __ldg(src + 1);
-                    }
+                    const uint4* src = reinterpret_cast<const uint4*>(p.items + idx);
+                    rec0 = __ldg(src);
+                    rec1 = __ldg(src + 1);
                     // A record that points outside the batch (only a damaged work list has one) ends this CTA's
                     // work and flags the run; nothing is read or written through it.
                     const int32_t r_req = (int32_t)rec0.x, r_g = (int32_t)rec0.y, r_kb = (int32_t)rec0.z, r_ke = (int32_t)rec0.w;
@@ -487,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
                                         r_kb % kTileKeys == 0 && r_kb < r_ke && r_ke <= p.max_pages * kPage && r_n >= 1 &&
                                         r_n <= 2 * tile_tok && r_q >= 0 && (int64_t)r_q + r_n <= p.total_q && r_pos >= 0 &&
                                         (int64_t)r_pos + r_n >= r_ke &&
-                                        (r_slot < 0 || (int64_t)r_slot + (int64_t)r_n * p.G <= p.n_part_slots);
+                                        r_slot < 0;  // (these batches' items are not cut)
                     if (!rec_ok) {
                         if (lane == 0) report(p.hdr, p.tag, kStatusBounds);
                         rec0 = rec1 = make_uint4(0, 0, 0, 0);
@@ -695,7 +657,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(const PrefillParam
         __syncthreads();
     }
     if (warp == 0) tmem_dealloc(tmem, Cfg::kTmemCols);
-    if (p.beside && blockIdx.x == 0) pdl_wait();  // this kernel's end also means that of the decode kernel beside it
 }
 
 }  // namespace
@@ -717,29 +678,19 @@ static ps_status launch_prefill_single(const RunArgs& a) {
     p.hdr = a.w.hdr;
     p.items = a.w.prefill;
     p.n_items = a.w.n_prefill;
-    p.cta_start = a.w.n_prefill_ctas > 0 ? a.w.prefill_cta_start : nullptr;
-    p.part_lse = a.w.part_lse;
-    p.part_o = a.w.part_o;
     p.Hq = a.shape.n_q_heads;
     p.Hkv = a.shape.n_kv_heads;
     p.G = p.Hq / p.Hkv;
     p.n_req = a.n_req;
     p.total_q = a.total_q;
-    p.n_part_slots = (int32_t)a.w.n_part_slots;
     p.wait_limit_ns = (uint32_t)a.wait_limit_ns;
-
     p.tag = a.tag;
-    p.inline_list = a.inline_items != nullptr;
-    p.beside = a.beside;
-    InlineItems inl;
-    fill_inline_items(a, inl);
-
     CUtensorMap q_map;
     const ps_status enc = encode_q_map(a, &q_map);
     if (enc != PS_OK) return enc;
 
-    const int grid = a.w.n_prefill_ctas > 0 ? a.w.n_prefill_ctas : (a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms);
-    return launch_kernel(prefill_kernel, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map, inl);
+    const int grid = a.w.n_prefill < a.pf_sms ? a.w.n_prefill : a.pf_sms;
+    return launch_kernel(prefill_kernel, grid, kThreads, Cfg::kSmemBytes, a.stream, 1, a.early, p, q_map);
 }
 
 ps_status launch_prefill(const RunArgs& a) {
