@@ -302,7 +302,7 @@ def cpu_baseline_record(batch, sample, timing):
 
 
 def components_alone(pa, batch, db, out, steps, peaks):
-    """Decode rows alone and prefill rows alone (each planned by itself on all SMs), for attribution in mixed batches.
+    """Decode rows alone and prefill rows alone (each planned by itself), for attribution in mixed batches.
     Returns one record per row class for the roofline's kernel list."""
     import torch
     import paper_2507_17769_b200 as ps
@@ -319,6 +319,8 @@ def components_alone(pa, batch, db, out, steps, peaks):
         q = db.q.index_select(0, torch.from_numpy(tok).to(db.q.device)).contiguous()
         o = torch.empty_like(q)
         prior, q_len = batch.prior[idx], batch.q_len[idx]
+
+        info = pa.plan(prior, q_len, batch.max_pages)
 
         def step():
             pa.plan(prior, q_len, batch.max_pages)
@@ -340,7 +342,7 @@ def components_alone(pa, batch, db, out, steps, peaks):
         pre_ms, dec_ms, _, _ = ps.ps_plan_get_timing(pa._plan, stream.cuda_stream)
         ps.ps_plan_set_timing(pa._plan, 0)
         if name == "decode":
-            res.append(kernel_record("decode_kernel", "decode rows alone on all SMs", dec_ms, float(batch.decode_bytes()), peaks,
+            res.append(kernel_record("decode_kernel", "decode rows alone on %d SMs" % info.decode_sms, dec_ms, float(batch.decode_bytes()), peaks,
                                      step_ms=step_ms))
         else:
             res.append(kernel_record(prefill_kernel_name(batch), "prefill rows alone on all SMs", pre_ms, float(batch.prefill_flops()), peaks,
@@ -350,8 +352,8 @@ def components_alone(pa, batch, db, out, steps, peaks):
 
 
 def prefill_kernel_name(batch):
-    """The kernel of the timed workloads' chunks (batches of many short ones would take prefill_kernel<128>)."""
-    return "prefill_pair_kernel" if batch.shape.head_dim == 128 else "prefill_kernel<64>"
+    """The kernel of the timed workloads' chunks (batches of many short ones would take prefill_kernel)."""
+    return "prefill_pair_kernel" if batch.shape.head_dim == 128 else "prefill_d64_kernel"
 
 
 def kernel_record(kernel, where, launch_ms, units, peaks, step_ms=None):

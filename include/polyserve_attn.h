@@ -187,7 +187,9 @@ typedef struct {
     int32_t decode_sms;        /* SMs the decode kernel is sized for */
     int32_t prefill_sms;       /* SMs the prefill kernel is sized for; in a mixed batch the two kernels run side by
                                   side on disjoint SMs when that is predicted to be faster (decode_sms + prefill_sms
-                                  = all SMs), otherwise one after the other on all of them */
+                                  = all SMs), otherwise one after the other on all of them.  Decode rows alone that
+                                  hold 0.75 GB of bf16 K/V or more are sized for at most 128 SMs: more ask for more
+                                  than the memory gives */
 } ps_plan_info;
 ps_status ps_plan_get_info(const ps_plan *plan, ps_plan_info *info_out);
 

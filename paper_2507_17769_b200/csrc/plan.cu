@@ -703,11 +703,12 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         }
         pl->dec_sms = pl->pf_sms = pl->num_sms;
         pl->concurrent = false;
-        // Decode rows alone stream a little faster from 128 SMs: all 148 ask for more than HBM gives, and their requests get in each
-        // other's way.  (bf16 cache; a launch on 148 / 128 SMs, us, on four GPUs: 512 rows lognormal 482 / 468, 256 rows of 8000
-        // tokens at 64 heads 1290 / 1230, or 2021 / 2024 for 299 of 11200; 140 of 1700 165 / 161; 256 of 3000 at head dimension 64 250 /
-        // 238; below the line 64 rows, 0.57 GB, 95.0 / 93.6, 32 of 1000 32.6 / 32.3.  Pages of the FP8 cache cost the SMs too much
-        // arithmetic for that.)
+        // Decode rows alone stream a little faster from 128 SMs on most GPUs: all 148 ask for more than HBM gives, and their requests get
+        // in each other's way.  (A number of SMs and no share of them, because it is their requests that count; 136 and 140 are slower
+        // than both.)  The time on 148 SMs over that on 128, both in turn on one GPU, 45 to 81 batches of 0.8 to 19 GB, head dimensions 64
+        // and 128, even, uniform and lognormal contexts, geometric means: 1.032, 1.033, 1.036, 1.031 on four GPUs and 0.975 on a fifth; at
+        // 0.8 GB 1.019 to 1.035 and 0.980, at 19 GB 1.039 to 1.049 and 0.972: no end of the range in sight.  Below the line, 0.4 and
+        // 0.6 GB, 0.99 to 1.01.  Not for the FP8 cache, whose pages cost the SMs too much arithmetic.
         if (pf_steps == 0 && shape->dtype == 0 && dec_bytes >= kDecodeManyBytes) pl->dec_sms = std::min(pl->num_sms, kDecodeAloneSms);
         if (dec_bytes > 0 && pf_steps > 0 && pl->num_sms >= 16) {
             // time models (seconds): decode = bytes / min(side-by-side peak, n * per-SM rate); prefill = steps * step time / m

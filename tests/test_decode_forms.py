@@ -30,3 +30,21 @@ def test_many_short_rows_take_24_warps(rows, ctx, warps):
 @pytest.mark.parametrize("rows,ctx,pages", [(30, 500, 5), (30, 1000, 9), (80, 480, 12)])
 def test_small_units_are_not_rounded_to_whole_stages(rows, ctx, pages):
     assert unit_pages(rows, ctx) == pages
+
+
+@pytest.mark.parametrize("heads,kv_heads,dim,dtype", [(32, 8, 128, 0), (64, 8, 128, 0), (8, 8, 64, 0), (4, 2, 64, 0), (32, 8, 128, 1)])
+@pytest.mark.parametrize("sms,above", [(148, 128), (132, 128), (128, 128), (64, 64)])
+def test_large_batches_of_decode_rows_alone_run_on_128_sms(heads, kv_heads, dim, dtype, sms, above):
+    shape = ps.make_shape(heads, kv_heads, dim, 16, dtype)
+    token = 2 * kv_heads * dim * 2
+    ctx = int(0.75e9 / token / 300)
+
+    def sized(prior, q_len):
+        plan, _ = ps.ps_attn_plan(shape, prior, q_len, (max(prior) + max(q_len) + 15) // 16, ps.ps_plan_opts(0, 0, sms))
+        info = ps.ps_plan_get_info(plan)
+        ps.ps_plan_free(plan)
+        return info.decode_sms
+
+    assert sized([ctx - 1] * 300, [1] * 300) == sms
+    assert sized([ctx] * 300, [1] * 300) == (above if dtype == 0 else sms)
+    assert sized([20 * ctx] * 300, [1] * 300) == (above if dtype == 0 else sms)
