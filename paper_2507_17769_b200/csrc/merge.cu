@@ -11,7 +11,7 @@
 // shuffle, so the rows cost about one round trip to L2 together, after the entry record, which belongs to the run's own list and
 // is read while the kernels before are still running.  (The partial rows are not read-only memory for this kernel: it may be there
 // while the prefill kernel still writes them.  They are ordinary loads, behind the wait.)  Bound by latency: rows of few segments go four to a warp, so that all
-// are under way at once (48 rows and two chunks at head dimension 64, whole iteration, 56.7 -> 55.8 us); rows of more than
+// are under way at once (48 rows and two chunks at head dimension 64, whole iteration, 56.2 -> 55.3 us); rows of more than
 // four segments, of which a batch has few, one to a warp with four segments in flight (100 tokens on 4000, ten segments, four rows
 // a warp with two in flight: 18.5 -> 20.8).
 #include <type_traits>

@@ -56,8 +56,11 @@ struct PrefillModel {
                           // more and a list that has to be uploaded
     int sms_per_worker;   // an item is worked on by one CTA, or by a pair of them
 };
-// prefill.cu (fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile)
-constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 3.0, 1};
+// prefill.cu (fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile).  Its items are never
+// cut: `cut` is how far its queue ends behind an even split at most, for the shares of mixed batches.  (Without it, by the longest item
+// alone: 239 rows of 359 tokens, 60 chunks of 24 and two of 953 and 555 102.7 -> 109.5 us, 40 rows of 2711 and 102 chunks 128.3 -> 135.9; 30
+// drawn mixed batches of many short chunks, geometric mean 1.008.)
+constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 0.0, 1};
 // prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
 // item; the merge kernel takes about 8 us).  Whole items, us, instead of cut ones: 8 items of 10 key tiles 25.9 -> 19.0, of 17
 // 26.9 -> 24.4, 40 of up to 26 35.8 -> 31.7, 16 of 33 35.3 -> 40.7 beside 6 decode rows, 8 of 63 31.2 -> 55.
@@ -731,9 +734,9 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
             // Once the decode rows saturate HBM the modelled time is flat in n; measured step times keep
             // improving a little as the decode kernel gets more SMs, as long as the prefill kernel still ends
-            // well before it.  Take the middle of that flat stretch.  (Not at head dimension 64, where it begins at 92 SMs and
-            // more of them gain nothing: 400 rows of about 1000 tokens and a 1024-token chunk 138.6 us at 88, 140 at 96, 146 at
-            // 112, the middle.)
+            // well before it.  Take the middle of that flat stretch.  (Not at head dimension 64, where it begins at some 84 SMs and
+            // more of them gain nothing: from its beginning / its middle 400 rows of about 1000 tokens and a fresh 1024-token chunk
+            // 133 / 140 us, on 2000 141 / 140, 256 of 2000 and 512 on 1000 166 / 176, 100 of 4000 and 700 on 500 129 / 137.)
             int hi = best_n;
             for (int nd = best_n; shape->head_dim == 128 && nd <= pl->num_sms - 8; nd += 4)
                 if (std::max(t_dec(nd), t_pf(nd)) <= 1.015 * best_t && t_pf(nd) <= 0.8 * t_dec(nd)) hi = nd;

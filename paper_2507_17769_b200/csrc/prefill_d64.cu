@@ -25,6 +25,10 @@
 //     8 q / 8 kv heads, 2048 tokens on 8192  72.6 -> 70.3 -> 61.4 -> 60.4 us      16 / 2  129.5 -> 123.6 -> 108.2 -> 105.9
 //     two chunks of 768 and 1224 on 3600     44.7 -> 42.6 -> 38.4 -> 38.3;  48 decode rows beside them, whole iteration, 65.9 -> 63.1
 // A chunk of 32 tokens on 100 takes 8.7 us instead of 11.3 (launch included).
+// The time depends on the data: an item with a row whose scores lie some 69 above its sample's runs three times.  With N(0, 1) keys
+// (whole run with append, 8/8 and 16/2 heads): 2048 tokens on 8192 64 and 111 us up to scores of standard deviation 8, and 16 at 8/8, 160
+// and 289 from 24 on (with a running maximum, as before, 82 and 145); fresh prompts of 900 to 2000 tokens 35 and 46 up to 16, 83 and 112 from
+// 24 on (49 and 55).
 #include "tcgen05.cuh"
 
 namespace ps {

@@ -1,4 +1,4 @@
-// What the two prefill kernels share: wrappers over the tcgen05 and tensor-map PTX they use, the matrix descriptors
+// What the three prefill kernels share: wrappers over the tcgen05 and tensor-map PTX they use, the matrix descriptors
 // and the tensor maps of Q and the pool.
 #pragma once
 
@@ -10,7 +10,6 @@
 
 namespace ps {
 
-// Q as a [T tokens][Hq heads][D] tensor; a box is one 64-element half of a q tile's 128 (token, head) rows.
 // (entries past the list's end are not read)
 inline void fill_inline_items(const RunArgs& a, InlineItems& inl) {
     if (!a.inline_items) return;
@@ -18,6 +17,7 @@ inline void fill_inline_items(const RunArgs& a, InlineItems& inl) {
     memcpy(inl.start, a.inline_starts, (a.w.n_prefill_ctas + 1) * sizeof(int32_t));
 }
 
+// Q as a [T tokens][Hq heads][D] tensor; a box is one 64-element half of a q tile's 128 (token, head) rows.
 ps_status encode_q_map(const RunArgs& a, CUtensorMap* map);
 // The pool as rows of 2 KB blocks (16 tokens x 64 elements); a box is one row, gathered four at a time.
 constexpr int kPoolBlock = kPage * 128;

@@ -1,5 +1,5 @@
-"""The prefill kernel of head dimension 64 where its own branches can go wrong: q tiles of one to seven key tiles (its score
-buffers, stages and barriers wrap at three, four and four), items of one q tile and of two that see different numbers of key
+"""The prefill kernel of head dimension 64 where its own branches can go wrong: q tiles of one to seven key tiles (its K and V
+stages wrap at four, the phases of its one score tile and one weight tile a q tile at two), items of one q tile and of two that see different numbers of key
 tiles, ragged ends, more items than its record ring holds, cut items of which a q tile sees nothing, and rows whose sums leave
 the range in which weights are taken without their row maximum.  Oracle and bounds: those of the CTA-pair kernel's tests."""
 import numpy as np
