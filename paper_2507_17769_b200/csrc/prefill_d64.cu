@@ -17,7 +17,7 @@
 // when they are done; PV of one tile runs under the softmax of the next.  Weights are relative to a sample of the row's own
 // scores instead of a running maximum, with rows whose sums leave the range run again, as in prefill_pair.cu.
 //
-// What bounds it: a 128-key step of both q tiles takes 2640 cycles, of which the exp2 unit needs 2048.  An mbarrier's answer takes
+// What bounds it: a 128-key step of both q tiles takes some 2700 cycles, of which the exp2 unit needs 2048.  An mbarrier's answer takes
 // a warp some 400 cycles beside those exponentials, whatever it is; so each q tile has an MMA warp of its own, which asks three
 // things a step (K and V land on one barrier, and it is asked together with the scores').
 // Measured (B200, N(0,1) data, kernel alone), before (two score tiles, a running maximum, one MMA warp) -> with one MMA warp and
