@@ -308,19 +308,24 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
 
 // Which form of the decode kernel with a unit per warp takes a batch at head dimension 64: two pages a stage on 12 warps an SM, or one
 // on 24.  A row costs a warp some 2 us beside its pages, so short rows of which a warp has several are done sooner by twice the warps:
-// from 1.2 (row, kv head)s a warp up to 5 pages a row, from 1.5 up to 9, where the smallest units do not leave warps idle anyway.
+// from 1.2 (row, kv head)s a warp up to 5 pages a row, from 1.5 up to 9, from 2 up to 15, where the smallest units do not leave warps idle
+// anyway.
 // Measured (12 warps / 24, us, 8 kv heads, 1 and 4 q heads each, contexts within half of the mean): 512 rows of 28 tokens 20.5 / 18.6,
-// of 40 22.6 / 19.3, of 64 26.1 / 24.3, of 96 30.0 / 30.7, of 128 35.9 / 34.7, of 256 55.5 / 55.3; 350 of 40 19.5 / 18.3, of 64 21.8 / 20.1, of
-// 96 25.2 / 23.6, of 128 28.7 / 28.0, of 192 35.3 / 35.2; 280 of 64 20.3 / 18.6, of 96 21.3 / 22.4, of 192 30.7 / 31.8; 230 of 64 18.5 / 18.4,
-// of 128 21.4 / 22.1; few pages: 512 of 20 16.0 / 16.4, 350 of 28 15.8 / 18.2; 2 kv heads: 512 of 128 18.7 / 19.5.
+// of 40 22.6 / 19.3, of 64 26.1 / 24.3, of 96 30.0 / 30.7, of 128 35.9 / 34.7, of 190 46.6 / 45.0, of 240 52.9 / 51.8, of 256 55.5 / 55.3; 700
+// of 210 62.6 / 61.2, of 240 67.9 / 68.5; 350 of 40 19.5 / 18.3, of 64 21.8 / 20.1, of 96 25.2 / 23.6, of 128 28.7 / 28.0, of 192 35.3 /
+// 35.2; 280 of 64 20.3 / 18.6, of 96 21.3 / 22.4, of 192 30.7 / 31.8; 230 of 64 18.5 / 18.4, of 128 21.4 / 22.1; few pages: 512 of 20
+// 16.0 / 16.4, 350 of 28 15.8 / 18.2; 2 kv heads: 512 of 128 18.7 / 19.5.
+// Twice the warps leave twice the partial rows, up to 15 MB with 8 q heads a kv head: ps_attn_plan() plans again on 12 where the built-in
+// scratch would no longer do.
 static bool one_page_a_stage(const ps_plan& pl, int64_t n_rows, int64_t total_pages) {
     const int64_t warps = (int64_t)pl.dec_sms * decode_unit_warps(64, 2);
     if (total_pages <= kDecodeMinPagesLo * warps) return false;
-    return (n_rows * 5 >= warps * 6 && total_pages <= 5 * n_rows) || (n_rows * 2 >= warps * 3 && total_pages <= 9 * n_rows);
+    return (n_rows * 5 >= warps * 6 && total_pages <= 5 * n_rows) || (n_rows * 2 >= warps * 3 && total_pages <= 9 * n_rows) ||
+           (n_rows >= warps * 2 && total_pages <= 15 * n_rows);
 }
 
 static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,
-                        const ps_plan_opts* opts, int64_t* n_slots) {
+                        const ps_plan_opts* opts, bool may_take_24_warps, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     int64_t total_pages = 0, longest = 0, n_rows = 0;  // (n_rows, total_pages: of all kv heads)
     for (int r = 0; r < pl->n; ++r)
@@ -339,7 +344,7 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     pl->cta_pieces = false;
     pl->info.decode_segment_tokens = 0;
     if (!(opts && opts->decode_segment_tokens > 0) && plan_decode_ctas(pl, prior, q_len, q_start, total_pages, longest, n_slots)) return;
-    pl->dec_pages = pl->shape.head_dim == 64 && !one_page_a_stage(*pl, n_rows, total_pages) ? 2 : 1;
+    pl->dec_pages = pl->shape.head_dim == 64 && !(may_take_24_warps && one_page_a_stage(*pl, n_rows, total_pages)) ? 2 : 1;
     const int64_t min_pages = std::min<int64_t>(kDecodeMinPagesHi, std::max<int64_t>(kDecodeMinPagesLo, (longest + kDecodePiecesPerRow - 1) / kDecodePiecesPerRow));
     int64_t per_unit;
     if (opts && opts->decode_segment_tokens > 0) {
@@ -760,9 +765,33 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         }
     }
     pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
+    const int d = shape->head_dim;
+    // (re)size the slots with headroom: a batch of the next iterations that needs a somewhat longer work list still fits, and the
+    // layout stays put
+    auto stride_for = [](size_t image_bytes) { return align_up(image_bytes + image_bytes / 2, 4096); };
+    auto lay_out_image = [pl]() {
+        size_t off = 256;  // WsHeader
+        pl->off_pieces = off;   off = align_up(off + pl->pieces.size() * sizeof(DecodePiece), 256);
+        pl->off_units = off;    off = align_up(off + pl->units.size() * sizeof(DecodeUnit), 256);
+        pl->off_prefill = off;  off = align_up(off + pl->prefill.size() * sizeof(PrefillItem), 256);
+        pl->off_merge = off;    off = align_up(off + pl->merge.size() * sizeof(MergeEntry), 256);
+        pl->off_dmerge = off;   off = align_up(off + pl->dmerge.size() * sizeof(DecodeMerge), 256);
+        pl->off_dmerge_cnt = off; off = align_up(off + pl->dmerge.size() * sizeof(int32_t), 256);
+        pl->off_cta_start = off; off = align_up(off + pl->prefill_cta_start.size() * sizeof(int32_t), 256);
+        pl->image_bytes = off;
+    };
     int64_t n_slots = 0;
-    plan_decode(pl, prior_host, q_len_host, q_start, opts, &n_slots);
     plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);
+    const int64_t prefill_slots = n_slots;
+    plan_decode(pl, prior_host, q_len_host, q_start, opts, true, &n_slots);
+    lay_out_image();
+    const size_t need = 2 * std::max(pl->slot_stride, pl->image_bytes > pl->slot_stride ? stride_for(pl->image_bytes) : 0) + (size_t)n_slots * (d + 1) * sizeof(float) + 512;
+    if (d == 64 && !pl->cta_pieces && pl->dec_pages == 1 && need > PS_STATIC_WORKSPACE_BYTES) {
+        n_slots = prefill_slots;
+        pl->decode_merge_rows = 0;
+        plan_decode(pl, prior_host, q_len_host, q_start, opts, false, &n_slots);
+        lay_out_image();
+    }
     pl->inline_list = (pl->pieces.empty() || (pl->cta_pieces && pl->dmerge.empty() && pl->pieces.size() <= kInlinePieces)) &&
                       (pl->prefill.empty() || (pl->prefill.size() <= kInlineItems && pl->merge.empty() && !pl->prefill_cta_start.empty() &&
                                                pl->prefill_cta_start.size() <= kInlineStarts));
@@ -771,23 +800,11 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         return fail(PS_ERR_UNSUPPORTED, "partial buffer would need %lld slots", (long long)n_slots);
     }
 
-    const int d = shape->head_dim;
-    size_t off = 256;  // WsHeader
-    pl->off_pieces = off;   off = align_up(off + pl->pieces.size() * sizeof(DecodePiece), 256);
-    pl->off_units = off;    off = align_up(off + pl->units.size() * sizeof(DecodeUnit), 256);
-    pl->off_prefill = off;  off = align_up(off + pl->prefill.size() * sizeof(PrefillItem), 256);
-    pl->off_merge = off;    off = align_up(off + pl->merge.size() * sizeof(MergeEntry), 256);
-    pl->off_dmerge = off;   off = align_up(off + pl->dmerge.size() * sizeof(DecodeMerge), 256);
-    pl->off_dmerge_cnt = off; off = align_up(off + pl->dmerge.size() * sizeof(int32_t), 256);
-    pl->off_cta_start = off; off = align_up(off + pl->prefill_cta_start.size() * sizeof(int32_t), 256);
-    pl->image_bytes = off;
     if (pl->image_bytes > pl->slot_stride) {
-        // (re)size the slots with headroom: a batch of the next iterations that needs a somewhat longer work list
-        // still fits, and the layout stays put
-        pl->slot_stride = align_up(pl->image_bytes + pl->image_bytes / 2, 4096);
+        pl->slot_stride = stride_for(pl->image_bytes);
         pl->layout_moved = true;
     }
-    off = 2 * pl->slot_stride;  // two image slots
+    size_t off = 2 * pl->slot_stride;  // two image slots
     pl->off_part_lse = off; off = align_up(off + (size_t)n_slots * sizeof(float), 256);
     pl->off_part_o = off;   off = align_up(off + (size_t)n_slots * d * sizeof(float), 256);
     pl->ws_bytes = off;

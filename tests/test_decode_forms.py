@@ -17,7 +17,8 @@ def unit_pages(rows, ctx, kv_heads=8, group=1, sms=148):
 
 
 @pytest.mark.parametrize("rows,ctx,warps", [
-    (512, 40, 24), (512, 144, 24), (512, 145, 12),  # nine pages a row, ten
+    (512, 40, 24), (512, 240, 24), (512, 241, 12),  # 15 pages a row, 16
+    (444, 240, 24), (443, 240, 12), (443, 144, 24), (443, 145, 12),  # two rows a warp, nine pages a row, ten
     (267, 80, 24), (266, 80, 12), (267, 81, 12),     # 1.2 rows a warp, five pages a row, six
     (333, 96, 24), (332, 96, 12),                   # 1.5 rows a warp
 ])
@@ -25,6 +26,19 @@ def test_many_short_rows_take_24_warps(rows, ctx, warps):
     pages = rows * 8 * ((ctx + 15) // 16)
     share = -(-pages // (148 * warps))
     assert unit_pages(rows, ctx) in ((max(4, share),) if warps == 24 else (max(4, share), max(4, share) + 1))
+
+
+@pytest.mark.parametrize("rows,ctx", [(500, 130), (600, 128), (950, 114), (1100, 210)])
+def test_24_warps_are_not_taken_beyond_the_built_in_scratch(rows, ctx):
+    """Eight q heads a kv head: the partial rows of 24 warps would need more than ps_attn_run_static has, those of 12 do not."""
+    shape = ps.make_shape(64, 8, 64)
+    plan, need = ps.ps_attn_plan(shape, np.full(rows, ctx - 1), np.ones(rows, dtype=np.int32), (ctx + 15) // 16, ps.ps_plan_opts(0, 0, 148))
+    items = ps.ps_plan_get_items(plan)[0]
+    slots = items[items[:, 6] >= 0, 6]
+    ps.ps_plan_free(plan)
+    assert need <= ps.PS_STATIC_WORKSPACE_BYTES
+    assert len(set(slots.tolist())) == len(slots)
+    assert unit_pages(rows, ctx, group=8) > unit_pages(rows, ctx, group=1)
 
 
 @pytest.mark.parametrize("rows,ctx,pages", [(30, 500, 5), (30, 1000, 9), (80, 480, 12)])
