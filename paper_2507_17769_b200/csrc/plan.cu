@@ -52,22 +52,27 @@ struct PrefillModel {
     double fixed;         // steps an item costs beyond its key tiles
     double masked_extra;  // and the diagonal tile's slower softmax
     double cut;           // steps that cutting items costs: partial rows, merge kernel
-    double whole;         // steps by which whole items may end later than an even split: what cutting costs a small batch, a kernel
-                          // more and a list that has to be uploaded
+    // Steps by which whole items may end later than an even split: what cutting costs a small batch, a kernel more and a list that has
+    // to be uploaded.  Of up to kFewItems items, whose merge is quick; of more.
+    double whole_few, whole;
     int sms_per_worker;   // an item is worked on by one CTA, or by a pair of them
 };
 // prefill.cu (fitted to per-CTA run times: 2.2 us per step, about 3 us per item, 1.2 us more for a masked tile).  Its items are never
 // cut: `cut` is how far its queue ends behind an even split at most, for the shares of mixed batches.  (Without it, by the longest item
 // alone: 239 rows of 359 tokens, 60 chunks of 24 and two of 953 and 555 102.7 -> 109.5 us, 40 rows of 2711 and 102 chunks 128.3 -> 135.9; 30
 // drawn mixed batches of many short chunks, geometric mean 1.008.)
-constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 0.0, 1};
+constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 0.0, 0.0, 1};
 // prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
-// item; the merge kernel takes about 8 us).  Whole items, us, instead of cut ones: 8 items of 10 key tiles 25.9 -> 19.0, of 17
-// 26.9 -> 24.4, 40 of up to 26 35.8 -> 31.7, 16 of 33 35.3 -> 40.7 beside 6 decode rows, 8 of 63 31.2 -> 55.
-constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 20.0, 2};
+// item; the merge kernel takes about 8 us).  A run with append, us, whole / cut, by the steps that whole items end later: 2 to 10 items
+// 12 steps 15 to 26 / 3 to 10 % more, 14 steps 21 / 20.5 to 21.4, 16 steps 23.2 / 22.6, 20 steps 24.9 / 20.7; 16 items 16.5 steps 2 to 3 % less
+// than cut, 18.8 steps the same; 24 items 17.9 steps 3 % less, 19.6 steps 3 % more; 32 items 16 steps 12 % less, 18.4 steps 2 %; 80 to 168
+// items 18.9 steps 2 % less, 19.1 steps 1 % more.
+constexpr int kFewItems = 12;
+constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 14.0, 18.5, 2};
 // prefill_d64.cu (148 CTAs of 1 to 3 items of 6 to 29 key tiles, beside a decode kernel: 9.4 us a CTA, 3.1 an item, 1.28 a step; the
-// merge kernel and the gap before it 7.5 us).  Whole items instead of cut ones: 8 of 10 key tiles 22.4 -> 18.4, of 17 22.1 -> 26.1.
-constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 10.0, 1};
+// merge kernel and the gap before it 7.5 us).  Whole / cut: 4 to 20 items 7.3 steps 1 to 20 % less, 8.2 steps 12 % less to 8 % more, 9.3
+// steps 5 % less to 11 % more.
+constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 8.0, 8.0, 1};
 static inline const PrefillModel& prefill_model(const ps_shape& sh, bool pairs) { return sh.head_dim == 64 ? kD64Model : pairs ? kPairModel : kSingleModel; }
 // Which kernel runs the prefill items.  Head dimension 64: a CTA per item.  128: a pair of CTAs, unless the items are short and
 // there are enough for all SMs.  An item costs a CTA 3.5 us and 2.2 more a key tile, a pair 3.2 us and 0.73, so up to some
@@ -502,9 +507,10 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 makespan = std::max(makespan, least.first);
                 std::push_heap(heap.begin(), heap.end(), std::greater<Slot>());
             }
+            const double whole = (int64_t)tiles.size() <= kFewItems ? cost.whole_few : cost.whole;
             // (cutting is not free either, and from four items a worker on it has less to gain than the partial rows cost in
             // space, 19 MB in a batch that needs none)
-            if ((int64_t)tiles.size() >= 4LL * pl->pf_workers || makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + cost.whole)) {
+            if ((int64_t)tiles.size() >= 4LL * pl->pf_workers || makespan <= std::max(kPrefillWholeItemSlack * total / n_cta, total / n_cta + whole)) {
                 for (int c = 0; c < n_cta; ++c) count[c + 1] += count[c];
                 pl->prefill_cta_start.assign(count.begin(), count.end());
                 std::vector<Tile> sorted(tiles.size());

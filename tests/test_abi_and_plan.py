@@ -343,3 +343,17 @@ def test_items_enough_for_a_queue_are_never_cut(d, n):
         assert info.n_prefill_items == 8 * n and info.n_partial_slots == 0 and ws <= ps.PS_STATIC_WORKSPACE_BYTES
     finally:
         ps.ps_plan_free(plan)
+
+
+@pytest.mark.parametrize("heads,kv_heads,d,chunk,last_whole", [
+    (32, 8, 128, 39, 14 * 128 - 39),  # eight items: 14 key tiles, 15
+])
+def test_short_items_stay_whole(heads, kv_heads, d, chunk, last_whole):
+    """A few items that end some key tiles later than an even split are not cut; later than that the merge kernel is worth it."""
+    for prior, launches in ((last_whole, 1), (last_whole + 1, 2)):
+        plan, _ = ps.ps_attn_plan(ps.make_shape(heads, kv_heads, d), np.array([prior], np.int32), np.array([chunk], np.int32), 2048, opts())
+        try:
+            info = ps.ps_plan_get_info(plan)
+            assert info.n_launches == launches and (info.n_prefill_items == kv_heads) == (launches == 1)
+        finally:
+            ps.ps_plan_free(plan)
