@@ -70,9 +70,21 @@ constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 0.0, 0.0, 1};
 constexpr int kFewItems = 12;
 constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 14.0, 18.5, 2};
 // prefill_d64.cu (148 CTAs of 1 to 3 items of 6 to 29 key tiles, beside a decode kernel: 9.4 us a CTA, 3.1 an item, 1.28 a step; the
-// merge kernel and the gap before it 7.5 us).  Whole / cut: 4 to 20 items 7.3 steps 1 to 20 % less, 8.2 steps 12 % less to 8 % more, 9.3
-// steps 5 % less to 11 % more.
-constexpr PrefillModel kD64Model = {1.28e-6, 2.0, 0.4, 6.0, 8.0, 8.0, 1};
+// merge kernel and the gap before it 7.5 us).  An item's 3.1 us are 2.4 steps; as 2, so that a smallest share holds two whole key tiles,
+// batches with cut items are 4 % faster: 256 tokens on 1500, 4 / 2 heads, 22.7 -> 20.4 us, 64 on 3000 18.3 -> 16.5, 700 and 300 on 1500 at 8 / 8
+// 26.4 -> 24.7 (30 batches; as 1.5 they gain as much, mixed batches lose).  Whole / cut: 4 to 20 items 7.3 steps 1 to 20 % less, 8.2 steps
+// 12 % less to 8 % more, 9.3 steps 5 % less to 11 % more.
+constexpr PrefillModel kD64Model = {1.28e-6, 1.5, 0.5, 6.0, 8.0, 8.0, 1};
+// An item's cost at head dimension 64 as measured, by which the SMs of mixed batches are shared out.
+static inline PrefillModel measured_model(const ps_shape& sh, PrefillModel m) {
+    if (sh.head_dim == 64) m.fixed = 2.0, m.masked_extra = 0.4;
+    return m;
+}
+// For plans that leave fewer partial rows, at the limit of the built-in scratch (ps_attn_plan()): items stay whole up to later ends, too.
+static inline PrefillModel lean_model(const ps_shape& sh, PrefillModel m) {
+    m.whole_few = m.whole = sh.head_dim == 64 ? 10.0 : 20.0;
+    return measured_model(sh, m);
+}
 static inline const PrefillModel& prefill_model(const ps_shape& sh, bool pairs) { return sh.head_dim == 64 ? kD64Model : pairs ? kPairModel : kSingleModel; }
 // Which kernel runs the prefill items.  Head dimension 64: a CTA per item.  128: a pair of CTAs, unless the items are short and
 // there are enough for all SMs.  An item costs a CTA 3.5 us and 2.2 more a key tile, a pair 3.2 us and 0.73, so up to some
@@ -193,6 +205,7 @@ struct ps_plan {
     bool pairs = false;      // prefill items go to CTA pairs
     int32_t pf_workers = 0;  // what they are handed to: CTAs, or CTA pairs (one SM each)
     bool concurrent = false;
+    bool cut_by_choice = false;  // prefill items are cut that a lean plan might leave whole
     bool tiny_as_rows = false;  // this batch runs its chunks of a few tokens as decode rows
     std::vector<DecodePiece> pieces;
     std::vector<DecodeUnit> units;
@@ -320,17 +333,18 @@ static bool plan_decode_ctas(ps_plan* pl, const int32_t* prior, const int32_t* q
 // of 210 62.6 / 61.2, of 240 67.9 / 68.5; 350 of 40 19.5 / 18.3, of 64 21.8 / 20.1, of 96 25.2 / 23.6, of 128 28.7 / 28.0, of 192 35.3 /
 // 35.2; 280 of 64 20.3 / 18.6, of 96 21.3 / 22.4, of 192 30.7 / 31.8; 230 of 64 18.5 / 18.4, of 128 21.4 / 22.1; few pages: 512 of 20
 // 16.0 / 16.4, 350 of 28 15.8 / 18.2; 2 kv heads: 512 of 128 18.7 / 19.5.
-// Twice the warps leave twice the partial rows, up to 15 MB with 8 q heads a kv head: ps_attn_plan() plans again on 12 where the built-in
-// scratch would no longer do.
 static bool one_page_a_stage(const ps_plan& pl, int64_t n_rows, int64_t total_pages) {
     const int64_t warps = (int64_t)pl.dec_sms * decode_unit_warps(64, 2);
     if (total_pages <= kDecodeMinPagesLo * warps) return false;
+    // (twice the warps leave twice the partial rows, two a unit and q head at most: not where the built-in scratch might no longer do)
+    const int64_t units = 2 * warps, G = pl.shape.n_q_heads / pl.shape.n_kv_heads;
+    if (2 * units * G * 65 * 4 + 3 * (n_rows + 2 * units) * (int64_t)sizeof(DecodePiece) > PS_STATIC_WORKSPACE_BYTES) return false;
     return (n_rows * 5 >= warps * 6 && total_pages <= 5 * n_rows) || (n_rows * 2 >= warps * 3 && total_pages <= 9 * n_rows) ||
            (n_rows >= warps * 2 && total_pages <= 15 * n_rows);
 }
 
 static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,
-                        const ps_plan_opts* opts, bool may_take_24_warps, int64_t* n_slots) {
+                        const ps_plan_opts* opts, bool lean, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     int64_t total_pages = 0, longest = 0, n_rows = 0;  // (n_rows, total_pages: of all kv heads)
     for (int r = 0; r < pl->n; ++r)
@@ -349,7 +363,7 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
     pl->cta_pieces = false;
     pl->info.decode_segment_tokens = 0;
     if (!(opts && opts->decode_segment_tokens > 0) && plan_decode_ctas(pl, prior, q_len, q_start, total_pages, longest, n_slots)) return;
-    pl->dec_pages = pl->shape.head_dim == 64 && !(may_take_24_warps && one_page_a_stage(*pl, n_rows, total_pages)) ? 2 : 1;
+    pl->dec_pages = pl->shape.head_dim == 64 && (lean || !one_page_a_stage(*pl, n_rows, total_pages)) ? 2 : 1;
     const int64_t min_pages = std::min<int64_t>(kDecodeMinPagesHi, std::max<int64_t>(kDecodeMinPagesLo, (longest + kDecodePiecesPerRow - 1) / kDecodePiecesPerRow));
     int64_t per_unit;
     if (opts && opts->decode_segment_tokens > 0) {
@@ -359,7 +373,7 @@ static void plan_decode(ps_plan* pl, const int32_t* prior, const int32_t* q_len,
         per_unit = std::max<int64_t>(min_pages, (total_pages + target - 1) / target);
         // With two pages a stage a unit's last stage should be full, but not at the price of a tenth of its pages more: 30 rows of 500 tokens,
         // 8 kv heads, with 6 pages instead of 5 19.1 us, 16.9; of 900, 10 instead of 9, 20.5, 18.7; 80 of 500, 12 instead of 11, 21.1, 22.2.
-        if (pl->dec_pages == 2 && per_unit > 10) per_unit += per_unit & 1;
+        if (pl->dec_pages == 2 && (lean || per_unit > 10)) per_unit += per_unit & 1;
     }
     pl->info.decode_segment_tokens = (int32_t)(per_unit * kPage);
 
@@ -429,10 +443,11 @@ constexpr double kPrefillWholeItemSlack = 1.12;  // uncut items are taken if the
 constexpr double kPrefillMinCtaCost = 4.0;  // do not spread the work thinner than this per CTA (two key tiles)
 
 static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len, const std::vector<int32_t>& q_start,
-                         const ps_plan_opts* opts, int64_t* n_slots) {
+                         const ps_plan_opts* opts, bool lean, int64_t* n_slots) {
     const int Hkv = pl->shape.n_kv_heads, G = pl->shape.n_q_heads / Hkv;
     const int tile_tok = kPrefillRowsPerItem / G;
-    const PrefillModel& cost = prefill_model(pl->shape, pl->pairs);
+    const PrefillModel usual = prefill_model(pl->shape, pl->pairs), lean_cost = lean_model(pl->shape, usual), &cost = lean ? lean_cost : usual;
+    pl->cut_by_choice = false;
     struct Tile { int r, g, tok0, n_tok, first_pos, key_tiles; };
     std::vector<Tile> tiles;
     size_t n_tiles = 0;
@@ -483,7 +498,7 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
         for (const Tile& t : tiles) total += cost.fixed + t.key_tiles + cost.masked_extra;
         // (No two items on one CTA while another has none: two fresh items of one key tile, 16 q / 2 kv heads of 64, 14.1 us on one
         // CTA, 9.7 on two; 56 items of 1 and 2 key tiles 15.2 on 50 CTAs, 12.0 on 56.)
-        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_workers, std::max<double>((double)tiles.size(), total / kPrefillMinCtaCost)));
+        const int n_cta = (int)std::max<double>(1, std::min<double>(pl->pf_workers, std::max<double>(lean ? 0 : (double)tiles.size(), total / kPrefillMinCtaCost)));
         // Many short items (fresh prompts): whole items, longest first, each to the CTA with the least work so far.
         // If that comes within kPrefillWholeItemSlack of an even split, nothing is cut: no partial rows, no merge
         // kernel, no item paying its fixed cost twice.
@@ -517,6 +532,8 @@ static void plan_prefill(ps_plan* pl, const int32_t* prior, const int32_t* q_len
                 for (int i : order) sorted[(size_t)count[owner[i]]++] = tiles[i];  // each CTA's items longest first
                 tiles.swap(sorted);
                 whole_items = true;
+            } else {
+                pl->cut_by_choice = makespan <= total / n_cta + lean_cost.whole + 1 || (int64_t)tiles.size() * 4 >= 15LL * pl->pf_workers;
             }
         }
         if (!whole_items) {
@@ -700,7 +717,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         double longest = 0;                  // steps of the longest prefill item
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
         const int G = shape->n_q_heads / shape->n_kv_heads;
-        const PrefillModel& cost = prefill_model(pl->shape, pl->pairs);
+        const PrefillModel cost = measured_model(pl->shape, prefill_model(pl->shape, pl->pairs));
         const int tile_tok = kPrefillRowsPerItem / G;
         for (int r = 0; r < n; ++r) {
             if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) {
@@ -769,8 +786,8 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
                 pl->concurrent = true;
             }
         }
+        pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
     }
-    pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
     const int d = shape->head_dim;
     // (re)size the slots with headroom: a batch of the next iterations that needs a somewhat longer work list still fits, and the
     // layout stays put
@@ -787,17 +804,21 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
         pl->image_bytes = off;
     };
     int64_t n_slots = 0;
-    plan_prefill(pl, prior_host, q_len_host, q_start, opts, &n_slots);
-    const int64_t prefill_slots = n_slots;
-    plan_decode(pl, prior_host, q_len_host, q_start, opts, true, &n_slots);
-    lay_out_image();
-    const size_t need = 2 * std::max(pl->slot_stride, pl->image_bytes > pl->slot_stride ? stride_for(pl->image_bytes) : 0) + (size_t)n_slots * (d + 1) * sizeof(float) + 512;
-    if (d == 64 && !pl->cta_pieces && pl->dec_pages == 1 && need > PS_STATIC_WORKSPACE_BYTES) {
-        n_slots = prefill_slots;
+    auto plan_items = [&](bool lean) {
+        pl->prefill.clear();
+        pl->merge.clear();
         pl->decode_merge_rows = 0;
-        plan_decode(pl, prior_host, q_len_host, q_start, opts, false, &n_slots);
+        n_slots = 0;
+        plan_decode(pl, prior_host, q_len_host, q_start, opts, lean, &n_slots);
+        plan_prefill(pl, prior_host, q_len_host, q_start, opts, lean, &n_slots);
         lay_out_image();
-    }
+        return 2 * std::max(pl->slot_stride, pl->image_bytes > pl->slot_stride ? stride_for(pl->image_bytes) : 0) + (size_t)n_slots * (d + 1) * sizeof(float) + 512;
+    };
+    // Items that are cut because their merge is quick, and twice the decode warps beside cut items, leave more partial rows: where the
+    // built-in scratch would no longer do because of them, the batch is planned with fewer.
+    const size_t need = plan_items(false);
+    const bool twice_the_warps = d == 64 && !pl->units.empty() && pl->dec_pages == 1 && !pl->merge.empty();
+    if (need > PS_STATIC_WORKSPACE_BYTES && (twice_the_warps || pl->cut_by_choice || (d == 64 && need <= PS_STATIC_WORKSPACE_BYTES / 10 * 11))) plan_items(true);
     pl->inline_list = (pl->pieces.empty() || (pl->cta_pieces && pl->dmerge.empty() && pl->pieces.size() <= kInlinePieces)) &&
                       (pl->prefill.empty() || (pl->prefill.size() <= kInlineItems && pl->merge.empty() && !pl->prefill_cta_start.empty() &&
                                                pl->prefill_cta_start.size() <= kInlineStarts));

@@ -347,6 +347,8 @@ def test_items_enough_for_a_queue_are_never_cut(d, n):
 
 @pytest.mark.parametrize("heads,kv_heads,d,chunk,last_whole", [
     (32, 8, 128, 39, 14 * 128 - 39),  # eight items: 14 key tiles, 15
+    (8, 8, 64, 39, 10 * 128 - 39),    # 10, 11
+    (4, 2, 64, 100, 10 * 128 - 100),
 ])
 def test_short_items_stay_whole(heads, kv_heads, d, chunk, last_whole):
     """A few items that end some key tiles later than an even split are not cut; later than that the merge kernel is worth it."""
@@ -354,6 +356,6 @@ def test_short_items_stay_whole(heads, kv_heads, d, chunk, last_whole):
         plan, _ = ps.ps_attn_plan(ps.make_shape(heads, kv_heads, d), np.array([prior], np.int32), np.array([chunk], np.int32), 2048, opts())
         try:
             info = ps.ps_plan_get_info(plan)
-            assert info.n_launches == launches and (info.n_prefill_items == kv_heads) == (launches == 1)
+            assert info.n_launches == launches and (info.n_partial_slots == 0) == (launches == 1)
         finally:
             ps.ps_plan_free(plan)
