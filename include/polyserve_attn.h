@@ -224,9 +224,10 @@ ps_status ps_plan_get_items(const ps_plan *plan, int32_t *decode_items_out, int6
  * run under the previous run's kernels), then the prefill, decode and merge
  * kernels run; for a batch with both row classes the prefill kernel may run
  * beside the decode kernel on disjoint SMs, launched when that one has begun
- * and ending after it.  (Long batches whose prefill items are queued, runs
- * that record events and captured ones put the decode kernel on a second
- * stream of the plan instead, which is joined back into `stream` before the
+ * and ending after it.  (Long batches whose prefill items are queued,
+ * batches with cut items whose decode rows take longer, runs that record
+ * events and captured ones put the decode kernel on a second stream of the
+ * plan instead, which is joined back into `stream` before the
  * call's work is complete in stream order.)
  * Small batches (at most 148 decode pieces and 64 prefill items, none of them
  * cut) differ: their work list travels with the kernels' parameters, nothing

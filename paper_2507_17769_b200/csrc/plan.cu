@@ -42,6 +42,7 @@ constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a
 static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 88e9; }
 static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;
+constexpr double kMergeUnderDecodeSec = 3e-6;
 constexpr double kDecodeManyBytes = 0.75e9;
 constexpr int kDecodeAloneSms = 128;
 
@@ -205,6 +206,7 @@ struct ps_plan {
     bool pairs = false;      // prefill items go to CTA pairs
     int32_t pf_workers = 0;  // what they are handed to: CTAs, or CTA pairs (one SM each)
     bool concurrent = false;
+    bool decode_last = false;    // side by side, the decode kernel is predicted to end well after the prefill kernel
     bool cut_by_choice = false;  // prefill items are cut that a lean plan might leave whole
     bool tiny_as_rows = false;  // this batch runs its chunks of a few tokens as decode rows
     std::vector<DecodePiece> pieces;
@@ -733,7 +735,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
             }
         }
         pl->dec_sms = pl->pf_sms = pl->num_sms;
-        pl->concurrent = false;
+        pl->concurrent = pl->decode_last = false;
         // Decode rows alone stream a little faster from 128 SMs on most GPUs: all 148 ask for more than HBM gives, and their requests get
         // in each other's way.  (A number of SMs and no share of them, because it is their requests that count; 136 and 140 are slower
         // than both.)  The time on 148 SMs over that on 128, both in turn on one GPU, 45 to 81 batches of 0.8 to 19 GB, head dimensions 64
@@ -784,6 +786,7 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
                 pl->dec_sms = best_n;
                 pl->pf_sms = pl->num_sms - best_n;
                 pl->concurrent = true;
+                pl->decode_last = t_dec(best_n) - t_pf(best_n) >= kMergeUnderDecodeSec;
             }
         }
         pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
@@ -1077,15 +1080,16 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
     bool merged = false;  // the merge kernel has been launched already
     // dynamic item queue with more items than workers: the decode kernel's SMs help once it has ended
     const bool helpers = a.w.n_prefill_ctas == 0 && a.w.n_prefill > pl->pf_workers;
-    if (pl->concurrent && !(rec && pl->side_stream) && (as_params || (!capturing && !helpers))) {
+    if (pl->concurrent && !(rec && pl->side_stream) && (as_params || (!capturing && !helpers && !(pl->decode_last && a.w.n_merge > 0)))) {
         // Mixed batch: both kernels on the caller's stream, the prefill kernel launched as soon as the decode kernel has begun and
         // waiting for its end only at its own, and the merge kernel behind both.  (A second stream costs two events, which take
         // some 3 us each between kernels: tiny mixed batch 22.5 -> 16.8 us, with the list as parameters; 32 rows of 2048 tokens
-        // beside a 512-token chunk 58.1 -> 57.2.  On a second stream the merge kernel could run while the decode kernel still
-        // does, which is worth no more than that even where it does for long: 200 rows of 2500 tokens and 40 on 8000 338 -> 330;
-        // where it ends first, 6 rows of 1500 and 500 on 1500 at head dimension 64 36.1 -> 29.0, 48 rows and two chunks 62.9 ->
-        // 57.5.  Helpers have to start as soon as the decode kernel ends, so batches with a queue keep the second stream.  So do
-        // runs that record events: one between the two launches would hold the prefill kernel back until the decode kernel's end.)
+        // beside a 512-token chunk 58.1 -> 57.2.)  On a second stream the merge kernel runs while the decode kernel still does: worth
+        // more where that one ends last by 3 us and more (60 rows of 2500 tokens and 300 on 5000 114.2 / 107.7, 150 of 1500 and 300 on 5000
+        // at 8 q / 2 kv heads 52.3 / 49.1, at head dimension 64 88.1 / 83.8; 58 batches 2 to 8 %), less where it does not (3 rows and 300 on
+        // 5000 30.9 / 34.7, at head dimension 64 24.7 / 28.7; 200 batches up to 20 %).  Helpers have to start as soon as the decode kernel
+        // ends, so batches with a queue keep the second stream.  So do runs that record events: one between the two launches would hold
+        // the prefill kernel back until the decode kernel's end.
         RunArgs ad = a;
         ad.sm_pairs = pl->pf_workers < pl->pf_sms;
         if (rec) cudaEventRecord(ev[2], s);  // (without a second stream the kernels follow one another)

@@ -33,10 +33,12 @@ def test_segments(shape, segments):
     (gen.Shape(8, 8, 64), [900] * 20 + [2100, 700], [1] * 20 + [300, 500]),
     (gen.Shape(8, 8, 64), [900] * 24 + [2500], [1] * 24 + [200]),
     (gen.Shape(8, 2, 128), [1999] * 30 + [6000], [1] * 30 + [300]),
-], ids=["d64-118-items", "d64-48-items", "d128"])
+    (gen.Shape(8, 2, 128), [2499] * 60 + [3000], [1] * 60 + [200]),  # (the decode kernel ends last: merged under it)
+    (gen.Shape(4, 2, 64), [1499] * 150 + [5000], [1] * 150 + [300]),
+], ids=["d64-118-items", "d64-48-items", "d128", "d128-decode-last", "d64-decode-last"])
 def test_mixed_batches_with_cut_items_back_to_back(shape, prior, q_len):
-    """Decode, prefill and merge kernel on one stream, each launched while the one before it runs, for queries that change from run to
-    run: bit for bit what a run gives whose kernels are recorded (decode kernel on a second stream) and one replayed from a graph."""
+    """Decode, prefill and merge kernel on one stream, each launched while the one before it runs, or on two, for queries that change from
+    run to run: bit for bit what a run gives whose kernels are recorded (decode kernel on a second stream) and one replayed from a graph."""
     import torch
     from workloads.device import DeviceBatch
 
