@@ -42,7 +42,9 @@ constexpr double kDecodeSharedPeakBytesPerSec = 6.0e12;  // decode rows beside a
 static inline double decode_alone_rate_per_sm(const ps_shape& sh) { return sh.head_dim == 128 ? 135e9 : 88e9; }
 static inline double decode_rate_per_sm(const ps_shape& sh) { return 0.85 * decode_alone_rate_per_sm(sh); }
 constexpr double kKernelFloorSec = 12e-6;
-constexpr double kMergeUnderDecodeSec = 3e-6;
+// The merge kernel runs under the decode kernel where that is predicted to end this much after the prefill kernel (ps_attn_run()), with what
+// a warp spends on each of its rows beside their pages, and on each segment of a row when it combines them.
+constexpr double kMergeUnderDecodeSec = 2.5e-6, kRowSec = 2e-6, kSegmentSec = 0.09e-6;
 constexpr double kDecodeManyBytes = 0.75e9;
 constexpr int kDecodeAloneSms = 128;
 
@@ -64,17 +66,18 @@ struct PrefillModel {
 // drawn mixed batches of many short chunks, geometric mean 1.008.)
 constexpr PrefillModel kSingleModel = {2.5e-6, 1.5, 0.5, 3.0, 0.0, 0.0, 1};
 // prefill_pair.cu (72, 144 and 288 equal items on 74 pairs with 11 to 67 key tiles: 0.70 us per step of a pair, 2.8 us per
-// item; the merge kernel takes about 8 us).  A run with append, us, whole / cut, by the steps that whole items end later: 2 to 10 items
-// 12 steps 15 to 26 / 3 to 10 % more, 14 steps 21 / 20.5 to 21.4, 16 steps 23.2 / 22.6, 20 steps 24.9 / 20.7; 16 items 16.5 steps 2 to 3 % less
-// than cut, 18.8 steps the same; 24 items 17.9 steps 3 % less, 19.6 steps 3 % more; 32 items 16 steps 12 % less, 18.4 steps 2 %; 80 to 168
-// items 18.9 steps 2 % less, 19.1 steps 1 % more.
+// item; the merge kernel takes about 8 us).  Cut instead of whole, a run with append, by the steps that whole items end later: 2 to 10
+// items 12 steps 3 to 10 % longer, 14 steps 2 % shorter to 2 % longer, 16 steps 3 % shorter, 19 steps 8 %, 20 steps 13 to 17 % (24.9 -> 20.7 us);
+// 16 items 16.5 steps 2 to 3 % longer, 18.8 steps the same; 24 items 17.9 steps 3 % longer, 19.6 steps 3 % shorter; 32 items 16 steps 12 %
+// longer, 18.4 steps 2 %; 80 to 168 items 18.9 steps 2 % longer, 19.1 steps 1 % shorter.
 constexpr int kFewItems = 12;
 constexpr PrefillModel kPairModel = {1.45e-6, 3.5, 0.5, 9.0, 14.0, 18.5, 2};
 // prefill_d64.cu (148 CTAs of 1 to 3 items of 6 to 29 key tiles, beside a decode kernel: 9.4 us a CTA, 3.1 an item, 1.28 a step; the
 // merge kernel and the gap before it 7.5 us).  An item's 3.1 us are 2.4 steps; as 2, so that a smallest share holds two whole key tiles,
-// batches with cut items are 4 % faster: 256 tokens on 1500, 4 / 2 heads, 22.7 -> 20.4 us, 64 on 3000 18.3 -> 16.5, 700 and 300 on 1500 at 8 / 8
-// 26.4 -> 24.7 (30 batches; as 1.5 they gain as much, mixed batches lose).  Whole / cut: 4 to 20 items 7.3 steps 1 to 20 % less, 8.2 steps
-// 12 % less to 8 % more, 9.3 steps 5 % less to 11 % more.
+// 30 batches with cut items are 4 % faster: 256 tokens on 1500, 4 / 2 heads, 22.7 -> 20.4 us, 64 on 3000 18.3 -> 16.5, 700 and 300 on 1500
+// at 8 / 8 26.4 -> 24.7.  Cut instead of whole, before that: 4 to 20 items 6.9 steps 1 to 40 % longer, 7.9 steps 8 % shorter to 12 % longer, 8.9
+// steps 11 % shorter to 5 % longer; now with a line of 7.5 instead of 8 items of ten key tiles 3 to 12 % longer (1633 and 1051 fresh
+// tokens beside 23 rows 29.5 -> 33.3) or 3 % shorter.
 constexpr PrefillModel kD64Model = {1.28e-6, 1.5, 0.5, 6.0, 8.0, 8.0, 1};
 // An item's cost at head dimension 64 as measured, by which the SMs of mixed batches are shared out.
 static inline PrefillModel measured_model(const ps_shape& sh, PrefillModel m) {
@@ -718,11 +721,13 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
     {
         double longest = 0;                  // steps of the longest prefill item
         double dec_bytes = 0, pf_steps = 0;  // KV bytes the decode rows stream; key-tile steps of the prefill items
+        double dec_rows = 0;                 // (row, kv head)s
         const int G = shape->n_q_heads / shape->n_kv_heads;
         const PrefillModel cost = measured_model(pl->shape, prefill_model(pl->shape, pl->pairs));
         const int tile_tok = kPrefillRowsPerItem / G;
         for (int r = 0; r < n; ++r) {
             if (runs_as_decode(*shape, pl->tiny_as_rows, prior_host[r], q_len_host[r])) {
+                dec_rows += (double)q_len_host[r] * shape->n_kv_heads;
                 for (int i = 0; i < q_len_host[r]; ++i)
                     dec_bytes += ((double)prior_host[r] + i + 1.0) * 2.0 * shape->n_kv_heads * shape->head_dim * 2.0;
             } else {
@@ -786,7 +791,9 @@ ps_status ps_attn_plan(const ps_shape* shape, const int32_t* prior_host, const i
                 pl->dec_sms = best_n;
                 pl->pf_sms = pl->num_sms - best_n;
                 pl->concurrent = true;
-                pl->decode_last = t_dec(best_n) - t_pf(best_n) >= kMergeUnderDecodeSec;
+                const double rows_per_warp = dec_rows / (best_n * decode_unit_warps(shape->head_dim, 2));
+                const double warp_sec = kRowSec * rows_per_warp + kSegmentSec * std::max(0.0, 1 / rows_per_warp - 1);
+                pl->decode_last = t_dec(best_n) + warp_sec - t_pf(best_n) >= kMergeUnderDecodeSec;
             }
         }
         pl->pf_workers = std::max(1, pl->pf_sms / prefill_model(pl->shape, pl->pairs).sms_per_worker);
@@ -1085,7 +1092,7 @@ ps_status ps_attn_run(ps_plan* pl, const ps_kv* kv, const void* q_dev, const int
         // waiting for its end only at its own, and the merge kernel behind both.  (A second stream costs two events, which take
         // some 3 us each between kernels: tiny mixed batch 22.5 -> 16.8 us, with the list as parameters; 32 rows of 2048 tokens
         // beside a 512-token chunk 58.1 -> 57.2.)  On a second stream the merge kernel runs while the decode kernel still does: worth
-        // more where that one ends last by 3 us and more (60 rows of 2500 tokens and 300 on 5000 114.2 / 107.7, 150 of 1500 and 300 on 5000
+        // more where that one ends last by 2.5 us and more (60 rows of 2500 tokens and 300 on 5000 114.2 / 107.7, 150 of 1500 and 300 on 5000
         // at 8 q / 2 kv heads 52.3 / 49.1, at head dimension 64 88.1 / 83.8; 58 batches 2 to 8 %), less where it does not (3 rows and 300 on
         // 5000 30.9 / 34.7, at head dimension 64 24.7 / 28.7; 200 batches up to 20 %).  Helpers have to start as soon as the decode kernel
         // ends, so batches with a queue keep the second stream.  So do runs that record events: one between the two launches would hold
